@@ -158,8 +158,8 @@ fsi_status fsi_jacobian_apply(fsi_mesh *mesh, fsi_prec prec, const void *U, cons
  * bitwise those of the two separate calls under the same brick schedule (the
  * element-to-node sums follow the bricks); in FSI_F64 and FSI_F32 they agree
  * with them to rounding (the compiler may contract differently).  The brick
- * schedule is op 2 of fsi_mesh_set_brick / fsi_mesh_autotune (default 8x4x4
- * elements, 256 threads: the pass needs twice the shared memory per brick).  On a
+ * schedule is op 2 of fsi_mesh_set_brick / fsi_mesh_autotune (by default one
+ * that fits the grid's size; the pass needs twice the shared memory per brick).  On a
  * tetrahedral mesh the two operators run one after the other.  Neither
  * output may alias an input or the other output.                          */
 fsi_status fsi_residual_jacobian_apply(fsi_mesh *mesh, fsi_prec prec, const void *U,
@@ -771,7 +771,7 @@ enum {
 /* Build a batch (descriptors, prefix sums and its own scratch) on `cuda_stream`.
  * All meshes must be on one device and uniform (no fsi_mesh_set_coordinates;
  * FSI_ERR_ARG otherwise).  The batch uses one brick shape for all instances
- * (default 8x8x4; see fsi_batch_autotune).                                 */
+ * (by default one that fits the instances' sizes; see fsi_batch_autotune).  */
 fsi_status fsi_batch_create(fsi_mesh *const *meshes, const fsi_batch_item *items, int count,
                             fsi_prec prec, void *cuda_stream, fsi_batch **out);
 void fsi_batch_destroy(fsi_batch *batch);
@@ -802,9 +802,11 @@ fsi_status fsi_batch_autotune(fsi_batch *batch, int reps, fsi_tune_report *repor
 
 /* Brick schedule of a single mesh for op 0 (residual), 1 (Jacobian) or 2
  * (both fused; twice the shared memory) in compute type
- * `prec` (FSI_F64, FSI_F32 or FSI_DF64, each its own): bx*by*bz elements per CTA of `threads` threads (8 lanes per element;
- * threads a multiple of 32 and at most 256; bx*by*bz*8 >= threads not
- * required).  Scratch grows as needed.                                     */
+ * `prec` (FSI_F64, FSI_F32 or FSI_DF64, each its own): bx*by columns of bz elements per CTA of `threads` threads (4 lanes
+ * per column; threads a multiple of 32 and at most 256).  A brick wider than the
+ * CTA has lanes for, or than its shared memory holds, is halved along its longest
+ * side until it fits; CTAs larger than 128 threads are not used.  Scratch grows
+ * as needed.  Without this call the library picks a schedule from the grid's size. */
 fsi_status fsi_mesh_set_brick(fsi_mesh *mesh, int op, fsi_prec prec, int bx, int by, int bz,
                               int threads);
 

@@ -53,17 +53,17 @@ __device__ __forceinline__ int find_instance(const int64_t *prefix, int count, i
     return lo;
 }
 
-template <typename T, bool JAC>
-__global__ void __launch_bounds__(256) batch_brick_kernel(const vmsd::VmsArgs<T> *desc,
+// residual and Jacobian apply of every instance in one pass
+template <typename T>
+__global__ void __launch_bounds__(vmsd::kBrickThreads, sizeof(T) == 4 ? 4 : 2) batch_brick_kernel(const vmsd::VmsArgs<T> *desc,
                                                           const int64_t *prefix, int count)
 {
     extern __shared__ __align__(32) unsigned char smem_raw[];
-    auto *rel = reinterpret_cast<vec4<T> *>(smem_raw);
     const int64_t total = prefix[count];
     for (int64_t item = blockIdx.x; item < total; item += gridDim.x) {
         const int inst = find_instance(prefix, count, item);
-        vmsd::brick_body<T, JAC>(desc[inst], (int)(item - prefix[inst]), rel);
-        __syncthreads();  // rel is reused by the next brick
+        vmsd::brick_body<T, true, false, true>(desc[inst], (int)(item - prefix[inst]), smem_raw);
+        __syncthreads();  // the shared memory is reused by the next brick
     }
 }
 
@@ -74,9 +74,8 @@ __global__ void batch_gather_kernel(const vmsd::VmsArgs<T> *desc, const int64_t 
     for (int64_t item = blockIdx.x; item < total; item += gridDim.x) {
         const int inst = find_instance(prefix, count, item);
         const vmsd::VmsArgs<T> &P = desc[inst];
-        const int n = (P.Nx + 1) * (P.Ny + 1) * (P.Nz + 1);
-        const int64_t node = (item - prefix[inst]) * kChunk + threadIdx.x;
-        if (node < n) vmsd::gather_node(P, (int)node);
+        const int q = (int)(item - prefix[inst]) * kChunk + threadIdx.x;
+        if (q < (int)vmsd::shared_nodes(P)) vmsd::gather_shared<T, true>(P, q);
     }
 }
 
@@ -301,9 +300,9 @@ struct fsi_batch {
     int ctas_per_sm;
     int sms;
     // device data
-    void *desc_res, *desc_jac, *desc_dlm;                      // descriptors
+    void *desc_vms, *desc_dlm;                                 // descriptors
     // [kRows][count+1]: bricks, node chunks, point chunks, spreading cell items,
-    // counter chunks (E+1 cells), scan tiles
+    // counter chunks (E+1 cells), scan tiles, chunks of shared nodes
     int64_t *prefix;
     void *blocks;
     size_t blocks_bytes;
@@ -317,7 +316,7 @@ struct fsi_batch {
     double *xi64;
     size_t xi64_bytes;
     bool locate;
-    int64_t totals[6];
+    int64_t totals[7];
     // CUDA graph of one batched step
     cudaGraph_t graph;
     cudaGraphExec_t graph_exec;
@@ -326,13 +325,14 @@ struct fsi_batch {
 namespace fsi {
 namespace {
 
-constexpr int kRows = 6;
+constexpr int kRows = 7;
 
 // (Re)build descriptors and scratch for the batch's current brick shape.
 template <typename T> fsi_status build_batch(fsi_batch *b)
 {
     const int C = b->count;
-    std::vector<vmsd::VmsArgs<T>> res(C), jac(C);
+    std::vector<vmsd::VmsArgs<T>> vms(C);
+    const Brick brick = vmsd::fit_brick(b->brick, (int)sizeof(T), true, true);
     std::vector<DlmDesc<T>> dlm(C);
     std::vector<int64_t> pre(kRows * (C + 1), 0);
     size_t blocks_need = 0, spread_need = 0, loc_need = 0, xi64_need = 0;
@@ -340,7 +340,7 @@ template <typename T> fsi_status build_batch(fsi_batch *b)
     for (int i = 0; i < C; ++i) {
         fsi_mesh *m = b->meshes[i];
         boff[i] = blocks_need;
-        blocks_need += vms_scratch_bytes_for(m, b->brick, sizeof(T));
+        blocks_need += vms_scratch_bytes_for(m, brick, 2 * sizeof(T));
         blocks_need = (blocks_need + 255) / 256 * 256;
         soff[i] = spread_need;
         spread_need += (size_t)m->n_elems * 24 * sizeof(T);
@@ -385,9 +385,10 @@ template <typename T> fsi_status build_batch(fsi_batch *b)
     for (int i = 0; i < C; ++i) {
         fsi_mesh *m = b->meshes[i];
         const fsi_batch_item &it = b->items[i];
-        res[i] = vmsd::make_args<T>(m, b->brick, it.U, it.A, it.f, nullptr, it.R);
-        jac[i] = vmsd::make_args<T>(m, b->brick, it.U, it.A, it.f, it.x, it.Jx);
-        res[i].blocks = jac[i].blocks = (vec4<T> *)((char *)b->blocks + boff[i]);
+        vms[i] = vmsd::make_args<T>(m, brick, it.U, it.A, it.f, it.x, it.Jx);
+        vms[i].blocks = (vec4<T> *)((char *)b->blocks + boff[i]);
+        vms[i].blocks2 = vms[i].blocks + vms_scratch_bytes_for(m, brick, sizeof(T)) / sizeof(vec4<T>);
+        vms[i].out2 = (vec4<T> *)it.R;
         DlmDesc<T> &D = dlm[i];
         D.g.Nx = m->grid.N[0];
         D.g.Ny = m->grid.N[1];
@@ -422,7 +423,7 @@ template <typename T> fsi_status build_batch(fsi_batch *b)
         } else {
             D.pairs = nullptr;
         }
-        const int64_t nb = (int64_t)res[i].nbx * res[i].nby * res[i].nbz;
+        const int64_t nb = (int64_t)vms[i].nbx * vms[i].nby * vms[i].nbz;
         pre[0 * (C + 1) + i + 1] = pre[0 * (C + 1) + i] + nb;
         pre[1 * (C + 1) + i + 1] = pre[1 * (C + 1) + i] + (m->n_nodes + kChunk - 1) / kChunk;
         pre[2 * (C + 1) + i + 1] = pre[2 * (C + 1) + i] + (it.m + kChunk - 1) / kChunk;
@@ -432,12 +433,13 @@ template <typename T> fsi_status build_batch(fsi_batch *b)
         const int64_t cells = it.X ? (m->n_elems + 1 + kChunk - 1) / kChunk : 0;
         pre[4 * (C + 1) + i + 1] = pre[4 * (C + 1) + i] + cells;
         pre[5 * (C + 1) + i + 1] = pre[5 * (C + 1) + i] + (it.X ? D.ntiles : 0);
+        pre[6 * (C + 1) + i + 1] =
+            pre[6 * (C + 1) + i] +
+            (vmsd::shared_nodes(vms[i]) + kChunk - 1) / kChunk;
     }
     for (int k = 0; k < kRows; ++k) b->totals[k] = pre[k * (C + 1) + C];
     cudaStream_t s = b->stream;
-    FSI_CUDA(cudaMemcpyAsync(b->desc_res, res.data(), C * sizeof(res[0]), cudaMemcpyHostToDevice, s),
-             "descriptor upload");
-    FSI_CUDA(cudaMemcpyAsync(b->desc_jac, jac.data(), C * sizeof(jac[0]), cudaMemcpyHostToDevice, s),
+    FSI_CUDA(cudaMemcpyAsync(b->desc_vms, vms.data(), C * sizeof(vms[0]), cudaMemcpyHostToDevice, s),
              "descriptor upload");
     FSI_CUDA(cudaMemcpyAsync(b->desc_dlm, dlm.data(), C * sizeof(dlm[0]), cudaMemcpyHostToDevice, s),
              "descriptor upload");
@@ -456,13 +458,18 @@ template <typename T> fsi_status build_batch(fsi_batch *b)
     return FSI_OK;
 }
 
-// phases of a batched step: 1 residual, 2 Jacobian apply, 4 interpolation and
-// spreading, 8 location and cell table (instances with raw points)
-constexpr int kAllPhases = 15;
+// phases of a batched step: 1 residual and Jacobian apply (one pass), 4
+// interpolation and spreading, 8 location and cell table (instances with raw
+// points)
+constexpr int kAllPhases = 13;
 
-int persistent_grid(const fsi_batch *b, int64_t items)
+// persistent grid of the VMS pass: ctas CTAs per SM (the autotuner's choice);
+// of the others, whose 256-thread CTAs are bound by the latency of their
+// gathers: as many as an SM holds
+constexpr int kPointCtas = 8;
+int persistent_grid(const fsi_batch *b, int64_t items, int ctas = kPointCtas)
 {
-    int64_t g = (int64_t)b->sms * b->ctas_per_sm;
+    int64_t g = (int64_t)b->sms * ctas;
     if (items < g) g = items;
     return (int)(g < 1 ? 1 : g);
 }
@@ -473,8 +480,6 @@ template <typename T> fsi_status run_batched(fsi_batch *b, int phases)
     cudaStream_t s = b->stream;
     const int C = b->count;
     const int64_t *pre = b->prefix;
-    const size_t smem = (size_t)vmsd::rel_records(b->brick.bx * b->brick.by * b->brick.bz) *
-                        sizeof(vec4<T>);
     if ((phases & 8) && b->locate) {
         const DlmDesc<T> *dd = (const DlmDesc<T> *)b->desc_dlm;
         batch_clear_kernel<T><<<persistent_grid(b, b->totals[4]), kChunk, 0, s>>>(
@@ -499,16 +504,14 @@ template <typename T> fsi_status run_batched(fsi_batch *b, int phases)
         FSI_TRY(check_launch("batched location kernels"));
     }
     if (phases & 1) {
-        batch_brick_kernel<T, false><<<persistent_grid(b, b->totals[0]), b->brick.threads, smem, s>>>(
-            (const vmsd::VmsArgs<T> *)b->desc_res, pre, C);
-        batch_gather_kernel<T><<<persistent_grid(b, b->totals[1]), kChunk, 0, s>>>(
-            (const vmsd::VmsArgs<T> *)b->desc_res, pre + (C + 1), C);
-    }
-    if (phases & 2) {
-        batch_brick_kernel<T, true><<<persistent_grid(b, b->totals[0]), b->brick.threads, smem, s>>>(
-            (const vmsd::VmsArgs<T> *)b->desc_jac, pre, C);
-        batch_gather_kernel<T><<<persistent_grid(b, b->totals[1]), kChunk, 0, s>>>(
-            (const vmsd::VmsArgs<T> *)b->desc_jac, pre + (C + 1), C);
+        const Brick k = vmsd::fit_brick(b->brick, (int)sizeof(T), true, true);
+        const size_t smem =
+            vmsd::brick_smem(k.bx, k.by, k.bz, k.threads, (int)sizeof(T), true, true);
+        batch_brick_kernel<T>
+            <<<persistent_grid(b, b->totals[0], b->ctas_per_sm), k.threads, smem, s>>>(
+                (const vmsd::VmsArgs<T> *)b->desc_vms, pre, C);
+        batch_gather_kernel<T><<<persistent_grid(b, b->totals[6]), kChunk, 0, s>>>(
+            (const vmsd::VmsArgs<T> *)b->desc_vms, pre + 6 * (C + 1), C);
     }
     if (phases & 4) {
         if (b->totals[2] > 0)
@@ -529,8 +532,8 @@ fsi_status run_per_instance(fsi_batch *b, int phases)
         const fsi_batch_item &it = b->items[i];
         cudaStream_t saved = m->stream;
         m->stream = b->stream;
-        fsi::Brick bsaved[2] = {m->brick[0][b->prec], m->brick[1][b->prec]};
-        m->brick[0][b->prec] = m->brick[1][b->prec] = b->brick;
+        const fsi::Brick bsaved = m->brick[2][b->prec];
+        m->brick[2][b->prec] = b->brick;
         fsi_status st = FSI_OK;
         if ((phases & 8) && it.X) {
             // FP64 xi straight into the item, or through the batch's FP64
@@ -545,17 +548,15 @@ fsi_status run_per_instance(fsi_batch *b, int phases)
                 st = check_launch("xi rounding kernel");
             }
         }
-        if (st == FSI_OK && (phases & 1)) st = fsi_residual(m, b->prec, it.U, it.A, it.f, it.R);
-        if (st == FSI_OK && (phases & 2))
-            st = fsi_jacobian_apply(m, b->prec, it.U, it.A, it.f, it.x, it.Jx);
+        if (st == FSI_OK && (phases & 1))
+            st = fsi_residual_jacobian_apply(m, b->prec, it.U, it.A, it.f, it.x, it.R, it.Jx);
         if (st == FSI_OK && (phases & 4)) {
             st = fsi_dlm_interp(m, b->prec, it.m, it.elem, it.xi, it.U, it.u);
             if (st == FSI_OK)
                 st = fsi_dlm_spread(m, b->prec, it.m, it.elem, it.xi, it.cell_start, it.perm,
                                     it.lam, it.w, it.F, 0);
         }
-        m->brick[0][b->prec] = bsaved[0];
-        m->brick[1][b->prec] = bsaved[1];
+        m->brick[2][b->prec] = bsaved;
         m->stream = saved;
         FSI_TRY(st);
     }
@@ -564,15 +565,9 @@ fsi_status run_per_instance(fsi_batch *b, int phases)
 
 fsi_status set_smem_attr(fsi_prec prec)
 {
-    const int bytes = 200 * 1024;
-    if (prec == FSI_F64) {
-        FSI_TRY(set_smem_limit((const void *)batch_brick_kernel<double, false>, bytes));
-        FSI_TRY(set_smem_limit((const void *)batch_brick_kernel<double, true>, bytes));
-    } else {
-        FSI_TRY(set_smem_limit((const void *)batch_brick_kernel<float, false>, bytes));
-        FSI_TRY(set_smem_limit((const void *)batch_brick_kernel<float, true>, bytes));
-    }
-    return FSI_OK;
+    return prec == FSI_F64
+               ? set_smem_limit((const void *)batch_brick_kernel<double>, vmsd::kBrickSmemMax)
+               : set_smem_limit((const void *)batch_brick_kernel<float>, vmsd::kBrickSmemMax);
 }
 
 fsi_status run_mode(fsi_batch *b, int mode, int phases)
@@ -665,13 +660,16 @@ fsi_status fsi_batch_create(fsi_mesh *const *meshes, const fsi_batch_item *items
     b->meshes.assign(meshes, meshes + count);
     b->items.assign(items, items + count);
     for (int i = 0; i < count; ++i) b->locate = b->locate || items[i].X != nullptr;
-    b->brick = Brick{8, 8, 4, 256};
-    b->ctas_per_sm = 2;
+    b->ctas_per_sm = 4;
     cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, device);
+    {
+        std::vector<int32_t> N(3 * (size_t)count);
+        for (int i = 0; i < count; ++i) std::copy_n(meshes[i]->grid.N, 3, &N[3 * (size_t)i]);
+        b->brick = default_brick((const int32_t (*)[3])N.data(), count, prec, 2, b->sms);
+    }
     const size_t vsz = prec == FSI_F64 ? sizeof(vmsd::VmsArgs<double>) : sizeof(vmsd::VmsArgs<float>);
     const size_t dsz = prec == FSI_F64 ? sizeof(DlmDesc<double>) : sizeof(DlmDesc<float>);
-    fsi_status st = check_cuda(cudaMalloc(&b->desc_res, count * vsz), "descriptors");
-    if (st == FSI_OK) st = check_cuda(cudaMalloc(&b->desc_jac, count * vsz), "descriptors");
+    fsi_status st = check_cuda(cudaMalloc(&b->desc_vms, count * vsz), "descriptors");
     if (st == FSI_OK) st = check_cuda(cudaMalloc(&b->desc_dlm, count * dsz), "descriptors");
     if (st == FSI_OK)
         st = check_cuda(cudaMalloc(&b->prefix, kRows * (count + 1) * sizeof(int64_t)), "prefix");
@@ -691,8 +689,7 @@ void fsi_batch_destroy(fsi_batch *b)
     cudaStreamSynchronize(b->stream);
     if (b->graph_exec) cudaGraphExecDestroy(b->graph_exec);
     if (b->graph) cudaGraphDestroy(b->graph);
-    cudaFree(b->desc_res);
-    cudaFree(b->desc_jac);
+    cudaFree(b->desc_vms);
     cudaFree(b->desc_dlm);
     cudaFree(b->prefix);
     cudaFree(b->blocks);
@@ -728,7 +725,7 @@ fsi_status fsi_batch_autotune(fsi_batch *b, int reps, fsi_tune_report *rep)
             b->ctas_per_sm = ctas;
             FSI_TRY(b->prec == FSI_F64 ? build_batch<double>(b) : build_batch<float>(b));
             double t = 0.0;
-            FSI_TRY(time_mode(b, FSI_BATCH_PERSISTENT, 3, reps, &t));
+            FSI_TRY(time_mode(b, FSI_BATCH_PERSISTENT, 1, reps, &t));
             if (tried < FSI_TUNE_MAX_CANDIDATES) {
                 rep->cand_bx[tried] = cand.bx;
                 rep->cand_by[tried] = cand.by;

@@ -79,8 +79,13 @@ template <typename T> __device__ __forceinline__ void st4(vec4<T> *p, vec4<T> v)
 // ---------------------------------------------------------------- tuning
 struct Brick {
     int bx, by, bz;  // elements per CTA along each axis
-    int threads;     // CTA size (multiple of 32; 8 lanes per element)
+    int threads;     // CTA size (multiple of 32; 4 lanes per bx x by column)
 };
+
+// Default brick schedule of one VMS operator (op 0 residual, 1 Jacobian apply, 2
+// both) in compute type prec for `count` grids run together (one mesh, or a
+// batch's instances), on sms SMs (vms.cu)
+Brick default_brick(const int32_t (*N)[3], int count, int prec, int op, int sms);
 
 struct NewtonWorkspace;
 struct PressureMG;

@@ -1,5 +1,6 @@
 // runtime.cu -- handles, errors, validation and the generalized-alpha stage
 // kernel of libfsi (C ABI in include/fsi.h).
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 #include <set>
@@ -243,11 +244,10 @@ fsi_status fsi_mesh_create(const fsi_grid *grid, const fsi_physics *phys, int de
     m->n_nodes = n;
     m->n_elems = E;
     derive(m);
-    // the fused pass keeps two element buffers in shared memory: half as many
-    // elements per brick keeps two CTAs per SM
     for (int op = 0; op < 3; ++op)
         for (int p = 0; p < 3; ++p)
-            m->brick[op][p] = op == 2 ? Brick{8, 4, 4, 256} : Brick{8, 8, 4, 256};
+            m->brick[op][p] = op == 1 ? m->brick[0][p]  // the residual's rule too
+                                      : default_brick(&m->grid.N, 1, p, op, sm_count());
     fsi_status st = FSI_OK;
     // cell-hash scratch: fill counters [E+1], scan scratch, counters; both
     // start at zero and every cell-table build leaves them so
@@ -264,7 +264,18 @@ fsi_status fsi_mesh_create(const fsi_grid *grid, const fsi_physics *phys, int de
     m->hash_clean = st == FSI_OK;
     if (st == FSI_OK)
         st = check_cuda(cudaMalloc(&m->dev_counters, 8 * sizeof(int64_t)), "counter scratch");
-    if (st == FSI_OK) st = ensure_vms_scratch(m, m->brick[1][0], sizeof(double));
+    if (st == FSI_OK) {
+        // node blocks of the default schedules, in one allocation
+        size_t need = 0;
+        for (int op = 0; op < 3; ++op)
+            for (int p = 0; p < 3; ++p)
+                need = std::max(need, vms_scratch_bytes_for(m, m->brick[op][p],
+                                                            (op == 2 ? 2 : 1) *
+                                                                (p == FSI_F32 ? sizeof(float)
+                                                                              : sizeof(double))));
+        st = check_cuda(cudaMalloc(&m->vms_scratch, need), "VMS scratch allocation");
+        if (st == FSI_OK) m->vms_scratch_bytes = need;
+    }
     if (st == FSI_OK) st = ensure_spread_scratch(m, (size_t)E * 24 * sizeof(double));
     if (st != FSI_OK) {
         fsi_mesh_destroy(m);

@@ -3,22 +3,21 @@
 // al. 2007).
 //
 // Layout of the work:
-//   * One CTA per brick of bx*by*bz elements.  Eight consecutive lanes own one
-//     element; lane g (bits gx, gy, gz) is first "node a = g" (it loads that
-//     node's record) and then "Gauss point g".  On the uniform grid the Q1
-//     basis is a tensor product of 1D linear functions, so the values and
-//     gradients at the 2x2x2 Gauss points follow from the nodal values by
-//     three butterfly stages over the lane bits (shfl.xor 1, 2, 4), and the
-//     test-function projection is the transposed butterfly.  No shape-function
-//     tables, no smem bank traffic for evaluation.
-//   * After the projection lane g holds the element's contribution to its
-//     local node g.  Contributions go to shared memory per element; after the
-//     brick is done every node of the brick's node block sums its (<= 8)
-//     element contributions in a fixed corner order (no atomics).
-//   * Bricks share the nodes on their faces, so each brick writes its whole
-//     node block to scratch, and a second kernel sums, for every node, the
-//     blocks that contain it in a fixed brick order.  The result is
-//     deterministic (bitwise reproducible) and atomic-free.
+//   * One CTA per brick of bx*by columns of bz elements, four lanes per column.
+//     A lane is first a node of the column's current plane, then the two Gauss
+//     points above it.  On the uniform grid the Q1 basis is a tensor product of
+//     1D linear functions: the x and y stages of the evaluation are butterflies
+//     over two lane bits, once per node plane; the z stage stays in the lane; the
+//     test-function projection is the transposed sequence, with the upper plane's
+//     part carried to the next element (brick_body in vms_device.cuh).
+//   * Contributions go to shared memory per column and plane; after the brick is
+//     done every node sums its (<= 4) columns' contributions in a fixed order (no
+//     atomics) and is written out, or, on a face between bricks, kept in the
+//     brick's node block.
+//   * A second kernel sums, for every node that several bricks share, the blocks
+//     that contain it in a fixed brick order.  The result is deterministic
+//     (bitwise reproducible) and atomic-free.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <type_traits>
@@ -32,21 +31,19 @@ namespace {
 
 using namespace vmsd;
 
-template <typename T, bool JAC, bool MAPPED, bool FUSED = false>
-__global__ void __launch_bounds__(256) vms_brick_kernel(const VmsArgs<T> P)
-{
-    extern __shared__ __align__(32) unsigned char smem_raw[];
-    brick_body<T, JAC, MAPPED, FUSED>(P, blockIdx.x, reinterpret_cast<vec4<T> *>(smem_raw));
-}
+// CTAs of 128 threads per SM that the registers are held to.  FP32: 4 (128
+// registers; 3 or 5 were within 1 %).  FP64: 2, since 8 warps keep its pipe busy
+// (85 % active) and no value has to be spilled.  Double-float: 3 (168 registers),
+// both operators at once 2 (254; at 3 it spills and takes 420 instead of 406 us at
+// 64^3).  On mapped grids FP32 spills a little at 4 and is still faster than at 3.
+template <typename T, bool FUSED>
+constexpr int kBrickCtas = sizeof(T) == 4 ? 4 : (std::is_same<T, double>::value || FUSED ? 2 : 3);
 
-// The same, held to 128 registers (two 256-thread CTAs per SM): used for the
-// mapped double-float kernels, whose Jacobian otherwise takes more registers
-// and runs 1.2x slower at one CTA per SM.
 template <typename T, bool JAC, bool MAPPED, bool FUSED = false>
-__global__ void __launch_bounds__(256, 2) vms_brick_kernel_capped(const VmsArgs<T> P)
+__global__ void __launch_bounds__(kBrickThreads, (kBrickCtas<T, FUSED>)) vms_brick_kernel(const VmsArgs<T> P)
 {
     extern __shared__ __align__(32) unsigned char smem_raw[];
-    brick_body<T, JAC, MAPPED, FUSED>(P, blockIdx.x, reinterpret_cast<vec4<T> *>(smem_raw));
+    brick_body<T, JAC, MAPPED, FUSED>(P, blockIdx.x, smem_raw);
 }
 
 // Geometry table of a mapped grid: 8 lanes per element (lane = node, then
@@ -115,12 +112,11 @@ template <typename T> fsi_status ensure_map_geo(fsi_mesh *m, const VmsArgs<T> &P
     return check_launch("mapped geometry kernel");
 }
 
-template <typename T, bool FUSED = false> __global__ void vms_gather_kernel(const VmsArgs<T> P)
+template <typename T, bool FUSED = false>
+__global__ void __launch_bounds__(256) vms_gather_kernel(const VmsArgs<T> P, int n)
 {
-    const int n = (P.Nx + 1) * (P.Ny + 1) * (P.Nz + 1);
-    for (int node = blockIdx.x * blockDim.x + threadIdx.x; node < n;
-         node += gridDim.x * blockDim.x)
-        gather_node<T, FUSED>(P, node);
+    const int q = blockIdx.x * 256 + threadIdx.x;
+    if (q < n) gather_shared<T, FUSED>(P, q);
 }
 
 // FUSED: the residual (R) and the Jacobian apply (out) at the same state in
@@ -131,7 +127,8 @@ fsi_status launch_geo(fsi_mesh *m, const void *U, const void *A, const void *f, 
                       void *out, void *R = nullptr)
 {
     using S = typename StorageOf<T>::type;
-    const Brick &b = m->brick[FUSED ? 2 : (JAC ? 1 : 0)][prec_slot<T>()];
+    const Brick b = fit_brick(m->brick[FUSED ? 2 : (JAC ? 1 : 0)][prec_slot<T>()],
+                              (int)sizeof(T), JAC, FUSED);
     FSI_TRY(ensure_vms_scratch(m, b, (FUSED ? 2 : 1) * sizeof(T)));
     VmsArgs<T> P = make_args<T>(m, b, U, A, f, x, out);
     if constexpr (MAPPED) {
@@ -143,19 +140,15 @@ fsi_status launch_geo(fsi_mesh *m, const void *U, const void *A, const void *f, 
         P.blocks2 = P.blocks + (size_t)nbricks * (b.bx + 1) * (b.by + 1) * (b.bz + 1);
         P.out2 = (vec4<S> *)R;
     }
-    const size_t smem = (FUSED ? 2 : 1) * (size_t)vmsd::rel_records(b.bx * b.by * b.bz) * sizeof(vec4<S>);
-    void (*kernel)(const VmsArgs<T>);
-    if constexpr (MAPPED && std::is_same<T, df64>::value)
-        kernel = vms_brick_kernel_capped<T, JAC, MAPPED, FUSED>;
-    else
-        kernel = vms_brick_kernel<T, JAC, MAPPED, FUSED>;
-    FSI_TRY(set_smem_limit((const void *)kernel, 200 * 1024));
+    const size_t smem = brick_smem(b.bx, b.by, b.bz, b.threads, (int)sizeof(T), JAC, FUSED);
+    void (*kernel)(const VmsArgs<T>) = vms_brick_kernel<T, JAC, MAPPED, FUSED>;
+    FSI_TRY(set_smem_limit((const void *)kernel, kBrickSmemMax));
     kernel<<<nbricks, b.threads, smem, m->stream>>>(P);
     FSI_TRY(check_launch("vms brick kernel"));
-    const int threads = 256;
-    int64_t nb = (m->n_nodes + threads - 1) / threads;
-    if (nb > sm_count() * 32) nb = sm_count() * 32;
-    vms_gather_kernel<T, FUSED><<<(int)nb, threads, 0, m->stream>>>(P);
+    const int64_t shared = shared_nodes(P);
+    if (shared == 0) return FSI_OK;
+    vms_gather_kernel<T, FUSED>
+        <<<(int)((shared + 255) / 256), 256, 0, m->stream>>>(P, (int)shared);
     return check_launch("vms gather kernel");
 }
 
@@ -177,9 +170,52 @@ fsi_status launch_fused(fsi_mesh *m, const void *U, const void *A, const void *f
     return launch_geo<T, true, false, true>(m, U, A, f, x, Jx, R);
 }
 
-// candidate brick shapes of the single-mesh autotuner: the default, smaller
-// bricks (more bricks per wave of resident CTAs on small grids), flatter and
-// longer ones, and 128-thread CTAs (more CTAs per SM)
+// Cost of a schedule in units of one warp's share of an element layer (8
+// columns): the warps' work over the SMs plus a quarter of one CTA's own
+// duration as the tail, but no less than one CTA alone takes.  `alone` is how much
+// longer a layer takes a warp that has an SM to itself than its share of a full
+// SM: measured on GB300, 24 us against 6.4 us (FP64, both operators), about
+// 10 : 1 in double-float and 16 : 1 in FP32.  A brick of bz layers spends 0.3 of a
+// layer more (its lowest plane, the carried parts), and its rim nodes go through
+// the node blocks.
+double brick_cost(const int32_t (*N)[3], int count, const Brick &b, double alone, int sms)
+{
+    const double layer = b.bz + 0.3;
+    const double rim = 1.0 + 0.06 * ((b.bx + 1.0) * (b.by + 1.0) / (b.bx * b.by) - 1.0);
+    double ctas = 0.0;
+    for (int i = 0; i < count; ++i)
+        ctas += (double)((N[i][0] + b.bx - 1) / b.bx) * ((N[i][1] + b.by - 1) / b.by) *
+                ((N[i][2] + b.bz - 1) / b.bz);
+    const double work = ctas / sms * (b.threads / 32) * layer * rim;
+    return std::max(work + 0.25 * alone * layer, alone * layer) + 0.01 * work;
+}
+
+}  // namespace
+
+Brick default_brick(const int32_t (*N)[3], int count, int prec, int op, int sms)
+{
+    const double alone = prec == FSI_F64 ? 4.0 : (prec == FSI_DF64 ? 10.0 : 16.0);
+    // both operators in an 8-byte type: taller bricks leave one CTA per SM
+    const int max_bz = op == 2 && prec != FSI_F32 ? 4 : 8;
+    Brick best{8, 4, max_bz, 128};
+    double cost = 1e300;
+    for (int bz = max_bz; bz >= 1; --bz)
+        for (int by = 1; by <= 16; ++by)
+            for (int bx = 1; bx * by <= 32 && bx <= 16; ++bx) {
+                const Brick b{bx, by, bz, (4 * bx * by + 31) / 32 * 32};
+                const double c = brick_cost(N, count, b, alone, sms);
+                if (c < cost * (1.0 - 1e-9)) {
+                    cost = c;
+                    best = b;
+                }
+            }
+    return best;
+}
+
+namespace {
+
+// candidate brick shapes of the single-mesh autotuner (fit_brick halves the ones
+// wider than a CTA has lanes for)
 const Brick kMeshBricks[] = {
     {8, 8, 4, 256}, {8, 4, 4, 256}, {8, 8, 2, 256}, {4, 4, 4, 256}, {4, 4, 8, 256},
     {16, 4, 4, 256}, {8, 4, 4, 128}, {4, 4, 4, 128}, {8, 4, 2, 128}, {4, 4, 2, 128},

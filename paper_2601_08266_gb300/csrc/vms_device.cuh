@@ -71,7 +71,8 @@ template <typename T> struct VmsArgs {
     T rho, mu, inv_rho;
     T G0, G1, G2, inv_trG, q0;  // q0 = C_T/dt^2 + C_I (mu/rho)^2 G:G
     T ih0, ih1, ih2;            // 1/h_k
-    T detJ;
+    T detJ, rdetJ;              // det J and rho det J of the uniform grid
+    T nu, nu2;                  // mu / rho and twice that
     T c_a, c_v;                 // d A / d y_v, d U / d y_v
     T c_av;                     // c_a / c_v
     T ct_dt2, CInu2;            // C_T/dt^2 and C_I (mu/rho)^2 (mapped grids: G per Gauss point)
@@ -226,24 +227,6 @@ template <typename T> __device__ __forceinline__ T eval_v_body(T u)
     return dot2_t(b1, t, b2, shx(t, 4));
 }
 
-// Transposed evaluation: with X the value coefficient and (Yx, Yy, Yz) the
-// gradient coefficients of one residual component at this lane's Gauss point,
-// returns sum_g [N_a(g) X(g) + grad N_a(g) . Y(g)] for the lane's node a.
-template <typename T>
-__device__ __forceinline__ T project_body(T X, T Yx, T Yy, T Yz, T sx, T sy, T sz)
-{
-    const T b1 = cB1<T>(), b2 = cB2<T>();
-    T Xo = shx(X, 4), Yzo = shx(Yz, 4), Yxo = shx(Yx, 4), Yyo = shx(Yy, 4);
-    T P1 = fma_t(sz, Yz + Yzo, dot2_t(b1, X, b2, Xo));
-    T P2 = dot2_t(b1, Yx, b2, Yxo);
-    T P3 = dot2_t(b1, Yy, b2, Yyo);
-    T P1o = shx(P1, 2), P2o = shx(P2, 2), P3o = shx(P3, 2);
-    T Q1 = fma_t(sy, P3 + P3o, dot2_t(b1, P1, b2, P1o));
-    T Q2 = dot2_t(b1, P2, b2, P2o);
-    T Q1o = shx(Q1, 1), Q2o = shx(Q2, 1);
-    return fma_t(sx, Q2 + Q2o, dot2_t(b1, Q1, b2, Q1o));
-}
-
 // Evaluation and projection entry points.  With OUT set, double-float calls
 // one out-of-line copy of each body instead of inlining it: inlined at all 8 +
 // 4 + 4 call sites the double-float Jacobian body outgrows what the
@@ -256,11 +239,6 @@ template <typename T> __device__ __noinline__ VG<T> eval_vg_ool(T u, T sx, T sy,
     return eval_vg_body(u, sx, sy, sz);
 }
 template <typename T> __device__ __noinline__ T eval_v_ool(T u) { return eval_v_body(u); }
-template <typename T>
-__device__ __noinline__ T project_ool(T X, T Yx, T Yy, T Yz, T sx, T sy, T sz)
-{
-    return project_body(X, Yx, Yy, Yz, sx, sy, sz);
-}
 // which compute types take the out-of-line copies when OUT is set
 template <typename T>
 constexpr bool kOutline = std::is_same<T, df64>::value || std::is_same<T, df64x2>::value;
@@ -279,15 +257,6 @@ template <bool OUT, typename T> __device__ __forceinline__ T eval_v(T u)
     else
         return eval_v_body(u);
 }
-template <bool OUT, typename T>
-__device__ __forceinline__ T project(T X, T Yx, T Yy, T Yz, T sx, T sy, T sz)
-{
-    if constexpr (OUT && kOutline<T>)
-        return project_ool(X, Yx, Yy, Yz, sx, sy, sz);
-    else
-        return project_body(X, Yx, Yy, Yz, sx, sy, sz);
-}
-
 // Four fields of a node record evaluated as two pairs (x, y) and (z, w):
 // float and double-float pairs run on the paired FP32 instructions (3-7 %
 // faster VMS kernels); double has no paired form and evaluates field by field.
@@ -324,24 +293,6 @@ template <bool OUT, typename T> __device__ __forceinline__ void eval_v2(T u, T w
     const auto r = eval_v<OUT>(PO::pack(u, w));
     ru = PO::first(r);
     rw = PO::second(r);
-}
-
-// projections of two residual components
-template <bool OUT, typename T>
-__device__ __forceinline__ void project2(T X0, const T (&Y0)[3], T X1, const T (&Y1)[3], T sx, T sy,
-                                         T sz, T &r0, T &r1)
-{
-    if constexpr (std::is_same<T, double>::value) {
-        r0 = project<OUT>(X0, Y0[0], Y0[1], Y0[2], sx, sy, sz);
-        r1 = project<OUT>(X1, Y1[0], Y1[1], Y1[2], sx, sy, sz);
-        return;
-    }
-    using PO = PairOf<T>;
-    const auto r = project<OUT>(PO::pack(X0, X1), PO::pack(Y0[0], Y1[0]), PO::pack(Y0[1], Y1[1]),
-                                PO::pack(Y0[2], Y1[2]), PO::pack(sx, sx), PO::pack(sy, sy),
-                                PO::pack(sz, sz));
-    r0 = PO::first(r);
-    r1 = PO::second(r);
 }
 
 template <typename T> __device__ __forceinline__ T inv_t(T v) { return T(1) / v; }
@@ -556,242 +507,702 @@ __device__ __forceinline__ void gp_jacobian_terms(const VmsArgs<T> &P, const GP<
     for (int j = 0; j < 3; ++j) Y[3][j] = -dup[j];
 }
 
-// One brick of elements: element contributions into rel (shared memory,
-// [bx*by*bz][8] node records), then the brick's node block into P.blocks.
-// FUSED (with JAC): the residual at the same Gauss-point state is projected
-// too, into rel + rel_records(bx*by*bz) and then P.blocks2; the evaluation of U and A
-// and the base state are shared by the two operators.
-// Element records in shared memory, corner-major with one padding record
-// per corner row: corner c of brick element `slot` at c (nel + 1) + slot.
-// The 8 lanes of an element then store to 8 different bank groups, and the
-// node sums read consecutive elements from consecutive threads (element-major
-// records, 8 apart, put a warp's 32 reads on the same banks: 8-way conflicts).
-__host__ __device__ __forceinline__ int rel_records(int nel) { return 8 * (nel + 1); }
-__device__ __forceinline__ int rel_at(int nel, int slot, int c) { return c * (nel + 1) + slot; }
+// ---------------------------------------------------------------- bricks
+// A brick is bx x by columns of bz elements; four lanes own a column and march
+// up its elements.  Lane (gx, gy) is first "node (gx, gy) of the plane" and
+// then "the two Gauss points above that corner" (gz = 0, 1), so
+//
+//   evaluation  the x and y stages of the butterfly run once per node plane
+//               (and serve the element below and the one above it), the z stage
+//               combines the two planes of an element in the lane's own
+//               registers, both Gauss points at once;
+//   algebra     both Gauss points of a lane as one pair: float and double-float
+//               on the paired FP32 instructions;
+//   projection  the transposed z stage leaves a lower and an upper part, the
+//               upper one is carried to the element above and added to its
+//               lower part, and the transposed y and x stages run once per plane.
+//
+// Against eight lanes per element (one per node and Gauss point, three shuffle
+// stages per field and element) this takes a quarter fewer floating-point
+// operations per Gauss point, a third of the shuffles and half of the node
+// loads.  Pressure and body force enter per unit of density (p/rho and a - f at
+// the nodes), rho and det J once per plane at the end.
+//
+// Bound: FP64 by its pipe (86 % active), FP32 by issue (70 %, FMA pipe 63 %),
+// double-float by the FP32 pipe and the latency of its dependent sequences.
+// Against eight lanes per element (GB300, brick and gather kernels, default
+// schedules): FP64 both operators at 64^3 2,073 -> 1,541 us; FP32 Jacobian apply
+// at 128^3 370 -> 228 us, residual 283 -> 177 us; double-float residual at 128^3
+// 1,524 -> 1,237 us, Jacobian apply 2,640 -> 2,230 us.  Tried and not kept: a
+// barrier and the node sums after every plane (less shared memory, taller
+// bricks) took the FP32 Jacobian apply from 296 to 376 us.
 
+// storage cell of a compute type in shared memory (double-float: one 8-byte pair)
+template <typename T> struct SmCell {
+    using type = T;
+};
+template <> struct SmCell<df64> {
+    using type = float2;
+};
+template <typename T> __device__ __forceinline__ T cell_ld(typename SmCell<T>::type v) { return v; }
+template <> __device__ __forceinline__ df64 cell_ld<df64>(float2 v) { return df64(v.x, v.y); }
+template <typename T> __device__ __forceinline__ typename SmCell<T>::type cell_st(T v) { return v; }
+template <> __device__ __forceinline__ float2 cell_st<df64>(df64 v) { return make_float2(v.hi, v.lo); }
+
+// Shared memory of a brick: rel[op][component][plane][corner][column], the
+// columns padded so that a warp's 8 columns x 4 corners fall on different
+// banks (4-byte cells: stride = 8 or 24 mod 32, 8-byte cells: 4 or 12 mod 16);
+// then, for the types whose lower plane and carried parts do not fit the
+// registers, lane[value][thread].
+__host__ __device__ __forceinline__ int rel_stride(int ncol, int cell)
+{
+    if (cell == 4) {
+        const int s = (ncol + 7) / 8 * 8;
+        return s % 16 == 8 ? s : s + 8;
+    }
+    const int s = (ncol + 3) / 4 * 4;
+    return s % 8 == 4 ? s : s + 4;
+}
+constexpr int kPlaneU = 16;  // plane values of U (4 x 3), A (3) and s
+constexpr int kPlaneX = 12;  // plane values of x (4 x 3)
+constexpr int kCarry = 12;   // carried values per operator (4 components x 3)
+constexpr int kAsyncRecs = 4;  // node records of U, A, x and f
+// 8-byte types: plane and carried values; float: two planes of node records
+__host__ __device__ __forceinline__ int lane_values(int cell, bool jac, bool fused)
+{
+    return cell == 4 ? 2 * kAsyncRecs * 4 : kPlaneU + (jac ? kPlaneX : 0) + kCarry * (fused ? 2 : 1);
+}
+__host__ __device__ __forceinline__ size_t brick_smem(int bx, int by, int bz, int threads, int cell,
+                                                      bool jac, bool fused)
+{
+    const size_t rel = (size_t)(fused ? 2 : 1) * 4 * (bz + 1) * 4 * rel_stride(bx * by, cell);
+    return cell * (rel + (size_t)lane_values(cell, jac, fused) * threads);
+}
+
+// x and y stages at one node plane: value and in-plane gradient (scaled by sx,
+// sy) above this lane's corner.  F: one field, or a pair of fields.
+template <typename F> struct Face {
+    F b, dx, dy;
+};
+template <typename F> __device__ __forceinline__ Face<F> face_body(F u, F sx, F sy)
+{
+    const F b1 = cB1<F>(), b2 = cB2<F>();
+    const F uo = shx(u, 1);
+    const F tB = dot2_t(b1, u, b2, uo), tD = u - uo;
+    const F tBo = shx(tB, 2), tDo = shx(tD, 2);
+    return {dot2_t(b1, tB, b2, tBo), sx * dot2_t(b1, tD, b2, tDo), sy * (tB - tBo)};
+}
+// native FP64 (one instruction per multiply, add or FMA alike): each
+// value-type output is one FMA on the difference the gradient needs anyway
+template <> __device__ __forceinline__ Face<double> face_body<double>(double u, double sx, double sy)
+{
+    const double b1 = kB1;
+    const double uo = shx(u, 1);
+    const double tD = u - uo, tB = fma(b1, tD, uo);
+    const double tBo = shx(tB, 2), tDo = shx(tD, 2);
+    const double d = tB - tBo;
+    return {fma(b1, d, tBo), sx * fma(b1, tD - tDo, tDo), sy * d};
+}
+template <typename F> __device__ __forceinline__ F face_v_body(F u)
+{
+    const F b1 = cB1<F>(), b2 = cB2<F>();
+    const F t = dot2_t(b1, u, b2, shx(u, 1));
+    return dot2_t(b1, t, b2, shx(t, 2));
+}
+// transposed y and x stages: node contributions from the accumulated z parts
+// (P1: value and z-gradient, P2 / P3: x- / y-gradient coefficients)
+template <typename F>
+__device__ __forceinline__ F face_project_body(F P1, F P2, F P3, F sx, F sy)
+{
+    const F b1 = cB1<F>(), b2 = cB2<F>();
+    const F P1o = shx(P1, 2), P2o = shx(P2, 2), P3o = shx(P3, 2);
+    const F Q1 = fma_t(sy, P3 + P3o, dot2_t(b1, P1, b2, P1o));
+    const F Q2 = dot2_t(b1, P2, b2, P2o);
+    const F Q1o = shx(Q1, 1), Q2o = shx(Q2, 1);
+    return fma_t(sx, Q2 + Q2o, dot2_t(b1, Q1, b2, Q1o));
+}
+// one out-of-line copy of each for double-float pairs (instruction cache)
+template <typename F> __device__ __noinline__ Face<F> face_ool(F u, F sx, F sy)
+{
+    return face_body(u, sx, sy);
+}
+template <typename F>
+__device__ __noinline__ F face_project_ool(F P1, F P2, F P3, F sx, F sy)
+{
+    return face_project_body(P1, P2, P3, sx, sy);
+}
+template <typename F> __device__ __forceinline__ Face<F> face(F u, F sx, F sy)
+{
+    if constexpr (kOutline<F>)
+        return face_ool(u, sx, sy);
+    else
+        return face_body(u, sx, sy);
+}
+template <typename F>
+__device__ __forceinline__ F face_project(F P1, F P2, F P3, F sx, F sy)
+{
+    if constexpr (kOutline<F>)
+        return face_project_ool(P1, P2, P3, sx, sy);
+    else
+        return face_project_body(P1, P2, P3, sx, sy);
+}
+
+// z stage: the two Gauss points between the plane values lo and hi
+template <typename T> __device__ __forceinline__ typename PairOf<T>::type z_val(T lo, T hi)
+{
+    const T d = hi - lo;
+    return PairOf<T>::pack(fma_t(cB2<T>(), d, lo), fma_t(cB1<T>(), d, lo));
+}
+template <> __device__ __forceinline__ df64x2 z_val<df64>(df64 lo, df64 hi)
+{
+    using PO = PairOf<df64>;
+    return pair_dot2(PO::pack(cB1<df64>(), cB2<df64>()), PO::pack(lo, lo),
+                     PO::pack(cB2<df64>(), cB1<df64>()), PO::pack(hi, hi));
+}
+// the same with the difference d = hi - lo at hand
+template <typename T> __device__ __forceinline__ typename PairOf<T>::type z_val_d(T lo, T hi, T d)
+{
+    (void)hi;
+    return PairOf<T>::pack(fma_t(cB2<T>(), d, lo), fma_t(cB1<T>(), d, lo));
+}
+template <> __device__ __forceinline__ df64x2 z_val_d<df64>(df64 lo, df64 hi, df64)
+{
+    return z_val(lo, hi);
+}
+
+// transposed z stage of one coefficient at the two Gauss points: tot = carry +
+// b1 X0 + b2 X1 goes to the lower plane, up = b2 X0 + b1 X1 to the upper one
+template <typename T>
+__device__ __forceinline__ void z_part(typename PairOf<T>::type X, T carry, T &tot, T &up)
+{
+    const T X0 = PairOf<T>::first(X), X1 = PairOf<T>::second(X);
+    const T d = X0 - X1;
+    tot = fma_t(cB1<T>(), d, carry + X1);
+    up = fma_t(-cB1<T>(), d, X0);
+}
+template <>
+__device__ __forceinline__ void z_part<df64>(df64x2 X, df64 carry, df64 &tot, df64 &up)
+{
+    using PO = PairOf<df64>;
+    const df64 X0 = PO::first(X), X1 = PO::second(X);
+    const df64x2 r = pair_dot2(PO::pack(cB1<df64>(), cB2<df64>()), PO::pack(X0, X0),
+                               PO::pack(cB2<df64>(), cB1<df64>()), PO::pack(X1, X1));
+    tot = carry + PO::first(r);
+    up = PO::second(r);
+}
+
+// 1/sqrt of both halves
+template <> __device__ __forceinline__ f32x2 rsqrt_t(f32x2 v)
+{
+    // hardware estimate and one Newton step: within an ulp, in a fifth of the
+    // instructions of an IEEE square root and division
+    const f32x2 y = {make_float2(rsqrtf(v.v.x), rsqrtf(v.v.y))};
+    const f32x2 one = {make_float2(1.0f, 1.0f)}, half = {make_float2(0.5f, 0.5f)};
+    const f32x2 t = v * y;
+    const f32x2 e = pair_fma({neg2(t.v)}, y, one);
+    return pair_fma(half * y, e, y);
+}
+template <> __device__ __forceinline__ pd rsqrt_t(pd v) { return {rsqrt(v.a), rsqrt(v.b)}; }
+template <> __device__ __forceinline__ df64x2 rsqrt_t(df64x2 x)
+{
+    // df_rsqrt on both halves
+    const df64x2 r = {make_float2(rsqrtf(x.hi.x), rsqrtf(x.hi.y)), make_float2(0.0f, 0.0f)};
+    const df64x2 one = {make_float2(1.0f, 1.0f), make_float2(0.0f, 0.0f)};
+    const df64x2 half = {make_float2(0.5f, 0.5f), make_float2(0.0f, 0.0f)};
+    const df64x2 corr = one - x * (r * r);
+    return r + r * (corr * half);
+}
+__device__ __forceinline__ pd operator-(pd x) { return {-x.a, -x.b}; }
+__device__ __forceinline__ f32x2 operator-(f32x2 x) { return {neg2(x.v)}; }
+
+// 16 bytes to shared memory asynchronously (zeros when !ok)
+__device__ __forceinline__ void cp_async16(void *dst, const void *src, bool ok)
+{
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(ok ? 16 : 0)
+                 : "memory");
+}
+
+// One brick: element contributions into rel (shared memory), then the node
+// sums: nodes inside the brick straight into P.out, nodes shared with a
+// neighbouring brick into the brick's node block in P.blocks (gather_node adds
+// those up).  FUSED (with JAC): the residual at the same Gauss-point state goes
+// to P.out2 / P.blocks2; the evaluation of U and A and the base state are
+// shared by the two operators.
 template <typename T, bool JAC, bool MAPPED = false, bool FUSED = false>
-__device__ __forceinline__ void brick_body(const VmsArgs<T> &P, int brick, vec4<T> *rel)
+__device__ __forceinline__ void brick_body(const VmsArgs<T> &P, int brick, unsigned char *smem)
 {
     static_assert(!FUSED || JAC, "the fused body computes the Jacobian apply too");
-    constexpr bool OUT = JAC;  // out-of-line double-float evaluation
-    const int g = threadIdx.x & 7;
+    using PO = PairOf<T>;
+    using C = typename PO::type;
+    using Cell = typename SmCell<T>::type;
+    using S = typename StorageOf<T>::type;
+    constexpr int kOps = FUSED ? 2 : 1;
+    constexpr bool kLaneSm = sizeof(T) == 8;
+    constexpr bool kAsync = sizeof(T) == 4;
+    const int tid = threadIdx.x, nthr = blockDim.x;
     const int bxi = brick % P.nbx, byi = (brick / P.nbx) % P.nby, bzi = brick / (P.nbx * P.nby);
     const int ex0 = bxi * P.bx, ey0 = byi * P.by, ez0 = bzi * P.bz;
-    const int nel = P.bx * P.by * P.bz;
-    const int groups = blockDim.x >> 3;
-    const int gx = g & 1, gy = (g >> 1) & 1, gz = (g >> 2) & 1;
+    const int ncol = P.bx * P.by, stride = rel_stride(ncol, (int)sizeof(T));
+    const int nl = min(P.bz, P.Nz - ez0);  // element layers of this brick
+    const int plane_cells = 4 * stride, comp_cells = (P.bz + 1) * plane_cells;
+    Cell *rel = reinterpret_cast<Cell *>(smem);
+    Cell *lane = rel + kOps * 4 * comp_cells + tid;
+    const int gx = tid & 1, gy = (tid >> 1) & 1;
     // gradient signs of the butterfly: physical (+-1/h) on the uniform grid,
     // reference (+-1/2 per unit of xi) on a mapped grid
     const T sx = MAPPED ? (gx ? T(0.5f) : T(-0.5f)) : (gx ? P.ih0 : -P.ih0);
     const T sy = MAPPED ? (gy ? T(0.5f) : T(-0.5f)) : (gy ? P.ih1 : -P.ih1);
-    const T sz = MAPPED ? (gz ? T(0.5f) : T(-0.5f)) : (gz ? P.ih2 : -P.ih2);
+    const T ihz = MAPPED ? T(0.5f) : P.ih2;
+    const C sx2 = PO::pack(sx, sx), sy2 = PO::pack(sy, sy);
+    const C nu = PO::pack(P.nu, P.nu), nu2 = PO::pack(P.nu2, P.nu2);
     const int NX1 = P.Nx + 1, NXY1 = (P.Nx + 1) * (P.Ny + 1);
+    // rho det J and det J of the momentum and continuity rows (mapped grids:
+    // det J per Gauss point)
+    const T scale_m = MAPPED ? P.rho : P.rdetJ, scale_c = MAPPED ? T(1) : P.detJ;
 
-    for (int base = 0; base < nel; base += groups) {
-        // the double-float body is long: a barrier per pass keeps the CTA's
-        // warps on the same stretch of it (instruction-cache locality; 3-5 %
-        // faster on GB300, a loss for the shorter float/double bodies)
-        if constexpr (std::is_same<T, df64>::value) __syncthreads();
-        const int slot = base + (threadIdx.x >> 3);
-        const int lx = slot % P.bx, ly = (slot / P.bx) % P.by, lz = slot / (P.bx * P.by);
-        const int ex = ex0 + lx, ey = ey0 + ly, ez = ez0 + lz;
-        const bool valid = slot < nel && ex < P.Nx && ey < P.Ny && ez < P.Nz;
-        const int node = valid ? (ex + gx) + NX1 * (ey + gy) + NXY1 * (ez + gz) : 0;
+    // plane values and carried parts: registers (float) or shared memory
+    T Lr[kLaneSm ? 1 : kPlaneU + (JAC ? kPlaneX : 0)];
+    T Cr[kLaneSm ? 1 : kCarry * kOps];
+    auto getL = [&](int q) -> T {
+        if constexpr (kLaneSm) return cell_ld<T>(lane[q * nthr]);
+        else return Lr[q];
+    };
+    auto setL = [&](int q, T v) {
+        if constexpr (kLaneSm) lane[q * nthr] = cell_st(v);
+        else Lr[q] = v;
+    };
+    constexpr int kC0 = kPlaneU + (JAC ? kPlaneX : 0);
+    auto getC = [&](int q) -> T {
+        if constexpr (kLaneSm) return cell_ld<T>(lane[(kC0 + q) * nthr]);
+        else return Cr[q];
+    };
+    auto setC = [&](int q, T v) {
+        if constexpr (kLaneSm) lane[(kC0 + q) * nthr] = cell_st(v);
+        else Cr[q] = v;
+    };
+
+    for (int base = 0; base < ncol; base += nthr >> 2) {
+        const int col = base + (tid >> 2);
+        const int lx = col % P.bx, ly = col / P.bx;
+        const int ex = ex0 + lx, ey = ey0 + ly;
+        const bool slot = col < ncol;
+        const bool valid = slot && ex < P.Nx && ey < P.Ny;
+        const int64_t node0 = valid ? (ex + gx) + (int64_t)NX1 * (ey + gy) + (int64_t)NXY1 * ez0 : 0;
         const vec4<T> zero = {T(0), T(0), T(0), T(0)};
-        vec4<T> u = valid ? load_c<T>(P.U + node) : zero;
-        vec4<T> ac = valid ? load_c<T>(P.A + node) : zero;
-        vec4<T> ff = (valid && P.f) ? load_c<T>(P.f + node) : zero;
-
-        Geo<T> geo;
-        if constexpr (MAPPED) {
-            // this lane's Gauss point from the geometry table; idle lanes
-            // take the identity (their result is discarded)
-            T gt[kMapGeo];
-            if (valid) {
-                const int64_t e = ex + (int64_t)P.Nx * (ey + (int64_t)P.Ny * ez);
-                const typename GeoStore<T>::type *gp = P.geo + e * (kMapGeo * 8) + g;
-#pragma unroll
-                for (int k = 0; k < kMapGeo; ++k) gt[k] = geo_ld<T>(gp + 8 * k);
+        // in-plane stages of the four fields of a record, of three or four values
+        auto faces4 = [&](const vec4<T> &u, Face<T> (&f)[4]) {
+            if constexpr (std::is_same<T, double>::value) {
+                f[0] = face(u.x, sx, sy);
+                f[1] = face(u.y, sx, sy);
+                f[2] = face(u.z, sx, sy);
+                f[3] = face(u.w, sx, sy);
             } else {
-#pragma unroll
-                for (int k = 0; k < kMapGeo; ++k) gt[k] = T(0);
-                gt[0] = gt[4] = gt[8] = gt[9] = gt[12] = gt[14] = gt[17] = T(1);
-                gt[15] = T(3);
-                gt[16] = T(1.0f / 3.0f);
+                const Face<C> a = face(PO::pack(u.x, u.y), sx2, sy2);
+                const Face<C> b = face(PO::pack(u.z, u.w), sx2, sy2);
+                f[0] = {PO::first(a.b), PO::first(a.dx), PO::first(a.dy)};
+                f[1] = {PO::second(a.b), PO::second(a.dx), PO::second(a.dy)};
+                f[2] = {PO::first(b.b), PO::first(b.dx), PO::first(b.dy)};
+                f[3] = {PO::second(b.b), PO::second(b.dx), PO::second(b.dy)};
             }
-            for (int i = 0; i < 3; ++i)
-                for (int j = 0; j < 3; ++j) geo.Ji[i][j] = gt[3 * i + j];
-            geo.G[0][0] = gt[9];
-            geo.G[0][1] = geo.G[1][0] = gt[10];
-            geo.G[0][2] = geo.G[2][0] = gt[11];
-            geo.G[1][1] = gt[12];
-            geo.G[1][2] = geo.G[2][1] = gt[13];
-            geo.G[2][2] = gt[14];
-            geo.q0 = P.ct_dt2 + P.CInu2 * gt[15];
-            geo.inv_trG = gt[16];
-            geo.det = gt[17];
-        }
-        GP<T> q;
+        };
+        auto faces_v = [&](const vec4<T> &a, T (&v)[4]) {
+            if constexpr (std::is_same<T, double>::value) {
+                v[0] = face_v_body(a.x);
+                v[1] = face_v_body(a.y);
+                v[2] = face_v_body(a.z);
+                v[3] = P.has_s ? face_v_body(a.w) : T(1);
+            } else {
+                const C p = face_v_body(PO::pack(a.x, a.y)), q = face_v_body(PO::pack(a.z, a.w));
+                v[0] = PO::first(p);
+                v[1] = PO::second(p);
+                v[2] = PO::first(q);
+                v[3] = PO::second(q);
+            }
+        };
+
+        // float: the node records of the next plane are on their way to shared
+        // memory (cp.async, each lane its own slots, no registers) while this
+        // plane's element layer is computed; its layers are short against the
+        // latency of the loads (Jacobian apply at 128^3: 290 us with plain loads,
+        // 239 us so; prefetching into registers gained nothing).  Idle lanes get
+        // zeros.
+        float4 *slot4 = reinterpret_cast<float4 *>(rel + kOps * 4 * comp_cells) + tid;
+        auto fetch = [&](int l) {
+            if constexpr (kAsync) {
+                if (l <= nl) {
+                    const int64_t nd = node0 + (valid ? (int64_t)NXY1 * l : 0);
+                    float4 *d = slot4 + (l & 1) * kAsyncRecs * nthr;
+                    cp_async16(d, P.U + nd, valid);
+                    cp_async16(d + nthr, P.A + nd, valid);
+                    if constexpr (JAC) cp_async16(d + 2 * nthr, P.x + nd, valid);
+                    if (P.f) cp_async16(d + 3 * nthr, P.f + nd, valid);
+                }
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            }
+        };
+        auto fetched = [&](int l, int r) {
+            const float4 v = slot4[((l & 1) * kAsyncRecs + r) * nthr];
+            return vec4<T>{T(v.x), T(v.y), T(v.z), T(v.w)};
+        };
+        // records of plane l: scaled to per-unit-density pressure, chain factor
+        auto load_u = [&](int l, int64_t nd) {
+            vec4<T> u;
+            if constexpr (kAsync) u = fetched(l, 0);
+            else u = valid ? load_c<T>(P.U + nd) : zero;
+            u.w = P.inv_rho * u.w;
+            return u;
+        };
+        auto load_a = [&](int l, int64_t nd) {
+            vec4<T> a, f;
+            if constexpr (kAsync) a = fetched(l, 1);
+            else a = valid ? load_c<T>(P.A + nd) : vec4<T>{T(0), T(0), T(0), T(1)};
+            if (P.f) {
+                if constexpr (kAsync) f = fetched(l, 3);
+                else f = valid ? load_c<T>(P.f + nd) : zero;
+                a.x = a.x - f.x;
+                a.y = a.y - f.y;
+                a.z = a.z - f.z;
+            }
+            return a;
+        };
+        auto load_x = [&](int l, int64_t nd) {
+            vec4<T> x;
+            if constexpr (kAsync) x = fetched(l, 2);
+            else x = valid ? load_c<T>(P.x + nd) : zero;
+            x.x = P.c_v * x.x;
+            x.y = P.c_v * x.y;
+            x.z = P.c_v * x.z;
+            x.w = P.inv_rho * x.w;
+            return x;
+        };
+        fetch(0);
+        fetch(1);
+        if constexpr (kAsync) asm volatile("cp.async.wait_group 1;" ::: "memory");
+
+        // ---- the lowest plane
         {
-            VG<T> e0, e1, e2, e3;
-            eval_vg4<OUT>(u, sx, sy, sz, e0, e1, e2, e3);
-            if constexpr (MAPPED) {
-                to_phys(geo, e0);
-                to_phys(geo, e1);
-                to_phys(geo, e2);
-                to_phys(geo, e3);
-            }
-            q.v[0] = e0.v; q.gv[0][0] = e0.gx; q.gv[0][1] = e0.gy; q.gv[0][2] = e0.gz;
-            q.v[1] = e1.v; q.gv[1][0] = e1.gx; q.gv[1][1] = e1.gy; q.gv[1][2] = e1.gz;
-            q.v[2] = e2.v; q.gv[2][0] = e2.gx; q.gv[2][1] = e2.gy; q.gv[2][2] = e2.gz;
-            q.p = e3.v; q.gp[0] = e3.gx; q.gp[1] = e3.gy; q.gp[2] = e3.gz;
-        }
-        eval_v2<OUT>(ac.x, ac.y, q.a[0], q.a[1]);
-        if constexpr (std::is_same<T, double>::value) {
-            q.a[2] = eval_v<OUT>(ac.z);
-            q.s = P.has_s ? eval_v<OUT>(ac.w) : T(1);
-        } else {  // the pair's second half is free
-            T sv;
-            eval_v2<OUT>(ac.z, ac.w, q.a[2], sv);
-            q.s = P.has_s ? sv : T(1);
-        }
-        if (P.f) {
-            eval_v2<OUT>(ff.x, ff.y, q.f[0], q.f[1]);
-            q.f[2] = eval_v<OUT>(ff.z);
-            for (int i = 0; i < 3; ++i) q.a[i] = q.a[i] - q.f[i];
-        } else {
-            q.f[0] = q.f[1] = q.f[2] = T(0);
-        }
-        if (!valid) q.s = T(1);  // keep tau finite on idle lanes
-        if constexpr (MAPPED)
-            base_state_g(P, geo, q);
-        else
-            base_state(P, q);
-
-        T X[4], Y[4][3];
-        if constexpr (FUSED) {
-            // the residual at this state, projected like the residual kernel's
-            gp_residual_terms(P, q, X, Y);
-            vec4<T> rr;
-            if constexpr (MAPPED) {
-                for (int c = 0; c < 4; ++c) {
-                    const T y0 = Y[c][0], y1 = Y[c][1], y2 = Y[c][2];
-                    Y[c][0] = geo.det * (geo.Ji[0][0] * y0 + geo.Ji[0][1] * y1 + geo.Ji[0][2] * y2);
-                    Y[c][1] = geo.det * (geo.Ji[1][0] * y0 + geo.Ji[1][1] * y1 + geo.Ji[1][2] * y2);
-                    Y[c][2] = geo.det * (geo.Ji[2][0] * y0 + geo.Ji[2][1] * y1 + geo.Ji[2][2] * y2);
-                    X[c] = geo.det * X[c];
-                }
-                project2<OUT>(X[0], Y[0], X[1], Y[1], sx, sy, sz, rr.x, rr.y);
-                project2<OUT>(X[2], Y[2], X[3], Y[3], sx, sy, sz, rr.z, rr.w);
-            } else {
-                project2<OUT>(X[0], Y[0], X[1], Y[1], sx, sy, sz, rr.x, rr.y);
-                project2<OUT>(X[2], Y[2], X[3], Y[3], sx, sy, sz, rr.z, rr.w);
-                rr.x = P.detJ * rr.x;
-                rr.y = P.detJ * rr.y;
-                rr.z = P.detJ * rr.z;
-                rr.w = P.detJ * rr.w;
-            }
-            if (slot < nel) rel[rel_records(nel) + rel_at(nel, slot, g)] = valid ? rr : zero;
-        }
-        if (!JAC) {
-            gp_residual_terms(P, q, X, Y);
-        } else {
-            vec4<T> xx = valid ? load_c<T>(P.x + node) : zero;
-            // native FP64: the chain factor c_v scales the direction's
-            // velocity at the node (3 multiplies instead of 12 at the Gauss
-            // point), and da = (c_a / c_v) dv
-            constexpr bool kNodeScale = std::is_same<T, double>::value;
-            if constexpr (kNodeScale) {
-                xx.x = P.c_v * xx.x;
-                xx.y = P.c_v * xx.y;
-                xx.z = P.c_v * xx.z;
-            }
-            T dv[3], dgv[3][3], da[3], dp, dgp[3];
-            {
-                VG<T> e0, e1, e2, e3;
-                eval_vg4<OUT>(xx, sx, sy, sz, e0, e1, e2, e3);
-                if constexpr (MAPPED) {
-                    to_phys(geo, e0);
-                    to_phys(geo, e1);
-                    to_phys(geo, e2);
-                    to_phys(geo, e3);
-                }
-                if constexpr (kNodeScale) {
-                    dv[0] = e0.v; da[0] = P.c_av * e0.v;
-                    dv[1] = e1.v; da[1] = P.c_av * e1.v;
-                    dv[2] = e2.v; da[2] = P.c_av * e2.v;
-                    dgv[0][0] = e0.gx; dgv[0][1] = e0.gy; dgv[0][2] = e0.gz;
-                    dgv[1][0] = e1.gx; dgv[1][1] = e1.gy; dgv[1][2] = e1.gz;
-                    dgv[2][0] = e2.gx; dgv[2][1] = e2.gy; dgv[2][2] = e2.gz;
-                } else {
-                    const T cv = P.c_v, ca = P.c_a;
-                    dv[0] = cv * e0.v; da[0] = ca * e0.v;
-                    dv[1] = cv * e1.v; da[1] = ca * e1.v;
-                    dv[2] = cv * e2.v; da[2] = ca * e2.v;
-                    dgv[0][0] = cv * e0.gx; dgv[0][1] = cv * e0.gy; dgv[0][2] = cv * e0.gz;
-                    dgv[1][0] = cv * e1.gx; dgv[1][1] = cv * e1.gy; dgv[1][2] = cv * e1.gz;
-                    dgv[2][0] = cv * e2.gx; dgv[2][1] = cv * e2.gy; dgv[2][2] = cv * e2.gz;
-                }
-                dp = e3.v; dgp[0] = e3.gx; dgp[1] = e3.gy; dgp[2] = e3.gz;
-            }
-            // d tau_M = -1/2 tau_M^3 s dQ with dQ = 2 v.G dv
-            T vGdv, q0;
-            if constexpr (MAPPED) {
-                vGdv = vGdv_full(geo, q, dv);
-                q0 = geo.q0;
-            } else {
-                vGdv = dot3_t(P.G0 * q.v[0], dv[0], P.G1 * q.v[1], dv[1], P.G2 * q.v[2], dv[2]);
-                q0 = P.q0;
-            }
-            gp_jacobian_terms(P, q, dv, dgv, da, dp, dgp, vGdv, q0, X, Y);
-        }
-        vec4<T> r;
-        if constexpr (MAPPED) {
-            // grad N . Y = grad_xi N . (Ji Y); det J per Gauss point
+            Face<T> f[4];
+            T v[4];
+            faces4(load_u(0, node0), f);
+#pragma unroll
             for (int c = 0; c < 4; ++c) {
-                const T y0 = Y[c][0], y1 = Y[c][1], y2 = Y[c][2];
-                Y[c][0] = geo.det * (geo.Ji[0][0] * y0 + geo.Ji[0][1] * y1 + geo.Ji[0][2] * y2);
-                Y[c][1] = geo.det * (geo.Ji[1][0] * y0 + geo.Ji[1][1] * y1 + geo.Ji[1][2] * y2);
-                Y[c][2] = geo.det * (geo.Ji[2][0] * y0 + geo.Ji[2][1] * y1 + geo.Ji[2][2] * y2);
-                X[c] = geo.det * X[c];
+                setL(3 * c, f[c].b);
+                setL(3 * c + 1, f[c].dx);
+                setL(3 * c + 2, f[c].dy);
             }
-            project2<OUT>(X[0], Y[0], X[1], Y[1], sx, sy, sz, r.x, r.y);
-            project2<OUT>(X[2], Y[2], X[3], Y[3], sx, sy, sz, r.z, r.w);
-        } else {
-            project2<OUT>(X[0], Y[0], X[1], Y[1], sx, sy, sz, r.x, r.y);
-            project2<OUT>(X[2], Y[2], X[3], Y[3], sx, sy, sz, r.z, r.w);
-            r.x = P.detJ * r.x;
-            r.y = P.detJ * r.y;
-            r.z = P.detJ * r.z;
-            r.w = P.detJ * r.w;
+            faces_v(load_a(0, node0), v);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) setL(12 + c, v[c]);
+            if constexpr (JAC) {
+                faces4(load_x(0, node0), f);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    setL(kPlaneU + 3 * c, f[c].b);
+                    setL(kPlaneU + 3 * c + 1, f[c].dx);
+                    setL(kPlaneU + 3 * c + 2, f[c].dy);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < kCarry * kOps; ++q) setC(q, T(0));
         }
-        if (slot < nel) rel[rel_at(nel, slot, g)] = valid ? r : zero;
+
+        // z parts of one component added to the carried ones; the totals of
+        // the lower plane in t, the upper parts become the carried ones
+        auto z_project = [&](int q0, const C &X, const C &Yx, const C &Yy, const C &Yz, T (&t)[3]) {
+            T up;
+            const T s = ihz * (PO::first(Yz) + PO::second(Yz));
+            z_part<T>(X, getC(q0), t[0], up);
+            t[0] = t[0] - s;
+            setC(q0, up + s);
+            z_part<T>(Yx, getC(q0 + 1), t[1], up);
+            setC(q0 + 1, up);
+            z_part<T>(Yy, getC(q0 + 2), t[2], up);
+            setC(q0 + 2, up);
+        };
+        // transposed in-plane stages of components c and c + 1 (op o) of plane l
+        auto put2 = [&](int o, int c, int l, const T (&t0)[3], const T (&t1)[3]) {
+            T r0, r1;
+            if constexpr (std::is_same<T, double>::value) {
+                r0 = face_project(t0[0], t0[1], t0[2], sx, sy);
+                r1 = face_project(t1[0], t1[1], t1[2], sx, sy);
+            } else {
+                const C r = face_project(PO::pack(t0[0], t1[0]), PO::pack(t0[1], t1[1]),
+                                         PO::pack(t0[2], t1[2]), sx2, sy2);
+                r0 = PO::first(r);
+                r1 = PO::second(r);
+            }
+            r0 = scale_m * r0;
+            r1 = (c == 2 ? scale_c : scale_m) * r1;
+            if (slot) {
+                Cell *d = rel + (4 * o + c) * comp_cells + l * plane_cells + (tid & 3) * stride + col;
+                d[0] = cell_st(r0);
+                d[comp_cells] = cell_st(r1);
+            }
+        };
+        // projection of one operator's coefficients (continuity: X3, Y3) of layer l
+        auto project_rows = [&](int o, int l, const C (&X)[4], const C (&Y)[4][3]) {
+            T t0[3], t1[3];
+#pragma unroll
+            for (int c = 0; c < 4; c += 2) {
+                z_project(kCarry * o + 3 * c, X[c], Y[c][0], Y[c][1], Y[c][2], t0);
+                z_project(kCarry * o + 3 * c + 3, X[c + 1], Y[c + 1][0], Y[c + 1][1], Y[c + 1][2], t1);
+                put2(o, c, l, t0, t1);
+            }
+        };
+
+        // ---- the elements, bottom to top
+        for (int l = 0; l < nl; ++l) {
+            // the double-float body is long: a barrier per layer keeps the
+            // CTA's warps on the same stretch of it (instruction cache)
+            if constexpr (std::is_same<T, df64>::value) __syncthreads();
+            const int64_t nd = node0 + (valid ? (int64_t)NXY1 * (l + 1) : 0);
+            fetch(l + 2);
+            if constexpr (kAsync) asm volatile("cp.async.wait_group 1;" ::: "memory");
+            // geometry of the lane's two Gauss points (mapped grids); idle
+            // lanes read element 0's
+            const typename GeoStore<T>::type *gp = nullptr;
+            if constexpr (MAPPED)
+                gp = P.geo + (tid & 3) +
+                     (valid ? (ex + (int64_t)P.Nx * (ey + (int64_t)P.Ny * (ez0 + l))) * (kMapGeo * 8)
+                            : 0);
+            auto geo = [&](int k) -> C {
+                return PO::pack(geo_ld<T>(gp + 8 * k), geo_ld<T>(gp + 8 * k + 4));
+            };
+            // value and gradient at the two points of the field at plane slot q
+            auto field = [&](int q, const Face<T> &h, C &v, C (&g)[3]) {
+                const T lb = getL(q), d = h.b - lb, gz = ihz * d;
+                v = z_val_d(lb, h.b, d);
+                g[2] = PO::pack(gz, gz);
+                g[0] = z_val(getL(q + 1), h.dx);
+                g[1] = z_val(getL(q + 2), h.dy);
+                setL(q, h.b);
+                setL(q + 1, h.dx);
+                setL(q + 2, h.dy);
+            };
+            auto to_physical = [&](C (&g)[3], const C (&Ji)[9]) {
+                const C a = g[0], b = g[1], c = g[2];
+                g[0] = dot3_t(a, Ji[0], b, Ji[3], c, Ji[6]);
+                g[1] = dot3_t(a, Ji[1], b, Ji[4], c, Ji[7]);
+                g[2] = dot3_t(a, Ji[2], b, Ji[5], c, Ji[8]);
+            };
+            C Ji[9];
+            if constexpr (MAPPED)
+#pragma unroll
+                for (int k = 0; k < 9; ++k) Ji[k] = geo(k);
+
+            // ---- base state: G[i][j] = d_j v_i, r = a + v.grad v + grad p / rho
+            C v[3], G[3][3], pr, gpr[3], a[3], s;
+            {
+                Face<T> f[4];
+                faces4(load_u(l + 1, nd), f);
+#pragma unroll
+                for (int i = 0; i < 3; ++i) field(3 * i, f[i], v[i], G[i]);
+                field(9, f[3], pr, gpr);
+                if constexpr (MAPPED) {
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) to_physical(G[i], Ji);
+                    to_physical(gpr, Ji);
+                }
+                T hv[4];
+                faces_v(load_a(l + 1, nd), hv);
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    a[i] = z_val(getL(12 + i), hv[i]);
+                    setL(12 + i, hv[i]);
+                }
+                if (P.has_s) {
+                    s = z_val(getL(15), hv[3]);
+                    setL(15, hv[3]);
+                }
+            }
+            C rM[3], up[3], w[3], gv[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                C t = a[i] + gpr[i];
+                t = fma_t(v[0], G[i][0], t);
+                t = fma_t(v[1], G[i][1], t);
+                rM[i] = fma_t(v[2], G[i][2], t);
+            }
+            const C rC = G[0][0] + G[1][1] + G[2][2];
+            C q0, itrG;
+            if constexpr (MAPPED) {
+                const C g00 = geo(9), g01 = geo(10), g02 = geo(11), g11 = geo(12), g12 = geo(13),
+                        g22 = geo(14);
+                gv[0] = dot3_t(g00, v[0], g01, v[1], g02, v[2]);
+                gv[1] = dot3_t(g01, v[0], g11, v[1], g12, v[2]);
+                gv[2] = dot3_t(g02, v[0], g12, v[1], g22, v[2]);
+                q0 = fma_t(PO::pack(P.CInu2, P.CInu2), geo(15), PO::pack(P.ct_dt2, P.ct_dt2));
+                itrG = geo(16);
+            } else {
+                gv[0] = PO::pack(P.G0, P.G0) * v[0];
+                gv[1] = PO::pack(P.G1, P.G1) * v[1];
+                gv[2] = PO::pack(P.G2, P.G2) * v[2];
+                q0 = PO::pack(P.q0, P.q0);
+                itrG = PO::pack(P.inv_trG, P.inv_trG);
+            }
+            // S = s (q0 + v.G v), tau_M = S^-1/2, tau_C = S tau_M / tr G
+            C Sq = q0 + dot3_t(gv[0], v[0], gv[1], v[1], gv[2], v[2]);
+            if (P.has_s) Sq = s * Sq;
+            const C tau = rsqrt_t(Sq);
+            const C ntau = -tau;
+            const C ntauC = Sq * ntau * itrG;
+            // u' = -tau_M r, p'/rho = -tau_C r_C, w = v + u'
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                up[i] = ntau * rM[i];
+                w[i] = v[i] + up[i];
+            }
+            const C pp = ntauC * rC;
+
+            // Y[c] -> det (Ji Y[c]) and X[c] -> det X[c] on mapped grids
+            auto to_reference = [&](C (&X)[4], C (&Y)[4][3]) {
+                const C det = geo(17);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const C y0 = Y[c][0], y1 = Y[c][1], y2 = Y[c][2];
+                    Y[c][0] = det * dot3_t(Ji[0], y0, Ji[1], y1, Ji[2], y2);
+                    Y[c][1] = det * dot3_t(Ji[3], y0, Ji[4], y1, Ji[5], y2);
+                    Y[c][2] = det * dot3_t(Ji[6], y0, Ji[7], y1, Ji[8], y2);
+                    X[c] = det * X[c];
+                }
+            };
+            // nu (g_ij + g_ji), both orders of the pair at once
+            auto viscous = [&](const C (&g)[3][3], C (&Y)[4][3]) {
+                Y[0][0] = nu2 * g[0][0];
+                Y[1][1] = nu2 * g[1][1];
+                Y[2][2] = nu2 * g[2][2];
+                Y[0][1] = Y[1][0] = nu * (g[0][1] + g[1][0]);
+                Y[0][2] = Y[2][0] = nu * (g[0][2] + g[2][0]);
+                Y[1][2] = Y[2][1] = nu * (g[1][2] + g[2][1]);
+            };
+            if constexpr (!JAC || FUSED) {
+                // residual: X_i = a_i + w.grad v_i,
+                // Y_ij = nu (d_j v_i + d_i v_j) - w_j u'_i - (p + p') delta_ij
+                C X[4], Y[4][3];
+                viscous(G, Y);
+                const C ptot = pr + pp;
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    C t = fma_t(w[0], G[i][0], a[i]);
+                    t = fma_t(w[1], G[i][1], t);
+                    X[i] = fma_t(w[2], G[i][2], t);
+                    const C nup = -up[i];
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) Y[i][j] = fma_t(w[j], nup, Y[i][j]);
+                    Y[i][i] = Y[i][i] - ptot;
+                    Y[3][i] = nup;
+                }
+                X[3] = rC;
+                if constexpr (MAPPED) to_reference(X, Y);
+                project_rows(FUSED ? 1 : 0, l, X, Y);
+            }
+            if constexpr (JAC) {
+                C dv[3], dG[3][3], dp, dgp[3];
+                {
+                    Face<T> f[4];
+                    faces4(load_x(l + 1, nd), f);
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) field(kPlaneU + 3 * i, f[i], dv[i], dG[i]);
+                    field(kPlaneU + 9, f[3], dp, dgp);
+                    if constexpr (MAPPED) {
+#pragma unroll
+                        for (int i = 0; i < 3; ++i) to_physical(dG[i], Ji);
+                        to_physical(dgp, Ji);
+                    }
+                }
+                // d tau_M = -k tau_M and d tau_C = k tau_C with k = tau_M^2 s v.G dv
+                const C vGdv = dot3_t(gv[0], dv[0], gv[1], dv[1], gv[2], dv[2]);
+                C k = tau * tau * vGdv;
+                if (P.has_s) k = s * k;
+                const C drC = dG[0][0] + dG[1][1] + dG[2][2];
+                const C cav = PO::pack(P.c_av, P.c_av);
+                C da[3], dup[3], dw[3];
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    da[i] = cav * dv[i];
+                    C t = da[i] + dgp[i];
+                    t = fma_t(v[0], dG[i][0], t);
+                    t = fma_t(v[1], dG[i][1], t);
+                    t = fma_t(v[2], dG[i][2], t);
+                    t = fma_t(dv[0], G[i][0], t);
+                    t = fma_t(dv[1], G[i][1], t);
+                    t = fma_t(dv[2], G[i][2], t);
+                    // du' = -d tau_M r - tau_M dr = -k u' - tau_M dr
+                    dup[i] = ntau * t - k * up[i];
+                }
+#pragma unroll
+                for (int i = 0; i < 3; ++i) dw[i] = dv[i] + dup[i];
+                // dp'/rho = -(d tau_C r_C + tau_C dr_C) = k p'/rho - tau_C dr_C
+                const C dptot = dp + dot2_t(k, pp, ntauC, drC);
+                C X[4], Y[4][3];
+                viscous(dG, Y);
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    C t = da[i];
+                    t = fma_t(dw[0], G[i][0], t);
+                    t = fma_t(dw[1], G[i][1], t);
+                    t = fma_t(dw[2], G[i][2], t);
+                    t = fma_t(w[0], dG[i][0], t);
+                    t = fma_t(w[1], dG[i][1], t);
+                    X[i] = fma_t(w[2], dG[i][2], t);
+                    const C nup = -up[i], ndup = -dup[i];
+#pragma unroll
+                    for (int j = 0; j < 3; ++j)
+                        Y[i][j] = fma_t(dw[j], nup, fma_t(w[j], ndup, Y[i][j]));
+                    Y[i][i] = Y[i][i] - dptot;
+                    Y[3][i] = ndup;
+                }
+                X[3] = drC;
+                if constexpr (MAPPED) to_reference(X, Y);
+                project_rows(0, l, X, Y);
+            }
+        }
+        // ---- the topmost plane: the carried parts alone
+#pragma unroll
+        for (int o = 0; o < kOps; ++o)
+#pragma unroll
+            for (int c = 0; c < 4; c += 2) {
+                const int q = kCarry * o + 3 * c;
+                const T t0[3] = {getC(q), getC(q + 1), getC(q + 2)};
+                const T t1[3] = {getC(q + 3), getC(q + 4), getC(q + 5)};
+                put2(o, c, nl, t0, t1);
+            }
     }
     __syncthreads();
 
-    // Node block of the brick: each node sums the contributions of the (up to
-    // 8) brick elements around it, corner by corner in a fixed order.
-    const int nx1 = P.bx + 1, ny1 = P.by + 1, nz1 = P.bz + 1;
-    const int nnodes = nx1 * ny1 * nz1;
-    constexpr int kOut = FUSED ? 2 : 1;
+    // Node sums: each node of the brick's node block adds the contributions of
+    // the (up to 4) columns around it in a fixed order.  A node that no other
+    // brick holds is done; the others go to the node block.
+    const int nx1 = P.bx + 1, ny1 = P.by + 1;
+    const int nxv = min(P.bx, P.Nx - ex0), nyv = min(P.by, P.Ny - ey0);  // columns in the grid
+    const int nin = (nxv + 1) * (nyv + 1) * (nl + 1);
+    for (int q = tid; q < nin; q += nthr) {
+        const int ix = q % (nxv + 1), iy = (q / (nxv + 1)) % (nyv + 1),
+                  iz = q / ((nxv + 1) * (nyv + 1));
+        const bool inner = (ix > 0 || ex0 == 0) && (ix < nxv || ex0 + nxv == P.Nx) &&
+                           (iy > 0 || ey0 == 0) && (iy < nyv || ey0 + nyv == P.Ny) &&
+                           (iz > 0 || ez0 == 0) && (iz < nl || ez0 + nl == P.Nz);
+        const int64_t node = ex0 + ix + (int64_t)NX1 * (ey0 + iy) + (int64_t)NXY1 * (ez0 + iz);
+        const size_t nb = (size_t)brick * (nx1 * ny1 * (P.bz + 1)) + ix + nx1 * (iy + ny1 * iz);
 #pragma unroll
-    for (int o = 0; o < kOut; ++o) {
-        vec4<T> *blk = (o ? P.blocks2 : P.blocks) + (size_t)brick * nnodes;
-        const vec4<T> *rl = rel + o * rel_records(nel);
-        for (int nl = threadIdx.x; nl < nnodes; nl += blockDim.x) {
-            const int ix = nl % nx1, iy = (nl / nx1) % ny1, iz = nl / (nx1 * ny1);
-            vec4<T> acc = {T(0), T(0), T(0), T(0)};
+        for (int o = 0; o < kOps; ++o) {
+            T acc[4] = {T(0), T(0), T(0), T(0)};
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const int lx = ix - (c & 1), ly = iy - ((c >> 1) & 1), lz = iz - ((c >> 2) & 1);
-                if (lx < 0 || ly < 0 || lz < 0 || lx >= P.bx || ly >= P.by || lz >= P.bz) continue;
-                const vec4<T> r = rl[rel_at(nel, (lz * P.by + ly) * P.bx + lx, c)];
-                acc.x += r.x;
-                acc.y += r.y;
-                acc.z += r.z;
-                acc.w += r.w;
+            for (int c = 0; c < 4; ++c) {
+                const int cx = ix - (c & 1), cy = iy - (c >> 1);
+                if (cx < 0 || cy < 0 || cx >= nxv || cy >= nyv) continue;
+                const Cell *r = rel + 4 * o * comp_cells + iz * plane_cells + c * stride + cy * P.bx + cx;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) acc[k] += cell_ld<T>(r[k * comp_cells]);
             }
-            blk[nl] = acc;
+            if (inner) {
+                vec4<S> *out = FUSED && o ? P.out2 : P.out;
+                out[node] = {to_s(acc[0]), to_s(acc[1]), to_s(acc[2]), to_s(acc[3])};
+            } else {
+                vec4<T> *blk = FUSED && o ? P.blocks2 : P.blocks;
+                blk[nb] = {acc[0], acc[1], acc[2], acc[3]};
+            }
         }
     }
 }
@@ -815,39 +1226,118 @@ static __device__ __forceinline__ int axis_candidates(int i, int b, int nb, int 
     return k;
 }
 
-// Sum, for one node, the (up to 8) brick node blocks that contain it, lower
-// bricks first (FUSED: the residual's blocks into out2 as well).
-template <typename T, bool FUSED = false>
-__device__ __forceinline__ void gather_node(const VmsArgs<T> &P, int node)
-{
-    using S = typename StorageOf<T>::type;
-    const int NX1 = P.Nx + 1, NY1 = P.Ny + 1;
-    const int nx1 = P.bx + 1, ny1 = P.by + 1, nz1 = P.bz + 1;
-    const int nnodes = nx1 * ny1 * nz1;
+// Sum, for one node shared by several bricks, the (up to 8) brick node blocks
+// that contain it, lower bricks first (FUSED: the residual's blocks into out2 as
+// well): the node's candidate bricks along x and y, the plane k's along z.
+struct AxisCandidates {
+    int n, b[2] = {0, 0}, l[2] = {0, 0};  // count, bricks, local indices
+    __device__ __forceinline__ AxisCandidates(int i, int size, int nb)
     {
-        const int i = node % NX1, j = (node / NX1) % NY1, k = node / (NX1 * NY1);
-        int cbx[2], clx[2], cby[2], cly[2], cbz[2], clz[2];
-        const int kx = axis_candidates(i, P.bx, P.nbx, cbx, clx);
-        const int ky = axis_candidates(j, P.by, P.nby, cby, cly);
-        const int kz = axis_candidates(k, P.bz, P.nbz, cbz, clz);
-        constexpr int kOut = FUSED ? 2 : 1;
+        n = axis_candidates(i, size, nb, b, l);
+    }
+};
+template <typename T, bool FUSED = false>
+__device__ __forceinline__ void gather_node(const VmsArgs<T> &P, const AxisCandidates &cx,
+                                            const AxisCandidates &cy, const AxisCandidates &cz,
+                                            int64_t node)
+{
+    const int nx1 = P.bx + 1, ny1 = P.by + 1;
+    const int nnodes = nx1 * ny1 * (P.bz + 1);
+    constexpr int kOut = FUSED ? 2 : 1;
 #pragma unroll
-        for (int o = 0; o < kOut; ++o) {
-            const vec4<T> *blocks = o ? P.blocks2 : P.blocks;
-            vec4<T> acc = {T(0), T(0), T(0), T(0)};
-            for (int c = 0; c < kz; ++c)
-                for (int b = 0; b < ky; ++b)
-                    for (int a = 0; a < kx; ++a) {
-                        const size_t brick = cbx[a] + P.nbx * (cby[b] + (size_t)P.nby * cbz[c]);
-                        const int nl = clx[a] + nx1 * (cly[b] + ny1 * clz[c]);
-                        const vec4<T> r = ld4_blk(blocks + brick * nnodes + nl);
-                        acc.x += r.x;
-                        acc.y += r.y;
-                        acc.z += r.z;
-                        acc.w += r.w;
-                    }
-            (o ? P.out2 : P.out)[node] = {to_s(acc.x), to_s(acc.y), to_s(acc.z), to_s(acc.w)};
+    for (int o = 0; o < kOut; ++o) {
+        const vec4<T> *blocks = o ? P.blocks2 : P.blocks;
+        // all loads before the first sum: they are independent, and a branch
+        // around each made the node wait for them one by one
+        vec4<T> r[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int a = q & 1, b = (q >> 1) & 1, c = q >> 2;
+            const bool in = a < cx.n && b < cy.n && c < cz.n;
+            const int brick = in ? cx.b[a] + P.nbx * (cy.b[b] + P.nby * cz.b[c]) : 0;
+            const int nl = in ? cx.l[a] + nx1 * (cy.l[b] + ny1 * cz.l[c]) : 0;
+            r[q] = vec4<T>{T(0), T(0), T(0), T(0)};
+            if (in) r[q] = ld4_blk(blocks + (int64_t)brick * nnodes + nl);
         }
+        vec4<T> acc = r[0];  // the first candidate always exists
+#pragma unroll
+        for (int q = 1; q < 8; ++q) {
+            // (an FP64 addition costs 16 cycles of an SM: none for a missing block)
+            if (!((q & 1) < cx.n && ((q >> 1) & 1) < cy.n && (q >> 2) < cz.n)) continue;
+            acc.x += r[q].x;
+            acc.y += r[q].y;
+            acc.z += r[q].z;
+            acc.w += r[q].w;
+        }
+        (o ? P.out2 : P.out)[node] = {to_s(acc.x), to_s(acc.y), to_s(acc.z), to_s(acc.w)};
+    }
+}
+// The nodes that several bricks share, numbered 0 .. shared_nodes() - 1 so that a
+// thread per shared node does nothing else: (a) whole planes between bricks along
+// z, (b) whole rows between bricks along y on the other planes, (c) the nodes
+// between bricks along x in what is left.  (A thread per grid node spent 33 us at
+// 129^3 finding out that its node was not shared; a warp per node row left too few
+// loads in flight.)
+template <typename T> __host__ __device__ __forceinline__ int64_t shared_nodes(const VmsArgs<T> &P)
+{
+    const int64_t nx = P.Nx + 1, ny = P.Ny + 1, nz = P.Nz + 1;
+    const int sx = P.nbx - 1, sy = P.nby - 1, sz = P.nbz - 1;
+    return sz * nx * ny + (nz - sz) * (sy * nx + (ny - sy) * sx);
+}
+// the r-th coordinate of an axis that no two of its bricks of b elements share
+__device__ __forceinline__ int unshared_coord(int r, int b, int N)
+{
+    if (r == 0) return 0;
+    const int g = b > 1 ? (r - 1) / (b - 1) : N;
+    return min(g * b + r - g * (b - 1), N);
+}
+template <typename T, bool FUSED = false>
+__device__ __forceinline__ void gather_shared(const VmsArgs<T> &P, int q)
+{
+    const int nx = P.Nx + 1, ny = P.Ny + 1;
+    const int sx = P.nbx - 1, sy = P.nby - 1, sz = P.nbz - 1;
+    int i, j, k;
+    if (q < sz * nx * ny) {
+        const int row = q / nx, pl = row / ny;
+        i = q - row * nx;
+        j = row - pl * ny;
+        k = (pl + 1) * P.bz;
+    } else {
+        q -= sz * nx * ny;
+        const int per = sy * nx + (ny - sy) * sx;  // of one plane
+        const int pl = q / per;
+        q -= pl * per;
+        k = unshared_coord(pl, P.bz, P.Nz);
+        if (q < sy * nx) {
+            const int row = q / nx;
+            i = q - row * nx;
+            j = (row + 1) * P.by;
+        } else {
+            q -= sy * nx;
+            const int row = q / sx;
+            i = (q - row * sx + 1) * P.bx;
+            j = unshared_coord(row, P.by, P.Ny);
+        }
+    }
+    gather_node<T, FUSED>(P, AxisCandidates(i, P.bx, P.nbx), AxisCandidates(j, P.by, P.nby),
+                          AxisCandidates(k, P.bz, P.nbz), i + (int64_t)nx * (j + (int64_t)ny * k));
+}
+
+// The schedule a kernel runs for a requested brick: the CTA no larger than the
+// brick's lanes need, and the brick halved along its longest side until its
+// shared memory fits.
+constexpr int kBrickSmemMax = 200 * 1024;
+constexpr int kBrickThreads = 128;  // CTA size limit of the brick kernels (their register caps)
+inline Brick fit_brick(Brick b, int cell, bool jac, bool fused)
+{
+    for (;;) {
+        const int lanes = (4 * b.bx * b.by + 31) / 32 * 32;
+        if (b.threads > lanes) b.threads = lanes;
+        if (b.threads > kBrickThreads) b.threads = kBrickThreads;
+        if (brick_smem(b.bx, b.by, b.bz, b.threads, cell, jac, fused) <= kBrickSmemMax) return b;
+        int &d = b.bz > 1 && b.bz >= b.bx && b.bz >= b.by ? b.bz : (b.bx >= b.by ? b.bx : b.by);
+        if (d == 1) return b;  // a single element always fits
+        d = (d + 1) / 2;
     }
 }
 
@@ -877,6 +1367,8 @@ VmsArgs<T> make_args(const fsi_mesh *m, const Brick &b, const void *U, const voi
     P.rho = (T)rho;
     P.mu = (T)mu;
     P.inv_rho = (T)(1.0 / rho);
+    P.nu = (T)nu;
+    P.nu2 = (T)(2.0 * nu);
     P.G0 = (T)G[0];
     P.G1 = (T)G[1];
     P.G2 = (T)G[2];
@@ -886,6 +1378,7 @@ VmsArgs<T> make_args(const fsi_mesh *m, const Brick &b, const void *U, const voi
     P.ih1 = (T)(1.0 / h[1]);
     P.ih2 = (T)(1.0 / h[2]);
     P.detJ = (T)(h[0] * h[1] * h[2] / 8.0);
+    P.rdetJ = (T)(rho * (h[0] * h[1] * h[2] / 8.0));
     P.c_a = (T)m->alpha_m;
     P.c_v = (T)(m->alpha_f * m->gamma * dt);
     P.c_av = (T)(m->alpha_m / (m->alpha_f * m->gamma * dt));
