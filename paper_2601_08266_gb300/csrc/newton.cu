@@ -866,7 +866,22 @@ fsi_status coupled_residual_impl(fsi_mesh *mesh, const fsi_step_state *st, doubl
     return point_mass_residual_add(mesh, st, R, prec);
 }
 
-// Working-precision copies of the linearisation point (after a residual).
+// The stage values the Jacobian is linearised at (for a hyperelastic body its
+// stage values too), as the coupled residual leaves them, without evaluating the
+// residual: fsi_coupled_jacobian_apply and fsi_block_diagonal need no more (the
+// native FP64 residual they used to evaluate was 0.82 of 1.45 ms on a 52 x 45 x
+// 48 mapped grid).
+fsi_status stage_linearisation(fsi_mesh *mesh, const fsi_step_state *st)
+{
+    Work &W = mesh->newton->w;
+    FSI_TRY(fsi_stage(mesh, FSI_F64, st->y, st->Vn, st->An, st->s, W.U, W.A));
+    if (!(st->m > 0 && st->body)) return FSI_OK;
+    FSI_TRY(fsi_dlm_interp(mesh, FSI_F64, st->m, st->elem, st->xi, st->y, W.pa));
+    return solid_stage_impl(st->body, st->us, st->vs, st->as, W.pa, W.bu, W.bv, W.ba);
+}
+
+// Working-precision copies of the linearisation point (after a residual or
+// stage_linearisation).
 template <typename T> fsi_status prepare_linearisation(fsi_mesh *mesh, const fsi_step_state *st)
 {
     Work &W = mesh->newton->w;
@@ -1380,7 +1395,7 @@ fsi_status fsi_coupled_jacobian_apply(fsi_mesh *mesh, fsi_prec prec, const fsi_s
     FSI_DEVICE(mesh->device);
     FSI_TRY(ensure_work(mesh, st->m, 1));
     Work &W = mesh->newton->w;
-    FSI_TRY(coupled_residual_impl(mesh, st, W.R));
+    FSI_TRY(stage_linearisation(mesh, st));
     if (prec == FSI_F64) {
         FSI_TRY(prepare_linearisation<double>(mesh, st));
         return coupled_jacobian_impl<double>(mesh, st, (const double *)x, (double *)Jx);
@@ -1399,7 +1414,7 @@ fsi_status fsi_block_diagonal(fsi_mesh *mesh, fsi_prec prec, const fsi_step_stat
     FSI_DEVICE(mesh->device);
     FSI_TRY(ensure_work(mesh, st->m, 1));
     Work &W = mesh->newton->w;
-    FSI_TRY(coupled_residual_impl(mesh, st, W.R));
+    FSI_TRY(stage_linearisation(mesh, st));
     const size_t bytes = (size_t)mesh->n_nodes * 16 * (prec == FSI_F64 ? 8 : 4);
     if (prec == FSI_F64) {
         FSI_TRY(prepare_linearisation<double>(mesh, st));
