@@ -183,8 +183,9 @@ void destroy_amg(fsi_mesh *m);
 // immersed hyperelastic solid (solid.cu)
 fsi_status solid_residual_impl(fsi_solid *b, const double *u_af, const double *v_af,
                                const double *a_am, const double *u_n, const double g[3], double *R);
-template <typename T>
-fsi_status solid_tangent_impl(fsi_solid *b, const T *u_af, const double *u_n, const T *x, T *Jx);
+// the tangent at (u_af, u_n): its state once, then applies (same T)
+template <typename T> fsi_status solid_linearise(fsi_solid *b, const T *u_af, const double *u_n);
+template <typename T> fsi_status solid_tangent_impl(fsi_solid *b, const T *x, T *Jx);
 fsi_status solid_stage_impl(fsi_solid *b, const double *u, const double *v, const double *a,
                             const double *a1, double *u_af, double *v_af, double *a_am);
 int64_t solid_nodes(const fsi_solid *b);

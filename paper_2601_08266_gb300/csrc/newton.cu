@@ -893,7 +893,10 @@ template <typename T> fsi_status prepare_linearisation(fsi_mesh *mesh, const fsi
     if (st->m > 0) {
         cast_kernel<double, T><<<grid1d(3 * st->m), 256, 0, s>>>(3 * st->m, st->xi, (T *)W.xiw);
         if (st->body)
+        {
             cast_kernel<double, T><<<grid1d(3 * st->m), 256, 0, s>>>(3 * st->m, W.bu, (T *)W.buw);
+            FSI_TRY(solid_linearise<T>(st->body, (const T *)W.buw, st->us));
+        }
         if (st->w) cast_kernel<double, T><<<grid1d(st->m), 256, 0, s>>>(st->m, st->w, (T *)W.ww);
     }
     return check_launch("linearisation casts");
@@ -916,8 +919,7 @@ fsi_status coupled_jacobian_impl(fsi_mesh *mesh, const fsi_step_state *st, const
     FSI_TRY(vms_jacobian(mesh, P, W.Uw, W.Aw, st->f ? W.fw : nullptr, x, Jx));
     if (st->m > 0 && st->body) {
         FSI_TRY(fsi_dlm_interp(mesh, P, st->m, st->elem, W.xiw, x, W.pu));
-        FSI_TRY(solid_tangent_impl<T>(st->body, (const T *)W.buw, st->us, (const T *)W.pu,
-                                      (T *)W.pw));
+        FSI_TRY(solid_tangent_impl<T>(st->body, (const T *)W.pu, (T *)W.pw));
         FSI_TRY(fsi_dlm_spread(mesh, P, st->m, st->elem, W.xiw, st->cell_start, st->perm, W.pw,
                                nullptr, Jx, 1));
     } else if (st->m > 0 && !overlap) {

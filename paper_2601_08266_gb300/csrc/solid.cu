@@ -15,11 +15,30 @@
 // w.r.t. uddot_{n+1} carries the chain factors alpha_m (inertia),
 // alpha_f beta dt^2 (stress), alpha_f gamma dt (viscous).
 //
-// GPU layout: one thread per element computes its 8 x 3 nodal contributions
-// (geometry from the reference coordinates at each Gauss point) into an
-// element scratch [es][8][3]; each node then sums its element slots through a
-// node -> (element, corner) table in a fixed order.  No atomics;
-// deterministic.
+// GPU layout: eight lanes per element; lane a is first "node a" (it loads the
+// node's record) and then "Gauss point a".  On the trilinear map values and
+// parent gradients follow from the nodal values by three butterfly stages over
+// the lane bits, and the projection onto the test functions is the transposed
+// butterfly.  All stresses are taken in the Kirchhoff form tau = P F^T, so that
+// one inverse per configuration, K = (dx/dxi)^-1 at the alpha level and Kn at the
+// start of the step, serves every gradient and every test function: the
+// reference configuration enters through det J0 and F = dx/dxi J0^-1 only.  With
+// H = grad_x(w) = (dw/dxi) K of the direction w,
+//
+//   tau       = mu (b - I) + lam ln J I,                    b = F F^T,
+//   dP F^T    = c_u (mu H b + (mu - lam ln J) H^T + lam tr H I).
+//
+// What the tangent needs of the state (K, Kn, mu b, mu - lam ln J, the viscous
+// scale, det J0: 27 values per Gauss point) is formed once per linearisation into
+// a table; a tangent apply reads it.  Contributions go to an element scratch
+// [es][8][3]; each node then sums its element slots through a node -> (element,
+// corner) table in a fixed order.  No atomics; deterministic.
+//
+// Bound: the FP64 pipe (2 operations per SM and clock).  One thread per element,
+// which formed dN/dX, F, F^-1 and both configurations' gradients of all 8 nodes at
+// every point of every apply, took 584 us per FP64 tangent apply of 20,736
+// hexahedra; an FP64 implicit step with that body on a 24^3 grid went from 76 to
+// 38 ms with this form.
 #include <cmath>
 #include <vector>
 
@@ -33,6 +52,7 @@ struct fsi_solid {
     int32_t *node_start; // [ns+1] CSR of element slots e*8+a per node
     int32_t *node_slot;  // [es*8]
     void *elem_f;        // [es][8][3] scratch, 8 bytes per value
+    void *state;         // [es][27][8] state of the tangent, 8 bytes per value
     double rho_s, mu_s, lam_s;
 };
 
@@ -80,179 +100,270 @@ struct SolidArgs {
     double c_a, c_u, c_v;  // tangent chain factors
 };
 
-// MODE 0: residual from (u_af, v_af, a_am, u_n); MODE 1: tangent apply along x
-// at (u_af, u_n).  T is the arithmetic and the array type of u_af, v_af,
-// a_am, x; u_n and X are FP64.
-template <typename T, int MODE>
-__global__ void solid_elem_kernel(SolidArgs s, const T *__restrict__ u_af, const T *__restrict__ v_af,
-                                  const T *__restrict__ a_am, const double *__restrict__ u_n,
-                                  const T *__restrict__ x, T *__restrict__ ef)
+constexpr double kGq = 0.57735026918962576451;  // 1/sqrt(3)
+
+template <typename T> __device__ __forceinline__ T shx(T v, int m)
 {
-    const T gq = T(0.57735026918962576451);  // 1/sqrt(3)
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < s.es;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        int nd[8];
-        T Xe[8][3], ue[8][3], un[8][3], ve[8][3], ae[8][3];
-#pragma unroll
-        for (int a = 0; a < 8; ++a) {
-            nd[a] = s.conn[8 * e + a];
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                const int64_t q = 3 * (int64_t)nd[a] + i;
-                Xe[a][i] = (T)s.X[q];
-                ue[a][i] = u_af[q];
-                un[a][i] = (T)u_n[q];
-                ve[a][i] = MODE == 0 ? v_af[q] : x[q];
-                ae[a][i] = MODE == 0 ? a_am[q] : x[q];
-            }
-        }
-        T out[8][3];
-#pragma unroll
-        for (int a = 0; a < 8; ++a) out[a][0] = out[a][1] = out[a][2] = T(0);
-        for (int qp = 0; qp < 8; ++qp) {
-            const T xi[3] = {(qp & 1) ? gq : -gq, (qp & 2) ? gq : -gq, (qp & 4) ? gq : -gq};
-            T N[8], dN[8][3];
-#pragma unroll
-            for (int a = 0; a < 8; ++a) {
-                T f[3];
-#pragma unroll
-                for (int k = 0; k < 3; ++k) f[k] = T(0.5) * (T(1) + (((a >> k) & 1) ? xi[k] : -xi[k]));
-                N[a] = f[0] * f[1] * f[2];
-                dN[a][0] = T(0.5) * (((a >> 0) & 1) ? T(1) : T(-1)) * f[1] * f[2];
-                dN[a][1] = T(0.5) * (((a >> 1) & 1) ? T(1) : T(-1)) * f[0] * f[2];
-                dN[a][2] = T(0.5) * (((a >> 2) & 1) ? T(1) : T(-1)) * f[0] * f[1];
-            }
-            // reference geometry: J0[i][k] = sum_a X_ai dN_a/dxi_k
-            M3<T> J0, J0i;
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    T t = T(0);
-#pragma unroll
-                    for (int a = 0; a < 8; ++a) t += Xe[a][i] * dN[a][k];
-                    J0.a[i][k] = t;
-                }
-            const T det0 = inv3(J0, J0i);
-            T gX[8][3];  // grad_X N_a = J0^{-T} dN_a/dxi
-#pragma unroll
-            for (int a = 0; a < 8; ++a)
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-                    gX[a][j] = dN[a][0] * J0i.a[0][j] + dN[a][1] * J0i.a[1][j] + dN[a][2] * J0i.a[2][j];
-            // deformation gradient at the alpha level
-            M3<T> F, Fi;
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    T t = i == j ? T(1) : T(0);
-#pragma unroll
-                    for (int a = 0; a < 8; ++a) t += ue[a][i] * gX[a][j];
-                    F.a[i][j] = t;
-                }
-            const T J = inv3(F, Fi);
-            const T lnJ = log_t(J);
-            const T mu = (T)s.mu, lam = (T)s.lam;
-            M3<T> P;
-            if (MODE == 0) {
-                // P = mu (F - F^-T) + lam ln J F^-T
-#pragma unroll
-                for (int i = 0; i < 3; ++i)
-#pragma unroll
-                    for (int j = 0; j < 3; ++j)
-                        P.a[i][j] = mu * (F.a[i][j] - Fi.a[j][i]) + lam * lnJ * Fi.a[j][i];
-            } else {
-                // dP = mu dF + (mu - lam ln J) F^-T dF^T F^-T + lam tr(F^-1 dF) F^-T,
-                // dF = c_u sum_a x_a (x) grad_X N_a
-                M3<T> dF;
-#pragma unroll
-                for (int i = 0; i < 3; ++i)
-#pragma unroll
-                    for (int j = 0; j < 3; ++j) {
-                        T t = T(0);
-#pragma unroll
-                        for (int a = 0; a < 8; ++a) t += ae[a][i] * gX[a][j];
-                        dF.a[i][j] = (T)s.c_u * t;
-                    }
-                T tr = T(0);
-#pragma unroll
-                for (int i = 0; i < 3; ++i)
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) tr += Fi.a[i][k] * dF.a[k][i];
-                // B = F^-T dF^T F^-T: B_ij = sum_kl Fi_ki dF_lk Fi_jl
-                M3<T> B1;  // dF^T F^-T: (B1)_kj = sum_l dF_lk Fi_jl
-#pragma unroll
-                for (int k = 0; k < 3; ++k)
-#pragma unroll
-                    for (int j = 0; j < 3; ++j)
-                        B1.a[k][j] = dF.a[0][k] * Fi.a[j][0] + dF.a[1][k] * Fi.a[j][1] + dF.a[2][k] * Fi.a[j][2];
-                const T c1 = mu - lam * lnJ, c2 = lam * tr;
-#pragma unroll
-                for (int i = 0; i < 3; ++i)
-#pragma unroll
-                    for (int j = 0; j < 3; ++j) {
-                        const T Bij = Fi.a[0][i] * B1.a[0][j] + Fi.a[1][i] * B1.a[1][j] + Fi.a[2][i] * B1.a[2][j];
-                        P.a[i][j] = mu * dF.a[i][j] + c1 * Bij + c2 * Fi.a[j][i];
-                    }
-            }
-            // inertia: N_a drho (uddot(g) - f) (MODE 1: c_a drho N_a x(g))
-            T ag[3];
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                T t = T(0);
-#pragma unroll
-                for (int a = 0; a < 8; ++a) t += N[a] * ae[a][i];
-                ag[i] = MODE == 0 ? (T)s.drho * (t - (T)s.g[i]) : (T)(s.c_a * s.drho) * t;
-            }
-            // viscous: configuration at the start of the step
-            M3<T> Fn, Fni;
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    T t = i == j ? T(1) : T(0);
-#pragma unroll
-                    for (int a = 0; a < 8; ++a) t += un[a][i] * gX[a][j];
-                    Fn.a[i][j] = t;
-                }
-            const T Jn = inv3(Fn, Fni);
-            T gx[8][3];  // grad_x N_a = grad_X N_a F_n^{-1}
-#pragma unroll
-            for (int a = 0; a < 8; ++a)
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-                    gx[a][j] = gX[a][0] * Fni.a[0][j] + gX[a][1] * Fni.a[1][j] + gX[a][2] * Fni.a[2][j];
-            M3<T> L;
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    T t = T(0);
-#pragma unroll
-                    for (int a = 0; a < 8; ++a) t += ve[a][i] * gx[a][j];
-                    L.a[i][j] = t;
-                }
-            const T vs = (T)(2.0 * s.mu_f) * Jn * (MODE == 0 ? T(1) : (T)s.c_v);
-            M3<T> D;  // 2 mu_f J_n D (times c_v for the tangent)
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < 3; ++j) D.a[i][j] = vs * T(0.5) * (L.a[i][j] + L.a[j][i]);
-#pragma unroll
-            for (int a = 0; a < 8; ++a)
-#pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    const T fint = P.a[i][0] * gX[a][0] + P.a[i][1] * gX[a][1] + P.a[i][2] * gX[a][2];
-                    const T fvis = D.a[i][0] * gx[a][0] + D.a[i][1] * gx[a][1] + D.a[i][2] * gx[a][2];
-                    out[a][i] += det0 * (N[a] * ag[i] + fint - fvis);
-                }
-        }
-#pragma unroll
-        for (int a = 0; a < 8; ++a)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) ef[(8 * e + a) * 3 + i] = out[a][i];
+    return __shfl_xor_sync(0xffffffffu, v, m);
+}
+
+// value and parent gradient at this lane's Gauss point of the trilinear field
+// whose value at this lane's node is u; s[k] = +-1/2 (the node's side along xi_k)
+template <typename T, bool VALUE>
+__device__ __forceinline__ T eval_parent(T u, const T (&s)[3], T (&g)[3])
+{
+    const T b1 = T(0.5 * (1.0 + kGq));
+    const T uo = shx(u, 1), tD = u - uo, tB = fma(b1, tD, uo);
+    const T tBo = shx(tB, 2), tDo = shx(tD, 2), tBD = tB - tBo;
+    const T tBB = fma(b1, tBD, tBo), tDB = fma(b1, tD - tDo, tDo);
+    const T tBBo = shx(tBB, 4), tBDo = shx(tBD, 4), tDBo = shx(tDB, 4), d = tBB - tBBo;
+    g[0] = s[0] * fma(b1, tDB - tDBo, tDBo);
+    g[1] = s[1] * fma(b1, tBD - tBDo, tBDo);
+    g[2] = s[2] * d;
+    return VALUE ? fma(b1, d, tBBo) : T(0);
+}
+
+// transposed: sum over the Gauss points of N_a X + dN_a/dxi . Y for this lane's node
+template <typename T>
+__device__ __forceinline__ T project_parent(T X, T Y0, T Y1, T Y2, const T (&s)[3])
+{
+    const T b1 = T(0.5 * (1.0 + kGq)), b2 = T(0.5 * (1.0 - kGq));
+    const T Xo = shx(X, 4), Y2o = shx(Y2, 4), Y0o = shx(Y0, 4), Y1o = shx(Y1, 4);
+    const T P1 = fma(s[2], Y2 + Y2o, fma(b1, X, b2 * Xo));
+    const T P2 = fma(b1, Y0, b2 * Y0o), P3 = fma(b1, Y1, b2 * Y1o);
+    const T P1o = shx(P1, 2), P2o = shx(P2, 2), P3o = shx(P3, 2);
+    const T Q1 = fma(s[1], P3 + P3o, fma(b1, P1, b2 * P1o));
+    const T Q2 = fma(b1, P2, b2 * P2o);
+    const T Q1o = shx(Q1, 1), Q2o = shx(Q2, 1);
+    return fma(s[0], Q2 + Q2o, fma(b1, Q1, b2 * Q1o));
+}
+
+// the lane's place: element, corner / Gauss point, node, gradient signs
+template <typename T> struct Lane {
+    int64_t e;
+    int node;
+    bool valid;
+    T s[3];
+    __device__ __forceinline__ Lane(const SolidArgs &a, int64_t t)
+    {
+        const int g = (int)(t & 7);
+        valid = (t >> 3) < a.es;
+        e = valid ? t >> 3 : 0;  // idle lanes repeat element 0, unused
+        node = a.conn[8 * e + g];
+        for (int k = 0; k < 3; ++k) s[k] = ((g >> k) & 1) ? T(0.5) : T(-0.5);
     }
+};
+
+// Kinematics of the configuration X + u at one Gauss point from the parent
+// gradient du of u: G = du/dX, K = (dx/dxi)^-1 = J0^-1 F^-1 with F = I + G;
+// returns det F
+template <typename T>
+__device__ __forceinline__ T kinematics(const M3<T> &du, const M3<T> &J0i, M3<T> &G, M3<T> &K)
+{
+    M3<T> F, Fi;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            G.a[i][j] = du.a[i][0] * J0i.a[0][j] + du.a[i][1] * J0i.a[1][j] + du.a[i][2] * J0i.a[2][j];
+            F.a[i][j] = (i == j ? T(1) : T(0)) + G.a[i][j];
+        }
+    const T J = inv3(F, Fi);
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+            K.a[k][j] = J0i.a[k][0] * Fi.a[0][j] + J0i.a[k][1] * Fi.a[1][j] + J0i.a[k][2] * Fi.a[2][j];
+    return J;
+}
+
+// State of one Gauss point: the two inverses, b - I (00 01 02 11 12 22), ln J,
+// J_n and det J0
+template <typename T> struct State {
+    M3<T> K, Kn;
+    T e[6], lnJ, Jn, det0;
+};
+template <typename T>
+__device__ __forceinline__ void solid_state(const SolidArgs &a, const Lane<T> &L,
+                                            const T *__restrict__ u_af,
+                                            const double *__restrict__ u_n, State<T> &q)
+{
+    M3<T> J0, J0i, d, G;
+    const int64_t n3 = 3 * (int64_t)L.node;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) eval_parent<T, false>((T)a.X[n3 + i], L.s, J0.a[i]);
+    q.det0 = inv3(J0, J0i);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) eval_parent<T, false>((T)u_n[n3 + i], L.s, d.a[i]);
+    q.Jn = kinematics(d, J0i, G, q.Kn);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) eval_parent<T, false>(u_af[n3 + i], L.s, d.a[i]);
+    q.lnJ = log_t(kinematics(d, J0i, G, q.K));
+    // b - I = G + G^T + G G^T: small strains keep their digits
+    int n = 0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = i; j < 3; ++j)
+            q.e[n++] = (G.a[i][j] + G.a[j][i]) +
+                       (G.a[i][0] * G.a[j][0] + G.a[i][1] * G.a[j][1] + G.a[i][2] * G.a[j][2]);
+}
+
+// Y = S K^T (ACC: -=), S symmetric given as 00 01 02 11 12 22
+template <typename T, bool SUB>
+__device__ __forceinline__ void sym_times_kt(const T (&S)[6], const M3<T> &K, M3<T> &Y)
+{
+    const int id[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const T s0 = S[id[i][0]], s1 = S[id[i][1]], s2 = S[id[i][2]];
+            if (SUB)
+                Y.a[i][k] = fma(-s2, K.a[k][2], fma(-s1, K.a[k][1], fma(-s0, K.a[k][0], Y.a[i][k])));
+            else
+                Y.a[i][k] = fma(s2, K.a[k][2], fma(s1, K.a[k][1], s0 * K.a[k][0]));
+        }
+}
+// D = vs (L + L^T), L = W Kn (00 01 02 11 12 22)
+template <typename T>
+__device__ __forceinline__ void viscous(const M3<T> &W, const M3<T> &Kn, T vs, T (&D)[6])
+{
+    M3<T> L;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+            L.a[i][j] = W.a[i][0] * Kn.a[0][j] + W.a[i][1] * Kn.a[1][j] + W.a[i][2] * Kn.a[2][j];
+    int n = 0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = i; j < 3; ++j) D[n++] = i == j ? (vs + vs) * L.a[i][i] : vs * (L.a[i][j] + L.a[j][i]);
+}
+template <typename T>
+__device__ __forceinline__ void project_store(const Lane<T> &L, const T (&X)[3], const M3<T> &Y,
+                                              T *__restrict__ ef, int64_t t)
+{
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const T r = project_parent(X[i], Y.a[i][0], Y.a[i][1], Y.a[i][2], L.s);
+        if (L.valid) ef[3 * t + i] = r;
+    }
+}
+
+// residual from (u_af, v_af, a_am, u_n), FP64
+__global__ void __launch_bounds__(128)
+    solid_residual_kernel(SolidArgs s, const double *__restrict__ u_af, const double *__restrict__ v_af,
+                          const double *__restrict__ a_am, const double *__restrict__ u_n,
+                          double *__restrict__ ef)
+{
+    using T = double;
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const Lane<T> L(s, t);
+    State<T> q;
+    solid_state<T>(s, L, u_af, u_n, q);
+    T S[6];
+    const T m0 = q.det0 * s.mu, l0 = q.det0 * s.lam * q.lnJ;
+#pragma unroll
+    for (int n = 0; n < 6; ++n) S[n] = m0 * q.e[n] + (n == 0 || n == 3 || n == 5 ? l0 : T(0));
+    M3<T> Y, W;
+    sym_times_kt<T, false>(S, q.K, Y);
+    const int64_t n3 = 3 * (int64_t)L.node;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) eval_parent<T, false>(v_af[n3 + i], L.s, W.a[i]);
+    viscous(W, q.Kn, q.det0 * s.mu_f * q.Jn, S);
+    sym_times_kt<T, true>(S, q.Kn, Y);
+    T X[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        T g[3];
+        X[i] = q.det0 * s.drho * (eval_parent<T, true>(a_am[n3 + i], L.s, g) - s.g[i]);
+    }
+    project_store(L, X, Y, ef, t);
+}
+
+// The tangent's state table, [element][value][Gauss point]: K, Kn, c_u mu b,
+// c_u (mu - lam ln J), c_v mu_f J_n and det J0, the stress terms times det J0
+constexpr int kState = 27;
+template <typename T>
+__global__ void __launch_bounds__(128)
+    solid_state_kernel(SolidArgs s, const T *__restrict__ u_af, const double *__restrict__ u_n,
+                       T *__restrict__ tab)
+{
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const Lane<T> L(s, t);
+    State<T> q;
+    solid_state<T>(s, L, u_af, u_n, q);
+    if (!L.valid) return;  // after the last shuffle
+    T *o = tab + L.e * (8 * kState) + (t & 7);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        o[8 * k] = q.K.a[k / 3][k % 3];
+        o[8 * (9 + k)] = q.Kn.a[k / 3][k % 3];
+    }
+    const T cu = (T)s.c_u * q.det0, m0 = cu * (T)s.mu;
+#pragma unroll
+    for (int n = 0; n < 6; ++n)
+        o[8 * (18 + n)] = m0 * (q.e[n] + (n == 0 || n == 3 || n == 5 ? T(1) : T(0)));
+    o[8 * 24] = m0 - cu * (T)s.lam * q.lnJ;
+    o[8 * 25] = q.det0 * (T)(s.c_v * s.mu_f) * q.Jn;
+    o[8 * 26] = q.det0;
+}
+
+// tangent apply along x from the state table
+template <typename T>
+__global__ void __launch_bounds__(128)
+    solid_tangent_kernel(SolidArgs s, const T *__restrict__ tab, const T *__restrict__ x,
+                         T *__restrict__ ef)
+{
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const Lane<T> L(s, t);
+    const T *o = tab + L.e * (8 * kState) + (t & 7);
+    M3<T> W, K, H, Y;
+    T X[3];
+    const T det0 = __ldg(o + 8 * 26);
+    const int64_t n3 = 3 * (int64_t)L.node;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+        X[i] = (T)(s.c_a * s.drho) * det0 * eval_parent<T, true>(x[n3 + i], L.s, W.a[i]);
+    // stress: S = mu H b + (mu - lam ln J) H^T + lam tr H I, H = W K
+#pragma unroll
+    for (int k = 0; k < 9; ++k) K.a[k / 3][k % 3] = __ldg(o + 8 * k);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+            H.a[i][j] = W.a[i][0] * K.a[0][j] + W.a[i][1] * K.a[1][j] + W.a[i][2] * K.a[2][j];
+    T b[6];
+#pragma unroll
+    for (int n = 0; n < 6; ++n) b[n] = __ldg(o + 8 * (18 + n));
+    const T c1 = __ldg(o + 8 * 24);
+    const T tr = (T)(s.c_u * s.lam) * det0 * (H.a[0][0] + H.a[1][1] + H.a[2][2]);
+    M3<T> S;
+    const int id[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            T v = c1 * H.a[j][i];
+            if (i == j) v += tr;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) v = fma(H.a[i][k], b[id[k][j]], v);
+            S.a[i][j] = v;
+        }
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            Y.a[i][k] = S.a[i][0] * K.a[k][0] + S.a[i][1] * K.a[k][1] + S.a[i][2] * K.a[k][2];
+    // artificial fluid, on the configuration at the start of the step
+#pragma unroll
+    for (int k = 0; k < 9; ++k) K.a[k / 3][k % 3] = __ldg(o + 8 * (9 + k));
+    T D[6];
+    viscous(W, K, __ldg(o + 8 * 25), D);
+    sym_times_kt<T, true>(D, K, Y);
+    project_store(L, X, Y, ef, t);
 }
 
 // R_b = sum of the element slots of node b (fixed order), overwrite
@@ -318,6 +429,9 @@ int grid_of(int64_t n, int threads = 128)
     return (int)(b < 1 ? 1 : (b > sm_count() * 32 ? sm_count() * 32 : b));
 }
 
+// eight lanes per element, 16 elements per CTA
+int lanes_grid(const fsi_solid *b) { return (int)((b->es + 15) / 16); }
+
 SolidArgs args_of(const fsi_solid *b, const double g[3])
 {
     const fsi_mesh *m = b->mesh;
@@ -345,29 +459,36 @@ fsi_status solid_residual_impl(fsi_solid *b, const double *u_af, const double *v
                                const double *a_am, const double *u_n, const double g[3], double *R)
 {
     cudaStream_t s = b->mesh->stream;
-    solid_elem_kernel<double, 0><<<grid_of(b->es), 128, 0, s>>>(
-        args_of(b, g), u_af, v_af, a_am, u_n, nullptr, (double *)b->elem_f);
+    solid_residual_kernel<<<lanes_grid(b), 128, 0, s>>>(args_of(b, g), u_af, v_af, a_am, u_n,
+                                                       (double *)b->elem_f);
     FSI_TRY(check_launch("solid element kernel"));
     solid_gather_kernel<double><<<grid_of(b->ns, 256), 256, 0, s>>>(
         b->ns, b->node_start, b->node_slot, (const double *)b->elem_f, R);
     return check_launch("solid gather kernel");
 }
 
-template <typename T>
-fsi_status solid_tangent_impl(fsi_solid *b, const T *u_af, const double *u_n, const T *x, T *Jx)
+// the tangent's state at (u_af, u_n) into the body's table
+template <typename T> fsi_status solid_linearise(fsi_solid *b, const T *u_af, const double *u_n)
+{
+    solid_state_kernel<T><<<lanes_grid(b), 128, 0, b->mesh->stream>>>(args_of(b, nullptr), u_af, u_n,
+                                                                     (T *)b->state);
+    return check_launch("solid state kernel");
+}
+// Jx = tangent x at the state of the last solid_linearise (same T)
+template <typename T> fsi_status solid_tangent_impl(fsi_solid *b, const T *x, T *Jx)
 {
     cudaStream_t s = b->mesh->stream;
-    solid_elem_kernel<T, 1><<<grid_of(b->es), 128, 0, s>>>(args_of(b, nullptr), u_af, nullptr,
-                                                          nullptr, u_n, x, (T *)b->elem_f);
+    solid_tangent_kernel<T><<<lanes_grid(b), 128, 0, s>>>(args_of(b, nullptr), (const T *)b->state, x,
+                                                         (T *)b->elem_f);
     FSI_TRY(check_launch("solid element kernel"));
     solid_gather_kernel<T><<<grid_of(b->ns, 256), 256, 0, s>>>(
         b->ns, b->node_start, b->node_slot, (const T *)b->elem_f, Jx);
     return check_launch("solid gather kernel");
 }
-template fsi_status solid_tangent_impl<double>(fsi_solid *, const double *, const double *,
-                                               const double *, double *);
-template fsi_status solid_tangent_impl<float>(fsi_solid *, const float *, const double *,
-                                              const float *, float *);
+template fsi_status solid_linearise<double>(fsi_solid *, const double *, const double *);
+template fsi_status solid_linearise<float>(fsi_solid *, const float *, const double *);
+template fsi_status solid_tangent_impl<double>(fsi_solid *, const double *, double *);
+template fsi_status solid_tangent_impl<float>(fsi_solid *, const float *, float *);
 
 fsi_status solid_stage_impl(fsi_solid *b, const double *u, const double *v, const double *a,
                             const double *a1, double *u_af, double *v_af, double *a_am)
@@ -432,7 +553,8 @@ fsi_status fsi_solid_create(fsi_mesh *mesh, int64_t n_nodes, int64_t n_elems, co
                {(void **)&b->conn, hconn.size() * sizeof(int32_t)},
                {(void **)&b->node_start, start.size() * sizeof(int32_t)},
                {(void **)&b->node_slot, slot.size() * sizeof(int32_t)},
-               {&b->elem_f, (size_t)n_elems * 24 * sizeof(double)}};
+               {&b->elem_f, (size_t)n_elems * 24 * sizeof(double)},
+               {&b->state, (size_t)n_elems * 8 * kState * sizeof(double)}};
     for (auto &r : req) {
         if (cudaMalloc(r.p, r.bytes) != cudaSuccess) {
             cudaGetLastError();
@@ -467,6 +589,7 @@ void fsi_solid_destroy(fsi_solid *b)
     cudaFree(b->node_start);
     cudaFree(b->node_slot);
     cudaFree(b->elem_f);
+    cudaFree(b->state);
     delete b;
 }
 
@@ -488,10 +611,12 @@ fsi_status fsi_solid_tangent_apply(fsi_solid *b, fsi_prec prec, const void *u_af
         return set_error(FSI_ERR_ARG, "fsi_solid_tangent_apply: NULL argument");
     if (prec != FSI_F64 && prec != FSI_F32) return set_error(FSI_ERR_ARG, "bad precision");
     FSI_DEVICE(b->mesh->device);
-    if (prec == FSI_F64)
-        return solid_tangent_impl<double>(b, (const double *)u_af, u_n, (const double *)x,
-                                          (double *)Jx);
-    return solid_tangent_impl<float>(b, (const float *)u_af, u_n, (const float *)x, (float *)Jx);
+    if (prec == FSI_F64) {
+        FSI_TRY(solid_linearise<double>(b, (const double *)u_af, u_n));
+        return solid_tangent_impl<double>(b, (const double *)x, (double *)Jx);
+    }
+    FSI_TRY(solid_linearise<float>(b, (const float *)u_af, u_n));
+    return solid_tangent_impl<float>(b, (const float *)x, (float *)Jx);
 }
 
 fsi_status fsi_solid_stage(fsi_solid *b, const double *u, const double *v, const double *a,
