@@ -211,10 +211,15 @@ struct TcGemm {
     const float *bias;  // [N] for TC_EPI_BIAS / TC_EPI_BIAS_RELU
     float *Cpre;        // pre-activation output for TC_EPI_BIAS_RELU (may be null)
     const float *mask;  // [M x N] (ldc) for TC_EPI_MASK: C *= (mask > 0)
-    int BN;             // set by tc_gemm: N rounded up to a multiple of 16
+    // set by tc_gemm: tile columns, K slices and their workspace, which operands
+    // (1: A, 2: B, 4: C) move in 16-byte pieces
+    int BN, splits, vec;
+    float *work;
 };
 size_t tc_gemm_work_floats();
 fsi_status tc_gemm(cudaStream_t s, const TcGemm &g, float *work, int *err);
+// up to three independent GEMMs in one launch
+fsi_status tc_gemm_group(cudaStream_t s, const TcGemm *g, int n, float *work, int *err);
 
 // fused tensor-core inference of the initial-guess network (mlp_tc.cu)
 size_t mlp_tc_packed_bytes();

@@ -55,7 +55,8 @@ TcGemm ga(int M, int N, int K, const float *A, int64_t lda, int tA, const float 
     g.A = A; g.lda = lda; g.transA = tA;
     g.B = B; g.ldb = ldb; g.transB = tB;
     g.C = C; g.ldc = ldc; g.epi = epi; g.bias = bias; g.Cpre = Cpre; g.mask = mask;
-    g.BN = 0;
+    g.BN = g.splits = g.vec = 0;
+    g.work = nullptr;
     return g;
 }
 
@@ -80,30 +81,34 @@ __global__ void loss_kernel(int64_t B, const float *O, const float *T, float *dO
     if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
 }
 
-__global__ void loss_final_kernel(int nb, const double *partial, float *loss)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int b = 0; b < nb; ++b) s += partial[b];
-        *loss = (float)s;
-    }
-}
-
-// db[j] = sum_i dZ[i][j] in two passes with a fixed order: CTA (cx, r) sums
-// its row slice of columns 32 cx .. 32 cx + 31 (thread (x, y): rows y, y + 8,
-// ... of the slice, then a tree over y) into part[r][j]; then the slices are
-// added in order.  FP32 sums of at most a few thousand rows.
+// The three bias gradients db[j] = sum_i dZ[i][j] in two passes with a fixed
+// order: CTA (cx, r) sums its row slice of 32 columns (thread (x, y): rows y, y +
+// 8, ... of the slice, then a tree over y) into part[r][j]; then the slices are
+// added in order.  FP32 sums of at most a few thousand rows.  One launch for the
+// three matrices each way; the second also sums the loss.
 constexpr int kColSlices = 16;
+struct ColSums {
+    const float *dZ[3];
+    float *db[3];
+    int N[3], col0[3];  // columns, and where a matrix's columns start in part
+    int cta0[4];        // column CTAs (32 columns each) of matrix q: cta0[q] ..
+    int cols;           // all columns
+};
 
-__global__ void colsum_partial_kernel(int64_t M, int N, const float *dZ, float *part)
+__global__ void colsum_partial_kernel(int64_t M, ColSums c, float *part)
 {
     __shared__ float red[8][33];
+    int q = 0;
+    while (q < 2 && (int)blockIdx.x >= c.cta0[q + 1]) ++q;
+    const int N = c.N[q];
+    const float *dZ = c.dZ[q];
     const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
-    const int j = blockIdx.x * 32 + x;
+    const int j = (blockIdx.x - c.cta0[q]) * 32 + x;
     const int64_t per = (M + gridDim.y - 1) / gridDim.y;
     const int64_t r0 = blockIdx.y * per, r1 = min(M, r0 + per);
     float acc = 0.f;
     if (j < N)
+#pragma unroll 8
         for (int64_t i = r0 + y; i < r1; i += 8) acc += dZ[i * N + j];
     red[y][x] = acc;
     __syncthreads();
@@ -111,16 +116,36 @@ __global__ void colsum_partial_kernel(int64_t M, int N, const float *dZ, float *
         if (y < st) red[y][x] += red[y + st][x];
         __syncthreads();
     }
-    if (y == 0 && j < N) part[(int64_t)blockIdx.y * N + j] = red[0][x];
+    if (y == 0 && j < N) part[(int64_t)blockIdx.y * c.cols + c.col0[q] + j] = red[0][x];
 }
 
-__global__ void colsum_final_kernel(int N, int slices, const float *part, float *db)
+// bias gradients from the slices (CTAs 1 ..), loss from its nb partial sums
+// (CTA 0: 256 threads, a fixed tree)
+__global__ void grad_final_kernel(ColSums c, int slices, const float *part, int nb,
+                                  const double *partial, float *loss)
 {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= N) return;
+    if (blockIdx.x == 0) {
+        __shared__ double red[256];
+        double v = 0.0;
+        for (int b = threadIdx.x; b < nb; b += 256) v += partial[b];
+        red[threadIdx.x] = v;
+        __syncthreads();
+        for (int s = 128; s > 0; s >>= 1) {
+            if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) *loss = (float)red[0];
+        return;
+    }
+    const int k = (blockIdx.x - 1) * 256 + threadIdx.x;
+    if (k >= c.cols) return;
+    int q = 0;
+    while (q < 2 && k >= c.col0[q + 1]) ++q;
     float s = 0.f;
-    for (int r = 0; r < slices; ++r) s += part[(int64_t)r * N + j];
-    db[j] = s;
+#pragma unroll
+    for (int r = 0; r < kColSlices; ++r) s += part[(int64_t)r * c.cols + k];
+    (void)slices;
+    c.db[q][k - c.col0[q]] = s;
 }
 
 __global__ void adam_kernel(int64_t n, float *p, const float *g, float *m, float *v, float lr,
@@ -168,22 +193,6 @@ __global__ void features_kernel(int Nx, int Ny, int Nz, int64_t base, int64_t k,
             const int f = 108 + c;
             const double e = 2.0 * d1[4 * (int64_t)node + c] - d2[4 * (int64_t)node + c];
             x[f] = (float)((e - mean[f]) / stdv[f]);
-        }
-    }
-}
-
-// y0 = y + e + (mean_c + std_c * O) for nodes [base, base + k)
-__global__ void predict_combine_kernel(int64_t base, int64_t k, const double *y, const double *d1,
-                                       const double *d2, const float *O, const float *omean,
-                                       const float *ostd, double *y0)
-{
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < k;
-         r += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t node = base + r;
-        for (int c = 0; c < 4; ++c) {
-            const int64_t q = 4 * node + c;
-            const double e = 2.0 * d1[q] - d2[q];
-            y0[q] = y[q] + e + ((double)omean[c] + (double)ostd[c] * (double)O[r * NO + c]);
         }
     }
 }
@@ -358,16 +367,6 @@ int blocks(int64_t n, int threads = 256, int cap = sm_count() * 16)
     return (int)(b < 1 ? 1 : (b > cap ? cap : b));
 }
 
-// db = column sums of dZ [M][N] (the bias gradient), through the split-K
-// workspace (free between GEMMs in stream order)
-fsi_status colsum(const fsi_mlp *h, int64_t M, int N, const float *dZ, float *db)
-{
-    dim3 grid((N + 31) / 32, kColSlices);
-    colsum_partial_kernel<<<grid, 256, 0, h->stream>>>(M, N, dZ, h->gemm_work);
-    colsum_final_kernel<<<(N + 255) / 256, 256, 0, h->stream>>>(N, kColSlices, h->gemm_work, db);
-    return check_launch("bias gradient");
-}
-
 fsi_status forward_impl(fsi_mlp *h, const float *P, const float *X, int64_t B, bool keep)
 {
     FSI_TRY(gemm(h, ga((int)B, NH, NI, X, NI, 0, P + OFF_W1, NH, 0, h->H1, NH, EPI_BIAS_RELU,
@@ -481,22 +480,30 @@ fsi_status fsi_mlp_loss_grad(fsi_mlp *h, const float *params, const float *X, co
     FSI_TRY(forward_impl(h, P, X, B, true));
     const int nb = 256;
     loss_kernel<<<nb, 256, 0, s>>>(B, h->O, T, h->dO, h->loss_partial);
-    loss_final_kernel<<<1, 32, 0, s>>>(nb, h->loss_partial, loss);
-    FSI_TRY(check_launch("loss kernels"));
+    FSI_TRY(check_launch("loss kernel"));
     const int M = (int)B;
-    // layer 3: dW3 = H2^T dO, db3 = colsum(dO), dZ2 = (dO W3^T) * (Z2 > 0)
-    FSI_TRY(gemm(h, ga(NH, NO, M, h->H2, NH, 1, h->dO, NO, 0, grad + OFF_W3, NO)));
-    FSI_TRY(colsum(h, B, NO, h->dO, grad + OFF_b3));
+    // dZ2 = (dO W3^T) * (Z2 > 0), dZ1 = (dZ2 W2^T) * (Z1 > 0)
     FSI_TRY(gemm(h, ga(M, NH, NO, h->dO, NO, 0, P + OFF_W3, NO, 1, h->dZ2, NH, EPI_MASK,
                        nullptr, nullptr, h->Z2)));
-    // layer 2: dW2 = H1^T dZ2, db2, dZ1 = (dZ2 W2^T) * (Z1 > 0)
-    FSI_TRY(gemm(h, ga(NH, NH, M, h->H1, NH, 1, h->dZ2, NH, 0, grad + OFF_W2, NH)));
-    FSI_TRY(colsum(h, B, NH, h->dZ2, grad + OFF_b2));
     FSI_TRY(gemm(h, ga(M, NH, NH, h->dZ2, NH, 0, P + OFF_W2, NH, 1, h->dZ1, NH, EPI_MASK,
                        nullptr, nullptr, h->Z1)));
-    // layer 1: dW1 = X^T dZ1, db1
-    FSI_TRY(gemm(h, ga(NI, NH, M, X, NI, 1, h->dZ1, NH, 0, grad + OFF_W1, NH)));
-    return colsum(h, B, NH, h->dZ1, grad + OFF_b1);
+    // dW2 = H1^T dZ2, dW1 = X^T dZ1, dW3 = H2^T dO in one launch
+    const TcGemm dW[3] = {ga(NH, NH, M, h->H1, NH, 1, h->dZ2, NH, 0, grad + OFF_W2, NH),
+                          ga(NI, NH, M, X, NI, 1, h->dZ1, NH, 0, grad + OFF_W1, NH),
+                          ga(NH, NO, M, h->H2, NH, 1, h->dO, NO, 0, grad + OFF_W3, NO)};
+    FSI_TRY(tc_gemm_group(s, dW, 3, h->gemm_work, h->tc_err));
+    // db1, db2, db3 and the loss
+    const ColSums c = {{h->dZ1, h->dZ2, h->dO},
+                       {grad + OFF_b1, grad + OFF_b2, grad + OFF_b3},
+                       {NH, NH, NO},
+                       {0, NH, 2 * NH},
+                       {0, NH / 32, 2 * (NH / 32), 2 * (NH / 32) + 1},
+                       2 * NH + NO};
+    float *part = h->gemm_work;  // the split-K workspace, free again in stream order
+    colsum_partial_kernel<<<dim3(c.cta0[3], kColSlices), 256, 0, s>>>(B, c, part);
+    grad_final_kernel<<<1 + (c.cols + 255) / 256, 256, 0, s>>>(c, kColSlices, part, nb,
+                                                              h->loss_partial, loss);
+    return check_launch("bias gradients");
 }
 
 fsi_status fsi_mlp_adam(fsi_mlp *h, float *params, const float *grad, float *m, float *v,
