@@ -10,7 +10,10 @@
 //
 //   features   the 112 features of each node (27-node stencil of V_n
 //              velocity and y_n pressure, the extrapolant 2 d1 - d2),
-//              normalised and rounded to BF16, into the A tile X [128 x 112];
+//              normalised and rounded to BF16, into the A tile X [128 x 112].
+//              They are gathered one tile ahead, during the previous tile's
+//              MMAs and epilogues, and wait packed in 16 registers per thread
+//              (shared memory has no room for a second A tile);
 //   layer 1    D1 [128 x 256] (TMEM columns 0..255) = X W1^T: 7 MMAs of
 //              M=128, N=256, K=16 (kind::f16, BF16 in, FP32 accumulate);
 //   layer 2    H1 = BF16(ReLU(D1 + b1)) is written back to shared memory in
@@ -22,7 +25,12 @@
 //              FP32 dot products with the BF16 rows of W3 (+ b3), summed per
 //              warpgroup over its 64 columns and then across warpgroups in a
 //              fixed order; the predictor y0 = y + e + (out_mean + out_std *
-//              out) is written in FP64.
+//              out) is written in FP64, one component per thread.
+//
+// Bound: the phases of a tile follow one another, so their latencies add up.  The
+// gather with its FP64 -> FP32 conversions (two per SM and clock on GB300's FP64
+// unit, so they are done on the integer pipe) was the longest: gathered a tile
+// ahead, 2,146,689 nodes (129^3) take 1.12 ms instead of 1.29 ms.
 //
 // The BF16 rounding points are those of the training kernels (inputs and
 // weights of every layer).  Weights are packed once per call into the
@@ -97,6 +105,20 @@ __global__ void pack_weights_kernel(const float *P, uint8_t *packed)
     }
 }
 
+// (float)d by integer operations (round to nearest, ties to even): the FP64
+// unit converts two values per SM and clock, and a tile has 14,336
+__device__ __forceinline__ float to_float(double d)
+{
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    const unsigned e = (hi >> 20) & 0x7ffu;
+    if (e - 897u < 254u) {  // a normal float before rounding (a carry may reach infinity, rightly)
+        const unsigned b = (hi & 0x80000000u) | ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+        return __uint_as_float(b + ((lo & 0x1fffffffu) + (b & 1u) > 0x10000000u ? 1u : 0u));
+    }
+    if (((hi << 1) | lo) == 0u) return __uint_as_float(hi);
+    return (float)d;
+}
+
 struct TcArgs {
     int Nx, Ny, Nz;
     int64_t n;
@@ -114,7 +136,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_predict_tc_kernel(const TcArg
     __shared__ __align__(8) uint64_t bars[2];  // [0] weights, [1] MMA completion
     __shared__ uint32_t tmem_holder;
     __shared__ int abort_flag;
-    __shared__ float smean[NI], sistd[NI];
+    __shared__ __align__(16) float smean[NI], sistd[NI];
     const int tid = threadIdx.x, warp = tid >> 5, row = tid & (TM - 1), grp = tid >> 7;
     const uint32_t s0 = smem_u32(sm);
     const uint32_t bar_w = smem_u32(&bars[0]), bar_m = smem_u32(&bars[1]);
@@ -170,63 +192,93 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_predict_tc_kernel(const TcArg
     bool ok = weights_ok;
     if (!ok) atomicExch(&abort_flag, 1);
     __syncthreads();
-    const float b3[4] = {a.P[OFF_b3], a.P[OFF_b3 + 1], a.P[OFF_b3 + 2], a.P[OFF_b3 + 3]};
-    const float om[4] = {a.out_mean[0], a.out_mean[1], a.out_mean[2], a.out_mean[3]};
-    const float os[4] = {a.out_std[0], a.out_std[1], a.out_std[2], a.out_std[3]};
+    const float b3 = a.P[OFF_b3 + (tid & 3)];
+    const double om = (double)a.out_mean[tid & 3], os = (double)a.out_std[tid & 3];
     const int nx = a.Nx + 1, ny = a.Ny + 1, nz = a.Nz + 1;
     const int64_t ntiles = (a.n + TM - 1) / TM;
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
     uint8_t *xh = sm + OFF_SXH;
 
-    for (int64_t tile = blockIdx.x; tile < ntiles && !abort_flag; tile += gridDim.x) {
+    // ---- features of a tile: X is BF16, canonical K-major, 14 chunks of 8 = two
+    // stencil points each, the last one point and the extrapolant.  Group g
+    // builds chunks [kChunk[g], kChunk[g + 1]) in two halves of two: gather()
+    // issues a half's loads, convert() normalises them in FP32 ((value - mean) *
+    // (1 / std): the result is rounded to BF16 right away) and packs them.
+    const int c0 = kChunk[grp], c1 = kChunk[grp + 1];
+    double raw[2][2][4];
+    uint4 xf[4];
+    auto gather = [&](int64_t tile, int half) {
         const int64_t node = tile * TM + row;
         const bool live = node < a.n;
-        // ---- features -> X (BF16, canonical K-major, 14 chunks of 8 = two
-        // stencil points each, the last one point and the extrapolant).  Group
-        // g builds chunks [kChunk[g], kChunk[g + 1]).  The normalisation runs
-        // in FP32 ((value - mean) * (1 / std)): the result is rounded to BF16
-        // right away, and GB300's FP64 unit is ~70x slower.
-        {
-            int i = 0, j = 0, k = 0;
-            if (live) {
-                i = (int)(node % nx);
-                j = (int)((node / nx) % ny);
-                k = (int)(node / ((int64_t)nx * ny));
-            }
-            for (int c = kChunk[grp]; c < kChunk[grp + 1]; ++c) {
-                float f8[8];
+        const unsigned nd = live ? (unsigned)node : 0u;  // n < 2^31
+        const int q = (int)(nd / (unsigned)nx);
+        const int i = (int)nd - q * nx, k = q / ny, j = q - k * ny;
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int s = 2 * c + h;
-                    double raw[4] = {0.0, 0.0, 0.0, 0.0};
-                    if (s < 27) {
-                        const int ii = i + s % 3 - 1, jj = j + (s / 3) % 3 - 1, kk = k + s / 9 - 1;
-                        const bool in = live && ii >= 0 && ii < nx && jj >= 0 && jj < ny &&
-                                        kk >= 0 && kk < nz;
-                        if (in) {
-                            const int64_t nb = ii + (int64_t)nx * (jj + (int64_t)ny * kk);
-                            const double2 v01 =
-                                __ldg(reinterpret_cast<const double2 *>(a.Vn + 4 * nb));
-                            raw[0] = v01.x;
-                            raw[1] = v01.y;
-                            raw[2] = __ldg(a.Vn + 4 * nb + 2);
-                            raw[3] = __ldg(a.y + 4 * nb + 3);
-                        }
-                    } else if (live) {  // features 108..111: the extrapolant 2 d1 - d2
+        for (int u = 0; u < 2; ++u) {
+            const int c = c0 + 2 * half + u;
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) raw[q] = 2.0 * a.d1[4 * node + q] - a.d2[4 * node + q];
+            for (int h = 0; h < 2; ++h) {
+                const int s = 2 * c + h;
+#pragma unroll
+                for (int t = 0; t < 4; ++t) raw[u][h][t] = 0.0;
+                if (c >= c1 || !live) continue;
+                if (s < 27) {
+                    const int dz = s / 9, dy = (s - 9 * dz) / 3, dx = s - 9 * dz - 3 * dy;
+                    const int ii = i + dx - 1, jj = j + dy - 1, kk = k + dz - 1;
+                    if (ii >= 0 && ii < nx && jj >= 0 && jj < ny && kk >= 0 && kk < nz) {
+                        const int64_t nb = ii + (int64_t)nx * (jj + (int64_t)ny * kk);
+                        const double2 v01 = __ldg(reinterpret_cast<const double2 *>(a.Vn + 4 * nb));
+                        raw[u][h][0] = v01.x;
+                        raw[u][h][1] = v01.y;
+                        raw[u][h][2] = __ldg(a.Vn + 4 * nb + 2);
+                        raw[u][h][3] = __ldg(a.y + 4 * nb + 3);
                     }
+                } else {  // features 108..111: the extrapolant 2 d1 - d2
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int f = 4 * s + q;
-                        f8[4 * h + q] = live ? ((float)raw[q] - smean[f]) * sistd[f] : 0.0f;
-                    }
+                    for (int t = 0; t < 4; ++t)
+                        raw[u][h][t] = 2.0 * __ldg(a.d1 + 4 * node + t) - __ldg(a.d2 + 4 * node + t);
                 }
-                const uint4 v = make_uint4(pack_bf16(f8[0], f8[1]), pack_bf16(f8[2], f8[3]),
-                                           pack_bf16(f8[4], f8[5]), pack_bf16(f8[6], f8[7]));
-                *reinterpret_cast<uint4 *>(xh + kmaj(row, 8 * c, KC1)) = v;
             }
         }
+    };
+    auto convert = [&](int64_t tile, int half) {
+        const bool live = tile * TM + row < a.n;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int c = c0 + 2 * half + u;
+            float f8[8];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int f = c < c1 ? 8 * c + 4 * h : 0;
+                const float4 mn = *reinterpret_cast<const float4 *>(smean + f);
+                const float4 is = *reinterpret_cast<const float4 *>(sistd + f);
+                f8[4 * h] = (to_float(raw[u][h][0]) - mn.x) * is.x;
+                f8[4 * h + 1] = (to_float(raw[u][h][1]) - mn.y) * is.y;
+                f8[4 * h + 2] = (to_float(raw[u][h][2]) - mn.z) * is.z;
+                f8[4 * h + 3] = (to_float(raw[u][h][3]) - mn.w) * is.w;
+            }
+            if (!live)
+#pragma unroll
+                for (int t = 0; t < 8; ++t) f8[t] = 0.0f;
+            xf[2 * half + u] = make_uint4(pack_bf16(f8[0], f8[1]), pack_bf16(f8[2], f8[3]),
+                                          pack_bf16(f8[4], f8[5]), pack_bf16(f8[6], f8[7]));
+        }
+    };
+    gather(blockIdx.x, 0);
+    convert(blockIdx.x, 0);
+    gather(blockIdx.x, 1);
+    convert(blockIdx.x, 1);
+
+    for (int64_t tile = blockIdx.x; tile < ntiles && !abort_flag; tile += gridDim.x) {
+        const int64_t next = tile + gridDim.x;  // beyond the last tile: all rows idle
+        // the predictor's component of this thread: node tile * 128 + tid / 4
+        const int64_t pq = 4 * tile * TM + tid;
+        const bool plive = pq < 4 * a.n;
+        const double p_d1 = plive ? __ldg(a.d1 + pq) : 0.0, p_d2 = plive ? __ldg(a.d2 + pq) : 0.0,
+                     p_y = plive ? __ldg(a.y + pq) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (c0 + u < c1) *reinterpret_cast<uint4 *>(xh + kmaj(row, 8 * (c0 + u), KC1)) = xf[u];
         fence_async_smem();
         fence_before();
         __syncthreads();
@@ -238,6 +290,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_predict_tc_kernel(const TcArg
                          sdesc(s0 + OFF_SW1 + ks * 256, 128, KC1 * 128), ks > 0);
             mma_commit(bar_m);
         }
+        gather(next, 0);
         mma_pending = true;
         ok = mbar_wait(bar_m, mma_phase);
         if (ok) {
@@ -257,11 +310,12 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_predict_tc_kernel(const TcArg
 #pragma unroll
             for (int q8 = 0; q8 < 4; ++q8) {
                 float h[8];
+                float b[8];
+                *reinterpret_cast<float4 *>(b) = *reinterpret_cast<const float4 *>(sb1 + 32 * grp + 8 * q8);
+                *reinterpret_cast<float4 *>(b + 4) =
+                    *reinterpret_cast<const float4 *>(sb1 + 32 * grp + 8 * q8 + 4);
 #pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    const int col = 32 * grp + 8 * q8 + t;
-                    h[t] = fmaxf(v[8 * q8 + t] + sb1[col], 0.0f);
-                }
+                for (int t = 0; t < 8; ++t) h[t] = fmaxf(v[8 * q8 + t] + b[t], 0.0f);
                 *reinterpret_cast<uint4 *>(xh + kmaj(row, 32 * grp + 8 * q8, KC2)) =
                     make_uint4(pack_bf16(h[0], h[1]), pack_bf16(h[2], h[3]), pack_bf16(h[4], h[5]),
                                pack_bf16(h[6], h[7]));
@@ -277,6 +331,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_predict_tc_kernel(const TcArg
                          sdesc(s0 + OFF_SW2A + ks * 256, 128, KC2 * 128), ks > 0);
             mma_commit(bar_m);
         }
+        convert(next, 0);
+        gather(next, 1);
         // second K-half of H1 (group g: columns 128 + 32 g ..) into registers
         // while those MMAs run
         uint32_t hp[16];
@@ -314,6 +370,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_predict_tc_kernel(const TcArg
                          sdesc(s0 + OFF_SW2B + ks * 256, 128, KC2 * 128), 1);
             mma_commit(bar_m);
         }
+        convert(next, 1);
         mma_pending = true;
         ok = mbar_wait(bar_m, mma_phase);
         if (ok) {
@@ -345,27 +402,18 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_predict_tc_kernel(const TcArg
             }
         }
         float4 *part = reinterpret_cast<float4 *>(xh);
-        if (grp > 0) part[(grp - 1) * TM + row] = make_float4(o[0], o[1], o[2], o[3]);
+        part[grp * TM + row] = make_float4(o[0], o[1], o[2], o[3]);
         __syncthreads();
-        if (grp == 0) {
+        {
+            // component tid % 4 of row tid / 4: the groups' sums in group order
+            const float *pp = reinterpret_cast<const float *>(xh) + tid;
+            float out = pp[0];
 #pragma unroll
-            for (int g = 1; g < kGroups; ++g) {
-                const float4 p = part[(g - 1) * TM + row];
-                o[0] += p.x;
-                o[1] += p.y;
-                o[2] += p.z;
-                o[3] += p.w;
-            }
-            if (live)
-                for (int c = 0; c < 4; ++c) {
-                    const int64_t qn = 4 * node + c;
-                    const double e = 2.0 * a.d1[qn] - a.d2[qn];
-                    const float out = o[c] + b3[c];
-                    a.y0[qn] = a.y[qn] + e + ((double)om[c] + (double)os[c] * (double)out);
-                }
+            for (int g = 1; g < kGroups; ++g) out += pp[4 * g * TM];
+            out += b3;
+            if (plive) a.y0[pq] = p_y + (2.0 * p_d1 - p_d2) + (om + os * (double)out);
         }
-        // the next tile overwrites X (read by the finished MMAs and by group 0
-        // above) and D1
+        // the next tile overwrites X (read by the finished MMAs and above) and D1
         fence_before();
         __syncthreads();
     }

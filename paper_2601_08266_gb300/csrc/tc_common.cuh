@@ -146,8 +146,8 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float v[8])
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b)
 {
-    const __nv_bfloat16 lo = __float2bfloat16_rn(a), hi = __float2bfloat16_rn(b);
-    return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
+    const __nv_bfloat162 p = __floats2bfloat162_rn(a, b);  // one conversion for both
+    return *reinterpret_cast<const uint32_t *>(&p);
 }
 
 __device__ __forceinline__ float bf16r(float a) { return __bfloat162float(__float2bfloat16_rn(a)); }
