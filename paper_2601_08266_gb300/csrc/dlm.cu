@@ -727,21 +727,21 @@ __global__ void __launch_bounds__(1024) dense_pairs_kernel(int64_t E, int64_t m,
 // --------------------------------------------------------------- interp / spread
 // FP32: two lanes per point (interp_point_pair; the loop bound is
 // warp-uniform); double-float and FP64: one lane per point
-template <typename T, typename S = typename StorageOf<T>::type>
+template <typename T, bool SCALED = false, typename S = typename StorageOf<T>::type>
 __global__ void interp_kernel(int64_t m, GridArgs g, const int32_t *__restrict__ elem,
                               const S *__restrict__ xi, const vec4<S> *__restrict__ U,
-                              S *__restrict__ u)
+                              S *__restrict__ u, S D = 1)
 {
     if constexpr (std::is_same<T, float>::value) {
         const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
         const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
         const int pair = (threadIdx.x & 31) >> 1;
         for (int64_t b0 = warp * 16; b0 < m; b0 += nwarps * 16)
-            interp_point_pair<T>(g, b0 + pair, b0 + pair < m, elem, xi, U, u);
+            interp_point_pair<T, SCALED>(g, b0 + pair, b0 + pair < m, elem, xi, U, u, D);
     } else {
         for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < m;
              b += (int64_t)gridDim.x * blockDim.x)
-            interp_point<T>(g, b, elem, xi, U, u);
+            interp_point<T, SCALED>(g, b, elem, xi, U, u, D);
     }
 }
 
@@ -943,6 +943,21 @@ template fsi_status spread_mass_diag<float>(fsi_mesh *, int64_t, const float *, 
 template fsi_status spread_mass_diag<double>(fsi_mesh *, int64_t, const double *,
                                              const int32_t *, const int32_t *, const double *,
                                              double, double *);
+
+template <typename T>
+fsi_status interp_scaled(fsi_mesh *mesh, int64_t m, const int32_t *elem, const T *xi, const T *U,
+                         T D, T *u)
+{
+    if (m == 0) return FSI_OK;
+    const int64_t lanes = sizeof(T) == 4 ? 2 * m : m;
+    interp_kernel<T, true><<<blocks_for(lanes, 256), 256, 0, mesh->stream>>>(
+        m, grid_args(mesh), elem, xi, (const vec4<T> *)U, u, D);
+    return check_launch("interp kernel");
+}
+template fsi_status interp_scaled<float>(fsi_mesh *, int64_t, const int32_t *, const float *,
+                                         const float *, float, float *);
+template fsi_status interp_scaled<double>(fsi_mesh *, int64_t, const int32_t *, const double *,
+                                          const double *, double, double *);
 
 }  // namespace fsi
 

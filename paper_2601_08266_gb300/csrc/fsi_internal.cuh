@@ -244,6 +244,11 @@ template <typename T>
 fsi_status spread_mass_diag(fsi_mesh *mesh, int64_t m, const T *xi, const int32_t *cell_start,
                             const int32_t *perm, const T *w, double dsq, T *F);
 
+// u = D C^T U at the points (dlm.cu; the interpolation, then the product, in T)
+template <typename T>
+fsi_status interp_scaled(fsi_mesh *mesh, int64_t m, const int32_t *elem, const T *xi, const T *U,
+                         T D, T *u);
+
 // the checks fsi_newton_step makes of a step state (newton.cu)
 fsi_status validate_step_state(const fsi_mesh *mesh, const fsi_step_state *st);
 

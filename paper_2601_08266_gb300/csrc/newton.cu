@@ -224,12 +224,73 @@ template <> struct DotAcc<float> {
     using type = Comp;
 };
 
+// Sums of kDotGroup values over a warp: each level halves the values a lane
+// carries, so the warp issues 9 FP64 additions instead of 40 (an FP64 addition
+// takes 16 cycles of a GB300 SM, and at 32^3 the 40 were most of the kernel: with
+// them, and 456 CTAs at every length, 15.9 us a launch and 7.9 us for the two small
+// launches behind it; now 10.4 us with everything).  Lanes with equal bits 2..4 end with value (bit 4, bit 3, bit 2).
+__device__ __forceinline__ double warp_sums8(double (&v)[kDotGroup], int lane)
+{
+    static_assert(kDotGroup == 8, "three halving levels");
+    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const double send = b4 ? v[k] : v[4 + k], keep = b4 ? v[4 + k] : v[k];
+        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const double send = b3 ? v[k] : v[2 + k], keep = b3 ? v[2 + k] : v[k];
+        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+    }
+    const double send = b2 ? v[0] : v[1], keep = b2 ? v[1] : v[0];
+    double t = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+    t += __shfl_xor_sync(0xffffffffu, t, 2);
+    return t + __shfl_xor_sync(0xffffffffu, t, 1);
+}
+
+// True in every thread of the CTA that finishes last; its partial sums and
+// everyone else's are then visible.  `ticket` counts the CTAs up and wraps to
+// zero by itself, so it needs no clearing; no CTA waits for another.
+__device__ __forceinline__ bool last_cta(unsigned *ticket)
+{
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
+// Kahan's test: 1 when |h[0..j]|^2 > |w|^2 / 2 (w . w in h[j + 1]), i.e. the
+// classical Gram-Schmidt pass lost orthogonality and a second pass is due; one
+// warp, lanes sum in a fixed order
+__device__ __forceinline__ void kahan_flag(int j, const volatile double *h, double *flag)
+{
+    double v = 0.0;
+    for (int i = threadIdx.x & 31; i <= j; i += 32) v += h[i] * h[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) *flag = (v <= 0.5 * h[j + 1]) ? 0.0 : 1.0;
+}
+
+// What the last CTA of a multi-dot launch does with the sums: mode 0 stores
+// them, 1 stores the square root (a norm); with kahan_j >= 0 (the launch of the
+// last group) Kahan's flag of the column h[0 .. kahan_j + 1] = out.
+struct DotFinal {
+    unsigned *ticket;
+    double *out;
+    int mode, kahan_j;
+    double *flag;
+};
+
 // (index self_k, when in [k0, k0+cnt), stands for w itself: w . w)
 // (cond, when not null, is a device flag: the kernel does nothing when it is 0)
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads, 3) multi_dot_partial_kernel(
     int k0, int cnt, int64_t len4, const vec4<T> *V, int64_t vstride, const vec4<T> *w,
-    double *partial, int self_k, const double *cond)
+    double *partial, int self_k, const double *cond, DotFinal fin)
 {
     if (cond && *cond == 0.0) return;
     using Acc = typename DotAcc<T>::type;
@@ -285,44 +346,34 @@ __global__ void __launch_bounds__(kRedThreads, 3) multi_dot_partial_kernel(
         }
     }
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    double v[kDotGroup];
 #pragma unroll
-    for (int j = 0; j < kDotGroup; ++j) {
-        double v = dot_value(acc[j]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) red[j][wid] = v;
-    }
+    for (int j = 0; j < kDotGroup; ++j) v[j] = dot_value(acc[j]);
+    const double t = warp_sums8(v, lane);
+    if ((lane & 3) == 0) red[lane >> 2][wid] = t;
     __syncthreads();
     if (threadIdx.x < cnt) {
         double v = 0.0;
         for (int q = 0; q < kRedThreads / 32; ++q) v += red[threadIdx.x][q];
         partial[(int64_t)(k0 + threadIdx.x) * kRedGrid + blockIdx.x] = v;
     }
-}
-
-// out[k] (+)= sum_b partial[k][b] for k < cnt; one block per k, fixed tree.
-// mode 0: store, 1: add, 2: store sqrt (norm)
-// (nb partials per k, rows kRedGrid apart)
-__global__ void multi_dot_final_kernel(int cnt, const double *partial, double *out, int mode,
-                                       const double *cond = nullptr, int nb = kRedGrid)
-{
-    if (cond && *cond == 0.0) return;
-    __shared__ double red[kRedThreads];
-    const int k = blockIdx.x;
-    double v = 0.0;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) v += partial[(int64_t)k * kRedGrid + b];
-    red[threadIdx.x] = v;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
+    // the last CTA adds up the CTAs' partial sums, one warp per vector, in a
+    // fixed order (a launch of its own for this cost a few microseconds per
+    // Krylov iteration)
+    if (!last_cta(fin.ticket)) return;
+    if (wid < cnt) {
+        const volatile double *p = partial + (int64_t)(k0 + wid) * kRedGrid;
+        double a = 0.0;
+        for (int b = lane; b < (int)gridDim.x; b += 32) a += p[b];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (lane == 0) fin.out[k0 + wid] = fin.mode ? sqrt(a) : a;
+    }
+    if (fin.kahan_j >= 0) {
+        __threadfence();
         __syncthreads();
+        if (wid == 0) kahan_flag(fin.kahan_j, fin.out, fin.flag);
     }
-    if (threadIdx.x == 0) {
-        if (mode == 0) out[k] = red[0];
-        else if (mode == 1) out[k] += red[0];
-        else out[k] = sqrt(red[0]);
-    }
-    (void)cnt;
 }
 
 // w_i -= sum_k V_k[i] h[k], k < cnt: FP64 vectors in FP64; FP32 vectors
@@ -330,13 +381,14 @@ __global__ void multi_dot_final_kernel(int cnt, const double *partial, double *o
 // 4-value record per thread and step, four basis vectors loaded ahead of their
 // FMAs (the FMA order per entry is k = 0, 1, 2, ...).  With norm_partial the
 // same pass sums |w_new|^2 (like the dots: FP64, or exact FP32 products in
-// double-float) per CTA into norm_partial[block] (launch on the fixed
-// kAxpyGrid x kRedThreads grid); with cond, nothing happens when *cond is 0.
+// double-float) per CTA into norm_partial[block], and the last CTA leaves its root
+// in *norm; with cond, nothing happens when *cond is 0.
 constexpr int kMaxAxpy = 256;
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads)
     multi_axpy_kernel(int cnt, int64_t len4, const vec4<T> *V, int64_t vstride, const double *h,
-                      vec4<T> *w, double *norm_partial, const double *cond)
+                      vec4<T> *w, double *norm_partial, const double *cond, unsigned *ticket,
+                      double *norm)
 {
     if (cond && *cond == 0.0) return;
     using Acc = typename DotAcc<T>::type;
@@ -391,19 +443,15 @@ __global__ void __launch_bounds__(kRedThreads)
             for (int q = 0; q < kRedThreads / 32; ++q) t += red[q];
             norm_partial[blockIdx.x] = t;
         }
-    }
-}
-
-// Kahan's test on the device: flag = 1 when |h[0..j]|^2 > |w|^2 / 2 (w . w in
-// h[j + 1]), i.e. the classical Gram-Schmidt pass lost orthogonality and a
-// second pass is due; lanes sum in a fixed order
-__global__ void kahan_flag_kernel(int j, const double *h, double *flag)
-{
-    double v = 0.0;
-    for (int i = threadIdx.x; i <= j; i += 32) v += h[i] * h[i];
+        // the last CTA: |w_new| = the root of the partial sums' sum
+        if (!last_cta(ticket) || wid != 0) return;
+        const volatile double *p = norm_partial;
+        double a = 0.0;
+        for (int b = lane; b < (int)gridDim.x; b += 32) a += p[b];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (threadIdx.x == 0) *flag = (v <= 0.5 * h[j + 1]) ? 0.0 : 1.0;
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (lane == 0) *norm = sqrt(a);
+    }
 }
 
 __global__ void add_if_kernel(int n, const double *x, double *y, const double *cond)
@@ -710,6 +758,7 @@ struct Work {
     void *blocks = nullptr, *inv = nullptr;  // [n][16]
     double *partial = nullptr;              // [restart+1][kRedGrid] + [kAxpyGrid]
     double *hcol = nullptr, *h2 = nullptr;  // [restart+2]
+    unsigned *ticket = nullptr;             // of the reductions' last CTA (zero between launches)
     double *hhost = nullptr;                // pinned
     int precond = 0;                        // 0 block-Jacobi, 1 Schur (pmg.cu)
     // the point-mass coupling of the Jacobian apply runs on a side stream
@@ -725,7 +774,8 @@ void free_work(Work &W)
 {
     void *ptrs[] = {W.U, W.A, W.R, W.V1, W.pa, W.pv, W.prs, W.Uw, W.Aw, W.fw, W.xiw, W.ww, W.pu,
                     W.bu, W.bv, W.ba, W.buw, W.pw,
-                    W.Vk, W.w, W.z, W.x, W.b, W.blocks, W.inv, W.partial, W.hcol, W.h2};
+                    W.Vk, W.w, W.z, W.x, W.b, W.blocks, W.inv, W.partial, W.hcol, W.h2,
+                    W.ticket};
     for (void *p : ptrs) cudaFree(p);
     cudaFree(W.ftmp);
     if (W.side) cudaStreamDestroy(W.side);
@@ -780,6 +830,7 @@ fsi_status ensure_work(fsi_mesh *mesh, int64_t m_pts, int restart)
         {(void **)&W.partial, ((size_t)(restart + 1) * kRedGrid + kAxpyGrid) * sizeof(double)},
         {(void **)&W.hcol, (size_t)(restart + 2) * sizeof(double)},
         {(void **)&W.h2, (size_t)(restart + 2) * sizeof(double)},
+        {(void **)&W.ticket, sizeof(double)},
     };
     for (auto &r : req) {
         cudaError_t e = cudaMalloc(r.p, r.bytes);
@@ -788,7 +839,13 @@ fsi_status ensure_work(fsi_mesh *mesh, int64_t m_pts, int restart)
             return check_cuda(e, "Newton workspace allocation");
         }
     }
-    cudaError_t e = cudaMallocHost((void **)&W.hhost, (size_t)(restart + 2) * sizeof(double));
+    cudaError_t e = cudaMemset(W.ticket, 0, sizeof(double));
+    if (e == cudaSuccess) e = cudaStreamSynchronize(0);
+    if (e != cudaSuccess) {
+        free_work(W);
+        return check_cuda(e, "Newton workspace");
+    }
+    e = cudaMallocHost((void **)&W.hhost, (size_t)(restart + 2) * sizeof(double));
     if (e != cudaSuccess) {
         free_work(W);
         return check_cuda(e, "pinned host buffer");
@@ -936,10 +993,7 @@ fsi_status coupled_jacobian_impl(fsi_mesh *mesh, const fsi_step_state *st, const
         const double D = st->drho_s + st->k_s * mesh->gamma * mesh->phys.dt * mesh->phys.dt;
         mesh->stream = W.side;
         const fsi_status cs = [&]() -> fsi_status {
-            FSI_TRY(fsi_dlm_interp(mesh, P, st->m, st->elem, W.xiw, x, W.pu));
-            scale_kernel<T><<<grid1d(3 * st->m), 256, 0, W.side>>>(3 * st->m, (T)D,
-                                                                  (const T *)W.pu, (T *)W.pu);
-            FSI_TRY(check_launch("scale kernel"));
+            FSI_TRY(interp_scaled<T>(mesh, st->m, st->elem, (const T *)W.xiw, x, (T)D, (T *)W.pu));
             return fsi_dlm_spread(mesh, P, st->m, st->elem, W.xiw, st->cell_start, st->perm,
                                   W.pu, st->w ? W.ww : nullptr, W.ftmp, 0);
         }();
@@ -1034,40 +1088,52 @@ fsi_status build_block_jacobi(fsi_mesh *mesh, const fsi_step_state *st, int prec
 }
 
 // ------------------------------------------------------------ Krylov helpers
-// out[k] = V_k . w for k < cnt (with self_k: out[self_k] = w . w)
+// CTAs of a reduction over len4 records: the fixed grid, or one record per thread
+// on short vectors (fewer partial sums to add up); a rule on the length alone, so
+// the sums of a vector length are always formed alike
+int red_grid(int64_t len4, int cap) { return grid1d(len4, kRedThreads, cap); }
+
+// out[k] = V_k . w for k < cnt (with self_k: out[self_k] = w . w); norm: the root.
+// kahan_j >= 0: Kahan's flag of the column too.
 template <typename T>
-fsi_status multi_dot(fsi_mesh *mesh, int cnt, const T *V, int64_t ld, const T *w, double *out,
-                     int mode, int self_k = -1, const double *cond = nullptr)
+void multi_dot_launch(cudaStream_t s, int64_t len, int cnt, const T *V, int64_t ld, const T *w,
+                      double *partial, unsigned *ticket, double *out, int norm, int self_k,
+                      const double *cond, int kahan_j, double *flag)
 {
-    Work &W = mesh->newton->w;
-    cudaStream_t s = mesh->stream;
-    const int64_t len = 4 * mesh->n_nodes;
+    const int grid = red_grid(len / 4, kRedGrid);
     for (int k0 = 0; k0 < cnt; k0 += kDotGroup) {
         const int c = cnt - k0 < kDotGroup ? cnt - k0 : kDotGroup;
-        multi_dot_partial_kernel<T><<<kRedGrid, kRedThreads, 0, s>>>(
-            k0, c, len / 4, (const vec4<T> *)V, ld / 4, (const vec4<T> *)w, W.partial, self_k,
-            cond);
+        const DotFinal fin = {ticket, out, norm, k0 + c == cnt ? kahan_j : -1, flag};
+        multi_dot_partial_kernel<T><<<grid, kRedThreads, 0, s>>>(
+            k0, c, len / 4, (const vec4<T> *)V, ld / 4, (const vec4<T> *)w, partial, self_k, cond,
+            fin);
     }
-    FSI_TRY(check_launch("multi-dot partial"));
-    multi_dot_final_kernel<<<cnt, kRedThreads, 0, s>>>(cnt, W.partial, out, mode, cond);
-    return check_launch("multi-dot final");
+}
+template <typename T>
+fsi_status multi_dot(fsi_mesh *mesh, int cnt, const T *V, int64_t ld, const T *w, double *out,
+                     int norm, int self_k = -1, const double *cond = nullptr, int kahan_j = -1,
+                     double *flag = nullptr)
+{
+    Work &W = mesh->newton->w;
+    multi_dot_launch<T>(mesh->stream, 4 * mesh->n_nodes, cnt, V, ld, w, W.partial, W.ticket, out, norm,
+                        self_k, cond, kahan_j, flag);
+    return check_launch("multi-dot");
 }
 
 // w -= V[:, :cnt] h (vectors of len = 4n entries, 16/32-byte aligned records);
-// with norm_partial also the CTA partial sums of |w|^2 (fixed grid); with
-// cond only when the device flag is set
+// with norm_partial also |w| into *norm; with cond only when the device flag is set
 template <typename T>
 void multi_axpy(cudaStream_t s, int cnt, int64_t len, const T *V, int64_t ld, const double *h,
-                T *w, double *norm_partial = nullptr, const double *cond = nullptr)
+                T *w, double *norm_partial = nullptr, const double *cond = nullptr,
+                unsigned *ticket = nullptr, double *norm = nullptr)
 {
-    multi_axpy_kernel<T><<<kAxpyGrid, kRedThreads, 0, s>>>(cnt, len / 4, (const vec4<T> *)V,
-                                                          ld / 4, h, (vec4<T> *)w, norm_partial,
-                                                          cond);
+    multi_axpy_kernel<T><<<red_grid(len / 4, kAxpyGrid), kRedThreads, 0, s>>>(
+        cnt, len / 4, (const vec4<T> *)V, ld / 4, h, (vec4<T> *)w, norm_partial, cond, ticket, norm);
 }
 
 template <typename T> fsi_status norm2(fsi_mesh *mesh, const T *x, double *dev_out)
 {
-    return multi_dot<T>(mesh, 1, x, 0, x, dev_out, 2);
+    return multi_dot<T>(mesh, 1, x, 0, x, dev_out, 1);
 }
 
 fsi_status host_scalar(fsi_mesh *mesh, const double *dev, double *out)
@@ -1172,20 +1238,18 @@ fsi_status gmres(fsi_mesh *mesh, const fsi_step_state *st, int restart, int max_
             // classical Gram-Schmidt, h = V^T w (and |w|^2 in the same pass), with
             // a second pass only when Kahan's criterion flags a loss of
             // orthogonality: |h|^2 > |w|^2 / 2, i.e. |w - V h| < |w| / sqrt(2)
-            // Kahan's test runs on the device and the second pass (when it is
-            // due) is launched conditionally, so the iteration needs one host
-            // synchronisation, at its end; |w|^2 of the orthogonalised vector is
-            // summed by the update pass itself
+            // Kahan's test runs on the device (in the dots' last CTA) and the
+            // second pass (when it is due) is launched conditionally, so the
+            // iteration needs one host synchronisation, at its end; |w| of the
+            // orthogonalised vector comes out of the update pass itself
             double *flag = W.h2 + restart + 1;
             double *npart = W.partial + (int64_t)(restart + 1) * kRedGrid;
-            FSI_TRY(multi_dot<T>(mesh, j + 2, V, ld, w, W.hcol, 0, j + 1));
-            kahan_flag_kernel<<<1, 32, 0, s>>>(j, W.hcol, flag);
-            multi_axpy<T>(s, j + 1, len, V, ld, W.hcol, w, npart);
+            double *norm = W.hcol + j + 1;
+            FSI_TRY(multi_dot<T>(mesh, j + 2, V, ld, w, W.hcol, 0, j + 1, nullptr, j, flag));
+            multi_axpy<T>(s, j + 1, len, V, ld, W.hcol, w, npart, nullptr, W.ticket, norm);
             FSI_TRY(multi_dot<T>(mesh, j + 1, V, ld, w, W.h2, 0, -1, flag));
-            multi_axpy<T>(s, j + 1, len, V, ld, W.h2, w, npart, flag);
+            multi_axpy<T>(s, j + 1, len, V, ld, W.h2, w, npart, flag, W.ticket, norm);
             add_if_kernel<<<1, 64, 0, s>>>(j + 1, W.h2, W.hcol, flag);
-            multi_dot_final_kernel<<<1, kRedThreads, 0, s>>>(1, npart, W.hcol + j + 1, 2, nullptr,
-                                                             kAxpyGrid);
             FSI_TRY(check_launch("Gram-Schmidt"));
             scale_basis(W.hcol + j + 1, V + (int64_t)(j + 1) * ld);
             FSI_CUDA(cudaMemcpyAsync(W.hhost, W.hcol, (j + 2) * sizeof(double),
@@ -1465,21 +1529,17 @@ fsi_status fsi_multi_dot(int device, fsi_prec prec, int64_t len, int nvec, const
     if (((uintptr_t)V | (uintptr_t)w) % (4 * esz) != 0)
         return set_error(FSI_ERR_ARG, "fsi_multi_dot: V and w must be aligned to 4 entries");
     FSI_DEVICE(device);
-    double *partial = nullptr;
-    FSI_CUDA(cudaMallocAsync((void **)&partial, (size_t)nvec * kRedGrid * sizeof(double), 0),
-             "partial sums");
-    for (int k0 = 0; k0 < nvec; k0 += kDotGroup) {
-        const int c = nvec - k0 < kDotGroup ? nvec - k0 : kDotGroup;
-        if (prec == FSI_F64)
-            multi_dot_partial_kernel<double><<<kRedGrid, kRedThreads, 0, 0>>>(
-                k0, c, len / 4, (const vec4<double> *)V, ldv / 4, (const vec4<double> *)w, partial,
-                -1, nullptr);
-        else
-            multi_dot_partial_kernel<float><<<kRedGrid, kRedThreads, 0, 0>>>(
-                k0, c, len / 4, (const vec4<float> *)V, ldv / 4, (const vec4<float> *)w, partial,
-                -1, nullptr);
-    }
-    multi_dot_final_kernel<<<nvec, kRedThreads, 0, 0>>>(nvec, partial, out, 0);
+    double *partial = nullptr;  // the partial sums, then the ticket
+    const size_t np = (size_t)nvec * kRedGrid;
+    FSI_CUDA(cudaMallocAsync((void **)&partial, (np + 1) * sizeof(double), 0), "partial sums");
+    unsigned *ticket = (unsigned *)(partial + np);
+    FSI_CUDA(cudaMemsetAsync(ticket, 0, sizeof(double), 0), "memset");
+    if (prec == FSI_F64)
+        multi_dot_launch<double>(0, len, nvec, (const double *)V, ldv, (const double *)w, partial,
+                                 ticket, out, 0, -1, nullptr, -1, nullptr);
+    else
+        multi_dot_launch<float>(0, len, nvec, (const float *)V, ldv, (const float *)w, partial,
+                                ticket, out, 0, -1, nullptr, -1, nullptr);
     const fsi_status st = check_launch("multi-dot kernels");
     cudaFreeAsync(partial, 0);
     return st;
@@ -1501,8 +1561,10 @@ fsi_status fsi_measure_blas1(int device, fsi_prec prec, int64_t len, int nvec, i
     fsi_status st = check_cuda(cudaMalloc(&V, (size_t)nvec * len * esz), "buffers");
     if (st == FSI_OK) st = check_cuda(cudaMalloc(&w, (size_t)len * esz), "buffers");
     if (st == FSI_OK)
-        st = check_cuda(cudaMalloc(&partial, (size_t)(nvec + 1) * kRedGrid * sizeof(double)),
+        st = check_cuda(cudaMalloc(&partial, ((size_t)nvec * kRedGrid + kAxpyGrid + 1) * sizeof(double)),
                         "buffers");
+    double *npart = partial + (size_t)nvec * kRedGrid;
+    unsigned *ticket = (unsigned *)(npart + kAxpyGrid);
     if (st == FSI_OK) st = check_cuda(cudaMalloc(&h, (size_t)(nvec + 1) * sizeof(double)), "buffers");
     if (st == FSI_OK) st = check_cuda(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking), "stream");
     if (st == FSI_OK) st = check_cuda(cudaEventCreate(&e0), "event");
@@ -1511,25 +1573,22 @@ fsi_status fsi_measure_blas1(int device, fsi_prec prec, int64_t len, int nvec, i
     if (st == FSI_OK) st = check_cuda(cudaMemsetAsync(w, 0, (size_t)len * esz, s), "memset");
     if (st == FSI_OK) st = check_cuda(cudaMemsetAsync(h, 0, (size_t)(nvec + 1) * sizeof(double), s),
                                       "memset");
+    if (st == FSI_OK) st = check_cuda(cudaMemsetAsync(ticket, 0, sizeof(double), s), "memset");
     auto dots = [&]() {
-        for (int k0 = 0; k0 < nvec; k0 += kDotGroup) {
-            const int c = nvec - k0 < kDotGroup ? nvec - k0 : kDotGroup;
-            if (prec == FSI_F64)
-                multi_dot_partial_kernel<double><<<kRedGrid, kRedThreads, 0, s>>>(
-                    k0, c, len / 4, (const vec4<double> *)V, len / 4, (const vec4<double> *)w,
-                    partial, -1, nullptr);
-            else
-                multi_dot_partial_kernel<float><<<kRedGrid, kRedThreads, 0, s>>>(
-                    k0, c, len / 4, (const vec4<float> *)V, len / 4, (const vec4<float> *)w,
-                    partial, -1, nullptr);
-        }
-        multi_dot_final_kernel<<<nvec, kRedThreads, 0, s>>>(nvec, partial, h, 0);
+        if (prec == FSI_F64)
+            multi_dot_launch<double>(s, len, nvec, (const double *)V, len, (const double *)w, partial,
+                                     ticket, h, 0, -1, nullptr, -1, nullptr);
+        else
+            multi_dot_launch<float>(s, len, nvec, (const float *)V, len, (const float *)w, partial,
+                                    ticket, h, 0, -1, nullptr, -1, nullptr);
     };
     auto axpy = [&]() {
         if (prec == FSI_F64)
-            multi_axpy<double>(s, nvec, len, (const double *)V, len, h, (double *)w, partial);
+            multi_axpy<double>(s, nvec, len, (const double *)V, len, h, (double *)w, npart, nullptr,
+                               ticket, h + nvec);
         else
-            multi_axpy<float>(s, nvec, len, (const float *)V, len, h, (float *)w, partial);
+            multi_axpy<float>(s, nvec, len, (const float *)V, len, h, (float *)w, npart, nullptr,
+                              ticket, h + nvec);
     };
     float ms = 0.f;
     for (int which = 0; st == FSI_OK && which < 2; ++which) {
