@@ -35,6 +35,8 @@
 // FP32 arithmetic follows the caller's precision.
 #include <algorithm>
 #include <cmath>
+#include <cooperative_groups.h>
+#include <cuda_pipeline.h>
 #include <type_traits>
 #include <vector>
 
@@ -74,6 +76,8 @@ namespace {
 
 // 1D coefficients of a level in the working type: mass and stiffness
 // entries of interior / boundary diagonals and of the off-diagonals.
+namespace cg = cooperative_groups;
+
 template <typename T> struct Axis {
     int N;
     T m_in, m_bd, m_off, k_in, k_bd, k_off;
@@ -758,6 +762,378 @@ fsi_status chebyshev(fsi_mesh *m, int l, int degree, double lo, double hi, const
     return check_launch("pressure smoother");
 }
 
+// ---------------------------------------------------------------- coarse levels
+// The V-cycle's FP32 levels of at most kCoarseNodes nodes, down to and with the
+// dense coarsest solve, as one cluster of CTAs: every vector of those levels lives
+// in shared memory, a pass is a loop over the level and passes are separated by
+// barriers.  As launches of their own these passes are 6 per level of 3 to 5 us
+// each, nearly all latency: at 32^3 a
+// mixed step with 56 V-cycles took 12.2 ms with them and takes 10.2 ms with this
+// kernel (41 us a launch; 47 us as one CTA).  In FP64 (two operations per SM and
+// clock) they stay spread over the chip, pass by pass.
+//
+// The first (largest) level is split into slabs of planes, one per CTA; a CTA keeps
+// all of the level's indexes but only its slab and the plane on either side hold
+// values, and a pass whose result the neighbours read stores their halo planes
+// into their shared memory (coarse_put).  Rank 0 alone does the levels below: they
+// have at most an eighth of the work, and a pass over the cluster costs a cluster
+// barrier.
+//
+// A stencil pass marches: a thread owns a column piece (i, j, planes k0 ..) and
+// folds each plane's 3 x 3 neighbourhood once, as march_kernel does.  The
+// arithmetic is march_kernel's; the sums along x are grouped differently.
+constexpr int kCoarseNodes = 4913;  // 17^3
+constexpr int kCoarseThreads = 1024;
+constexpr int kCoarseCtas = 8;
+constexpr int kCoarseSmemMax = 224 * 1024;
+constexpr int kCoarseSplit = 1000;  // nodes from which the first level is split
+constexpr int kCoarseMaxLevels = 8;
+struct CoarseLevel {
+    LevelArgs<float> A;
+    int n;
+    float inv_theta, c1, c2;  // Chebyshev degree 2 over [hi/4, hi]
+    int off;                  // of b, v, t in shared memory (3 n floats)
+};
+struct CoarseCycle {
+    int nlev;  // smoothed levels; the dense level follows
+    CoarseLevel lev[kCoarseMaxLevels];
+    LevelArgs<float> Ad;  // the dense level
+    int nd, off_d;        // its nodes and the place of its b, x
+    int off_inv;          // of the dense inverse in shared memory; 0: left in global
+    const float *inv;
+    const float *b;  // right-hand side of the first level
+    float *x;        // result
+};
+
+// One column piece of a level: its node of k = 0, planes [k0, k1), the operator's
+// weights along x and y (zero towards eliminated nodes) and the neighbours' columns
+struct CoarseCol {
+    int q;  // which piece (-1: none yet)
+    int i, j, c, k0, k1;
+    bool el;
+    float mx[3], kx[3], my[3], ky[3];  // ky: with kappa times the mass
+    float A1, A2, iDi, iDb;            // column's D = A1 mz(0) + A2 kz(0), inverse inside/at the ends
+    int at[9];
+};
+
+__device__ __forceinline__ void coarse_col(const LevelArgs<float> &L, int q, int z0, int z1, int cols,
+                                           int len, CoarseCol &c)
+{
+    const int piece = q / cols;
+    c.q = q;
+    c.c = q - piece * cols;
+    c.j = c.c / L.NX1;
+    c.i = c.c - c.j * L.NX1;
+    c.k0 = z0 + piece * len;
+    c.k1 = min(z1, c.k0 + len);
+    const Axis<float> &ax = L.a[0], &ay = L.a[1], &az = L.a[2];
+    // coordinates of an axis whose nodes the operator has as columns
+    const int lo0 = L.faces[0] ? 1 : 0, lo1 = L.faces[2] ? 1 : 0;
+    const int hi0 = L.NX1 - (L.faces[1] ? 2 : 1), hi1 = L.NY1 - (L.faces[3] ? 2 : 1);
+#pragma unroll
+    for (int d = -1; d <= 1; ++d) {
+        const bool inx = c.i + d >= lo0 && c.i + d <= hi0, iny = c.j + d >= lo1 && c.j + d <= hi1;
+        c.mx[d + 1] = inx ? (d ? ax.m_off : md_of(ax, c.i)) : 0.f;
+        c.kx[d + 1] = inx ? (d ? ax.k_off : kd_of(ax, c.i)) : 0.f;
+        c.my[d + 1] = iny ? (d ? ay.m_off : md_of(ay, c.j)) : 0.f;
+        c.ky[d + 1] = iny ? (d ? ay.k_off : kd_of(ay, c.j)) + L.kappa * c.my[d + 1] : 0.f;
+    }
+#pragma unroll
+    for (int p = 0; p < 9; ++p) {
+        const int ii = c.i + p % 3 - 1, jj = c.j + p / 3 - 1;
+        c.at[p] = (ii >= lo0 && ii <= hi0 ? ii : c.i) + L.NX1 * (jj >= lo1 && jj <= hi1 ? jj : c.j);
+    }
+    const float mdx = md_of(ax, c.i), kdx = kd_of(ax, c.i), mdy = md_of(ay, c.j), kdy = kd_of(ay, c.j);
+    c.A1 = kdx * mdy + mdx * kdy + L.kappa * mdx * mdy;
+    c.A2 = mdx * mdy;
+    c.iDi = 1.f / (c.A1 * az.m_in + c.A2 * az.k_in);
+    c.iDb = 1.f / (c.A1 * az.m_bd + c.A2 * az.k_bd);
+    c.el = c.i < lo0 || c.i > hi0 || c.j < lo1 || c.j > hi1;
+}
+
+// f(column) for this thread's column pieces of the planes [z0, z1); `col` is kept
+// from pass to pass (a thread has one piece unless the level is wide and flat)
+template <typename F>
+__device__ __forceinline__ void coarse_columns(const LevelArgs<float> &L, int z0, int z1, CoarseCol &col,
+                                               F f)
+{
+    if (z0 >= z1) return;
+    const int cols = L.NX1 * L.NY1;
+    const int pieces = max(1, kCoarseThreads / cols), len = (z1 - z0 + pieces - 1) / pieces;
+    for (int q = threadIdx.x; q < cols * pieces; q += kCoarseThreads) {
+        if (q != col.q) coarse_col(L, q, z0, z1, cols, len, col);
+        if (col.k0 < col.k1) f(col);
+    }
+}
+
+// out(node, plane, A v, v, 1/D) for the nodes of [z0, z1), v in shared memory
+template <typename F>
+__device__ __forceinline__ void coarse_stencil(const LevelArgs<float> &L, int z0, int z1, CoarseCol &col,
+                                               const float *v, F out)
+{
+    const int plane = L.NX1 * L.NY1, lo2 = L.faces[4] ? 1 : 0, hi2 = L.NZ1 - (L.faces[5] ? 2 : 1);
+    const Axis<float> &az = L.a[2];
+    coarse_columns(L, z0, z1, col, [&](const CoarseCol &c) {
+        float Pm = 0.f, Qm = 0.f, P0 = 0.f, Q0 = 0.f;
+        const float *pl = v + (c.k0 - 1) * plane;
+        for (int kk = c.k0 - 1; kk <= c.k1; ++kk, pl += plane) {
+            float P = 0.f, Q = 0.f;
+            if (kk >= lo2 && kk <= hi2) {
+                float w[9];
+#pragma unroll
+                for (int p = 0; p < 9; ++p) w[p] = pl[c.at[p]];
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    const float sk = c.kx[0] * w[3 * d] + c.kx[1] * w[3 * d + 1] + c.kx[2] * w[3 * d + 2];
+                    const float sm = c.mx[0] * w[3 * d] + c.mx[1] * w[3 * d + 1] + c.mx[2] * w[3 * d + 2];
+                    P += sk * c.my[d] + sm * c.ky[d];
+                    Q += sm * c.my[d];
+                }
+            }
+            const int k = kk - 1;
+            if (k >= c.k0 && k < c.k1) {
+                const bool bd = k == 0 || k == L.NZ1 - 1, el = c.el || k < lo2 || k > hi2;
+                const float mdz = bd ? az.m_bd : az.m_in, kdz = bd ? az.k_bd : az.k_in;
+                const float own = pl[c.c - plane];
+                const float Av = el ? (c.A1 * mdz + c.A2 * kdz) * own
+                                    : az.m_off * (Pm + P) + az.k_off * (Qm + Q) + P0 * mdz + Q0 * kdz;
+                out(c.c + k * plane, k, Av, own, bd ? c.iDb : c.iDi);
+            }
+            Pm = P0;
+            Qm = Q0;
+            P0 = P;
+            Q0 = Q;
+        }
+    });
+}
+
+__global__ void __launch_bounds__(kCoarseThreads, 1) coarse_cycle_kernel(const CoarseCycle C)
+{
+    extern __shared__ float cs[];
+    cg::cluster_group cl = cg::this_cluster();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nr = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    // this CTA's planes [z0, z1) of the first level
+    const int NZ = C.lev[0].A.NZ1, zl = (NZ + nr - 1) / nr;
+    const int s0 = min(rank * zl, NZ), s1 = min(s0 + zl, NZ);
+    auto sync = [&](bool split) {
+        if (split && nr > 1) cl.sync();
+        else __syncthreads();
+    };
+    // a value of plane k of the slab, also into the neighbours' halo planes
+    auto put = [&](float *at, int k, float val) {
+        *at = val;
+        if (nr > 1) {
+            if (k == s0 && s0 > 0) *cl.map_shared_rank(at, rank - 1) = val;
+            if (k == s1 - 1 && s1 < NZ) *cl.map_shared_rank(at, rank + 1) = val;
+        }
+    };
+    {
+        float *b = cs + C.lev[0].off;
+        const int plane = C.lev[0].n / NZ, q1 = min(s1 + 1, NZ) * plane;
+        if (s0 < s1)
+            for (int q = max(s0 - 1, 0) * plane + tid; q < q1; q += kCoarseThreads) b[q] = C.b[q];
+        // the dense inverse on its way (see off_inv)
+        if (rank == 0 && C.off_inv)
+            for (int q = tid; q < C.nd * C.nd; q += kCoarseThreads) __pipeline_memcpy_async(cs + C.off_inv + q, C.inv + q, 4);
+        __pipeline_commit();
+    }
+    CoarseCol col;
+    sync(true);
+    // down: pre-smoothing from zero into t, residual into v, its restriction
+    for (int l = 0; l < C.nlev; ++l) {
+        if (l > 0 && rank > 0) break;
+        const CoarseLevel &L = C.lev[l];
+        const LevelArgs<float> &A = L.A;
+        const int z0 = l ? 0 : s0, z1 = l ? A.NZ1 : s1, plane = A.NX1 * A.NY1;
+        const bool split = l == 0;
+        float *b = cs + L.off, *v = b + L.n, *t = v + L.n;
+        col.q = -1;
+        // d0, on the halo planes too
+        coarse_columns(A, z0, z1, col, [&](const CoarseCol &c) {
+            const int ka = c.k0 == z0 ? max(z0 - 1, 0) : c.k0, kb = c.k1 == z1 ? min(z1 + 1, A.NZ1) : c.k1;
+            for (int k = ka; k < kb; ++k)
+                v[c.c + k * plane] = L.inv_theta * b[c.c + k * plane] * (k == 0 || k == A.NZ1 - 1 ? c.iDb : c.iDi);
+        });
+        __syncthreads();
+        coarse_stencil(A, z0, z1, col, v, [&](int q, int k, float Av, float d0, float iD) {
+            const float y = d0 + (L.c1 * d0 + L.c2 * ((b[q] - Av) * iD));
+            if (split) put(t + q, k, y);
+            else t[q] = y;
+        });
+        sync(split);
+        coarse_stencil(A, z0, z1, col, t, [&](int q, int k, float Av, float, float) {
+            if (split) put(v + q, k, b[q] - Av);
+            else v[q] = b[q] - Av;
+        });
+        sync(split);
+        // restriction of the coarse planes whose fine plane is in the slab, to rank 0
+        const bool last = l + 1 == C.nlev;
+        const LevelArgs<float> &B = last ? C.Ad : C.lev[l + 1].A;
+        float *bc = cs + (last ? C.off_d : C.lev[l + 1].off);
+        if (split && rank > 0) bc = cl.map_shared_rank(bc, 0);
+        const int cplane = B.NX1 * B.NY1, K0 = (z0 + 1) / 2, K1 = z0 < z1 ? (z1 - 1) / 2 + 1 : 0;
+        for (int q = K0 * cplane + tid; q < K1 * cplane; q += kCoarseThreads) {
+            const int row = q / B.NX1, I = q - row * B.NX1, K = row / B.NY1, J = row - K * B.NY1;
+            float acc = 0.f;
+#pragma unroll
+            for (int dk = -1; dk <= 1; ++dk)
+#pragma unroll
+                for (int dj = -1; dj <= 1; ++dj) {
+                    const int k = 2 * K + dk, j = 2 * J + dj;
+                    if (k < 0 || k >= A.NZ1 || j < 0 || j >= A.NY1) continue;
+                    const float *rw = v + A.NX1 * (j + A.NY1 * k) + 2 * I;
+                    float sum = rw[0];
+                    if (I > 0) sum += 0.5f * rw[-1];
+                    if (2 * I + 1 < A.NX1) sum += 0.5f * rw[1];
+                    acc += (dj ? 0.5f : 1.f) * (dk ? 0.5f : 1.f) * sum;
+                }
+            bc[q] = eliminated(B, I, J, K) ? 0.f : acc;
+        }
+        sync(split);
+    }
+    // the dense inverse: a warp per row, lanes in dense_apply_kernel's order
+    if (rank == 0) {
+        const float *b = cs + C.off_d;
+        float *x = cs + C.off_d + C.nd;
+        const float *inv = C.off_inv ? cs + C.off_inv : C.inv;
+        __pipeline_wait_prior(0);
+        __syncthreads();
+        for (int row = warp; row < C.nd; row += kCoarseThreads / 32) {
+            float sum = 0.f;
+            for (int c = lane; c < C.nd; c += 32) sum += inv[row * C.nd + c] * b[c];
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            if (lane == 0) x[row] = sum;
+        }
+        __syncthreads();
+    }
+    // up: prolongation into t, post-smoothing from t
+    for (int l = C.nlev - 1; l >= 0; --l) {
+        if (l > 0 && rank > 0) continue;
+        const CoarseLevel &L = C.lev[l];
+        const LevelArgs<float> &A = L.A;
+        const int z0 = l ? 0 : s0, z1 = l ? A.NZ1 : s1, plane = A.NX1 * A.NY1;
+        const bool split = l == 0;
+        float *b = cs + L.off, *v = b + L.n, *t = v + L.n;
+        const bool last = l + 1 == C.nlev;
+        const LevelArgs<float> &B = last ? C.Ad : C.lev[l + 1].A;
+        // the level below leaves its result in its t (the dense level after its b)
+        float *xc = last ? cs + C.off_d + C.nd : cs + C.lev[l + 1].off + 2 * C.lev[l + 1].n;
+        const int cplane = B.NX1 * B.NY1;
+        if (split && nr > 1) {
+            // rank 0's result is there; the planes this slab and its halo read
+            cl.sync();
+            if (rank > 0 && z0 < z1) {
+                const float *x0 = cl.map_shared_rank(xc, 0);
+                const int q1 = min(z1 / 2 + 2, B.NZ1) * cplane;
+                for (int q = ((z0 - 1) / 2) * cplane + tid; q < q1; q += kCoarseThreads) xc[q] = x0[q];
+            }
+            __syncthreads();
+        }
+        if (!split || (rank == 0 && C.nlev > 1)) col.q = -1;
+        coarse_columns(A, z0, z1, col, [&](const CoarseCol &c) {
+            const int ka = c.k0 == z0 ? max(z0 - 1, 0) : c.k0, kb = c.k1 == z1 ? min(z1 + 1, A.NZ1) : c.k1;
+            // trilinear: along x and y between the column's (up to) four coarse ones
+            const int dx = c.i & 1, dy = (c.j & 1) ? B.NX1 : 0;
+            const float w = (dx ? 0.5f : 1.f) * (dy ? 0.5f : 1.f);
+            for (int k = ka; k < kb; ++k) {
+                const float *r0 = xc + (c.i >> 1) + B.NX1 * (c.j >> 1) + (k >> 1) * cplane;
+                float s = r0[0];
+                if (dx) s += r0[1];
+                if (dy) s += r0[dy] + (dx ? r0[dy + 1] : 0.f);
+                if (k & 1) {
+                    const float *r1 = r0 + cplane;
+                    float s1 = r1[0];
+                    if (dx) s1 += r1[1];
+                    if (dy) s1 += r1[dy] + (dx ? r1[dy + 1] : 0.f);
+                    s = 0.5f * (s + s1);
+                }
+                t[c.c + k * plane] += w * s;
+            }
+        });
+        __syncthreads();
+        // the first direction d0 from x = t; then v = t + d0, d0 kept in t
+        coarse_stencil(A, z0, z1, col, t, [&](int q, int, float Av, float, float iD) {
+            v[q] = L.inv_theta * (b[q] - Av) * iD;
+        });
+        __syncthreads();
+        coarse_columns(A, z0, z1, col, [&](const CoarseCol &c) {
+            for (int k = c.k0; k < c.k1; ++k) {
+                const int q = c.c + k * plane;
+                const float d0 = v[q], y = t[q] + d0;
+                t[q] = d0;
+                if (split) put(v + q, k, y);
+                else v[q] = y;
+            }
+        });
+        sync(split);
+        coarse_stencil(A, z0, z1, col, v, [&](int q, int, float Av, float xv, float iD) {
+            const float y = xv + (L.c1 * t[q] + L.c2 * ((b[q] - Av) * iD));
+            t[q] = y;
+            if (l == 0) C.x[q] = y;
+        });
+        __syncthreads();
+    }
+}
+
+// The first level of the FP32 V-cycle that coarse_cycle_kernel takes, or -1: a
+// level below the finest, small enough, with the levels after it fitting the
+// kernel and a dense coarsest solve
+int coarse_first(const PressureMG &P)
+{
+    if (!P.direct) return -1;
+    for (int l = 1; l < P.nlev - 1; ++l)
+        if (P.lev[l].n <= kCoarseNodes) return P.nlev - 1 - l <= kCoarseMaxLevels ? l : -1;
+    return -1;
+}
+
+fsi_status coarse_cycle(fsi_mesh *m, int l0, const float *b, float *x)
+{
+    const PressureMG &P = *m->pmg;
+    CoarseCycle C{};
+    C.nlev = P.nlev - 1 - l0;
+    int off = 0;
+    for (int l = 0; l < C.nlev; ++l) {
+        const PmgLevel &L = P.lev[l0 + l];
+        const double hi = L.hi, lo = hi / 4.0, theta = 0.5 * (hi + lo), delta = 0.5 * (hi - lo),
+                     s1 = theta / delta, rho = 1.0 / s1, rho_new = 1.0 / (2.0 * s1 - rho);
+        C.lev[l].A = level_args<float>(P, l0 + l);
+        C.lev[l].n = (int)L.n;
+        C.lev[l].inv_theta = (float)(1.0 / theta);
+        C.lev[l].c1 = (float)(rho_new * rho);
+        C.lev[l].c2 = (float)(2.0 * rho_new / delta);
+        C.lev[l].off = off;
+        off += 3 * (int)L.n;
+    }
+    C.Ad = level_args<float>(P, P.nlev - 1);
+    C.nd = (int)P.nc;
+    C.off_d = off;
+    off += 2 * C.nd;
+    C.inv = P.inv32;
+    C.b = b;
+    C.x = x;
+    if (C.nd <= 181 && (off + C.nd * C.nd) * (int)sizeof(float) <= kCoarseSmemMax) {
+        C.off_inv = off;
+        off += C.nd * C.nd;
+    }
+    const int bytes = off * (int)sizeof(float);
+    FSI_TRY(set_smem_limit((const void *)coarse_cycle_kernel, kCoarseSmemMax));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = cfg.blockDim = dim3(1, 1, 1);
+    cfg.gridDim.x = C.lev[0].n >= kCoarseSplit ? kCoarseCtas : 1;
+    cfg.blockDim.x = kCoarseThreads;
+    cfg.dynamicSmemBytes = bytes;
+    cfg.stream = m->stream;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = cfg.gridDim.x;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    FSI_CUDA(cudaLaunchKernelEx(&cfg, coarse_cycle_kernel, C), "pressure coarse levels");
+    return check_launch("pressure coarse levels");
+}
+
 template <typename T> fsi_status coarse_solve(fsi_mesh *m, const T *b, T *x)
 {
     PressureMG &P = *m->pmg;
@@ -781,6 +1157,8 @@ fsi_status vcycle_level(fsi_mesh *m, int l, const T *b, T *x, const SchurOut<T> 
 {
     PressureMG &P = *m->pmg;
     if (l == P.nlev - 1) return coarse_solve<T>(m, b, x);
+    if constexpr (std::is_same<T, float>::value)
+        if (l == coarse_first(P)) return coarse_cycle(m, l, b, x);
     PmgLevel &L = P.lev[l], &Lc = P.lev[l + 1];
     const double hi = L.hi;
     T *t = vec<T>(L.t);
