@@ -395,14 +395,12 @@ template <typename T> __device__ __forceinline__ T shape_1d(T xi, int side)
 // Interpolation for one point b (u = C^T V, Eq. nodal_solid_velo) by one
 // lane (the double-float and FP64 kernels: issue-bound, so no work is
 // duplicated).  T is the compute type; xi, U and u are in StorageOf<T>.
-// SCALED: the interpolated values times D (the product after the rounding to
-// storage, as a pass of its own would form it).
-template <typename T, bool SCALED = false>
+template <typename T>
 __device__ __forceinline__ void interp_point(
     const GridArgs &g, int64_t b, const int32_t *__restrict__ elem,
     const typename StorageOf<T>::type *__restrict__ xi,
     const vec4<typename StorageOf<T>::type> *__restrict__ U,
-    typename StorageOf<T>::type *__restrict__ u, typename StorageOf<T>::type D = 1)
+    typename StorageOf<T>::type *__restrict__ u)
 {
     const int NX1 = g.Nx + 1, NXY1 = (g.Nx + 1) * (g.Ny + 1);
     const int E = g.Nx * g.Ny * g.Nz;
@@ -424,9 +422,9 @@ __device__ __forceinline__ void interp_point(
             uz = madd(Na, to_c<T>(v.z), uz);
         }
     }
-    u[3 * b] = SCALED ? D * to_s(ux) : to_s(ux);
-    u[3 * b + 1] = SCALED ? D * to_s(uy) : to_s(uy);
-    u[3 * b + 2] = SCALED ? D * to_s(uz) : to_s(uz);
+    u[3 * b] = to_s(ux);
+    u[3 * b + 1] = to_s(uy);
+    u[3 * b + 2] = to_s(uz);
 }
 
 // The same by two adjacent lanes of a warp (the FP32 kernels: bound by the
@@ -436,12 +434,12 @@ __device__ __forceinline__ void interp_point(
 // lane adds the other half and writes u.  Every lane of the warp calls this
 // (valid == false: no point, no memory access), because of the shuffle.  T
 // is the compute type; xi, U and u are in StorageOf<T>.
-template <typename T, bool SCALED = false>
+template <typename T>
 __device__ __forceinline__ void interp_point_pair(
     const GridArgs &g, int64_t b, bool valid, const int32_t *__restrict__ elem,
     const typename StorageOf<T>::type *__restrict__ xi,
     const vec4<typename StorageOf<T>::type> *__restrict__ U,
-    typename StorageOf<T>::type *__restrict__ u, typename StorageOf<T>::type D = 1)
+    typename StorageOf<T>::type *__restrict__ u)
 {
     const int NX1 = g.Nx + 1, NXY1 = (g.Nx + 1) * (g.Ny + 1);
     const int E = g.Nx * g.Ny * g.Nz;
@@ -469,9 +467,9 @@ __device__ __forceinline__ void interp_point_pair(
     uy = uy + shfl_x(uy, 1);
     uz = uz + shfl_x(uz, 1);
     if (valid && ax == 0) {
-        u[3 * b] = SCALED ? D * to_s(ux) : to_s(ux);
-        u[3 * b + 1] = SCALED ? D * to_s(uy) : to_s(uy);
-        u[3 * b + 2] = SCALED ? D * to_s(uz) : to_s(uz);
+        u[3 * b] = to_s(ux);
+        u[3 * b + 1] = to_s(uy);
+        u[3 * b + 2] = to_s(uz);
     }
 }
 

@@ -244,10 +244,19 @@ template <typename T>
 fsi_status spread_mass_diag(fsi_mesh *mesh, int64_t m, const T *xi, const int32_t *cell_start,
                             const int32_t *perm, const T *w, double dsq, T *F);
 
-// u = D C^T U at the points (dlm.cu; the interpolation, then the product, in T)
+// The point-mass coupling C D W C^T of a step as one matrix per occupied cell
+// (dlm.cu): build for the cell table's points (list: coupling_cells + 1 ints, M: 36
+// values per cell), apply into the mesh's spreading scratch, and add the nodal
+// forces to y, with the Dirichlet rows y = x (mask may be null; 4-byte aligned)
+int64_t coupling_cells(const fsi_mesh *mesh, int64_t m);
 template <typename T>
-fsi_status interp_scaled(fsi_mesh *mesh, int64_t m, const int32_t *elem, const T *xi, const T *U,
-                         T D, T *u);
+fsi_status coupling_build(fsi_mesh *mesh, int64_t m, const T *xi, const int32_t *cell_start,
+                          const int32_t *perm, const T *w, T D, int32_t *list, T *M);
+template <typename T>
+fsi_status coupling_apply(fsi_mesh *mesh, int64_t m, const int32_t *list, const T *M, const T *x);
+template <typename T>
+fsi_status coupling_finish(fsi_mesh *mesh, const int32_t *cell_start, const uint8_t *mask, const T *x,
+                           T *y);
 
 // the checks fsi_newton_step makes of a step state (newton.cu)
 fsi_status validate_step_state(const fsi_mesh *mesh, const fsi_step_state *st);

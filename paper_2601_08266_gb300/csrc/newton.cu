@@ -98,46 +98,6 @@ __global__ void solid_force_kernel(int64_t m, const int32_t *elem, const double 
     }
 }
 
-// y[i].xyz += f[i].xyz (the coupling's nodal forces into the Jacobian apply)
-template <typename T>
-__global__ void add_xyz_kernel(int64_t n, const vec4<T> *__restrict__ f, vec4<T> *__restrict__ y)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const vec4<T> a = f[i];
-        vec4<T> b = y[i];
-        b.x += a.x;
-        b.y += a.y;
-        b.z += a.z;
-        y[i] = b;
-    }
-}
-
-// the same followed by the Dirichlet rows (Jx = x where mask), one pass
-template <typename T>
-__global__ void add_xyz_rows_kernel(int64_t n, const vec4<T> *__restrict__ f,
-                                    const uchar4 *__restrict__ mask, const vec4<T> *__restrict__ x,
-                                    vec4<T> *__restrict__ y)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const vec4<T> a = f[i];
-        const uchar4 mk = mask[i];
-        vec4<T> b = y[i];
-        b.x += a.x;
-        b.y += a.y;
-        b.z += a.z;
-        if (mk.x | mk.y | mk.z | mk.w) {
-            const vec4<T> xv = x[i];
-            if (mk.x) b.x = xv.x;
-            if (mk.y) b.y = xv.y;
-            if (mk.z) b.z = xv.z;
-            if (mk.w) b.w = xv.w;
-        }
-        y[i] = b;
-    }
-}
-
 template <typename T> __global__ void scale_kernel(int64_t n, T alpha, const T *x, T *y)
 {
     GRID_STRIDE(i, n) y[i] = alpha * x[i];
@@ -758,6 +718,9 @@ struct Work {
     void *blocks = nullptr, *inv = nullptr;  // [n][16]
     double *partial = nullptr;              // [restart+1][kRedGrid] + [kAxpyGrid]
     double *hcol = nullptr, *h2 = nullptr;  // [restart+2]
+    int32_t *clist = nullptr;               // occupied cells and their count
+    void *cmat = nullptr;                   // [cells][36] coupling matrices
+    bool cells = false;                     // they hold this call's step (and type)
     unsigned *ticket = nullptr;             // of the reductions' last CTA (zero between launches)
     double *hhost = nullptr;                // pinned
     int precond = 0;                        // 0 block-Jacobi, 1 Schur (pmg.cu)
@@ -775,7 +738,7 @@ void free_work(Work &W)
     void *ptrs[] = {W.U, W.A, W.R, W.V1, W.pa, W.pv, W.prs, W.Uw, W.Aw, W.fw, W.xiw, W.ww, W.pu,
                     W.bu, W.bv, W.ba, W.buw, W.pw,
                     W.Vk, W.w, W.z, W.x, W.b, W.blocks, W.inv, W.partial, W.hcol, W.h2,
-                    W.ticket};
+                    W.ticket, W.clist, W.cmat};
     for (void *p : ptrs) cudaFree(p);
     cudaFree(W.ftmp);
     if (W.side) cudaStreamDestroy(W.side);
@@ -816,6 +779,7 @@ fsi_status ensure_work(fsi_mesh *mesh, int64_t m_pts, int restart)
     W.restart = restart;
     const size_t v = (size_t)n * 4 * sizeof(double);
     const size_t pm = (size_t)(m_pts > 0 ? m_pts : 1) * 3 * sizeof(double);
+    const int64_t cells = mesh->tet ? 0 : coupling_cells(mesh, m_pts);
     struct {
         void **p;
         size_t bytes;
@@ -831,6 +795,8 @@ fsi_status ensure_work(fsi_mesh *mesh, int64_t m_pts, int restart)
         {(void **)&W.hcol, (size_t)(restart + 2) * sizeof(double)},
         {(void **)&W.h2, (size_t)(restart + 2) * sizeof(double)},
         {(void **)&W.ticket, sizeof(double)},
+        {(void **)&W.clist, (size_t)(cells + 1) * sizeof(int32_t)},
+        {&W.cmat, (size_t)(cells + 1) * 36 * sizeof(double)},
     };
     for (auto &r : req) {
         cudaError_t e = cudaMalloc(r.p, r.bytes);
@@ -931,10 +897,17 @@ fsi_status coupled_residual_impl(fsi_mesh *mesh, const fsi_step_state *st, doubl
 fsi_status stage_linearisation(fsi_mesh *mesh, const fsi_step_state *st)
 {
     Work &W = mesh->newton->w;
+    W.cells = false;
     FSI_TRY(fsi_stage(mesh, FSI_F64, st->y, st->Vn, st->An, st->s, W.U, W.A));
     if (!(st->m > 0 && st->body)) return FSI_OK;
     FSI_TRY(fsi_dlm_interp(mesh, FSI_F64, st->m, st->elem, st->xi, st->y, W.pa));
     return solid_stage_impl(st->body, st->us, st->vs, st->as, W.pa, W.bu, W.bv, W.ba);
+}
+
+// point masses on a structured grid: the coupling by the cells' matrices
+bool coupling_by_cells(const fsi_mesh *mesh, const fsi_step_state *st)
+{
+    return st->m > 0 && !st->body && !mesh->tet;
 }
 
 // Working-precision copies of the linearisation point (after a residual or
@@ -967,7 +940,7 @@ fsi_status coupled_jacobian_impl(fsi_mesh *mesh, const fsi_step_state *st, const
     const int64_t n = mesh->n_nodes;
     const fsi_prec P = prec_of<T>();
     // point masses on a structured grid: the coupling overlaps the VMS Jacobian
-    const bool overlap = st->m > 0 && !st->body && !mesh->tet;
+    const bool overlap = coupling_by_cells(mesh, st);
     if (overlap) {
         // x is ready on s: the side stream may start the coupling
         FSI_CUDA(cudaEventRecord(W.ev_fork, s), "event record");
@@ -988,28 +961,28 @@ fsi_status coupled_jacobian_impl(fsi_mesh *mesh, const fsi_step_state *st, const
         FSI_TRY(fsi_dlm_spread(mesh, P, st->m, st->elem, W.xiw, st->cell_start, st->perm, W.pu,
                                st->w ? W.ww : nullptr, Jx, 1));
     } else if (st->m > 0) {
-        // C D C^T x on the side stream (D = w (drho + k gamma dt^2)): it needs
-        // only x, so it overlaps the VMS Jacobian issued above on s
-        const double D = st->drho_s + st->k_s * mesh->gamma * mesh->phys.dt * mesh->phys.dt;
+        // C D C^T x on the side stream by the cells' matrices: it needs only x,
+        // so it overlaps the VMS Jacobian issued above on s
         mesh->stream = W.side;
         const fsi_status cs = [&]() -> fsi_status {
-            FSI_TRY(interp_scaled<T>(mesh, st->m, st->elem, (const T *)W.xiw, x, (T)D, (T *)W.pu));
-            return fsi_dlm_spread(mesh, P, st->m, st->elem, W.xiw, st->cell_start, st->perm,
-                                  W.pu, st->w ? W.ww : nullptr, W.ftmp, 0);
+            if (!W.cells) {
+                // the first application of a step: the points stay where they are
+                const double D = st->drho_s + st->k_s * mesh->gamma * mesh->phys.dt * mesh->phys.dt;
+                FSI_TRY(coupling_build<T>(mesh, st->m, (const T *)W.xiw, st->cell_start, st->perm,
+                                          st->w ? (const T *)W.ww : nullptr, (T)D, W.clist,
+                                          (T *)W.cmat));
+            }
+            return coupling_apply<T>(mesh, st->m, W.clist, (const T *)W.cmat, x);
         }();
         mesh->stream = s;
+        W.cells = cs == FSI_OK;
         FSI_TRY(cs);
         FSI_CUDA(cudaEventRecord(W.ev_join, W.side), "event record");
         FSI_CUDA(cudaStreamWaitEvent(s, W.ev_join, 0), "stream wait");
-        if (st->mask && (reinterpret_cast<uintptr_t>(st->mask) & 3) == 0) {
-            // the coupling's forces and the Dirichlet rows in one pass
-            add_xyz_rows_kernel<T><<<grid1d(n), 256, 0, s>>>(
-                n, (const vec4<T> *)W.ftmp, (const uchar4 *)st->mask, (const vec4<T> *)x,
-                (vec4<T> *)Jx);
-            return check_launch("coupling add kernel");
-        }
-        add_xyz_kernel<T><<<grid1d(n), 256, 0, s>>>(n, (const vec4<T> *)W.ftmp, (vec4<T> *)Jx);
-        FSI_TRY(check_launch("coupling add kernel"));
+        // the coupling's forces and the Dirichlet rows in one pass
+        const bool rows = (reinterpret_cast<uintptr_t>(st->mask) & 3) == 0;
+        FSI_TRY(coupling_finish<T>(mesh, st->cell_start, rows ? st->mask : nullptr, x, Jx));
+        if (rows) return FSI_OK;
     }
     if (st->mask) {
         dirichlet_rows_kernel<T><<<grid1d(4 * n), 256, 0, s>>>(4 * n, st->mask, x, Jx);
@@ -1317,6 +1290,7 @@ fsi_status newton_impl(fsi_mesh *mesh, const fsi_newton_opts *o, const fsi_step_
 {
     Work &W = mesh->newton->w;
     cudaStream_t s = mesh->stream;
+    W.cells = false;
     const int64_t len = 4 * mesh->n_nodes;
     const fsi_prec rp = o->residual_prec == FSI_DF64 ? FSI_DF64 : FSI_F64;
     if (o->R0 && !(st->m > 0 && st->body)) {
@@ -1388,6 +1362,7 @@ fsi_status coupled_jacobian_f32(fsi_mesh *mesh, const fsi_step_state *st, int k,
 {
     FSI_TRY(ensure_work(mesh, st->m, 1));
     Work &W = mesh->newton->w;
+    W.cells = false;
     const bool body = st->m > 0 && st->body;
     if (body) FSI_TRY(coupled_residual_impl(mesh, st, R_fit ? R_fit : W.R, R_fit ? FSI_DF64 : FSI_F64));
     else FSI_TRY(fsi_stage(mesh, FSI_F64, st->y, st->Vn, st->An, st->s, W.U, W.A));
