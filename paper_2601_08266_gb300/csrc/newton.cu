@@ -24,6 +24,9 @@ constexpr int kRedGrid = 456;   // fixed partial-sum grid (3 CTAs per SM): deter
 constexpr int kAxpyGrid = 608;
 constexpr int kRedThreads = 256;
 constexpr int kDotGroup = 8;    // vectors per multi-dot pass
+// vectors the fused Gram-Schmidt pass holds in registers (an FP64 record takes
+// twice the registers of an FP32 one)
+template <typename T> constexpr int kFuseMax = sizeof(T) == 4 ? 16 : 8;
 static_assert(kDotGroup % 2 == 0, "the FP32 multi-dot pairs vectors");
 
 int grid1d(int64_t n, int threads = 256, int cap = sm_count() * 16)
@@ -243,6 +246,7 @@ struct DotFinal {
     double *out;
     int mode, kahan_j;
     double *flag;
+    double *add;  // when set: add[k] += the sum too
 };
 
 // (index self_k, when in [k0, k0+cnt), stands for w itself: w . w)
@@ -327,7 +331,10 @@ __global__ void __launch_bounds__(kRedThreads, 3) multi_dot_partial_kernel(
         for (int b = lane; b < (int)gridDim.x; b += 32) a += p[b];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        if (lane == 0) fin.out[k0 + wid] = fin.mode ? sqrt(a) : a;
+        if (lane == 0) {
+            fin.out[k0 + wid] = fin.mode ? sqrt(a) : a;
+            if (fin.add) fin.add[k0 + wid] += a;
+        }
     }
     if (fin.kahan_j >= 0) {
         __threadfence();
@@ -414,10 +421,111 @@ __global__ void __launch_bounds__(kRedThreads)
     }
 }
 
-__global__ void add_if_kernel(int n, const double *x, double *y, const double *cond)
+// The first Gram-Schmidt update and what follows it, in one pass over the basis:
+// w_i -= sum_k V_k[i] h[k] as multi_axpy_kernel does it (same order), then with
+// *flag set the second pass's dots V_k . w_new (as multi_dot_partial_kernel
+// forms them) into fin.out and added to fin.add, else |w_new| into *norm.  A
+// thread keeps its record of all cnt <= G vectors in registers between the
+// two, so the pass that the dots made over the basis is gone: Kahan's flag is
+// nearly always set with a good preconditioner, and at 128^3 the basis comes
+// from HBM each time (8 vectors: 102 us for the update and the dots as two launches,
+// 45 us here; at 32^3 19.5 -> 10.2 us).
+template <typename T, int G>
+__global__ void __launch_bounds__(kRedThreads, G * sizeof(T) <= 32 ? 3 : 2)
+    gs_update_kernel(int cnt, int64_t len4, const vec4<T> *V, int64_t vstride, const double *h,
+                     vec4<T> *w, double *partial, DotFinal fin, double *norm)
 {
-    if (*cond == 0.0) return;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) y[i] += x[i];
+    using Acc = typename DotAcc<T>::type;
+    __shared__ double red[G][kRedThreads / 32];
+    __shared__ T hs[G];
+    const bool second = *fin.flag != 0.0;
+    if (threadIdx.x < G) hs[threadIdx.x] = threadIdx.x < cnt ? (T)h[threadIdx.x] : T(0);
+    __syncthreads();
+    Acc acc[G];
+#pragma unroll
+    for (int j = 0; j < G; ++j) acc[j] = Acc(0);
+    GRID_STRIDE(i, len4)
+    {
+        vec4<T> wi = w[i];
+        vec4<T> v[G];
+#pragma unroll
+        for (int j = 0; j < G; ++j)
+            v[j] = j < cnt ? ld4(V + (int64_t)j * vstride + i) : vec4<T>{T(0), T(0), T(0), T(0)};
+#pragma unroll
+        for (int j = 0; j < G; ++j)
+            if (j < cnt) {
+                const T hk = hs[j];
+                wi.x = fma_rn(-v[j].x, hk, wi.x);
+                wi.y = fma_rn(-v[j].y, hk, wi.y);
+                wi.z = fma_rn(-v[j].z, hk, wi.z);
+                wi.w = fma_rn(-v[j].w, hk, wi.w);
+            }
+        w[i] = wi;
+        if (!second) {
+            dot_acc(acc[0], wi.x, wi.x);
+            dot_acc(acc[0], wi.y, wi.y);
+            dot_acc(acc[0], wi.z, wi.z);
+            dot_acc(acc[0], wi.w, wi.w);
+            dot_renorm(acc[0]);
+            continue;
+        }
+#pragma unroll
+        for (int j = 0; j < G; j += 2)
+            if (j < cnt) {
+                if constexpr (sizeof(T) == 4) {
+                    Comp2 a2{make_float2(acc[j].s, acc[j + 1].s),
+                             make_float2(acc[j].c, acc[j + 1].c)};
+                    dot_acc2(a2, make_float2(v[j].x, v[j + 1].x), make_float2(wi.x, wi.x));
+                    dot_acc2(a2, make_float2(v[j].y, v[j + 1].y), make_float2(wi.y, wi.y));
+                    dot_acc2(a2, make_float2(v[j].z, v[j + 1].z), make_float2(wi.z, wi.z));
+                    dot_acc2(a2, make_float2(v[j].w, v[j + 1].w), make_float2(wi.w, wi.w));
+                    dot_renorm2(a2);
+                    acc[j].s = a2.s.x;
+                    acc[j].c = a2.c.x;
+                    acc[j + 1].s = a2.s.y;
+                    acc[j + 1].c = a2.c.y;
+                } else {
+#pragma unroll
+                    for (int q = j; q < j + 2; ++q)
+                        if (q < cnt) {
+                            dot_acc(acc[q], v[q].x, wi.x);
+                            dot_acc(acc[q], v[q].y, wi.y);
+                            dot_acc(acc[q], v[q].z, wi.z);
+                            dot_acc(acc[q], v[q].w, wi.w);
+                        }
+                }
+            }
+    }
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, n = second ? cnt : 1;
+#pragma unroll
+    for (int g = 0; g < G; g += kDotGroup)
+        if (g < n) {
+            double v[kDotGroup];
+#pragma unroll
+            for (int j = 0; j < kDotGroup; ++j) v[j] = dot_value(acc[g + j]);
+            const double t = warp_sums8(v, lane);
+            if ((lane & 3) == 0) red[g + (lane >> 2)][wid] = t;
+        }
+    __syncthreads();
+    if (threadIdx.x < n) {
+        double v = 0.0;
+        for (int q = 0; q < kRedThreads / 32; ++q) v += red[threadIdx.x][q];
+        partial[(int64_t)threadIdx.x * kRedGrid + blockIdx.x] = v;
+    }
+    if (!last_cta(fin.ticket)) return;
+    for (int j = wid; j < n; j += kRedThreads / 32) {
+        const volatile double *p = partial + (int64_t)j * kRedGrid;
+        double a = 0.0;
+        for (int b = lane; b < (int)gridDim.x; b += 32) a += p[b];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (lane == 0) {
+            if (second) {
+                fin.out[j] = a;
+                fin.add[j] += a;
+            } else *norm = sqrt(a);
+        }
+    }
 }
 
 // y = x / *den (0 when the norm vanished: lucky breakdown), in the vector's
@@ -1071,12 +1179,12 @@ int red_grid(int64_t len4, int cap) { return grid1d(len4, kRedThreads, cap); }
 template <typename T>
 void multi_dot_launch(cudaStream_t s, int64_t len, int cnt, const T *V, int64_t ld, const T *w,
                       double *partial, unsigned *ticket, double *out, int norm, int self_k,
-                      const double *cond, int kahan_j, double *flag)
+                      const double *cond, int kahan_j, double *flag, double *add = nullptr)
 {
     const int grid = red_grid(len / 4, kRedGrid);
     for (int k0 = 0; k0 < cnt; k0 += kDotGroup) {
         const int c = cnt - k0 < kDotGroup ? cnt - k0 : kDotGroup;
-        const DotFinal fin = {ticket, out, norm, k0 + c == cnt ? kahan_j : -1, flag};
+        const DotFinal fin = {ticket, out, norm, k0 + c == cnt ? kahan_j : -1, flag, add};
         multi_dot_partial_kernel<T><<<grid, kRedThreads, 0, s>>>(
             k0, c, len / 4, (const vec4<T> *)V, ld / 4, (const vec4<T> *)w, partial, self_k, cond,
             fin);
@@ -1102,6 +1210,35 @@ void multi_axpy(cudaStream_t s, int cnt, int64_t len, const T *V, int64_t ld, co
 {
     multi_axpy_kernel<T><<<red_grid(len / 4, kAxpyGrid), kRedThreads, 0, s>>>(
         cnt, len / 4, (const vec4<T> *)V, ld / 4, h, (vec4<T> *)w, norm_partial, cond, ticket, norm);
+}
+
+// Classical Gram-Schmidt of w against V[:, :cnt], h = V^T w formed (in h): the update,
+// and with *flag the second pass, whose coefficients are added to h; |w| into
+// *norm.  Of a longer basis than the fused pass holds, the vectors behind it are
+// subtracted before it and dotted after it.
+template <typename T>
+void gram_schmidt(fsi_mesh *mesh, int cnt, const T *V, int64_t ld, double *h, T *w, double *flag,
+                  double *norm)
+{
+    Work &W = mesh->newton->w;
+    cudaStream_t s = mesh->stream;
+    const int64_t len = 4 * mesh->n_nodes;
+    double *npart = W.partial + (int64_t)(W.restart + 1) * kRedGrid;
+    const int c = cnt < kFuseMax<T> ? cnt : kFuseMax<T>, rest = cnt - c;
+    const DotFinal fin = {W.ticket, W.h2, 0, -1, flag, h};
+    // (two resident CTAs an SM with 64 registers of vectors, three with 32)
+    const int grid = red_grid(len / 4, c <= kDotGroup && sizeof(T) == 4 ? kRedGrid : kRedGrid * 2 / 3);
+    if (rest) multi_axpy<T>(s, rest, len, V + c * ld, ld, h + c, w);
+    if (c <= kDotGroup)
+        gs_update_kernel<T, kDotGroup><<<grid, kRedThreads, 0, s>>>(
+            c, len / 4, (const vec4<T> *)V, ld / 4, h, (vec4<T> *)w, W.partial, fin, norm);
+    else
+        gs_update_kernel<T, kFuseMax<T>><<<grid, kRedThreads, 0, s>>>(
+            c, len / 4, (const vec4<T> *)V, ld / 4, h, (vec4<T> *)w, W.partial, fin, norm);
+    if (rest)
+        multi_dot_launch<T>(s, len, rest, V + c * ld, ld, w, W.partial, W.ticket, W.h2 + c, 0, -1, flag,
+                            -1, nullptr, h + c);
+    multi_axpy<T>(s, cnt, len, V, ld, W.h2, w, npart, flag, W.ticket, norm);
 }
 
 template <typename T> fsi_status norm2(fsi_mesh *mesh, const T *x, double *dev_out)
@@ -1216,13 +1353,8 @@ fsi_status gmres(fsi_mesh *mesh, const fsi_step_state *st, int restart, int max_
             // iteration needs one host synchronisation, at its end; |w| of the
             // orthogonalised vector comes out of the update pass itself
             double *flag = W.h2 + restart + 1;
-            double *npart = W.partial + (int64_t)(restart + 1) * kRedGrid;
-            double *norm = W.hcol + j + 1;
             FSI_TRY(multi_dot<T>(mesh, j + 2, V, ld, w, W.hcol, 0, j + 1, nullptr, j, flag));
-            multi_axpy<T>(s, j + 1, len, V, ld, W.hcol, w, npart, nullptr, W.ticket, norm);
-            FSI_TRY(multi_dot<T>(mesh, j + 1, V, ld, w, W.h2, 0, -1, flag));
-            multi_axpy<T>(s, j + 1, len, V, ld, W.h2, w, npart, flag, W.ticket, norm);
-            add_if_kernel<<<1, 64, 0, s>>>(j + 1, W.h2, W.hcol, flag);
+            gram_schmidt<T>(mesh, j + 1, V, ld, W.hcol, w, flag, W.hcol + j + 1);
             FSI_TRY(check_launch("Gram-Schmidt"));
             scale_basis(W.hcol + j + 1, V + (int64_t)(j + 1) * ld);
             FSI_CUDA(cudaMemcpyAsync(W.hhost, W.hcol, (j + 2) * sizeof(double),

@@ -1,8 +1,9 @@
-"""The Krylov solver's parts that change with a size: the V-cycle's coarse levels
-by their shape."""
+"""The Krylov solver's parts that change with a size: the Gram-Schmidt update
+by the number of basis vectors, the V-cycle's coarse levels by their shape."""
 import numpy as np
 import pytest
 
+import test_gpu_newton as newton_case
 import test_gpu_precond as precond_case
 
 pytestmark = pytest.mark.gpu
@@ -15,6 +16,26 @@ def fsi():
         pytest.skip("no CUDA device")
     import paper_2601_08266_gb300 as pkg
     return pkg
+
+
+# basis lengths at the edges of 8 (one group of dots), 16 (the vectors an FP32
+# update holds) and beyond; with block Jacobi the solves use the whole restart
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("restart", [7, 8, 9, 16, 17, 40])
+def test_newton_step_by_restart_length(fsi, oracle, mixed, restart):
+    """Every solve reaches the residual reduction that was planned for it, so
+    the step converges in as many Newton iterations as with a long basis."""
+    mesh, st, dev, P, y0 = newton_case.setup(fsi, oracle, N=6, m=200, seed=3)
+    code, rep = fsi.fsi_newton_step(mesh, st, mixed=mixed, restart=restart, max_newton=12,
+                                    max_krylov=4000, newton_rtol=1e-8, krylov_rtol=1e-3, precond=0)
+    assert code == 0 and rep["converged"] == 1
+    assert rep["krylov_iters"] > restart, rep
+    r = np.linalg.norm(P.residual(newton_case.H(dev["y"])))
+    assert r <= 1.01e-8 * rep["r_ref"], (r, rep)
+    mesh2, st2, _, _, _ = newton_case.setup(fsi, oracle, N=6, m=200, seed=3)
+    _, full = fsi.fsi_newton_step(mesh2, st2, mixed=mixed, restart=150, max_newton=12,
+                                  max_krylov=4000, newton_rtol=1e-8, krylov_rtol=1e-3, precond=0)
+    assert rep["newton_iters"] <= full["newton_iters"] + 1, (rep, full)
 
 
 # first coarse levels of 1,331 nodes (split, 2 planes a slab), 729 (not split),
