@@ -177,7 +177,7 @@ __global__ void tet_geo_kernel(int64_t E, const int4 *__restrict__ tets,
         T g[kTetGeo];
         tet_geometry(c, g);
 #pragma unroll
-        for (int k = 0; k < kTetGeo; ++k) geo[e * kTetGeo + k] = g[k];
+        for (int k = 0; k < kTetGeo; ++k) geo[k * E + e] = g[k];
     }
 }
 
@@ -187,10 +187,13 @@ template <typename T> struct TetArgs {
     int64_t E;
     const vec4<S> *X;
     const int4 *tets;
-    const T *geo;  // [E][kTetGeo]
+    const T *geo;  // [kTetGeo][E]
     vec4<T> *slots;
 };
 
+// Four lanes per element (lane = node, then quadrature point): used on small
+// meshes, where it spreads an element over four threads; every lane repeats the
+// element's gradients (the rule: tet_by_element).
 template <typename T, bool JAC> __global__ void __launch_bounds__(256) tet_vms_kernel(TetArgs<T> P)
 {
     using S = typename StorageOf<T>::type;
@@ -217,20 +220,20 @@ template <typename T, bool JAC> __global__ void __launch_bounds__(256) tet_vms_k
         Geo<T> geo;
         T GG;
         if (valid) {
-            const T *g = P.geo + e * kTetGeo;
+            auto g = [&](int k) { return P.geo[k * P.E + e]; };
 #pragma unroll
             for (int i = 0; i < 3; ++i)
 #pragma unroll
-                for (int k = 0; k < 3; ++k) geo.Ji[i][k] = g[3 * i + k];
-            geo.G[0][0] = g[9];
-            geo.G[0][1] = geo.G[1][0] = g[10];
-            geo.G[0][2] = geo.G[2][0] = g[11];
-            geo.G[1][1] = g[12];
-            geo.G[1][2] = geo.G[2][1] = g[13];
-            geo.G[2][2] = g[14];
-            GG = g[15];
-            geo.inv_trG = g[16];
-            geo.det = g[17];  // holds the quadrature weight |det J| / 24
+                for (int k = 0; k < 3; ++k) geo.Ji[i][k] = g(3 * i + k);
+            geo.G[0][0] = g(9);
+            geo.G[0][1] = geo.G[1][0] = g(10);
+            geo.G[0][2] = geo.G[2][0] = g(11);
+            geo.G[1][1] = g(12);
+            geo.G[1][2] = geo.G[2][1] = g(13);
+            geo.G[2][2] = g(14);
+            GG = g(15);
+            geo.inv_trG = g(16);
+            geo.det = g(17);  // holds the quadrature weight |det J| / 24
         } else {
 #pragma unroll
             for (int i = 0; i < 3; ++i)
@@ -335,23 +338,423 @@ template <typename T, bool JAC> __global__ void __launch_bounds__(256) tet_vms_k
     }
 }
 
-template <typename T>
-__global__ void tet_gather_kernel(int64_t n, const int32_t *__restrict__ start,
-                                  const int32_t *__restrict__ slot, const vec4<T> *__restrict__ in,
-                                  vec4<typename StorageOf<T>::type> *__restrict__ out)
+// One thread per element.  On a linear tetrahedron the gradients, the divergence
+// and the viscous stress are the same at all four quadrature points, so they are
+// formed once: about 760 operations per Jacobian element against 1,400 of the
+// four-lane kernel, and no shuffles.  float and double-float take their points two
+// at a time on the paired FP32 instructions; float is fully unrolled, the 8-byte
+// types run a rolled loop (their records come again from L1), which keeps the
+// registers and the instruction footprint small.  Pressure enters per unit of
+// density, rho at the end, as in the hexahedral kernels (vms_device.cuh, brick_body).
+template <typename T> struct Points {  // quadrature points per pass
+    static constexpr int n = 1;
+    using C = T;
+    static __device__ __forceinline__ C set(T a, T) { return a; }
+    static __device__ __forceinline__ T first(C a) { return a; }
+    static __device__ __forceinline__ T second(C) { return T(0); }
+    static __device__ __forceinline__ T sum(C a) { return a; }
+};
+template <> struct Points<df64> {
+    static constexpr int n = 2;
+    using C = df64x2;
+    static __device__ __forceinline__ C set(df64 a, df64 b) { return PairOf<df64>::pack(a, b); }
+    static __device__ __forceinline__ df64 first(C a) { return PairOf<df64>::first(a); }
+    static __device__ __forceinline__ df64 second(C a) { return PairOf<df64>::second(a); }
+    static __device__ __forceinline__ df64 sum(C a) { return first(a) + second(a); }
+};
+template <> struct Points<float> {
+    static constexpr int n = 2;
+    using C = f32x2;
+    static __device__ __forceinline__ C set(float a, float b) { return {make_float2(a, b)}; }
+    static __device__ __forceinline__ float first(C a) { return a.v.x; }
+    static __device__ __forceinline__ float second(C a) { return a.v.y; }
+    static __device__ __forceinline__ float sum(C a) { return a.v.x + a.v.y; }
+};
+
+template <typename T, bool JAC>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 || (!JAC && std::is_same<T, df64>::value) ? 4 : 3)
+    tet_vms_elem_kernel(TetArgs<T> P)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        vec4<T> acc = {T(0), T(0), T(0), T(0)};
-        for (int k = start[i]; k < start[i + 1]; ++k) {
-            const vec4<T> r = ld4_blk(in + slot[k]);
-            acc.x += r.x;
-            acc.y += r.y;
-            acc.z += r.z;
-            acc.w += r.w;
+    using S = typename StorageOf<T>::type;
+    using PT = Points<T>;
+    using C = typename PT::C;
+    const VmsArgs<T> &V = P.V;
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e >= P.E) return;
+    const int *nodes = reinterpret_cast<const int *>(P.tets + e);
+    auto geo = [&](int k) -> T {
+        return geo_ld<T>(reinterpret_cast<const typename GeoStore<T>::type *>(P.geo) + k * P.E + e);
+    };
+    auto load_u = [&](int n) {
+        vec4<T> u = load_c<T>(V.U + n);
+        u.w = V.inv_rho * u.w;
+        return u;
+    };
+    auto load_a = [&](int n) {
+        vec4<T> a = load_c<T>(V.A + n);
+        if (V.f) {
+            const vec4<T> f = load_c<T>(V.f + n);
+            a.x = a.x - f.x;
+            a.y = a.y - f.y;
+            a.z = a.z - f.z;
         }
-        out[i] = {to_s(acc.x), to_s(acc.y), to_s(acc.z), to_s(acc.w)};
+        return a;
+    };
+    auto load_x = [&](int n) {
+        vec4<T> x = load_c<T>(V.x + n);
+        x.x = V.c_v * x.x;
+        x.y = V.c_v * x.y;
+        x.z = V.c_v * x.z;
+        x.w = V.inv_rho * x.w;
+        return x;
+    };
+    // double-float: the records' values for the points' loop, converted once, in this
+    // thread's column of shared memory (u, v, w, A and s, x)
+    constexpr bool kKeep = std::is_same<T, df64>::value;
+    constexpr int kVals = JAC ? 10 : 7;
+    __shared__ float2 kept[kKeep ? 4 * kVals * 128 : 1];
+    auto keep = [&](int node, int val, T t) {
+        if constexpr (kKeep) kept[(node * kVals + val) * 128 + threadIdx.x] = make_float2(t.hi, t.lo);
+    };
+    auto keep3 = [&](int node, int val, const vec4<T> &t) {
+        keep(node, val, t.x);
+        keep(node, val + 1, t.y);
+        keep(node, val + 2, t.z);
+    };
+    auto get3 = [&](int node, int val) {
+        vec4<T> t;
+        if constexpr (kKeep) {
+            const float2 *q = kept + (node * kVals + val) * 128 + threadIdx.x;
+            t = {T(q[0].x, q[0].y), T(q[128].x, q[128].y), T(q[256].x, q[256].y), T(0)};
+        }
+        return t;
+    };
+    auto get1 = [&](int node, int val) {
+        T t;
+        if constexpr (kKeep) {
+            const float2 q = kept[(node * kVals + val) * 128 + threadIdx.x];
+            t = T(q.x, q.y);
+        }
+        return t;
+    };
+    auto bc = [](T a) { return PT::set(a, a); };
+    const T be = tet_be<T>(), amb = tet_al<T>() - be;
+    T Ji[3][3];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) Ji[k / 3][k % 3] = geo(k);
+
+    // be x (sum over the nodes), and the gradients from the differences to
+    // node 0: d_j w = sum_k Ji[k][j] (w_{k+1} - w_0)
+    T su[4], sa[4], sx[4], G[4][3], dG[4][3];
+    T Sp, Sdp;  // sums of the pressures over the points = over the nodes
+    {
+        const vec4<T> u0 = load_u(nodes[0]), a0 = load_a(nodes[0]);
+        keep3(0, 0, u0);
+        keep3(0, 3, a0);
+        if (V.has_s) keep(0, 6, a0.w);
+        const T w0[4] = {u0.x, u0.y, u0.z, u0.w};
+        T x0[4] = {T(0), T(0), T(0), T(0)};
+        if constexpr (JAC) {
+            const vec4<T> v = load_x(nodes[0]);
+            keep3(0, 7, v);
+            x0[0] = v.x, x0[1] = v.y, x0[2] = v.z, x0[3] = v.w;
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) su[c] = w0[c], sx[c] = x0[c];
+        sa[0] = a0.x, sa[1] = a0.y, sa[2] = a0.z, sa[3] = a0.w;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int n = nodes[k + 1];
+            const vec4<T> uk = load_u(n), ak = load_a(n);
+            keep3(k + 1, 0, uk);
+            keep3(k + 1, 3, ak);
+            if (V.has_s) keep(k + 1, 6, ak.w);
+            const T w[4] = {uk.x, uk.y, uk.z, uk.w};
+            sa[0] = sa[0] + ak.x;
+            sa[1] = sa[1] + ak.y;
+            sa[2] = sa[2] + ak.z;
+            if (V.has_s) sa[3] = sa[3] + ak.w;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                su[c] = su[c] + w[c];
+                const T d = w[c] - w0[c];
+#pragma unroll
+                for (int j = 0; j < 3; ++j) G[c][j] = k ? fma_t(Ji[k][j], d, G[c][j]) : Ji[k][j] * d;
+            }
+            if constexpr (JAC) {
+                const vec4<T> xk = load_x(n);
+                keep3(k + 1, 7, xk);
+                const T y[4] = {xk.x, xk.y, xk.z, xk.w};
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    sx[c] = sx[c] + y[c];
+                    const T d = y[c] - x0[c];
+#pragma unroll
+                    for (int j = 0; j < 3; ++j)
+                        dG[c][j] = k ? fma_t(Ji[k][j], d, dG[c][j]) : Ji[k][j] * d;
+                }
+            }
+        }
+        Sp = su[3];
+        Sdp = sx[3];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            su[c] = be * su[c];
+            if (c < 3 || V.has_s) sa[c] = be * sa[c];
+            if constexpr (JAC) sx[c] = be * sx[c];
+        }
     }
+    const T rC = G[0][0] + G[1][1] + G[2][2];
+    const T drC = JAC ? dG[0][0] + dG[1][1] + dG[2][2] : T(0);
+    const T q0 = fma_t(V.CInu2, geo(15), V.ct_dt2), itrG = geo(16);
+
+    // sums over the points of the coefficients: Y without the viscous part and
+    // with the pressures' sum apart; X at each point for the projection
+    T SY[4][3], SX[3], Spp = T(0), Xp[4][3];
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) SY[c][j] = T(0);
+    SX[0] = SX[1] = SX[2] = T(0);
+#pragma unroll(sizeof(T) == 4 ? 2 : 1)
+    for (int g = 0; g < 4; g += PT::n) {
+        [[maybe_unused]] const int n0 = nodes[g], n1 = nodes[g + PT::n - 1];
+        auto at = [&](T s, T a, T b) { return fma_t(bc(amb), PT::set(a, b), bc(s)); };
+        C v[3], r[3], a[3], s;
+        {
+            vec4<T> u0, a0, u1, a1;
+            if constexpr (kKeep) {
+                u0 = get3(g, 0), a0 = get3(g, 3), u1 = get3(g + 1, 0), a1 = get3(g + 1, 3);
+                if (V.has_s) a0.w = get1(g, 6), a1.w = get1(g + 1, 6);
+            } else {
+                u0 = load_u(n0), a0 = load_a(n0);
+                u1 = u0, a1 = a0;
+                if constexpr (PT::n == 2) u1 = load_u(n1), a1 = load_a(n1);
+            }
+            v[0] = at(su[0], u0.x, u1.x);
+            v[1] = at(su[1], u0.y, u1.y);
+            v[2] = at(su[2], u0.z, u1.z);
+            a[0] = at(sa[0], a0.x, a1.x);
+            a[1] = at(sa[1], a0.y, a1.y);
+            a[2] = at(sa[2], a0.z, a1.z);
+            if (V.has_s) s = at(sa[3], a0.w, a1.w);
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            C t = a[i] + bc(G[3][i]);
+            t = fma_t(v[0], bc(G[i][0]), t);
+            t = fma_t(v[1], bc(G[i][1]), t);
+            r[i] = fma_t(v[2], bc(G[i][2]), t);
+        }
+        // S = s (q0 + v.G v), tau_M = S^-1/2, tau_C = S tau_M / tr G
+        const C g01 = bc(geo(10)), g02 = bc(geo(11)), g12 = bc(geo(13));
+        const C gv[3] = {dot3_t(bc(geo(9)), v[0], g01, v[1], g02, v[2]),
+                         dot3_t(g01, v[0], bc(geo(12)), v[1], g12, v[2]),
+                         dot3_t(g02, v[0], g12, v[1], bc(geo(14)), v[2])};
+        C Sq = bc(q0) + dot3_t(gv[0], v[0], gv[1], v[1], gv[2], v[2]);
+        if (V.has_s) Sq = s * Sq;
+        const C tau = rsqrt_t(Sq), ntau = -tau, ntauC = Sq * ntau * bc(itrG);
+        C up[3], w[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            up[i] = ntau * r[i];
+            w[i] = v[i] + up[i];
+        }
+        const C pp = ntauC * bc(rC);
+        C X[3];
+        if constexpr (!JAC) {
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                C t = fma_t(w[0], bc(G[i][0]), a[i]);
+                t = fma_t(w[1], bc(G[i][1]), t);
+                X[i] = fma_t(w[2], bc(G[i][2]), t);
+                const C nup = -up[i];
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    if constexpr (PT::n == 1) SY[i][j] = fma_t(w[j], nup, SY[i][j]);
+                    else if constexpr (sizeof(T) == 8)
+                        SY[i][j] = fma_t(PT::second(w[j]), PT::second(nup),
+                                         fma_t(PT::first(w[j]), PT::first(nup), SY[i][j]));
+                    else SY[i][j] = SY[i][j] + PT::sum(w[j] * nup);
+                }
+                SY[3][i] = SY[3][i] + PT::sum(nup);
+            }
+            Spp = Spp + PT::sum(pp);
+        } else {
+            C dv[3];
+            {
+                vec4<T> x0, x1;
+                if constexpr (kKeep) {
+                    x0 = get3(g, 7), x1 = get3(g + 1, 7);
+                } else {
+                    x0 = load_x(n0), x1 = x0;
+                    if constexpr (PT::n == 2) x1 = load_x(n1);
+                }
+                dv[0] = at(sx[0], x0.x, x1.x);
+                dv[1] = at(sx[1], x0.y, x1.y);
+                dv[2] = at(sx[2], x0.z, x1.z);
+            }
+            const C vGdv = dot3_t(gv[0], dv[0], gv[1], dv[1], gv[2], dv[2]);
+            C k = tau * tau * vGdv;
+            if (V.has_s) k = s * k;
+            C da[3], dup[3], dw[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                da[i] = bc(V.c_av) * dv[i];
+                C t = da[i] + bc(dG[3][i]);
+                t = fma_t(v[0], bc(dG[i][0]), t);
+                t = fma_t(v[1], bc(dG[i][1]), t);
+                t = fma_t(v[2], bc(dG[i][2]), t);
+                t = fma_t(dv[0], bc(G[i][0]), t);
+                t = fma_t(dv[1], bc(G[i][1]), t);
+                t = fma_t(dv[2], bc(G[i][2]), t);
+                dup[i] = ntau * t - k * up[i];
+            }
+#pragma unroll
+            for (int i = 0; i < 3; ++i) dw[i] = dv[i] + dup[i];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                C t = fma_t(dw[0], bc(G[i][0]), da[i]);
+                t = fma_t(dw[1], bc(G[i][1]), t);
+                t = fma_t(dw[2], bc(G[i][2]), t);
+                t = fma_t(w[0], bc(dG[i][0]), t);
+                t = fma_t(w[1], bc(dG[i][1]), t);
+                X[i] = fma_t(w[2], bc(dG[i][2]), t);
+                const C nup = -up[i], ndup = -dup[i];
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    if constexpr (PT::n == 1)
+                        SY[i][j] = fma_t(dw[j], nup, fma_t(w[j], ndup, SY[i][j]));
+                    else
+                        SY[i][j] = SY[i][j] + PT::sum(fma_t(dw[j], nup, w[j] * ndup));
+                }
+                SY[3][i] = SY[3][i] + PT::sum(ndup);
+            }
+            Spp = Spp + PT::sum(dot2_t(k, pp, ntauC, bc(drC)));
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            SX[i] = SX[i] + PT::sum(X[i]);
+            if constexpr (kKeep) {  // over u, which these points no longer need
+                keep(g, i, PT::first(X[i]));
+                keep(g + 1, i, PT::second(X[i]));
+            } else {
+                Xp[g][i] = PT::first(X[i]);
+                if constexpr (PT::n == 2) Xp[g + 1][i] = PT::second(X[i]);
+            }
+        }
+    }
+    // the parts that are the same at every point: viscous stress, pressure sums
+    {
+        const T(&H)[4][3] = JAC ? dG : G;
+        const T nu4 = V.nu2 + V.nu2, nu8 = nu4 + nu4;  // 4 nu, 8 nu
+        const T p = JAC ? Sdp + Spp : Sp + Spp;
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = i; j < 3; ++j) {
+                if (i == j) {
+                    SY[i][i] = fma_t(nu8, H[i][i], SY[i][i]) - p;
+                } else {
+                    const T m = H[i][j] + H[j][i];
+                    SY[i][j] = fma_t(nu4, m, SY[i][j]);
+                    SY[j][i] = fma_t(nu4, m, SY[j][i]);
+                }
+            }
+    }
+    // projection: node a gets amb X(a) + be sum X + grad N_a . SY, the continuity
+    // row div + grad N_a . SY_3; grad N_0 = -(sum of the others)
+    // (double-float reads Ji again: its 18 registers are worth more in the loop)
+    if constexpr (kKeep)
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            float2 t;
+            asm volatile("ld.global.v2.f32 {%0, %1}, [%2];"
+                         : "=f"(t.x), "=f"(t.y)
+                         : "l"(reinterpret_cast<const float2 *>(P.geo) + k * P.E + e));
+            Ji[k / 3][k % 3] = T(t.x, t.y);
+        }
+    const T wc = geo(17), wm = V.rho * wc;
+    T q[4][4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            q[k + 1][c] = dot3_t(Ji[k][0], SY[c][0], Ji[k][1], SY[c][1], Ji[k][2], SY[c][2]);
+        q[0][c] = -(q[1][c] + q[2][c] + q[3][c]);
+    }
+    const T div = JAC ? drC : rC;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        T o[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) o[i] = wm * (fma_t(amb, kKeep ? get1(a, i) : Xp[a][i], fma_t(be, SX[i], q[a][i])));
+        P.slots[4 * e + a] = vec4<T>{o[0], o[1], o[2], wc * (div + q[a][3])};
+    }
+}
+
+// Which of the two kernels.  A thread per element needs enough elements to fill the
+// chip: in FP32 the two are level below 10,000 elements, in FP64 a mesh of 3,072 takes
+// 37.2 us by elements against 35.2 us by lanes, and double-float, with its long
+// dependent operations, is level at 24,576 (10,368: 20.8 against 16.8 us).  At 279,936
+// elements, residual / Jacobian with their gathers, by lanes -> by elements: FP32
+// 36.1/43.5 -> 27.0/32.8 us, FP64 508/787 -> 291/466 us, double-float 126/181 ->
+// 93/145 us.
+template <typename T> bool tet_by_element(int64_t E)
+{
+    return E >= (std::is_same<T, df64>::value ? 25000 : 10000);
+}
+
+// Sums over the four lanes of a node of four values each: lane q ends with value q.
+template <typename T> __device__ __forceinline__ T quad_sum4(const T (&v)[4], int q)
+{
+    const bool b1 = q & 2, b0 = q & 1;
+    T h[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const T send = b1 ? v[k] : v[2 + k], keep = b1 ? v[2 + k] : v[k];
+        h[k] = keep + shfl_x(send, 2);
+    }
+    const T send = b0 ? h[0] : h[1], keep = b0 ? h[1] : h[0];
+    return keep + shfl_x(send, 1);
+}
+
+// Element slots to nodes: a node's slots (24 on average) in four lanes, four
+// slots a lane in flight.  Bound by the latency of two dependent reads: one
+// thread per node, slot after slot, took 23 us at
+// 279,936 elements, this 14 us.
+template <typename T>
+__global__ void __launch_bounds__(256)
+    tet_gather_kernel(int64_t n, const int32_t *__restrict__ start, const int32_t *__restrict__ slot,
+                      const vec4<T> *__restrict__ in, typename StorageOf<T>::type *__restrict__ out)
+{
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, i = t >> 2;
+    const int q = (int)(t & 3);
+    int k = 0, k1 = 0;
+    if (i < n) {
+        k = start[i] + q;
+        k1 = start[i + 1];
+    }
+    T acc[4] = {T(0), T(0), T(0), T(0)};
+    for (; k < k1; k += 16) {
+        int sl[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) sl[u] = k + 4 * u < k1 ? slot[k + 4 * u] : -1;
+        vec4<T> v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (sl[u] >= 0) v[u] = ld4_blk(in + sl[u]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (sl[u] >= 0) {
+                acc[0] += v[u].x;
+                acc[1] += v[u].y;
+                acc[2] += v[u].z;
+                acc[3] += v[u].w;
+            }
+    }
+    const T sum = quad_sum4<T>(acc, q);
+    if (i < n) out[t] = to_s(sum);
 }
 
 // ------------------------------------------------------------------ location
@@ -420,68 +823,149 @@ __device__ __forceinline__ int screen32(const float4 &x0, const float4 &x1, cons
     return lmin >= -1e-5f ? 2 : 1;
 }
 
-__global__ void tet_locate_kernel(int64_t m, BucketArgs B, const double4 *__restrict__ X64,
-                                  const float4 *__restrict__ X32, const int4 *__restrict__ tets,
-                                  const int32_t *__restrict__ bstart,
-                                  const int32_t *__restrict__ btets, const double *__restrict__ P,
-                                  int32_t *__restrict__ elem, double *__restrict__ lam_out,
-                                  int32_t *__restrict__ count, unsigned long long *n_out)
+// A warp takes npw points (4, 8 or 16, few enough to fill the chip), each in a lane.
+// Screening: eight lanes test eight
+// elements of a point's list at a time in FP32, until every point has an element
+// that holds it almost surely, four candidates, or no list left.  Then the exact FP64
+// test runs over all (point, candidate) pairs of the warp, packed over the lanes, and
+// a point takes its first candidate that passes, in list order.  Bound by the
+// FP64 unit (about 120 operations a test, 16 cycles each) and by the latency of
+// the screening's dependent reads; with a point's screening and tests in its own
+// lane, lists of unequal length and candidate numbers left most lanes idle (50,000 points in
+// 279,936 elements: 76 us, now 46 us).
+constexpr int kLocThreads = 128, kLocCand = 4;
+__global__ void __launch_bounds__(kLocThreads)
+    tet_locate_kernel(int64_t m, BucketArgs B, const double4 *__restrict__ X64,
+                      const float4 *__restrict__ X32, const int4 *__restrict__ tets,
+                      const int32_t *__restrict__ bstart, const int32_t *__restrict__ btets,
+                      const double *__restrict__ P, int npw, int32_t *__restrict__ elem,
+                      double *__restrict__ lam_out, int32_t *__restrict__ count,
+                      unsigned long long *n_out)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const double p[3] = {P[3 * i], P[3 * i + 1], P[3 * i + 2]};
-        int found = -1;
-        double lam[4] = {0.0, 0.0, 0.0, 0.0};
-        bool inbox = true;
-        for (int k = 0; k < 3; ++k)
-            inbox = inbox && p[k] >= B.box_lo[k] && p[k] <= B.box_hi[k];  // NaN: outside
-        if (inbox) {
-            int bi[3];
+    constexpr unsigned kAll = 0xffffffffu;
+    __shared__ int cand_s[kLocThreads / 32][32 * kLocCand], pair_s[kLocThreads / 32][32 * kLocCand];
+    __shared__ uint8_t owner_s[kLocThreads / 32][32 * kLocCand];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int *cand = cand_s[wid] + lane * kLocCand, *pairs = pair_s[wid];
+    uint8_t *owners = owner_s[wid];
+    const int64_t step = (int64_t)gridDim.x * (kLocThreads / 32) * npw;
+    for (int64_t i0 = (blockIdx.x * (int64_t)(kLocThreads / 32) + wid) * npw; i0 < m; i0 += step) {
+        const int64_t i = lane < npw ? i0 + lane : m;
+        double p[3] = {0.0, 0.0, 0.0};
+        int found = -1, c = 0, cend = 0;
+        double l1 = 0.0, l2 = 0.0, l3 = 0.0;
+        if (i < m) {
+            bool inbox = true;
             for (int k = 0; k < 3; ++k) {
-                int v = (int)floor((p[k] - B.lo[k]) * B.inv_cell[k]);
-                bi[k] = v < 0 ? 0 : (v >= B.nb[k] ? B.nb[k] - 1 : v);
+                p[k] = P[3 * i + k];
+                inbox = inbox && p[k] >= B.box_lo[k] && p[k] <= B.box_hi[k];  // NaN: outside
             }
-            const int64_t bk = bi[0] + (int64_t)B.nb[0] * (bi[1] + (int64_t)B.nb[1] * bi[2]);
-            const float pf[3] = {(float)p[0], (float)p[1], (float)p[2]};
-            // the FP32 screen collects candidates in list order (up to four,
-            // or up to one it finds almost surely inside), then the exact FP64
-            // test runs on them in that order; the lanes of a warp reach the
-            // FP64 block together far more often than if each ran it at its
-            // own position in the list
-            int c = bstart[bk];
-            const int cend = bstart[bk + 1];
-            while (c < cend && found < 0) {
-                int cand[4], nc = 0;
-                bool likely = false;
-                for (; c < cend && nc < 4 && !likely; ++c) {
-                    const int e = btets[c];
-                    const int4 t = tets[e];
-                    const int sc = screen32(X32[t.x], X32[t.y], X32[t.z], X32[t.w], pf);
-                    if (sc > 0) cand[nc++] = e;
-                    likely = sc == 2;
+            if (inbox) {
+                int bi[3];
+                for (int k = 0; k < 3; ++k) {
+                    int v = (int)floor((p[k] - B.lo[k]) * B.inv_cell[k]);
+                    bi[k] = v < 0 ? 0 : (v >= B.nb[k] ? B.nb[k] - 1 : v);
                 }
-                for (int k = 0; k < nc; ++k) {
-                    const int4 t = tets[cand[k]];
-                    barycentric64(X64[t.x], X64[t.y], X64[t.z], X64[t.w], p, lam);
-                    if (lam[0] >= -1e-12 && lam[1] >= -1e-12 && lam[2] >= -1e-12 &&
-                        lam[3] >= -1e-12) {
-                        found = cand[k];
-                        break;
+                const int64_t bk = bi[0] + (int64_t)B.nb[0] * (bi[1] + (int64_t)B.nb[1] * bi[2]);
+                c = bstart[bk];
+                cend = bstart[bk + 1];
+            }
+        }
+        const float pf[3] = {(float)p[0], (float)p[1], (float)p[2]};
+        while (__any_sync(kAll, found < 0 && c < cend)) {
+            int nc = 0;
+            bool more = found < 0 && c < cend;
+            while (unsigned need = __ballot_sync(kAll, more)) {
+#pragma unroll 2
+                for (int g = 0; g < npw / 4; ++g) {
+                    if (!((need >> (4 * g)) & 15u)) continue;  // none of these four points
+                    const int src = 4 * g + (lane >> 3);
+                    const int k = __shfl_sync(kAll, c, src) + (lane & 7);
+                    const int ke = __shfl_sync(kAll, cend, src);
+                    const float q[3] = {__shfl_sync(kAll, pf[0], src), __shfl_sync(kAll, pf[1], src),
+                                        __shfl_sync(kAll, pf[2], src)};
+                    int sc = 0;
+                    if (((need >> src) & 1u) && k < ke) {
+                        const int4 t = tets[btets[k]];
+                        sc = screen32(X32[t.x], X32[t.y], X32[t.z], X32[t.w], q);
+                    }
+                    const unsigned some = __ballot_sync(kAll, sc > 0), sure = __ballot_sync(kAll, sc == 2);
+                    if (more && (lane >> 2) == g) {
+                        unsigned m1 = (some >> (8 * (lane & 3))) & 255u;
+                        const unsigned m2 = (sure >> (8 * (lane & 3))) & 255u;
+                        int next = c + 8;
+                        if (m2) {
+                            const int f = __ffs((int)m2);  // up to and with the first sure one
+                            m1 &= (1u << f) - 1u;
+                            next = c + f;
+                            more = false;
+                        }
+                        while (m1) {
+                            const int f = __ffs((int)m1);
+                            m1 &= m1 - 1u;
+                            cand[nc++] = c + f - 1;
+                            if (nc == kLocCand) {
+                                next = c + f;
+                                more = false;
+                                break;
+                            }
+                        }
+                        c = next < cend ? next : cend;
+                        more = more && c < cend;
                     }
                 }
             }
+            // the pairs of all points, point by point
+            int first = nc;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(kAll, first, o);
+                if (lane >= o) first += v;
+            }
+            const int total = __shfl_sync(kAll, first, 31);
+            first -= nc;
+            for (int k = 0; k < nc; ++k) {
+                pairs[first + k] = cand[k];
+                owners[first + k] = (uint8_t)lane;
+            }
+            __syncwarp();
+            for (int b = 0; b < total; b += 32) {
+                const bool live = b + lane < total;
+                const int own = live ? owners[b + lane] : lane, e = live ? btets[pairs[b + lane]] : 0;
+                const double pp[3] = {__shfl_sync(kAll, p[0], own), __shfl_sync(kAll, p[1], own),
+                                      __shfl_sync(kAll, p[2], own)};
+                double lam[4] = {0.0, 0.0, 0.0, 0.0};
+                bool ok = false;
+                if (live) {
+                    const int4 t = tets[e];
+                    barycentric64(X64[t.x], X64[t.y], X64[t.z], X64[t.w], pp, lam);
+                    ok = lam[0] >= -1e-12 && lam[1] >= -1e-12 && lam[2] >= -1e-12 && lam[3] >= -1e-12;
+                }
+                // this point's pairs among these 32
+                const int lo = max(first - b, 0), hi = min(first + nc - b, 32);
+                unsigned hit = __ballot_sync(kAll, ok);
+                hit = lo < hi ? (hit >> lo) << lo & (kAll >> (32 - hi)) : 0u;
+                const bool take = found < 0 && hit;
+                const int src = take ? __ffs((int)hit) - 1 : lane;
+                const int fe = __shfl_sync(kAll, e, src);
+                const double f1 = __shfl_sync(kAll, lam[1], src), f2 = __shfl_sync(kAll, lam[2], src),
+                             f3 = __shfl_sync(kAll, lam[3], src);
+                if (take) {
+                    found = fe;
+                    l1 = f1;
+                    l2 = f2;
+                    l3 = f3;
+                }
+            }
+            __syncwarp();
         }
-        if (found < 0) {
-            elem[i] = -1;
-            lam_out[3 * i] = lam_out[3 * i + 1] = lam_out[3 * i + 2] = 0.0;
-            atomicAdd(n_out, 1ull);
-            continue;
-        }
+        if (i >= m) continue;
         elem[i] = found;
-        lam_out[3 * i] = lam[1];
-        lam_out[3 * i + 1] = lam[2];
-        lam_out[3 * i + 2] = lam[3];
-        if (count) atomicAdd(count + found, 1);
+        lam_out[3 * i] = l1;
+        lam_out[3 * i + 1] = l2;
+        lam_out[3 * i + 2] = l3;
+        if (found < 0) atomicAdd(n_out, 1ull);
+        else if (count) atomicAdd(count + found, 1);
     }
 }
 
@@ -578,34 +1062,40 @@ __global__ void tet_spread_cells_kernel(int64_t E, const S *__restrict__ lam,
 }
 
 template <typename T, typename S = typename StorageOf<T>::type>
-__global__ void tet_spread_nodes_kernel(int64_t n, const int32_t *__restrict__ nstart,
-                                        const int32_t *__restrict__ nslot,
-                                        const int32_t *__restrict__ start,
-                                        const T *__restrict__ Ssum, S *__restrict__ F,
-                                        int accumulate)
+__global__ void __launch_bounds__(256)
+    tet_spread_nodes_kernel(int64_t n, const int32_t *__restrict__ nstart,
+                            const int32_t *__restrict__ nslot, const int32_t *__restrict__ start,
+                            const T *__restrict__ Ssum, S *__restrict__ F, int accumulate)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        T fx = T(0), fy = T(0), fz = T(0);
-        for (int k = nstart[i]; k < nstart[i + 1]; ++k) {
-            const int sl = nslot[k];
-            const int e = sl >> 2;
-            if (start[e + 1] == start[e]) continue;
-            const T *src = Ssum + (int64_t)e * 12 + 3 * (sl & 3);
-            fx += src[0];
-            fy += src[1];
-            fz += src[2];
-        }
-        if (accumulate) {
-            F[4 * i] = to_s(to_c<T>(F[4 * i]) + fx);
-            F[4 * i + 1] = to_s(to_c<T>(F[4 * i + 1]) + fy);
-            F[4 * i + 2] = to_s(to_c<T>(F[4 * i + 2]) + fz);
-        } else {
-            F[4 * i] = to_s(fx);
-            F[4 * i + 1] = to_s(fy);
-            F[4 * i + 2] = to_s(fz);
-        }
+    // four lanes per node, four slots a lane in flight, as in tet_gather_kernel
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, i = t >> 2;
+    const int q = (int)(t & 3);
+    int k = 0, k1 = 0;
+    if (i < n) {
+        k = nstart[i] + q;
+        k1 = nstart[i + 1];
     }
+    T acc[4] = {T(0), T(0), T(0), T(0)};
+    for (; k < k1; k += 16) {
+        int sl[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) sl[u] = k + 4 * u < k1 ? nslot[k + 4 * u] : -1;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int e = sl[u] >= 0 ? sl[u] >> 2 : 0;
+            if (start[e + 1] == start[e]) sl[u] = -1;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (sl[u] >= 0) {
+                const T *src = Ssum + 3 * (int64_t)sl[u];
+                acc[0] += src[0];
+                acc[1] += src[1];
+                acc[2] += src[2];
+            }
+    }
+    const T sum = quad_sum4<T>(acc, q);
+    if (i < n && q < 3) F[t] = to_s(accumulate ? to_c<T>(F[t]) + sum : sum);
 }
 
 __global__ void pad_tet_coords_kernel(int64_t n, const double *X, double4 *X64, float4 *X32)
@@ -642,6 +1132,9 @@ TetArgs<T> tet_args(fsi_tetmesh *m, const void *U, const void *A, const void *f,
     P.V.inv_rho = T(1.0 / rho);
     P.V.c_a = T(m->alpha_m);
     P.V.c_v = T(m->alpha_f * m->gamma * dt);
+    P.V.c_av = T(m->alpha_m / (m->alpha_f * m->gamma * dt));
+    P.V.nu = T(nu);
+    P.V.nu2 = T(2.0 * nu);
     P.V.ct_dt2 = T(m->phys.C_T / (dt * dt));
     P.V.CInu2 = T(m->phys.C_I * nu * nu);
     P.V.has_s = m->phys.has_s != 0;
@@ -692,11 +1185,15 @@ fsi_status tet_vms(fsi_tetmesh *m, const void *U, const void *A, const void *f, 
     FSI_TRY(ensure_geo<T>(m));
     TetArgs<T> P = tet_args<T>(m, U, A, f, x);
     P.geo = (const T *)m->geo[geo_slot<T>()];
-    const int64_t threads = 4 * m->n_elems;
-    tet_vms_kernel<T, JAC><<<grid_for(threads, 256, sm_count() * 64), 256, 0, m->stream>>>(P);
+    if (tet_by_element<T>(m->n_elems)) {
+        tet_vms_elem_kernel<T, JAC><<<(int)((m->n_elems + 127) / 128), 128, 0, m->stream>>>(P);
+    } else {
+        const int64_t threads = 4 * m->n_elems;
+        tet_vms_kernel<T, JAC><<<grid_for(threads, 256, sm_count() * 64), 256, 0, m->stream>>>(P);
+    }
     FSI_TRY(check_launch("tet vms kernel"));
-    tet_gather_kernel<T><<<grid_for(m->n_nodes, 256), 256, 0, m->stream>>>(
-        m->n_nodes, m->node_start, m->node_slot, P.slots, (vec4<S> *)out);
+    tet_gather_kernel<T><<<(int)((4 * m->n_nodes + 255) / 256), 256, 0, m->stream>>>(
+        m->n_nodes, m->node_start, m->node_slot, P.slots, (S *)out);
     return check_launch("tet gather kernel");
 }
 
@@ -1034,8 +1531,10 @@ fsi_status fsi_tet_locate(fsi_tetmesh *m, int64_t np, const double *P, int32_t *
             B.box_lo[k] = m->box_lo[k];
             B.box_hi[k] = m->box_hi[k];
         }
-        tet_locate_kernel<<<grid_for(np, 128), 128, 0, s>>>(
-            np, B, m->X64, m->X32, m->tets, m->bucket_start, m->bucket_tets, P, elem, lam,
+        int npw = 4;
+        while (npw < 16 && np > (int64_t)npw * 16 * sm_count()) npw *= 2;
+        tet_locate_kernel<<<grid_for((np + npw - 1) / npw * 32, kLocThreads), kLocThreads, 0, s>>>(
+            np, B, m->X64, m->X32, m->tets, m->bucket_start, m->bucket_tets, P, npw, elem, lam,
             table ? m->fill : nullptr, m->nout);
         FSI_TRY(check_launch("tet locate kernel"));
     }
@@ -1088,7 +1587,7 @@ fsi_status fsi_tet_spread(fsi_tetmesh *m, fsi_prec prec, int64_t np, const int32
     FSI_DEVICE(m->device);
     const int64_t E = m->n_elems;
     const int cg = grid_for((E + 7) / 8 * 32, 256, sm_count() * 64);
-    const int ng = grid_for(m->n_nodes, 256);
+    const int ng = (int)((4 * m->n_nodes + 255) / 256);
     cudaStream_t s = m->stream;
     if (prec == FSI_F64) {
         tet_spread_cells_kernel<double><<<cg, 256, 0, s>>>(E, (const double *)lam, cell_start, perm,
