@@ -765,23 +765,25 @@ fsi_status chebyshev(fsi_mesh *m, int l, int degree, double lo, double hi, const
 // ---------------------------------------------------------------- coarse levels
 // The V-cycle's FP32 levels of at most kCoarseNodes nodes, down to and with the
 // dense coarsest solve, as one cluster of CTAs: every vector of those levels lives
-// in shared memory, a pass is a loop over the level and passes are separated by
-// barriers.  As launches of their own these passes are 6 per level of 3 to 5 us
-// each, nearly all latency: at 32^3 a
-// mixed step with 56 V-cycles took 12.2 ms with them and takes 10.2 ms with this
-// kernel (41 us a launch; 47 us as one CTA).  In FP64 (two operations per SM and
-// clock) they stay spread over the chip, pass by pass.
+// in shared memory and passes are separated by barriers.  As launches of their own
+// these passes are 6 per level of 3 to 5 us each, nearly all latency: at 32^3 a
+// mixed step with 56 V-cycles took 12.2 ms with them, and about 46 us a cycle less with this
+// kernel (24.6 us).  In FP64 (two
+// operations per SM and clock) they stay spread over the chip, pass by pass.
 //
-// The first (largest) level is split into slabs of planes, one per CTA; a CTA keeps
-// all of the level's indexes but only its slab and the plane on either side hold
-// values, and a pass whose result the neighbours read stores their halo planes
-// into their shared memory (coarse_put).  Rank 0 alone does the levels below: they
-// have at most an eighth of the work, and a pass over the cluster costs a cluster
-// barrier.
+// A pass is bound by the length of one thread's instruction stream (a kernel of
+// this form with a marching stencil, a thread per column piece, took 41 us), so a
+// thread has one node and its weights stay in registers from pass to pass:
+// the operator is symmetric along every axis, so a row is 8 weights times sums of
+// neighbours (none, along x, along y, both; in the plane and off it).  Vectors
+// that a stencil reads are padded by zeros, and they are zero at eliminated nodes,
+// whose rows are their diagonal alone.
 //
-// A stencil pass marches: a thread owns a column piece (i, j, planes k0 ..) and
-// folds each plane's 3 x 3 neighbourhood once, as march_kernel does.  The
-// arithmetic is march_kernel's; the sums along x are grouped differently.
+// The first (largest) level is split into slabs of planes, one per CTA; a CTA has
+// the whole level's indexes, but only its slab and the plane on either side hold
+// values: what the neighbours read is stored into their shared memory as well.
+// Rank 0 alone does the levels below: at most an eighth of the work, and a pass over
+// the cluster costs a cluster barrier.
 constexpr int kCoarseNodes = 4913;  // 17^3
 constexpr int kCoarseThreads = 1024;
 constexpr int kCoarseCtas = 8;
@@ -792,7 +794,8 @@ struct CoarseLevel {
     LevelArgs<float> A;
     int n;
     float inv_theta, c1, c2;  // Chebyshev degree 2 over [hi/4, hi]
-    int off;                  // of b, v, t in shared memory (3 n floats)
+    int sy, sz;               // strides of the padded vectors
+    int b, e, v, t;           // places in shared memory: b, e [n], v, t padded
 };
 struct CoarseCycle {
     int nlev;  // smoothed levels; the dense level follows
@@ -800,280 +803,262 @@ struct CoarseCycle {
     LevelArgs<float> Ad;  // the dense level
     int nd, off_d;        // its nodes and the place of its b, x
     int off_inv;          // of the dense inverse in shared memory; 0: left in global
+    int pads0, pads1;     // the padded vectors' range
     const float *inv;
     const float *b;  // right-hand side of the first level
     float *x;        // result
 };
 
-// One column piece of a level: its node of k = 0, planes [k0, k1), the operator's
-// weights along x and y (zero towards eliminated nodes) and the neighbours' columns
-struct CoarseCol {
-    int q;  // which piece (-1: none yet)
-    int i, j, c, k0, k1;
-    bool el;
-    float mx[3], kx[3], my[3], ky[3];  // ky: with kappa times the mass
-    float A1, A2, iDi, iDb;            // column's D = A1 mz(0) + A2 kz(0), inverse inside/at the ends
-    int at[9];
+// One node of a level and its row of the operator: A v = sum_c wA[c] S_c + wB[c] Z_c,
+// S_c the neighbours' sum of class c (0: the node, 1: along x, 2: along y, 3: both) in
+// the node's plane, Z_c in the two planes beside it
+struct CoarseNode {
+    int q;  // which (-1: none yet)
+    int k, p;
+    float wA[4], wB[4], iD;
 };
 
-__device__ __forceinline__ void coarse_col(const LevelArgs<float> &L, int q, int z0, int z1, int cols,
-                                           int len, CoarseCol &c)
+__device__ __forceinline__ void coarse_node(const CoarseLevel &L, int q, CoarseNode &N)
 {
-    const int piece = q / cols;
-    c.q = q;
-    c.c = q - piece * cols;
-    c.j = c.c / L.NX1;
-    c.i = c.c - c.j * L.NX1;
-    c.k0 = z0 + piece * len;
-    c.k1 = min(z1, c.k0 + len);
-    const Axis<float> &ax = L.a[0], &ay = L.a[1], &az = L.a[2];
-    // coordinates of an axis whose nodes the operator has as columns
-    const int lo0 = L.faces[0] ? 1 : 0, lo1 = L.faces[2] ? 1 : 0;
-    const int hi0 = L.NX1 - (L.faces[1] ? 2 : 1), hi1 = L.NY1 - (L.faces[3] ? 2 : 1);
+    const LevelArgs<float> &A = L.A;
+    const Axis<float> &ax = A.a[0], &ay = A.a[1], &az = A.a[2];
+    const int row = q / A.NX1, i = q - row * A.NX1, k = row / A.NY1, j = row - k * A.NY1;
+    N.q = q;
+    N.k = k;
+    N.p = (i + 1) + L.sy * (j + 1) + L.sz * (k + 1);
+    const float mx = md_of(ax, i), kx = kd_of(ax, i), my = md_of(ay, j), mz = md_of(az, k), kz = kd_of(az, k);
+    const float ky = kd_of(ay, j) + A.kappa * my, kyo = ay.k_off + A.kappa * ay.m_off;
+    const float P[4] = {kx * my + mx * ky, ax.k_off * my + ax.m_off * ky, kx * ay.m_off + mx * kyo,
+                        ax.k_off * ay.m_off + ax.m_off * kyo};
+    const float Q[4] = {mx * my, ax.m_off * my, mx * ay.m_off, ax.m_off * ay.m_off};
+    const bool el = eliminated(A, i, j, k);
 #pragma unroll
-    for (int d = -1; d <= 1; ++d) {
-        const bool inx = c.i + d >= lo0 && c.i + d <= hi0, iny = c.j + d >= lo1 && c.j + d <= hi1;
-        c.mx[d + 1] = inx ? (d ? ax.m_off : md_of(ax, c.i)) : 0.f;
-        c.kx[d + 1] = inx ? (d ? ax.k_off : kd_of(ax, c.i)) : 0.f;
-        c.my[d + 1] = iny ? (d ? ay.m_off : md_of(ay, c.j)) : 0.f;
-        c.ky[d + 1] = iny ? (d ? ay.k_off : kd_of(ay, c.j)) + L.kappa * c.my[d + 1] : 0.f;
+    for (int c = 0; c < 4; ++c) {
+        N.wA[c] = el && c ? 0.f : P[c] * mz + Q[c] * kz;
+        N.wB[c] = el ? 0.f : P[c] * az.m_off + Q[c] * az.k_off;
     }
-#pragma unroll
-    for (int p = 0; p < 9; ++p) {
-        const int ii = c.i + p % 3 - 1, jj = c.j + p / 3 - 1;
-        c.at[p] = (ii >= lo0 && ii <= hi0 ? ii : c.i) + L.NX1 * (jj >= lo1 && jj <= hi1 ? jj : c.j);
-    }
-    const float mdx = md_of(ax, c.i), kdx = kd_of(ax, c.i), mdy = md_of(ay, c.j), kdy = kd_of(ay, c.j);
-    c.A1 = kdx * mdy + mdx * kdy + L.kappa * mdx * mdy;
-    c.A2 = mdx * mdy;
-    c.iDi = 1.f / (c.A1 * az.m_in + c.A2 * az.k_in);
-    c.iDb = 1.f / (c.A1 * az.m_bd + c.A2 * az.k_bd);
-    c.el = c.i < lo0 || c.i > hi0 || c.j < lo1 || c.j > hi1;
+    N.iD = 1.f / N.wA[0];
 }
 
-// f(column) for this thread's column pieces of the planes [z0, z1); `col` is kept
-// from pass to pass (a thread has one piece unless the level is wide and flat)
+// f(node) for this thread's nodes of the planes [z0, z1); N is kept from pass to
+// pass (a thread has one node unless a plane has more than kCoarseThreads)
 template <typename F>
-__device__ __forceinline__ void coarse_columns(const LevelArgs<float> &L, int z0, int z1, CoarseCol &col,
-                                               F f)
+__device__ __forceinline__ void coarse_nodes(const CoarseLevel &L, int z0, int z1, CoarseNode &N, F f)
 {
-    if (z0 >= z1) return;
-    const int cols = L.NX1 * L.NY1;
-    const int pieces = max(1, kCoarseThreads / cols), len = (z1 - z0 + pieces - 1) / pieces;
-    for (int q = threadIdx.x; q < cols * pieces; q += kCoarseThreads) {
-        if (q != col.q) coarse_col(L, q, z0, z1, cols, len, col);
-        if (col.k0 < col.k1) f(col);
+    const int plane = L.A.NX1 * L.A.NY1;
+    for (int q = z0 * plane + threadIdx.x; q < z1 * plane; q += kCoarseThreads) {
+        if (q != N.q) coarse_node(L, q, N);
+        f(N);
     }
 }
 
-// out(node, plane, A v, v, 1/D) for the nodes of [z0, z1), v in shared memory
-template <typename F>
-__device__ __forceinline__ void coarse_stencil(const LevelArgs<float> &L, int z0, int z1, CoarseCol &col,
-                                               const float *v, F out)
+__device__ __forceinline__ float coarse_row(const CoarseLevel &L, const CoarseNode &N, const float *v)
 {
-    const int plane = L.NX1 * L.NY1, lo2 = L.faces[4] ? 1 : 0, hi2 = L.NZ1 - (L.faces[5] ? 2 : 1);
-    const Axis<float> &az = L.a[2];
-    coarse_columns(L, z0, z1, col, [&](const CoarseCol &c) {
-        float Pm = 0.f, Qm = 0.f, P0 = 0.f, Q0 = 0.f;
-        const float *pl = v + (c.k0 - 1) * plane;
-        for (int kk = c.k0 - 1; kk <= c.k1; ++kk, pl += plane) {
-            float P = 0.f, Q = 0.f;
-            if (kk >= lo2 && kk <= hi2) {
-                float w[9];
+    float S[3][3], Z[3][3];  // [y][x]
 #pragma unroll
-                for (int p = 0; p < 9; ++p) w[p] = pl[c.at[p]];
+    for (int d = 0; d < 3; ++d) {
+        const float *r = v + N.p + (d - 1) * L.sy;
 #pragma unroll
-                for (int d = 0; d < 3; ++d) {
-                    const float sk = c.kx[0] * w[3 * d] + c.kx[1] * w[3 * d + 1] + c.kx[2] * w[3 * d + 2];
-                    const float sm = c.mx[0] * w[3 * d] + c.mx[1] * w[3 * d + 1] + c.mx[2] * w[3 * d + 2];
-                    P += sk * c.my[d] + sm * c.ky[d];
-                    Q += sm * c.my[d];
-                }
-            }
-            const int k = kk - 1;
-            if (k >= c.k0 && k < c.k1) {
-                const bool bd = k == 0 || k == L.NZ1 - 1, el = c.el || k < lo2 || k > hi2;
-                const float mdz = bd ? az.m_bd : az.m_in, kdz = bd ? az.k_bd : az.k_in;
-                const float own = pl[c.c - plane];
-                const float Av = el ? (c.A1 * mdz + c.A2 * kdz) * own
-                                    : az.m_off * (Pm + P) + az.k_off * (Qm + Q) + P0 * mdz + Q0 * kdz;
-                out(c.c + k * plane, k, Av, own, bd ? c.iDb : c.iDi);
-            }
-            Pm = P0;
-            Qm = Q0;
-            P0 = P;
-            Q0 = Q;
+        for (int x = 0; x < 3; ++x) {
+            S[d][x] = r[x - 1];
+            Z[d][x] = r[x - 1 - L.sz] + r[x - 1 + L.sz];
         }
-    });
+    }
+    const float a0 = N.wA[0] * S[1][1] + N.wB[0] * Z[1][1];
+    const float a1 = N.wA[1] * (S[1][0] + S[1][2]) + N.wB[1] * (Z[1][0] + Z[1][2]);
+    const float a2 = N.wA[2] * (S[0][1] + S[2][1]) + N.wB[2] * (Z[0][1] + Z[2][1]);
+    const float a3 = N.wA[3] * ((S[0][0] + S[0][2]) + (S[2][0] + S[2][2])) +
+                     N.wB[3] * ((Z[0][0] + Z[0][2]) + (Z[2][0] + Z[2][2]));
+    return (a0 + a1) + (a2 + a3);
 }
 
-__global__ void __launch_bounds__(kCoarseThreads, 1) coarse_cycle_kernel(const CoarseCycle C)
+__global__ void __launch_bounds__(kCoarseThreads, 1) coarse_cycle_kernel(const __grid_constant__ CoarseCycle C)
 {
-    extern __shared__ float cs[];
+    extern __shared__ __align__(16) float cs[];
     cg::cluster_group cl = cg::this_cluster();
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x;
     const int nr = (int)cl.num_blocks(), rank = (int)cl.block_rank();
-    // this CTA's planes [z0, z1) of the first level
+    // this CTA's planes [s0, s1) of the first level
     const int NZ = C.lev[0].A.NZ1, zl = (NZ + nr - 1) / nr;
     const int s0 = min(rank * zl, NZ), s1 = min(s0 + zl, NZ);
     auto sync = [&](bool split) {
         if (split && nr > 1) cl.sync();
         else __syncthreads();
     };
-    // a value of plane k of the slab, also into the neighbours' halo planes
-    auto put = [&](float *at, int k, float val) {
+    // a value of plane k, with split also into the neighbours' halo planes
+    auto put = [&](bool split, float *at, int k, float val) {
         *at = val;
-        if (nr > 1) {
+        if (split && nr > 1) {
             if (k == s0 && s0 > 0) *cl.map_shared_rank(at, rank - 1) = val;
             if (k == s1 - 1 && s1 < NZ) *cl.map_shared_rank(at, rank + 1) = val;
         }
     };
-    {
-        float *b = cs + C.lev[0].off;
-        const int plane = C.lev[0].n / NZ, q1 = min(s1 + 1, NZ) * plane;
-        if (s0 < s1)
-            for (int q = max(s0 - 1, 0) * plane + tid; q < q1; q += kCoarseThreads) b[q] = C.b[q];
-        // the dense inverse on its way (see off_inv)
-        if (rank == 0 && C.off_inv)
-            for (int q = tid; q < C.nd * C.nd; q += kCoarseThreads) __pipeline_memcpy_async(cs + C.off_inv + q, C.inv + q, 4);
-        __pipeline_commit();
-    }
-    CoarseCol col;
+    // the dense inverse on its way (see off_inv)
+    if (rank == 0 && C.off_inv)
+        for (int q = tid; q < C.nd * C.nd; q += kCoarseThreads)
+            __pipeline_memcpy_async(cs + C.off_inv + q, C.inv + q, 4);
+    __pipeline_commit();
+    for (int q = C.pads0 + tid; q < C.pads1; q += kCoarseThreads) cs[q] = 0.f;
+    CoarseNode N;
+    N.q = -1;
+    coarse_nodes(C.lev[0], s0, s1, N, [&](const CoarseNode &N) { cs[C.lev[0].b + N.q] = __ldg(C.b + N.q); });
     sync(true);
     // down: pre-smoothing from zero into t, residual into v, its restriction
     for (int l = 0; l < C.nlev; ++l) {
-        if (l > 0 && rank > 0) break;
-        const CoarseLevel &L = C.lev[l];
-        const LevelArgs<float> &A = L.A;
-        const int z0 = l ? 0 : s0, z1 = l ? A.NZ1 : s1, plane = A.NX1 * A.NY1;
         const bool split = l == 0;
-        float *b = cs + L.off, *v = b + L.n, *t = v + L.n;
-        col.q = -1;
-        // d0, on the halo planes too
-        coarse_columns(A, z0, z1, col, [&](const CoarseCol &c) {
-            const int ka = c.k0 == z0 ? max(z0 - 1, 0) : c.k0, kb = c.k1 == z1 ? min(z1 + 1, A.NZ1) : c.k1;
-            for (int k = ka; k < kb; ++k)
-                v[c.c + k * plane] = L.inv_theta * b[c.c + k * plane] * (k == 0 || k == A.NZ1 - 1 ? c.iDb : c.iDi);
-        });
-        __syncthreads();
-        coarse_stencil(A, z0, z1, col, v, [&](int q, int k, float Av, float d0, float iD) {
-            const float y = d0 + (L.c1 * d0 + L.c2 * ((b[q] - Av) * iD));
-            if (split) put(t + q, k, y);
-            else t[q] = y;
+        if (!split && rank > 0) break;
+        const CoarseLevel &L = C.lev[l];
+        const int z0 = l ? 0 : s0, z1 = l ? L.A.NZ1 : s1;
+        const float *b = cs + L.b;
+        float *v = cs + L.v, *t = cs + L.t;
+        if (!split) N.q = -1;
+        coarse_nodes(L, z0, z1, N, [&](const CoarseNode &N) {  // d0
+            put(split, v + N.p, N.k, L.inv_theta * b[N.q] * N.iD);
         });
         sync(split);
-        coarse_stencil(A, z0, z1, col, t, [&](int q, int k, float Av, float, float) {
-            if (split) put(v + q, k, b[q] - Av);
-            else v[q] = b[q] - Av;
+        coarse_nodes(L, z0, z1, N, [&](const CoarseNode &N) {
+            const float d0 = v[N.p];
+            put(split, t + N.p, N.k, d0 + (L.c1 * d0 + L.c2 * ((b[N.q] - coarse_row(L, N, v)) * N.iD)));
+        });
+        sync(split);
+        coarse_nodes(L, z0, z1, N, [&](const CoarseNode &N) {
+            put(split, v + N.p, N.k, b[N.q] - coarse_row(L, N, t));
         });
         sync(split);
         // restriction of the coarse planes whose fine plane is in the slab, to rank 0
         const bool last = l + 1 == C.nlev;
         const LevelArgs<float> &B = last ? C.Ad : C.lev[l + 1].A;
-        float *bc = cs + (last ? C.off_d : C.lev[l + 1].off);
-        if (split && rank > 0) bc = cl.map_shared_rank(bc, 0);
+        float *bc = cs + (last ? C.off_d : C.lev[l + 1].b);
+        if (rank > 0) bc = cl.map_shared_rank(bc, 0);
         const int cplane = B.NX1 * B.NY1, K0 = (z0 + 1) / 2, K1 = z0 < z1 ? (z1 - 1) / 2 + 1 : 0;
         for (int q = K0 * cplane + tid; q < K1 * cplane; q += kCoarseThreads) {
             const int row = q / B.NX1, I = q - row * B.NX1, K = row / B.NY1, J = row - K * B.NY1;
-            float acc = 0.f;
+            const float *c = v + (2 * I + 1) + L.sy * (2 * J + 1) + L.sz * (2 * K + 1);
+            float acc[3];
 #pragma unroll
-            for (int dk = -1; dk <= 1; ++dk)
+            for (int dk = -1; dk <= 1; ++dk) {
+                float r[3];
 #pragma unroll
                 for (int dj = -1; dj <= 1; ++dj) {
-                    const int k = 2 * K + dk, j = 2 * J + dj;
-                    if (k < 0 || k >= A.NZ1 || j < 0 || j >= A.NY1) continue;
-                    const float *rw = v + A.NX1 * (j + A.NY1 * k) + 2 * I;
-                    float sum = rw[0];
-                    if (I > 0) sum += 0.5f * rw[-1];
-                    if (2 * I + 1 < A.NX1) sum += 0.5f * rw[1];
-                    acc += (dj ? 0.5f : 1.f) * (dk ? 0.5f : 1.f) * sum;
+                    const float *rw = c + dk * L.sz + dj * L.sy;
+                    r[dj + 1] = rw[0] + 0.5f * (rw[-1] + rw[1]);
                 }
-            bc[q] = eliminated(B, I, J, K) ? 0.f : acc;
+                acc[dk + 1] = r[1] + 0.5f * (r[0] + r[2]);
+            }
+            bc[q] = eliminated(B, I, J, K) ? 0.f : acc[1] + 0.5f * (acc[0] + acc[2]);
         }
         sync(split);
     }
-    // the dense inverse: a warp per row, lanes in dense_apply_kernel's order
+    // the dense inverse: eight threads per row
     if (rank == 0) {
         const float *b = cs + C.off_d;
         float *x = cs + C.off_d + C.nd;
         const float *inv = C.off_inv ? cs + C.off_inv : C.inv;
         __pipeline_wait_prior(0);
         __syncthreads();
-        for (int row = warp; row < C.nd; row += kCoarseThreads / 32) {
-            float sum = 0.f;
-            for (int c = lane; c < C.nd; c += 32) sum += inv[row * C.nd + c] * b[c];
-            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            if (lane == 0) x[row] = sum;
+        for (int r0 = 0; r0 < C.nd; r0 += kCoarseThreads / 8) {
+            const int row = r0 + (tid >> 3);
+            float s0 = 0.f, s1 = 0.f;
+            if (row < C.nd) {
+                const float *m = inv + row * C.nd;
+                int c = tid & 7;
+                for (; c + 8 < C.nd; c += 16) {
+                    s0 += m[c] * b[c];
+                    s1 += m[c + 8] * b[c + 8];
+                }
+                if (c < C.nd) s0 += m[c] * b[c];
+            }
+            s0 += s1;
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+            if (row < C.nd && (tid & 7) == 0) x[row] = s0;
         }
         __syncthreads();
     }
     // up: prolongation into t, post-smoothing from t
     for (int l = C.nlev - 1; l >= 0; --l) {
-        if (l > 0 && rank > 0) continue;
-        const CoarseLevel &L = C.lev[l];
-        const LevelArgs<float> &A = L.A;
-        const int z0 = l ? 0 : s0, z1 = l ? A.NZ1 : s1, plane = A.NX1 * A.NY1;
         const bool split = l == 0;
-        float *b = cs + L.off, *v = b + L.n, *t = v + L.n;
+        if (!split && rank > 0) continue;
+        const CoarseLevel &L = C.lev[l];
+        const int z0 = l ? 0 : s0, z1 = l ? L.A.NZ1 : s1;
+        const float *b = cs + L.b;
+        float *e = cs + L.e, *v = cs + L.v, *t = cs + L.t;
+        // the level below leaves its result in its t (the dense level after its b)
         const bool last = l + 1 == C.nlev;
         const LevelArgs<float> &B = last ? C.Ad : C.lev[l + 1].A;
-        // the level below leaves its result in its t (the dense level after its b)
-        float *xc = last ? cs + C.off_d + C.nd : cs + C.lev[l + 1].off + 2 * C.lev[l + 1].n;
-        const int cplane = B.NX1 * B.NY1;
+        const int cy = last ? B.NX1 : C.lev[l + 1].sy, cz = last ? B.NX1 * B.NY1 : C.lev[l + 1].sz;
+        const float *xc = cs + (last ? C.off_d + C.nd : C.lev[l + 1].t + 1 + cy + cz);
         if (split && nr > 1) {
-            // rank 0's result is there; the planes this slab and its halo read
-            cl.sync();
-            if (rank > 0 && z0 < z1) {
-                const float *x0 = cl.map_shared_rank(xc, 0);
-                const int q1 = min(z1 / 2 + 2, B.NZ1) * cplane;
-                for (int q = ((z0 - 1) / 2) * cplane + tid; q < q1; q += kCoarseThreads) xc[q] = x0[q];
-            }
-            __syncthreads();
+            cl.sync();  // rank 0's result is there
+            if (rank > 0) xc = cl.map_shared_rank(xc, 0);
         }
-        if (!split || (rank == 0 && C.nlev > 1)) col.q = -1;
-        coarse_columns(A, z0, z1, col, [&](const CoarseCol &c) {
-            const int ka = c.k0 == z0 ? max(z0 - 1, 0) : c.k0, kb = c.k1 == z1 ? min(z1 + 1, A.NZ1) : c.k1;
-            // trilinear: along x and y between the column's (up to) four coarse ones
-            const int dx = c.i & 1, dy = (c.j & 1) ? B.NX1 : 0;
-            const float w = (dx ? 0.5f : 1.f) * (dy ? 0.5f : 1.f);
-            for (int k = ka; k < kb; ++k) {
-                const float *r0 = xc + (c.i >> 1) + B.NX1 * (c.j >> 1) + (k >> 1) * cplane;
-                float s = r0[0];
-                if (dx) s += r0[1];
-                if (dy) s += r0[dy] + (dx ? r0[dy + 1] : 0.f);
-                if (k & 1) {
-                    const float *r1 = r0 + cplane;
-                    float s1 = r1[0];
-                    if (dx) s1 += r1[1];
-                    if (dy) s1 += r1[dy] + (dx ? r1[dy + 1] : 0.f);
-                    s = 0.5f * (s + s1);
-                }
-                t[c.c + k * plane] += w * s;
-            }
-        });
-        __syncthreads();
-        // the first direction d0 from x = t; then v = t + d0, d0 kept in t
-        coarse_stencil(A, z0, z1, col, t, [&](int q, int, float Av, float, float iD) {
-            v[q] = L.inv_theta * (b[q] - Av) * iD;
-        });
-        __syncthreads();
-        coarse_columns(A, z0, z1, col, [&](const CoarseCol &c) {
-            for (int k = c.k0; k < c.k1; ++k) {
-                const int q = c.c + k * plane;
-                const float d0 = v[q], y = t[q] + d0;
-                t[q] = d0;
-                if (split) put(v + q, k, y);
-                else v[q] = y;
-            }
+        if (!split || (rank == 0 && C.nlev > 1)) N.q = -1;
+        coarse_nodes(L, z0, z1, N, [&](const CoarseNode &N) {
+            // trilinear: the mean of the two (or, on a coarse line, twice the one) along each axis
+            const int row = N.q / L.A.NX1, i = N.q - row * L.A.NX1, j = row - N.k * L.A.NY1;
+            const float *r = xc + (i >> 1) + cy * (j >> 1) + cz * (N.k >> 1);
+            const int dx = i & 1, dy = (j & 1) ? cy : 0, dz = (N.k & 1) ? cz : 0;
+            const float s = ((r[0] + r[dx]) + (r[dy] + r[dx + dy])) +
+                            ((r[dz] + r[dx + dz]) + (r[dy + dz] + r[dx + dy + dz]));
+            put(split, t + N.p, N.k, t[N.p] + 0.125f * s);
         });
         sync(split);
-        coarse_stencil(A, z0, z1, col, v, [&](int q, int, float Av, float xv, float iD) {
-            const float y = xv + (L.c1 * t[q] + L.c2 * ((b[q] - Av) * iD));
-            t[q] = y;
-            if (l == 0) C.x[q] = y;
+        // the first direction d0 from x = t; then v = t + d0, d0 kept in e
+        coarse_nodes(L, z0, z1, N, [&](const CoarseNode &N) {
+            const float d0 = L.inv_theta * (b[N.q] - coarse_row(L, N, t)) * N.iD;
+            e[N.q] = d0;
+            put(split, v + N.p, N.k, t[N.p] + d0);
+        });
+        sync(split);
+        coarse_nodes(L, z0, z1, N, [&](const CoarseNode &N) {
+            const float y = v[N.p] + (L.c1 * e[N.q] + L.c2 * ((b[N.q] - coarse_row(L, N, v)) * N.iD));
+            if (l == 0) C.x[N.q] = y;
+            else t[N.p] = y;
         });
         __syncthreads();
     }
+}
+
+// The levels from l0 on as coarse_cycle_kernel's arguments; the shared memory they
+// need in bytes
+int coarse_plan(const PressureMG &P, int l0, CoarseCycle &C)
+{
+    C.nlev = P.nlev - 1 - l0;
+    int off = 0;
+    for (int l = 0; l < C.nlev; ++l) {
+        const PmgLevel &L = P.lev[l0 + l];
+        CoarseLevel &D = C.lev[l];
+        const double hi = L.hi, lo = hi / 4.0, theta = 0.5 * (hi + lo), delta = 0.5 * (hi - lo),
+                     s1 = theta / delta, rho = 1.0 / s1, rho_new = 1.0 / (2.0 * s1 - rho);
+        D.A = level_args<float>(P, l0 + l);
+        D.n = (int)L.n;
+        D.inv_theta = (float)(1.0 / theta);
+        D.c1 = (float)(rho_new * rho);
+        D.c2 = (float)(2.0 * rho_new / delta);
+        D.sy = D.A.NX1 + 2;
+        D.sz = D.sy * (D.A.NY1 + 2);
+        const int padded = D.sz * (D.A.NZ1 + 2);
+        D.v = off;
+        D.t = off + padded;
+        off += 2 * padded;
+    }
+    C.pads0 = 0;
+    C.pads1 = off;
+    for (int l = 0; l < C.nlev; ++l) {
+        C.lev[l].b = off;
+        C.lev[l].e = off + C.lev[l].n;
+        off += 2 * C.lev[l].n;
+    }
+    C.Ad = level_args<float>(P, P.nlev - 1);
+    C.nd = (int)P.nc;
+    C.off_d = off;
+    off += 2 * C.nd;
+    C.inv = P.inv32;
+    if (C.nd <= 181 && (off + C.nd * C.nd) * (int)sizeof(float) <= kCoarseSmemMax) {
+        C.off_inv = off;
+        off += C.nd * C.nd;
+    }
+    return off * (int)sizeof(float);
 }
 
 // The first level of the FP32 V-cycle that coarse_cycle_kernel takes, or -1: a
@@ -1082,41 +1067,20 @@ __global__ void __launch_bounds__(kCoarseThreads, 1) coarse_cycle_kernel(const C
 int coarse_first(const PressureMG &P)
 {
     if (!P.direct) return -1;
-    for (int l = 1; l < P.nlev - 1; ++l)
-        if (P.lev[l].n <= kCoarseNodes) return P.nlev - 1 - l <= kCoarseMaxLevels ? l : -1;
+    for (int l = 1; l < P.nlev - 1; ++l) {
+        if (P.lev[l].n > kCoarseNodes || P.nlev - 1 - l > kCoarseMaxLevels) continue;
+        CoarseCycle C{};
+        if (coarse_plan(P, l, C) <= kCoarseSmemMax) return l;
+    }
     return -1;
 }
 
 fsi_status coarse_cycle(fsi_mesh *m, int l0, const float *b, float *x)
 {
-    const PressureMG &P = *m->pmg;
     CoarseCycle C{};
-    C.nlev = P.nlev - 1 - l0;
-    int off = 0;
-    for (int l = 0; l < C.nlev; ++l) {
-        const PmgLevel &L = P.lev[l0 + l];
-        const double hi = L.hi, lo = hi / 4.0, theta = 0.5 * (hi + lo), delta = 0.5 * (hi - lo),
-                     s1 = theta / delta, rho = 1.0 / s1, rho_new = 1.0 / (2.0 * s1 - rho);
-        C.lev[l].A = level_args<float>(P, l0 + l);
-        C.lev[l].n = (int)L.n;
-        C.lev[l].inv_theta = (float)(1.0 / theta);
-        C.lev[l].c1 = (float)(rho_new * rho);
-        C.lev[l].c2 = (float)(2.0 * rho_new / delta);
-        C.lev[l].off = off;
-        off += 3 * (int)L.n;
-    }
-    C.Ad = level_args<float>(P, P.nlev - 1);
-    C.nd = (int)P.nc;
-    C.off_d = off;
-    off += 2 * C.nd;
-    C.inv = P.inv32;
+    const int bytes = coarse_plan(*m->pmg, l0, C);
     C.b = b;
     C.x = x;
-    if (C.nd <= 181 && (off + C.nd * C.nd) * (int)sizeof(float) <= kCoarseSmemMax) {
-        C.off_inv = off;
-        off += C.nd * C.nd;
-    }
-    const int bytes = off * (int)sizeof(float);
     FSI_TRY(set_smem_limit((const void *)coarse_cycle_kernel, kCoarseSmemMax));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = cfg.blockDim = dim3(1, 1, 1);
