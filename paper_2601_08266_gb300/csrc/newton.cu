@@ -772,31 +772,218 @@ __global__ void schur_split_kernel(int n, const T *inv, const T *v, T *z, T *bp)
 
 // The GMRES basis scaling V = w / den fused with the Schur split of V for
 // the next preconditioner application (the arithmetic of scale_by_inv_kernel
-// and schur_split_kernel, one pass)
+// and schur_split_kernel, one pass); inv null: the scaling alone
+template <typename T>
+__device__ __forceinline__ void scale_split_node(int64_t node, vec4<T> x, double den, vec4<T> *V,
+                                                 const T *inv, vec4<T> *z, T *bp)
+{
+    const T sc = (T)(den > 0.0 ? 1.0 / den : 0.0);
+    x.x *= sc;
+    x.y *= sc;
+    x.z *= sc;
+    x.w *= sc;
+    V[node] = x;
+    if (!inv) return;
+    const vec4<T> *M = (const vec4<T> *)(inv + 16 * node);
+    vec4<T> zr;
+    const vec4<T> m0 = ld4(M), m1 = ld4(M + 1), m2 = ld4(M + 2);
+    zr.x = m0.x * x.x + m0.y * x.y + m0.z * x.z;
+    zr.y = m1.x * x.x + m1.y * x.y + m1.z * x.z;
+    zr.z = m2.x * x.x + m2.y * x.y + m2.z * x.z;
+    zr.w = T(0);
+    z[node] = zr;
+    bp[node] = x.w;
+}
 template <typename T>
 __global__ void scale_split_kernel(int n, const double *den, const T *w, T *V, const T *inv, T *z,
                                    T *bp)
 {
     const double dd = *den;
-    const T sc = (T)(dd > 0.0 ? 1.0 / dd : 0.0);
     GRID_STRIDE(node, n)
-    {
-        vec4<T> x = ld4((const vec4<T> *)w + node);
-        x.x *= sc;
-        x.y *= sc;
-        x.z *= sc;
-        x.w *= sc;
-        ((vec4<T> *)V)[node] = x;
-        const vec4<T> *M = (const vec4<T> *)(inv + 16 * node);
-        vec4<T> zr;
-        const vec4<T> m0 = ld4(M), m1 = ld4(M + 1), m2 = ld4(M + 2);
-        zr.x = m0.x * x.x + m0.y * x.y + m0.z * x.z;
-        zr.y = m1.x * x.x + m1.y * x.y + m1.z * x.z;
-        zr.z = m2.x * x.x + m2.y * x.y + m2.z * x.z;
-        zr.w = T(0);
-        ((vec4<T> *)z)[node] = zr;
-        bp[node] = x.w;
+    scale_split_node<T>(node, ld4((const vec4<T> *)w + node), dd, (vec4<T> *)V, inv, (vec4<T> *)z, bp);
+}
+
+// ------------------------------------------------ one launch per Gram-Schmidt
+// On short vectors every pass above is a launch of 9 to 16 us that moves a few MB:
+// its time is the launch, the FP64 reductions and the sum over the CTAs.  Here a
+// thread keeps one record of w and of all the basis vectors in registers for the
+// whole orthogonalisation -- dots, Kahan's test, update, second dots and update,
+// norm, scaling and Schur split -- and the CTAs, all resident (a cooperative
+// launch), meet at each sum: the last to arrive adds up the partial sums and
+// releases the others.  At 32^3 31 us an iteration (FP32, 10 vectors) against 38 to 50
+// us for the passes, and no gaps between them: a mixed step 8.95 -> 8.15 ms; FP64 at
+// 24^3 36.2 -> 35.1 ms.  Above 304 CTAs the records don't fit the registers.
+template <typename T> constexpr int kOrthoThreads = sizeof(T) == 4 ? 256 : 128;
+constexpr int kOrthoMax = 16;                 // basis vectors held
+constexpr unsigned kOrthoPolls = 1u << 22;    // a wait gives up after a few seconds
+
+template <typename T> struct OrthoArgs {
+    int cnt;
+    int64_t n;
+    const vec4<T> *V;
+    int64_t vstride;
+    const vec4<T> *w;
+    vec4<T> *Vnew;
+    const T *inv;
+    vec4<T> *z;
+    T *bp;
+    double *partial, *h, *h2, *flag, *err;
+    unsigned *bar;  // arrivals, generation
+};
+
+// Every CTA arrives; the last one runs fin() (all its threads), then all go on.
+// The wait is bounded: when it runs out *err is set, later waits are skipped and the
+// kernel ends with meaningless results.
+template <typename F>
+__device__ __forceinline__ void grid_step(unsigned *bar, double *err, int &last_or_bad, F fin)
+{
+    __syncthreads();
+    unsigned gen = 0;
+    const bool bad = last_or_bad == 2;
+    if (threadIdx.x == 0) {
+        gen = *(volatile unsigned *)(bar + 1);
+        __threadfence();
+        const bool last = atomicAdd(bar, 1u) == gridDim.x - 1;
+        if (!bad) last_or_bad = last;
     }
+    __syncthreads();
+    if (last_or_bad == 1) {
+        __threadfence();
+        fin();
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            atomicExch(bar, 0u);
+            __threadfence();
+            atomicAdd(bar + 1, 1u);
+        }
+    } else if (threadIdx.x == 0 && !bad) {
+        unsigned polls = 0;
+        while (*(volatile unsigned *)(bar + 1) == gen)
+            if (++polls == kOrthoPolls) {
+                *err = 1.0;
+                last_or_bad = 2;
+                break;
+            }
+        __threadfence();
+    }
+    __syncthreads();
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kOrthoThreads<T>, 2) ortho_kernel(const OrthoArgs<T> P)
+{
+    constexpr int G = kOrthoMax, NT = kOrthoThreads<T>, NW = NT / 32, Q = (G + NW) / NW;
+    using Acc = typename DotAcc<T>::type;
+    __shared__ double red[G + 1][NW];
+    __shared__ double sums[G + 1];
+    __shared__ T hs[G];
+    __shared__ int state;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, cnt = P.cnt;
+    const int64_t i = blockIdx.x * (int64_t)NT + tid;
+    const bool live = i < P.n;
+    const vec4<T> zero = {T(0), T(0), T(0), T(0)};
+    if (tid == 0) state = 0;
+    vec4<T> w = live ? ld4(P.w + i) : zero, v[G];
+#pragma unroll
+    for (int j = 0; j < G; ++j) v[j] = live && j < cnt ? ld4(P.V + (int64_t)j * P.vstride + i) : zero;
+
+    // V_j . w for all j (and w . w behind them) into this CTA's partial sums
+    auto dots = [&](bool self, int nv) {
+#pragma unroll
+        for (int g = 0; g < G; g += kDotGroup)
+            if (g < nv) {
+                double d[kDotGroup];
+#pragma unroll
+                for (int j = 0; j < kDotGroup; ++j) {
+                    Acc a = Acc(0);
+                    if (g + j < nv) {
+                        dot_acc(a, v[g + j].x, w.x);
+                        dot_acc(a, v[g + j].y, w.y);
+                        dot_acc(a, v[g + j].z, w.z);
+                        dot_acc(a, v[g + j].w, w.w);
+                    }
+                    d[j] = dot_value(a);
+                }
+                const double t = warp_sums8(d, lane);
+                if ((lane & 3) == 0) red[g + (lane >> 2)][wid] = t;
+            }
+        if (self) {
+            Acc a = Acc(0);
+            dot_acc(a, w.x, w.x);
+            dot_acc(a, w.y, w.y);
+            dot_acc(a, w.z, w.z);
+            dot_acc(a, w.w, w.w);
+            double d = dot_value(a);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+            if (lane == 0) red[G][wid] = d;
+        }
+        __syncthreads();
+        if (tid < nv + (self ? 1 : 0)) {
+            const double *row = red[tid < nv ? tid : G];
+            double d = 0.0;
+            for (int q = 0; q < NW; ++q) d += row[q];
+            P.partial[(int64_t)tid * kRedGrid + blockIdx.x] = d;
+        }
+    };
+    // (the last CTA) the sums over the CTAs of nv rows into `sums`
+    auto total = [&](int nv) {
+        double a[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) a[q] = 0.0;
+        for (int b = lane; b < (int)gridDim.x; b += 32)
+#pragma unroll
+            for (int q = 0; q < Q; ++q)
+                if (wid + q * NW < nv) a[q] += __ldcg(P.partial + (int64_t)(wid + q * NW) * kRedGrid + b);
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+            if (wid + q * NW < nv) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) a[q] += __shfl_xor_sync(0xffffffffu, a[q], o);
+                if (lane == 0) sums[wid + q * NW] = a[q];
+            }
+        __syncthreads();
+    };
+    // w -= V h, in the order of multi_axpy_kernel
+    auto update = [&](const double *h) {
+        if (tid < cnt) hs[tid] = (T)__ldcg(h + tid);
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < G; ++j)
+            if (j < cnt) {
+                const T hk = hs[j];
+                w.x = fma_rn(-v[j].x, hk, w.x);
+                w.y = fma_rn(-v[j].y, hk, w.y);
+                w.z = fma_rn(-v[j].z, hk, w.z);
+                w.w = fma_rn(-v[j].w, hk, w.w);
+            }
+    };
+    dots(true, cnt);
+    grid_step(P.bar, P.err, state, [&]() {
+        total(cnt + 1);
+        if (tid <= cnt) P.h[tid] = sums[tid];
+        if (wid == 0) kahan_flag(cnt - 1, sums, P.flag);
+    });
+    const bool second = __ldcg(P.flag) != 0.0;
+    update(P.h);
+    if (second) {
+        dots(false, cnt);
+        grid_step(P.bar, P.err, state, [&]() {
+            total(cnt);
+            if (tid < cnt) {
+                P.h2[tid] = sums[tid];
+                P.h[tid] += sums[tid];
+            }
+        });
+        update(P.h2);
+    }
+    dots(true, 0);
+    grid_step(P.bar, P.err, state, [&]() {
+        total(1);
+        if (tid == 0) P.h[cnt] = sqrt(sums[0]);
+    });
+    if (live) scale_split_node<T>(i, w, __ldcg(P.h + cnt), P.Vnew, P.inv, P.z, P.bp);
 }
 
 // z_p = V-cycle result / sigma, or z_p = v_p on Dirichlet pressure rows
@@ -825,11 +1012,12 @@ struct Work {
     void *w = nullptr, *z = nullptr, *x = nullptr, *b = nullptr;
     void *blocks = nullptr, *inv = nullptr;  // [n][16]
     double *partial = nullptr;              // [restart+1][kRedGrid] + [kAxpyGrid]
-    double *hcol = nullptr, *h2 = nullptr;  // [restart+2]
+    double *hcol = nullptr, *h2 = nullptr;  // [restart+4], [restart+2]
     int32_t *clist = nullptr;               // occupied cells and their count
     void *cmat = nullptr;                   // [cells][36] coupling matrices
     bool cells = false;                     // they hold this call's step (and type)
-    unsigned *ticket = nullptr;             // of the reductions' last CTA (zero between launches)
+    unsigned *ticket = nullptr;             // of the reductions' last CTA (zero between launches),
+                                            // then arrivals and generation of ortho_kernel
     double *hhost = nullptr;                // pinned
     int precond = 0;                        // 0 block-Jacobi, 1 Schur (pmg.cu)
     // the point-mass coupling of the Jacobian apply runs on a side stream
@@ -900,9 +1088,9 @@ fsi_status ensure_work(fsi_mesh *mesh, int64_t m_pts, int restart)
         {&W.Vk, v * (size_t)(restart + 1)}, {&W.w, v}, {&W.z, v}, {&W.x, v}, {&W.b, v},
         {&W.blocks, v * 4}, {&W.inv, v * 4}, {&W.ftmp, v},
         {(void **)&W.partial, ((size_t)(restart + 1) * kRedGrid + kAxpyGrid) * sizeof(double)},
-        {(void **)&W.hcol, (size_t)(restart + 2) * sizeof(double)},
+        {(void **)&W.hcol, (size_t)(restart + 4) * sizeof(double)},
         {(void **)&W.h2, (size_t)(restart + 2) * sizeof(double)},
-        {(void **)&W.ticket, sizeof(double)},
+        {(void **)&W.ticket, 4 * sizeof(unsigned)},
         {(void **)&W.clist, (size_t)(cells + 1) * sizeof(int32_t)},
         {&W.cmat, (size_t)(cells + 1) * 36 * sizeof(double)},
     };
@@ -913,13 +1101,13 @@ fsi_status ensure_work(fsi_mesh *mesh, int64_t m_pts, int restart)
             return check_cuda(e, "Newton workspace allocation");
         }
     }
-    cudaError_t e = cudaMemset(W.ticket, 0, sizeof(double));
+    cudaError_t e = cudaMemset(W.ticket, 0, 4 * sizeof(unsigned));
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) {
         free_work(W);
         return check_cuda(e, "Newton workspace");
     }
-    e = cudaMallocHost((void **)&W.hhost, (size_t)(restart + 2) * sizeof(double));
+    e = cudaMallocHost((void **)&W.hhost, (size_t)(restart + 4) * sizeof(double));
     if (e != cudaSuccess) {
         free_work(W);
         return check_cuda(e, "pinned host buffer");
@@ -1241,6 +1429,41 @@ void gram_schmidt(fsi_mesh *mesh, int cnt, const T *V, int64_t ld, double *h, T 
     multi_axpy<T>(s, cnt, len, V, ld, W.h2, w, npart, flag, W.ticket, norm);
 }
 
+// The whole orthogonalisation, scaling and Schur split in one launch where the basis
+// fits the registers and every CTA can be resident; false: not this size (or the
+// device has no room for a cooperative launch right now)
+template <typename T>
+bool ortho_launch(fsi_mesh *mesh, int cnt, const T *V, int64_t ld, double *flag, double *err, const T *inv,
+                  T *z, T *bp)
+{
+    Work &W = mesh->newton->w;
+    const int64_t n = mesh->n_nodes, grid = (n + kOrthoThreads<T> - 1) / kOrthoThreads<T>;
+    if (cnt > kOrthoMax || grid > kRedGrid || grid > 2 * (int64_t)sm_count()) return false;
+    OrthoArgs<T> P;
+    P.cnt = cnt;
+    P.n = n;
+    P.V = (const vec4<T> *)V;
+    P.vstride = ld / 4;
+    P.w = (const vec4<T> *)W.w;
+    P.Vnew = (vec4<T> *)((T *)W.Vk + (int64_t)cnt * ld);
+    P.inv = inv;
+    P.z = (vec4<T> *)z;
+    P.bp = bp;
+    P.partial = W.partial;
+    P.h = W.hcol;
+    P.h2 = W.h2;
+    P.flag = flag;
+    P.err = err;
+    P.bar = W.ticket + 2;
+    void *args[] = {&P};
+    if (cudaLaunchCooperativeKernel((const void *)ortho_kernel<T>, dim3((unsigned)grid),
+                                    dim3(kOrthoThreads<T>), args, 0, mesh->stream) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return true;
+}
+
 template <typename T> fsi_status norm2(fsi_mesh *mesh, const T *x, double *dev_out)
 {
     return multi_dot<T>(mesh, 1, x, 0, x, dev_out, 1);
@@ -1307,6 +1530,7 @@ fsi_status gmres(fsi_mesh *mesh, const fsi_step_state *st, int restart, int max_
     std::vector<double> H((size_t)(restart + 1) * restart, 0.0), cs(restart), sn(restart),
         g(restart + 1), y(restart);
     zero_kernel<T><<<grid1d(len), 256, 0, s>>>(len, x);
+    zero_kernel<double><<<1, 32, 0, s>>>(2, W.hcol + restart + 2);
     FSI_TRY(check_launch("zero"));
     // r = b (x0 = 0)
     cudaMemcpyAsync(w, b, len * sizeof(T), cudaMemcpyDeviceToDevice, s);
@@ -1352,19 +1576,22 @@ fsi_status gmres(fsi_mesh *mesh, const fsi_step_state *st, int restart, int max_
             // second pass (when it is due) is launched conditionally, so the
             // iteration needs one host synchronisation, at its end; |w| of the
             // orthogonalised vector comes out of the update pass itself
-            double *flag = W.h2 + restart + 1;
-            FSI_TRY(multi_dot<T>(mesh, j + 2, V, ld, w, W.hcol, 0, j + 1, nullptr, j, flag));
-            gram_schmidt<T>(mesh, j + 1, V, ld, W.hcol, w, flag, W.hcol + j + 1);
-            FSI_TRY(check_launch("Gram-Schmidt"));
-            scale_basis(W.hcol + j + 1, V + (int64_t)(j + 1) * ld);
-            FSI_CUDA(cudaMemcpyAsync(W.hhost, W.hcol, (j + 2) * sizeof(double),
-                                     cudaMemcpyDeviceToHost, s),
-                     "memcpy");
-            FSI_CUDA(cudaMemcpyAsync(W.hhost + j + 2, flag, sizeof(double),
+            double *flag = W.hcol + restart + 2, *err = flag + 1;
+            if (!ortho_launch<T>(mesh, j + 1, V, ld, flag, err, fuse ? (const T *)W.inv : nullptr, z, bp)) {
+                FSI_TRY(multi_dot<T>(mesh, j + 2, V, ld, w, W.hcol, 0, j + 1, nullptr, j, flag));
+                gram_schmidt<T>(mesh, j + 1, V, ld, W.hcol, w, flag, W.hcol + j + 1);
+                FSI_TRY(check_launch("Gram-Schmidt"));
+                scale_basis(W.hcol + j + 1, V + (int64_t)(j + 1) * ld);
+            }
+            FSI_CUDA(cudaMemcpyAsync(W.hhost, W.hcol, (restart + 4) * sizeof(double),
                                      cudaMemcpyDeviceToHost, s),
                      "memcpy");
             FSI_CUDA(cudaStreamSynchronize(s), "GMRES sync");
-            if (W.hhost[j + 2] != 0.0) ++W.reorth;
+            if (W.hhost[restart + 3] != 0.0) {
+                cudaMemsetAsync(W.ticket, 0, 4 * sizeof(unsigned), s);
+                return set_error(FSI_ERR_TIMEOUT, "GMRES: a wait between CTAs ran out");
+            }
+            if (W.hhost[restart + 2] != 0.0) ++W.reorth;
             ++its;
             double *h = &H[(size_t)j * (restart + 1)];
             for (int i = 0; i <= j + 1; ++i) h[i] = W.hhost[i];
