@@ -175,41 +175,32 @@ __global__ void cheb0_kernel(LevelArgs<T> L, const T *__restrict__ b, T inv_thet
 }
 
 // ---------------------------------------------------------------- z-marching stencil
-// The operator A = K + kappa M of a level is a tensor product of 1D Q1 rows
-// (stiffness k, mass m per axis), so (A v)_node = sum_dk [P(k+dk) mz(dk) +
-// Q(k+dk) kz(dk)] with, per plane k', P = Ax + By + kappa C and Q = C, where
-// Ax = sum_dj sK_x(j+dj) my(dj), By = sum_dj sM_x(j+dj) ky(dj), C = sum_dj
-// sM_x(j+dj) my(dj), and sK_x / sM_x the 1D stiffness / mass rows along x.
-// A CTA of 32 x 8 threads owns a 32 x 8 column of nodes and marches up kz
-// planes (as many as leave about 16 CTAs per SM, 2 to 16): per plane it
-// stages v (with a one-node
-// halo, zero outside the grid and on eliminated nodes, whose columns A does
-// not have) in shared memory, forms the x rows once per position, and each
-// thread folds its 3 x 3 neighbourhood into (P, Q) for the plane; the z fold
-// uses the three most recent planes held in registers.  The next plane's
-// loads are issued before the current plane is folded, so their latency
-// overlaps the work.  Every v is read once per plane (plus halos) instead of
-// 27 times, and the per-node work is ~30 operations.  Rows of eliminated
-// nodes keep only the diagonal.  The sums run in a fixed order
-// (deterministic).  (One thread per column marching without shared memory,
-// reading its 3 x 3 neighbourhood through L1, measured 1.8x slower; two
-// rows per thread, 8 apart, measured 1.3x slower at 129^3: 88-94 registers
-// leave 2 CTAs per SM.)  The source of v (x, d or x + d) is a template
-// parameter, so no pass tests for null vectors per load.
-constexpr int kMarchX = 32, kMarchTY = 8, kMarchRows = 1;    // threads x, threads y, rows per thread
-constexpr int kMarchY = kMarchTY * kMarchRows;                   // node rows per CTA
-constexpr int kMarchThreads = kMarchX * kMarchTY;
-constexpr int kStage = (kMarchY + 2) * (kMarchX + 2);            // staged values per plane
-constexpr int kStagePer = (kStage + kMarchThreads - 1) / kMarchThreads;
-constexpr int kXRows = (kMarchY + 2) * kMarchX;                  // x-row positions per plane
-constexpr int kXRowPer = (kXRows + kMarchThreads - 1) / kMarchThreads;
+// The operator A = K + kappa M of a level is a tensor product of symmetric 1D Q1
+// rows (stiffness k, mass m per axis), so with S_0 the node's value, S_x the sum of
+// its two x neighbours, S_y of the y neighbours and S_xy of the four diagonal ones
+// in a plane, (A v)(k) = PA(k) + PB(k - 1) + PB(k + 1), PA = sum_c A_c S_c and PB =
+// sum_c B_c S_c.  The 8 weights depend on the node's place along x only: a
+// boundary node's own 1D entries are exactly half of an inner one's, so on a
+// boundary row S_0 and S_x, and on a boundary plane PA, count half, and 1/D takes
+// factors of two.
+//
+// A lane owns a column in x, a warp 32 of them (the outer two are halo: 30 give
+// results) by R rows, and marches up kz planes: x neighbours come by shuffles, y
+// neighbours are the lane's own rows, the z fold is held in registers; the next
+// plane's loads are in flight while a plane is folded.  No shared memory and no
+// barrier: with both (x rows formed once per CTA, three barriers a plane) the four
+// passes of a smoothing at 129^3 took 145 us in FP32, now 88 us.  v is zero
+// outside the grid and on eliminated nodes (whose columns A does not have); rows of
+// eliminated nodes keep only the diagonal.  Fixed order of sums (deterministic).
+constexpr int kMarchOut = 30;    // columns of results per warp
+constexpr int kMarchWarps = 4;   // warps per CTA, one row group each
 
 template <typename T> struct March {
     const T *x, *d;  // v = x + d (VX selects which are present)
     const T *b;
     T c1, c2, inv_theta;
     T *y, *x_next, *d_next, *x_final;
-    int kz;          // planes per CTA
+    int kz;          // planes per warp
     // with z4 (a step's x_final): the result goes to z4[4 node + 3] as
     // x_final * inv_sigma, or v4[4 node + 3] where m4[4 node + 3] is set
     T *z4;
@@ -234,239 +225,162 @@ __device__ __forceinline__ T kd_of(const Axis<T> &a, int i)
 {
     return (i == 0 || i == a.N) ? a.k_bd : a.k_in;
 }
-template <typename T, int VX> __device__ __forceinline__ T vsrc(const March<T> &M, int64_t q)
+template <typename T, int MODE, int VX, int R>
+__global__ void __launch_bounds__(32 * kMarchWarps) march_kernel(LevelArgs<T> L, March<T> M)
 {
-    if constexpr (VX == kVd) return M.d[q];
-    else if constexpr (VX == kVx) return M.x[q];
-    else return M.x[q] + M.d[q];
-}
-
-template <typename T, int MODE, int VX>
-__global__ void __launch_bounds__(kMarchThreads) march_kernel(LevelArgs<T> L, March<T> M)
-{
-    __shared__ T vt[kStage];                      // [kMarchY + 2][kMarchX + 2]
-    __shared__ T sk[kXRows], sm[kXRows];          // [kMarchY + 2][kMarchX]
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + kMarchX * ty;
-    const int i0 = blockIdx.x * kMarchX, j0 = blockIdx.y * kMarchY, k0 = blockIdx.z * M.kz;
-    const int i = i0 + tx;
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x;
+    const int i = blockIdx.x * kMarchOut + lane - 1, j0 = (blockIdx.y * kMarchWarps + threadIdx.y) * R;
+    const int k0 = blockIdx.z * M.kz, k1 = min(k0 + M.kz, L.NZ1);  // planes k0 .. k1-1 are output
+    if (j0 >= L.NY1) return;
     const Axis<T> &ax = L.a[0], &ay = L.a[1], &az = L.a[2];
     const int64_t plane_n = (int64_t)L.NX1 * L.NY1;
-    // per thread, once: the staged slots' in-plane offsets and masks (x, y
-    // faces), the x-row slots' centre coefficients and staged indices
-    int64_t s_off[kStagePer];
-    bool s_in[kStagePer];
-    // kVb: 1/D of the staged column's nodes on an interior / boundary plane
-    T s_iDi[kStagePer], s_iDb[kStagePer];
+    const bool inx = i >= 0 && i < L.NX1;
+    const bool elx = (L.faces[0] && i == 0) || (L.faces[1] && i == L.NX1 - 1);
+    // rows j0 - 1 .. j0 + R: in the grid, not eliminated, half weights
+    bool in[R + 2], ok[R + 2];
 #pragma unroll
-    for (int r = 0; r < kStagePer; ++r) {
-        const int q = tid + r * kMarchThreads;
-        const int gi = i0 - 1 + q % (kMarchX + 2), gj = j0 - 1 + q / (kMarchX + 2);
-        s_in[r] = q < kStage && gi >= 0 && gj >= 0 && gi < L.NX1 && gj < L.NY1 &&
-                  !((L.faces[0] && gi == 0) || (L.faces[1] && gi == L.NX1 - 1) ||
-                    (L.faces[2] && gj == 0) || (L.faces[3] && gj == L.NY1 - 1));
-        s_off[r] = gi + (int64_t)L.NX1 * gj;
-        if constexpr (VX == kVb) {
-            const T mx = md_of(L.a[0], gi), kx = kd_of(L.a[0], gi);
-            const T my = md_of(L.a[1], gj), ky = kd_of(L.a[1], gj);
-            const T a1 = kx * my + mx * ky + L.kappa * mx * my, a2 = mx * my;
-            s_iDi[r] = T(1) / (a1 * L.a[2].m_in + a2 * L.a[2].k_in);
-            s_iDb[r] = T(1) / (a1 * L.a[2].m_bd + a2 * L.a[2].k_bd);
+    for (int r = 0; r < R + 2; ++r) {
+        const int j = j0 - 1 + r;
+        in[r] = inx && j >= 0 && j < L.NY1;
+        ok[r] = in[r] && !elx && !((L.faces[2] && j == 0) || (L.faces[3] && j == L.NY1 - 1));
+    }
+    auto bdy = [&](int r) { const int j = j0 - 1 + r; return j == 0 || j == L.NY1 - 1; };
+    T A[4], B[4];
+    {
+        const T mx = md_of(ax, i), kx = kd_of(ax, i);
+        const T ky = ay.k_in + L.kappa * ay.m_in, kyo = ay.k_off + L.kappa * ay.m_off;
+        const T P[4] = {kx * ay.m_in + mx * ky, ax.k_off * ay.m_in + ax.m_off * ky,
+                        kx * ay.m_off + mx * kyo, ax.k_off * ay.m_off + ax.m_off * kyo};
+        const T Q[4] = {mx * ay.m_in, ax.m_off * ay.m_in, mx * ay.m_off, ax.m_off * ay.m_off};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            A[c] = P[c] * az.m_in + Q[c] * az.k_in;
+            B[c] = P[c] * az.m_off + Q[c] * az.k_off;
         }
     }
-    T x_k[kXRowPer], x_m[kXRowPer];
-    int x_v[kXRowPer];
+    const T iA0 = T(1) / A[0];
+    const int64_t off = i + (int64_t)L.NX1 * (j0 - 1);
+    auto elz = [&](int k) { return (L.faces[4] && k == 0) || (L.faces[5] && k == L.NZ1 - 1); };
+    auto bdz = [&](int k) { return k == 0 || k == L.NZ1 - 1; };
+
+    // a plane as loaded: x (or b, VX = kVb) and d
+    struct Raw {
+        T x[R + 2], d[R + 2];
+    };
+    auto load = [&](int k, Raw &w) {
+        const bool inz = k >= 0 && k < L.NZ1;
+        const int64_t q = off + plane_n * k;
 #pragma unroll
-    for (int r = 0; r < kXRowPer; ++r) {
-        const int q = tid + r * kMarchThreads;
-        const int cx = q % kMarchX, cy = q / kMarchX;
-        x_k[r] = kd_of(ax, i0 + cx);
-        x_m[r] = md_of(ax, i0 + cx);
-        x_v[r] = cy * (kMarchX + 2) + cx;
-    }
-    // this thread's nodes (i, j0 + ty + kMarchTY * rr): D = A1 mz(0) + A2 kz(0)
-    const T mdx = md_of(ax, i), kdx = kd_of(ax, i);
-    T mdy[kMarchRows], kdy[kMarchRows], A1[kMarchRows], A2[kMarchRows], iDb[kMarchRows],
-        iDi[kMarchRows];
-    bool own[kMarchRows], exy[kMarchRows];
-    int64_t off[kMarchRows];
-#pragma unroll
-    for (int rr = 0; rr < kMarchRows; ++rr) {
-        const int j = j0 + ty + kMarchTY * rr;
-        own[rr] = i < L.NX1 && j < L.NY1;
-        mdy[rr] = md_of(ay, j);
-        kdy[rr] = kd_of(ay, j);
-        A1[rr] = kdx * mdy[rr] + mdx * kdy[rr] + L.kappa * mdx * mdy[rr];
-        A2[rr] = mdx * mdy[rr];
-        iDb[rr] = T(1) / (A1[rr] * az.m_bd + A2[rr] * az.k_bd);
-        iDi[rr] = T(1) / (A1[rr] * az.m_in + A2[rr] * az.k_in);
-        exy[rr] = (L.faces[0] && i == 0) || (L.faces[1] && i == L.NX1 - 1) ||
-                  (L.faces[2] && j == 0) || (L.faces[3] && j == L.NY1 - 1);
-        off[rr] = i + (int64_t)L.NX1 * j;
-    }
-    const int klast = min(k0 + M.kz, L.NZ1);  // planes k0 .. klast-1 are output
-    auto stage = [&](int kk, T (&v)[kStagePer]) {
-        const bool zcut = kk < 0 || kk >= L.NZ1 || (L.faces[4] && kk == 0) ||
-                          (L.faces[5] && kk == L.NZ1 - 1);
-        if constexpr (VX == kVb) {
-            const bool zb = kk == 0 || kk == L.NZ1 - 1;
-#pragma unroll
-            for (int r = 0; r < kStagePer; ++r)
-                v[r] = (s_in[r] && !zcut) ? M.inv_theta * M.b[s_off[r] + plane_n * kk] *
-                                                (zb ? s_iDb[r] : s_iDi[r])
-                                          : T(0);
-        } else {
-#pragma unroll
-            for (int r = 0; r < kStagePer; ++r)
-                v[r] = (s_in[r] && !zcut) ? vsrc<T, VX>(M, s_off[r] + plane_n * kk) : T(0);
+        for (int r = 0; r < R + 2; ++r) {
+            const bool g = inz && in[r];
+            if constexpr (VX != kVd) w.x[r] = g ? __ldg((VX == kVb ? M.b : M.x) + q + (int64_t)L.NX1 * r) : T(0);
+            if constexpr (VX == kVd || VX == kVxd) w.d[r] = g ? __ldg(M.d + q + (int64_t)L.NX1 * r) : T(0);
         }
     };
-    // per row: (P, Q) of planes k-1, k; the node inputs of the next output
-    // plane (b, d, v) loaded one plane ahead, the staged planes two ahead
-    T Pm[kMarchRows], P0[kMarchRows], Qm[kMarchRows], Q0[kMarchRows];
-    T b_nx[kMarchRows], d_nx[kMarchRows], v_nx[kMarchRows];
+    // v from a loaded plane's row
+    auto value = [&](const Raw &w, int r, T gz) {
+        if constexpr (VX == kVd) return w.d[r];
+        else if constexpr (VX == kVx) return w.x[r];
+        else if constexpr (VX == kVxd) return w.x[r] + w.d[r];
+        else return M.inv_theta * w.x[r] * (iA0 * (bdy(r) ? gz + gz : gz));
+    };
+
+    // per output row: fz PA(k) + PB(k - 1) and PB(k) of the plane k below the
+    // current one, and that plane's v, d and b at the node
+    T acc[R], PBk[R], vk[R], dk[R], bk[R];
 #pragma unroll
-    for (int rr = 0; rr < kMarchRows; ++rr)
-        Pm[rr] = P0[rr] = Qm[rr] = Q0[rr] = b_nx[rr] = d_nx[rr] = v_nx[rr] = T(0);
-    auto plane = [&](int kk, T (&cur)[kStagePer]) {
+    for (int r = 0; r < R; ++r) acc[r] = PBk[r] = vk[r] = dk[r] = bk[r] = T(0);
+    Raw nx;
+    load(k0 - 1, nx);
+    for (int kk = k0 - 1; kk <= k1; ++kk) {
+        const Raw w = nx;
+        if (kk < k1) load(kk + 1, nx);
+        const bool zb = bdz(kk), vz = kk >= 0 && kk < L.NZ1 && !elz(kk);
+        const T gz = zb ? T(2) : T(1), fz = zb ? T(0.5) : T(1);
+        // the node inputs of this plane's results, used one plane later
+        T bn[R];
+        const bool mine = kk >= k0 && kk < k1;
 #pragma unroll
-        for (int r = 0; r < kStagePer; ++r)
-            if (tid + r * kMarchThreads < kStage) vt[tid + r * kMarchThreads] = cur[r];
-        __syncthreads();
-        T b_cur[kMarchRows], d_cur[kMarchRows], v_cur[kMarchRows];
-#pragma unroll
-        for (int rr = 0; rr < kMarchRows; ++rr) {
-            b_cur[rr] = b_nx[rr];
-            d_cur[rr] = d_nx[rr];
-            v_cur[rr] = v_nx[rr];
+        for (int r = 0; r < R; ++r) {
+            bn[r] = T(0);
+            if constexpr (VX == kVb) bn[r] = w.x[r + 1];
+            else if (M.b && mine && in[r + 1])
+                bn[r] = __ldg(M.b + off + plane_n * kk + (int64_t)L.NX1 * (r + 1));
         }
-        // the loads two planes ahead are in flight while this plane is folded
-        if (kk + 2 <= klast) stage(kk + 2, cur);
-        const bool ez = (L.faces[4] && kk == 0) || (L.faces[5] && kk == L.NZ1 - 1);
-        if (kk >= k0 && kk < klast) {
+        T v[R + 2], X[R + 2];
 #pragma unroll
-            for (int rr = 0; rr < kMarchRows; ++rr)
-                if (own[rr]) {
-                    const int64_t nd = off[rr] + plane_n * kk;
-                    if (M.b) b_nx[rr] = M.b[nd];
-                    if constexpr (VX == kVb) {
-                        // v = d0 at the node (staged, unless eliminated)
-                        const bool zb = kk == 0 || kk == L.NZ1 - 1;
-                        v_nx[rr] = (exy[rr] || ez)
-                                       ? M.inv_theta * b_nx[rr] * (zb ? iDb[rr] : iDi[rr])
-                                       : vt[(ty + kMarchTY * rr + 1) * (kMarchX + 2) + tx + 1];
-                        d_nx[rr] = v_nx[rr];
-                    } else {
-                        if (MODE == kMarchStep) d_nx[rr] = M.d[nd];
-                        // v at the node: staged, unless eliminated (staged as 0)
-                        v_nx[rr] = (exy[rr] || ez)
-                                       ? vsrc<T, VX>(M, nd)
-                                       : vt[(ty + kMarchTY * rr + 1) * (kMarchX + 2) + tx + 1];
-                    }
-                }
+        for (int r = 0; r < R + 2; ++r) {
+            v[r] = vz && ok[r] ? value(w, r, gz) : T(0);
+            X[r] = __shfl_up_sync(kAll, v[r], 1) + __shfl_down_sync(kAll, v[r], 1);
         }
-        // the x rows of the plane at the CTA's columns, rows j0-1 .. j0+kMarchY
+        const int k = kk - 1;  // the plane that is complete now
+        const bool out = k >= k0 && inx && lane >= 1 && lane <= kMarchOut;
+        const bool kb = bdz(k), kel = elz(k);
 #pragma unroll
-        for (int r = 0; r < kXRowPer; ++r) {
-            const int q = tid + r * kMarchThreads;
-            if (q < kXRows) {
-                const T vm = vt[x_v[r]], v0 = vt[x_v[r] + 1], vp = vt[x_v[r] + 2];
-                T a = T(0), c = T(0);
-                a += ax.k_off * vm;
-                c += ax.m_off * vm;
-                a += x_k[r] * v0;
-                c += x_m[r] * v0;
-                a += ax.k_off * vp;
-                c += ax.m_off * vp;
-                sk[q] = a;
-                sm[q] = c;
-            }
-        }
-        __syncthreads();
-        const int k = kk - 1;  // output plane: k-1, k, k+1 = (Pm, P0, Pp)
-        const bool out = k >= k0 && k < klast;
-        const bool bd = k == 0 || k == L.NZ1 - 1;
-        const bool elim_z = (L.faces[4] && k == 0) || (L.faces[5] && k == L.NZ1 - 1);
-        const T mdz = bd ? az.m_bd : az.m_in, kdz = bd ? az.k_bd : az.k_in;
-#pragma unroll
-        for (int rr = 0; rr < kMarchRows; ++rr) {
-            // y fold for this row's column on plane kk
-            const int c0 = (ty + kMarchTY * rr) * kMarchX + tx;
-            T Ax = T(0), By = T(0), C = T(0);
-            Ax += sk[c0] * ay.m_off;
-            By += sm[c0] * ay.k_off;
-            C += sm[c0] * ay.m_off;
-            Ax += sk[c0 + kMarchX] * mdy[rr];
-            By += sm[c0 + kMarchX] * kdy[rr];
-            C += sm[c0 + kMarchX] * mdy[rr];
-            Ax += sk[c0 + 2 * kMarchX] * ay.m_off;
-            By += sm[c0 + 2 * kMarchX] * ay.k_off;
-            C += sm[c0 + 2 * kMarchX] * ay.m_off;
-            const T Pp = Ax + By + L.kappa * C, Qp = C;
-            if (out && own[rr]) {
-                const int64_t node = off[rr] + plane_n * k;
-                T Av = T(0);
-                Av += Pm[rr] * az.m_off;
-                Av += Qm[rr] * az.k_off;
-                Av += P0[rr] * mdz;
-                Av += Q0[rr] * kdz;
-                Av += Pp * az.m_off;
-                Av += Qp * az.k_off;
-                const T inv_D = bd ? iDb[rr] : iDi[rr];
-                if (exy[rr] || elim_z) Av = (A1[rr] * mdz + A2[rr] * kdz) * v_cur[rr];
+        for (int r = 0; r < R; ++r) {
+            const T fy = bdy(r + 1) ? T(0.5) : T(1);
+            const T S0 = fy * v[r + 1], Sx = fy * X[r + 1], Sy = v[r] + v[r + 2], Sxy = X[r] + X[r + 2];
+            const T PA = A[0] * S0 + A[1] * Sx + A[2] * Sy + A[3] * Sxy;
+            const T PB = B[0] * S0 + B[1] * Sx + B[2] * Sy + B[3] * Sxy;
+            if (out && in[r + 1]) {
+                const int64_t node = off + plane_n * k + (int64_t)L.NX1 * (r + 1);
+                const T g = (kb ? T(2) : T(1)) * (bdy(r + 1) ? T(2) : T(1)), inv_D = iA0 * g;
+                const T Av = ok[r + 1] && !kel ? acc[r] + PB : A[0] * (fy * (kb ? T(0.5) : T(1))) * vk[r];
                 if constexpr (MODE == kMarchApply) {
-                    M.y[node] = M.b ? b_cur[rr] - Av : Av;
+                    M.y[node] = M.b ? bk[r] - Av : Av;
                 } else if constexpr (MODE == kMarchCheb0) {
                     // first Chebyshev direction from x (not null here)
-                    const T d0 = M.inv_theta * (b_cur[rr] - Av) * inv_D;
+                    const T d0 = M.inv_theta * (bk[r] - Av) * inv_D;
                     if (M.x_final)
-                        M.x_final[node] = v_cur[rr] + d0;
+                        M.x_final[node] = vk[r] + d0;
                     else
                         M.d_next[node] = d0;
                 } else {
-                    const T dn = M.c1 * d_cur[rr] + M.c2 * ((b_cur[rr] - Av) * inv_D);
+                    const T dn = M.c1 * dk[r] + M.c2 * ((bk[r] - Av) * inv_D);
                     if (M.z4) {
-                        M.z4[4 * node + 3] = (M.m4 && M.m4[4 * node + 3])
-                                                 ? M.v4[4 * node + 3]
-                                                 : (v_cur[rr] + dn) * M.inv_sigma;
+                        M.z4[4 * node + 3] = (M.m4 && M.m4[4 * node + 3]) ? M.v4[4 * node + 3]
+                                                                         : (vk[r] + dn) * M.inv_sigma;
                     } else if (M.x_final) {
-                        M.x_final[node] = v_cur[rr] + dn;
+                        M.x_final[node] = vk[r] + dn;
                     } else {
-                        M.x_next[node] = v_cur[rr];
+                        M.x_next[node] = vk[r];
                         M.d_next[node] = dn;
                     }
                 }
             }
-            Pm[rr] = P0[rr];
-            Qm[rr] = Q0[rr];
-            P0[rr] = Pp;
-            Q0[rr] = Qp;
+            acc[r] = fz * PA + PBk[r];
+            PBk[r] = PB;
+            vk[r] = value(w, r + 1, gz);  // also where it is eliminated
+            if constexpr (MODE == kMarchStep) dk[r] = VX == kVb ? vk[r] : w.d[r + 1];
+            bk[r] = bn[r];
         }
-        __syncthreads();
-    };
-    T pa[kStagePer], pb[kStagePer];
-    stage(k0 - 1, pa);
-    stage(k0, pb);
-    for (int kk = k0 - 1; kk <= klast; kk += 2) {
-        plane(kk, pa);
-        if (kk + 1 <= klast) plane(kk + 1, pb);
     }
 }
 
-const dim3 kMarchBlock(kMarchX, kMarchTY);
-
-template <typename T, int MODE, int VX>
-fsi_status march_launch(const PressureMG &P, int l, cudaStream_t s, March<T> M)
+template <typename T, int MODE, int VX, int R>
+fsi_status march_rows(const PressureMG &P, int l, cudaStream_t s, March<T> M)
 {
     const PmgLevel &L = P.lev[l];
     const int nz1 = L.N[2] + 1;
-    const int gx = (L.N[0] + 1 + kMarchX - 1) / kMarchX, gy = (L.N[1] + 1 + kMarchY - 1) / kMarchY;
-    // planes per CTA: about 8 CTAs per SM in all (each CTA's planes are a
-    // serial chain of shared-memory passes), at least 2, at most 16
-    const int64_t cols = (int64_t)gx * gy;
-    M.kz = (int)std::max<int64_t>(2, std::min<int64_t>(16, nz1 * cols / (16 * sm_count())));
-    const dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)((nz1 + M.kz - 1) / M.kz));
-    march_kernel<T, MODE, VX><<<grid, kMarchBlock, 0, s>>>(level_args<T>(P, l), M);
+    const int gx = (L.N[0] + kMarchOut) / kMarchOut, gy = (L.N[1] + R) / R;
+    // planes per warp: 12 warps an SM (a warp reads two planes more than it
+    // writes, and its planes are a serial chain), 1 to 16
+    M.kz = (int)std::max<int64_t>(1, std::min<int64_t>(16, (int64_t)nz1 * gx * gy / (12 * sm_count())));
+    const dim3 grid((unsigned)gx, (unsigned)((gy + kMarchWarps - 1) / kMarchWarps),
+                    (unsigned)((nz1 + M.kz - 1) / M.kz));
+    march_kernel<T, MODE, VX, R><<<grid, dim3(32, kMarchWarps), 0, s>>>(level_args<T>(P, l), M);
     return check_launch("pressure stencil");
+}
+// Rows per warp: more rows share their neighbours' loads, fewer give short vectors
+// more warps (a mixed step at 32^3 with 4, 2, 1 rows: 7.93, 7.77, 7.65 ms; FP64 at
+// 24^3: 37.2, 33.2, 31.1 ms; 129^3 gains from 4, 65^3 is level between 2 and 4)
+template <typename T, int MODE, int VX>
+fsi_status march_launch(const PressureMG &P, int l, cudaStream_t s, const March<T> &M)
+{
+    if (P.lev[l].n >= 400000) return march_rows<T, MODE, VX, 4>(P, l, s, M);
+    if (P.lev[l].n >= 100000) return march_rows<T, MODE, VX, 2>(P, l, s, M);
+    return march_rows<T, MODE, VX, 1>(P, l, s, M);
 }
 
 // the stencil pass in MODE: on v = M.x (apply, first Chebyshev direction) or
@@ -498,58 +412,68 @@ fsi_status level_apply(const PressureMG &P, int l, cudaStream_t s, const T *x, c
 }
 
 // b_c = P^T r: each coarse node gathers the fine nodes within one fine cell,
-// weights 1 (coincident) and 1/2 (neighbour) per axis; zero on eliminated nodes
+// weights 1 (coincident) and 1/2 (neighbour) per axis; zero on eliminated nodes.
+// A thread has a coarse column (I, J) and goes up kz coarse planes: a fine plane's
+// 3 x 3 sum is formed once for the two coarse planes that it belongs to
 template <typename T>
-__global__ void restrict_kernel(LevelArgs<T> F, LevelArgs<T> C, const T *__restrict__ r,
+__global__ void restrict_kernel(LevelArgs<T> F, LevelArgs<T> C, int kz, const T *__restrict__ r,
                                 T *__restrict__ bc)
 {
-    NODE3(C, I, J, K)
-    {
-        const int64_t node = I + (int64_t)C.NX1 * (J + (int64_t)C.NY1 * K);
-        T acc = T(0);
-        for (int dk = -1; dk <= 1; ++dk) {
-            const int k = 2 * K + dk;
-            if (k < 0 || k >= F.NZ1) continue;
-            const T wk = dk ? T(0.5) : T(1);
-            for (int dj = -1; dj <= 1; ++dj) {
-                const int j = 2 * J + dj;
-                if (j < 0 || j >= F.NY1) continue;
-                const T wjk = (dj ? T(0.5) : T(1)) * wk;
-                const T *row = r + (int64_t)F.NX1 * (j + (int64_t)F.NY1 * k);
-                T s = T(0);
-                for (int di = -1; di <= 1; ++di) {
-                    const int i = 2 * I + di;
-                    if (i < 0 || i >= F.NX1) continue;
-                    s += (di ? T(0.5) : T(1)) * row[i];
-                }
-                acc += wjk * s;
-            }
-        }
-        bc[node] = eliminated(C, I, J, K) ? T(0) : acc;
+    const int I = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y * blockDim.y + threadIdx.y;
+    if (I >= C.NX1 || J >= C.NY1) return;
+    const int K0 = blockIdx.z * kz, K1 = min(K0 + kz, C.NZ1);
+    const int xl = I > 0 ? 1 : 0, xr = 2 * I + 1 < F.NX1 ? 1 : 0, yl = J > 0 ? F.NX1 : 0,
+              yr = 2 * J + 1 < F.NY1 ? F.NX1 : 0;
+    const T wl = xl ? T(0.5) : T(0), wr = xr ? T(0.5) : T(0), vl = yl ? T(0.5) : T(0),
+            vr = yr ? T(0.5) : T(0);
+    const int64_t plane_n = (int64_t)F.NX1 * F.NY1, off = 2 * I + (int64_t)F.NX1 * (2 * J);
+    auto plane = [&](int k) {
+        if (k < 0 || k >= F.NZ1) return T(0);
+        const T *q = r + off + plane_n * k;
+        const T a = q[0] + wl * q[-xl] + wr * q[xr];
+        const T b = q[-yl] + wl * q[-yl - xl] + wr * q[xr - yl];
+        const T c = q[yr] + wl * q[yr - xl] + wr * q[yr + xr];
+        return a + vl * b + vr * c;
+    };
+    T below = plane(2 * K0 - 1);
+#pragma unroll 2
+    for (int K = K0; K < K1; ++K) {
+        const T at = plane(2 * K), above = plane(2 * K + 1);
+        bc[I + (int64_t)C.NX1 * (J + (int64_t)C.NY1 * K)] =
+            eliminated(C, I, J, K) ? T(0) : at + T(0.5) * (below + above);
+        below = above;
     }
 }
 
-// x += P x_c: trilinear interpolation of the coarse correction
+// x += P x_c: trilinear interpolation of the coarse correction.  A thread has a
+// fine column (i, j) and goes up kz coarse planes, two fine nodes for each: the mean
+// of the (one, two or four) coarse values around the column in a plane is formed
+// once per coarse plane.  (A node at a time with its loops over the coarse
+// neighbours took 22 us at 129^3 in FP32, now 12 us.)
 template <typename T>
-__global__ void prolong_kernel(LevelArgs<T> F, LevelArgs<T> C, const T *__restrict__ xc,
+__global__ void prolong_kernel(LevelArgs<T> F, LevelArgs<T> C, int kz, const T *__restrict__ xc,
                                T *__restrict__ x)
 {
-    NODE3(F, i, j, k)
-    {
-        const int64_t node = i + (int64_t)F.NX1 * (j + (int64_t)F.NY1 * k);
-        const int i0 = i >> 1, j0 = j >> 1, k0 = k >> 1;
-        const int ni = (i & 1) ? 2 : 1, nj = (j & 1) ? 2 : 1, nk = (k & 1) ? 2 : 1;
-        const T wi = (i & 1) ? T(0.5) : T(1), wj = (j & 1) ? T(0.5) : T(1),
-                wk = (k & 1) ? T(0.5) : T(1);
-        T acc = T(0);
-        for (int c = 0; c < nk; ++c)
-            for (int bb = 0; bb < nj; ++bb) {
-                const T *row = xc + (int64_t)C.NX1 * ((j0 + bb) + (int64_t)C.NY1 * (k0 + c));
-                T s = T(0);
-                for (int a = 0; a < ni; ++a) s += row[i0 + a];
-                acc += (wj * wk) * (wi * s);
-            }
-        x[node] += acc;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+    if (i >= F.NX1 || j >= F.NY1) return;
+    const int K0 = blockIdx.z * kz, K1 = min(K0 + kz, C.NZ1);
+    const int dx = i & 1, dy = (j & 1) ? C.NX1 : 0;
+    const int64_t plane_n = (int64_t)F.NX1 * F.NY1, plane_c = (int64_t)C.NX1 * C.NY1;
+    const T *c = xc + (i >> 1) + (int64_t)C.NX1 * (j >> 1);
+    T *f = x + i + (int64_t)F.NX1 * j;
+    auto plane = [&](int K) {
+        const T *q = c + plane_c * K;
+        return T(0.25) * ((q[0] + q[dx]) + (q[dy] + q[dy + dx]));
+    };
+    T at = plane(K0);
+#pragma unroll 2
+    for (int K = K0; K < K1; ++K) {
+        f[plane_n * (2 * K)] += at;
+        if (2 * K + 1 < F.NZ1) {
+            const T above = plane(K + 1);
+            f[plane_n * (2 * K + 1)] += T(0.5) * (at + above);
+            at = above;
+        }
     }
 }
 
@@ -578,18 +502,18 @@ __global__ void dense_apply_kernel(int64_t nc, const T *__restrict__ Ainv, const
 
 int grid_for(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, sm_count() * 16)); }
 
-// node kernels: CTAs of 32 nodes along x by 4 along y (at 129 nodes per row:
-// 81 % of the lanes busy, against 50 % for 128-node rows of CTAs), one plane
-// per grid layer
+// transfers: CTAs of 32 nodes along x by 4 along y of L (at 129 nodes per row:
+// 81 % of the lanes busy, against 50 % for 128-node rows of CTAs), and along z the
+// coarse planes, up to four per thread where that leaves 8 CTAs per SM
 const dim3 kRowBlock(32, 4);
-dim3 grid3(const PmgLevel &L)
+dim3 transfer_grid(const PmgLevel &L, const PmgLevel &Lc, int &kz)
 {
-    return dim3((unsigned)((L.N[0] + 1 + 31) / 32), (unsigned)((L.N[1] + 1 + 3) / 4),
-                (unsigned)(L.N[2] + 1));
+    const int gx = (L.N[0] + 1 + 31) / 32, gy = (L.N[1] + 1 + 3) / 4;
+    kz = (int)std::max<int64_t>(1, std::min<int64_t>(4, (int64_t)gx * gy * (Lc.N[2] + 1) / (8 * sm_count())));
+    return dim3((unsigned)gx, (unsigned)gy, (unsigned)((Lc.N[2] + kz) / kz));
 }
-// the same with about 16 CTAs per SM in all, each striding over planes (for
-// the purely pointwise first smoother direction: 13 -> 8 us at 129^3; the
-// transfers are faster one plane per CTA)
+// node kernels with about 16 CTAs per SM in all, each striding over planes (the
+// purely pointwise first smoother direction: 13 -> 8 us at 129^3)
 dim3 grid3_strided(const PmgLevel &L)
 {
     const int gx = (L.N[0] + 1 + 31) / 32, gy = (L.N[1] + 1 + 3) / 4;
@@ -1128,11 +1052,14 @@ fsi_status vcycle_level(fsi_mesh *m, int l, const T *b, T *x, const SchurOut<T> 
     T *t = vec<T>(L.t);
     FSI_TRY(chebyshev<T>(m, l, kPmgNu, hi / 4.0, hi, b, (const T *)nullptr, t));
     const LevelArgs<T> A = level_args<T>(P, l), Ac = level_args<T>(P, l + 1);
+    int kz = 1;
     FSI_TRY(level_apply<T>(P, l, m->stream, t, b, vec<T>(L.r)));
-    restrict_kernel<T><<<grid3(Lc), kRowBlock, 0, m->stream>>>(A, Ac, vec<T>(L.r), vec<T>(Lc.b));
+    const dim3 gr = transfer_grid(Lc, Lc, kz);
+    restrict_kernel<T><<<gr, kRowBlock, 0, m->stream>>>(A, Ac, kz, vec<T>(L.r), vec<T>(Lc.b));
     FSI_TRY(check_launch("pressure restrict"));
     FSI_TRY(vcycle_level<T>(m, l + 1, vec<T>(Lc.b), vec<T>(Lc.x)));
-    prolong_kernel<T><<<grid3(L), kRowBlock, 0, m->stream>>>(A, Ac, vec<T>(Lc.x), t);
+    const dim3 gp = transfer_grid(L, Lc, kz);
+    prolong_kernel<T><<<gp, kRowBlock, 0, m->stream>>>(A, Ac, kz, vec<T>(Lc.x), t);
     FSI_TRY(check_launch("pressure prolong"));
     return chebyshev<T>(m, l, kPmgNu, hi / 4.0, hi, b, t, x, so);
 }
@@ -1404,14 +1331,15 @@ fsi_status fsi_pressure_restrict(fsi_mesh *mesh, fsi_prec prec, int32_t level, c
     FSI_TRY(pmg_ensure(mesh));
     FSI_TRY(check_level(mesh, level, true));
     PressureMG &P = *mesh->pmg;
-    const dim3 g = grid3(P.lev[level + 1]);
+    int kz = 1;
+    const dim3 g = transfer_grid(P.lev[level + 1], P.lev[level + 1], kz);
     if (prec == FSI_F64)
         restrict_kernel<double><<<g, kRowBlock, 0, mesh->stream>>>(
-            level_args<double>(P, level), level_args<double>(P, level + 1), (const double *)r,
+            level_args<double>(P, level), level_args<double>(P, level + 1), kz, (const double *)r,
             (double *)b);
     else
         restrict_kernel<float><<<g, kRowBlock, 0, mesh->stream>>>(
-            level_args<float>(P, level), level_args<float>(P, level + 1), (const float *)r,
+            level_args<float>(P, level), level_args<float>(P, level + 1), kz, (const float *)r,
             (float *)b);
     return check_launch("pressure restrict");
 }
@@ -1427,14 +1355,15 @@ fsi_status fsi_pressure_prolong_add(fsi_mesh *mesh, fsi_prec prec, int32_t level
     FSI_TRY(pmg_ensure(mesh));
     FSI_TRY(check_level(mesh, level, true));
     PressureMG &P = *mesh->pmg;
-    const dim3 g = grid3(P.lev[level]);
+    int kz = 1;
+    const dim3 g = transfer_grid(P.lev[level], P.lev[level + 1], kz);
     if (prec == FSI_F64)
         prolong_kernel<double><<<g, kRowBlock, 0, mesh->stream>>>(
-            level_args<double>(P, level), level_args<double>(P, level + 1), (const double *)xc,
+            level_args<double>(P, level), level_args<double>(P, level + 1), kz, (const double *)xc,
             (double *)x);
     else
         prolong_kernel<float><<<g, kRowBlock, 0, mesh->stream>>>(
-            level_args<float>(P, level), level_args<float>(P, level + 1), (const float *)xc,
+            level_args<float>(P, level), level_args<float>(P, level + 1), kz, (const float *)xc,
             (float *)x);
     return check_launch("pressure prolong");
 }
