@@ -806,14 +806,17 @@ __global__ void scale_split_kernel(int n, const double *den, const T *w, T *V, c
 // ------------------------------------------------ one launch per Gram-Schmidt
 // On short vectors every pass above is a launch of 9 to 16 us that moves a few MB:
 // its time is the launch, the FP64 reductions and the sum over the CTAs.  Here a
-// thread keeps one record of w and of all the basis vectors in registers for the
+// thread keeps one or two records of w and of all the basis vectors in registers for the
 // whole orthogonalisation -- dots, Kahan's test, update, second dots and update,
 // norm, scaling and Schur split -- and the CTAs, all resident (a cooperative
 // launch), meet at each sum: the last to arrive adds up the partial sums and
 // releases the others.  At 32^3 31 us an iteration (FP32, 10 vectors) against 38 to 50
 // us for the passes, and no gaps between them: a mixed step 8.95 -> 8.15 ms; FP64 at
 // 24^3 36.2 -> 35.1 ms.  Above 304 CTAs the records don't fit the registers.
-template <typename T> constexpr int kOrthoThreads = sizeof(T) == 4 ? 256 : 128;
+// Two records a thread in FP32: the FP64 sums over a warp (16 cycles an operation)
+// cost the same for twice the vector.
+constexpr int kOrthoThreads = 128;
+template <typename T> constexpr int kOrthoRec = sizeof(T) == 4 ? 2 : 1;
 constexpr int kOrthoMax = 16;                 // basis vectors held
 constexpr unsigned kOrthoPolls = 1u << 22;    // a wait gives up after a few seconds
 
@@ -871,22 +874,27 @@ __device__ __forceinline__ void grid_step(unsigned *bar, double *err, int &last_
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kOrthoThreads<T>, 2) ortho_kernel(const OrthoArgs<T> P)
+__global__ void __launch_bounds__(kOrthoThreads, 2) ortho_kernel(const OrthoArgs<T> P)
 {
-    constexpr int G = kOrthoMax, NT = kOrthoThreads<T>, NW = NT / 32, Q = (G + NW) / NW;
+    constexpr int G = kOrthoMax, R = kOrthoRec<T>, NT = kOrthoThreads, NW = NT / 32, Q = (G + NW) / NW;
     using Acc = typename DotAcc<T>::type;
     __shared__ double red[G + 1][NW];
     __shared__ double sums[G + 1];
     __shared__ T hs[G];
     __shared__ int state;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, cnt = P.cnt;
-    const int64_t i = blockIdx.x * (int64_t)NT + tid;
-    const bool live = i < P.n;
+    const int64_t i = blockIdx.x * (int64_t)(NT * R) + tid;
     const vec4<T> zero = {T(0), T(0), T(0), T(0)};
     if (tid == 0) state = 0;
-    vec4<T> w = live ? ld4(P.w + i) : zero, v[G];
+    vec4<T> w[R], v[R][G];
 #pragma unroll
-    for (int j = 0; j < G; ++j) v[j] = live && j < cnt ? ld4(P.V + (int64_t)j * P.vstride + i) : zero;
+    for (int q = 0; q < R; ++q) {
+        const bool live = i + q * NT < P.n;
+        w[q] = live ? ld4(P.w + i + q * NT) : zero;
+#pragma unroll
+        for (int j = 0; j < G; ++j)
+            v[q][j] = live && j < cnt ? ld4(P.V + (int64_t)j * P.vstride + i + q * NT) : zero;
+    }
 
     // V_j . w for all j (and w . w behind them) into this CTA's partial sums
     auto dots = [&](bool self, int nv) {
@@ -897,12 +905,15 @@ __global__ void __launch_bounds__(kOrthoThreads<T>, 2) ortho_kernel(const OrthoA
 #pragma unroll
                 for (int j = 0; j < kDotGroup; ++j) {
                     Acc a = Acc(0);
-                    if (g + j < nv) {
-                        dot_acc(a, v[g + j].x, w.x);
-                        dot_acc(a, v[g + j].y, w.y);
-                        dot_acc(a, v[g + j].z, w.z);
-                        dot_acc(a, v[g + j].w, w.w);
-                    }
+                    if (g + j < nv)
+#pragma unroll
+                        for (int q = 0; q < R; ++q) {
+                            dot_acc(a, v[q][g + j].x, w[q].x);
+                            dot_acc(a, v[q][g + j].y, w[q].y);
+                            dot_acc(a, v[q][g + j].z, w[q].z);
+                            dot_acc(a, v[q][g + j].w, w[q].w);
+                            dot_renorm(a);
+                        }
                     d[j] = dot_value(a);
                 }
                 const double t = warp_sums8(d, lane);
@@ -910,10 +921,14 @@ __global__ void __launch_bounds__(kOrthoThreads<T>, 2) ortho_kernel(const OrthoA
             }
         if (self) {
             Acc a = Acc(0);
-            dot_acc(a, w.x, w.x);
-            dot_acc(a, w.y, w.y);
-            dot_acc(a, w.z, w.z);
-            dot_acc(a, w.w, w.w);
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                dot_acc(a, w[q].x, w[q].x);
+                dot_acc(a, w[q].y, w[q].y);
+                dot_acc(a, w[q].z, w[q].z);
+                dot_acc(a, w[q].w, w[q].w);
+                dot_renorm(a);
+            }
             double d = dot_value(a);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
@@ -953,10 +968,13 @@ __global__ void __launch_bounds__(kOrthoThreads<T>, 2) ortho_kernel(const OrthoA
         for (int j = 0; j < G; ++j)
             if (j < cnt) {
                 const T hk = hs[j];
-                w.x = fma_rn(-v[j].x, hk, w.x);
-                w.y = fma_rn(-v[j].y, hk, w.y);
-                w.z = fma_rn(-v[j].z, hk, w.z);
-                w.w = fma_rn(-v[j].w, hk, w.w);
+#pragma unroll
+                for (int q = 0; q < R; ++q) {
+                    w[q].x = fma_rn(-v[q][j].x, hk, w[q].x);
+                    w[q].y = fma_rn(-v[q][j].y, hk, w[q].y);
+                    w[q].z = fma_rn(-v[q][j].z, hk, w[q].z);
+                    w[q].w = fma_rn(-v[q][j].w, hk, w[q].w);
+                }
             }
     };
     dots(true, cnt);
@@ -983,7 +1001,10 @@ __global__ void __launch_bounds__(kOrthoThreads<T>, 2) ortho_kernel(const OrthoA
         total(1);
         if (tid == 0) P.h[cnt] = sqrt(sums[0]);
     });
-    if (live) scale_split_node<T>(i, w, __ldcg(P.h + cnt), P.Vnew, P.inv, P.z, P.bp);
+    const double den = __ldcg(P.h + cnt);
+#pragma unroll
+    for (int q = 0; q < R; ++q)
+        if (i + q * NT < P.n) scale_split_node<T>(i + q * NT, w[q], den, P.Vnew, P.inv, P.z, P.bp);
 }
 
 // z_p = V-cycle result / sigma, or z_p = v_p on Dirichlet pressure rows
@@ -1437,7 +1458,8 @@ bool ortho_launch(fsi_mesh *mesh, int cnt, const T *V, int64_t ld, double *flag,
                   T *z, T *bp)
 {
     Work &W = mesh->newton->w;
-    const int64_t n = mesh->n_nodes, grid = (n + kOrthoThreads<T> - 1) / kOrthoThreads<T>;
+    const int64_t n = mesh->n_nodes, per = kOrthoThreads * kOrthoRec<T>,
+                  grid = (n + per - 1) / per;
     if (cnt > kOrthoMax || grid > kRedGrid || grid > 2 * (int64_t)sm_count()) return false;
     OrthoArgs<T> P;
     P.cnt = cnt;
@@ -1457,7 +1479,7 @@ bool ortho_launch(fsi_mesh *mesh, int cnt, const T *V, int64_t ld, double *flag,
     P.bar = W.ticket + 2;
     void *args[] = {&P};
     if (cudaLaunchCooperativeKernel((const void *)ortho_kernel<T>, dim3((unsigned)grid),
-                                    dim3(kOrthoThreads<T>), args, 0, mesh->stream) != cudaSuccess) {
+                                    dim3(kOrthoThreads), args, 0, mesh->stream) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
