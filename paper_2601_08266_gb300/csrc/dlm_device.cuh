@@ -24,6 +24,10 @@ struct GridArgs {
     int sx, sy, sz;
     long long dmax_bits[3];
     int zero_origin;  // x0_k == 0 (either sign) on every axis
+    // otherwise: 1/h_k rounded to nearest (0: out of the range that grid_coord's
+    // division needs) and the bit patterns of N_k as doubles
+    double ix, iy, iz;
+    long long nmax_bits[3];
     // exact division of an element index e < 2^31 by Nx and by Ny:
     // e / N = (e * div_m) >> div_k (see division_magic)
     unsigned long long div_mx, div_my;
@@ -71,17 +75,43 @@ inline void set_reciprocals(GridArgs &g)
     g.zero_origin = g.x0 == 0.0 && g.y0 == 0.0 && g.z0 == 0.0;
     division_magic(g.Nx, g.div_mx, g.div_kx);
     division_magic(g.Ny, g.div_my, g.div_ky);
+    double *inv[3] = {&g.ix, &g.iy, &g.iz};
+    for (int k = 0; k < 3; ++k) {
+        *inv[k] = h[k] > 0x1p-500 && h[k] < 0x1p500 ? 1.0 / h[k] : 0.0;
+        const double nmax = N[k];
+        std::memcpy(&g.nmax_bits[k], &nmax, sizeof nmax);
+    }
     g.sx = sh[0];
     g.sy = sh[1];
     g.sz = sh[2];
 }
 
-// (X - x0) / h as IEEE FP64 division, by the exact multiply when h is a
-// power of two (GB300's FP64 division is a long dependent sequence)
-__device__ __forceinline__ double grid_coord(double X, double x0, double h, double r)
+// (X - x0) / h as IEEE FP64 division.  By the exact multiply when h is a power
+// of two; else from y = 1/h rounded to nearest by two corrections of the quotient
+// with their exact remainders (P. Markstein, IBM J. Res. Dev. 34, 1990: the
+// last one rounds correctly): five FP64 operations instead of a general
+// division's dozen.  The remainders are exact while nothing underflows, so tiny
+// numerators divide.  (A zero comes out as +0.)
+__device__ __forceinline__ double grid_coord(double X, double x0, double h, double r, double y)
 {
     const double d = X - x0;
-    return r != 0.0 ? d * r : d / h;
+    if (r != 0.0) return d * r;
+    const unsigned hw = (unsigned)__double2hiint(d) & 0x7fffffffu;
+    if (y == 0.0 || (hw < (123u << 20) && (hw | (unsigned)__double2loint(d)) != 0u)) return d / h;
+    double q = d * y;
+    q = fma(fma(-h, q, d), y, q);
+    return fma(fma(-h, q, d), y, q);
+}
+
+// min(floor(t), N - 1) and 2 (t - that) - 1 for 0 <= t <= N, else false; the
+// comparisons on the bit patterns (NaN and negative values are above N's as
+// unsigned numbers; -0 is inside)
+__device__ __forceinline__ bool cell_of(double t, long long nmax_bits, int N, int &e, double &xi)
+{
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(t);
+    e = min(__double2int_rd(t), N - 1);
+    xi = fma(2.0, t - (double)e, -1.0);  // 2 (t - e) is exact
+    return bits <= (unsigned long long)nmax_bits || bits == 0x8000000000000000ull;
 }
 
 // ------------------------------------------------------------ location
@@ -212,11 +242,12 @@ __device__ __forceinline__ int locate_point(const GridArgs &g, int64_t b,
         elem[b] = e;
         return e;
     }
-    const double tx = grid_coord(X[3 * b + 0], g.x0, g.hx, g.rx);
-    const double ty = grid_coord(X[3 * b + 1], g.y0, g.hy, g.ry);
-    const double tz = grid_coord(X[3 * b + 2], g.z0, g.hz, g.rz);
-    const bool in = (tx >= 0.0 && tx <= (double)g.Nx) && (ty >= 0.0 && ty <= (double)g.Ny) &&
-                    (tz >= 0.0 && tz <= (double)g.Nz);
+    int ex, ey, ez;
+    double qx, qy, qz;
+    const bool in =
+        cell_of(grid_coord(X[3 * b + 0], g.x0, g.hx, g.rx, g.ix), g.nmax_bits[0], g.Nx, ex, qx) &
+        cell_of(grid_coord(X[3 * b + 1], g.y0, g.hy, g.ry, g.iy), g.nmax_bits[1], g.Ny, ey, qy) &
+        cell_of(grid_coord(X[3 * b + 2], g.z0, g.hz, g.rz, g.iz), g.nmax_bits[2], g.Nz, ez, qz);
     if (!in) {
         elem[b] = -1;
         xi[3 * b + 0] = S(0);
@@ -224,12 +255,9 @@ __device__ __forceinline__ int locate_point(const GridArgs &g, int64_t b,
         xi[3 * b + 2] = S(0);
         return -1;
     }
-    const int ex = min((int)floor(tx), g.Nx - 1);
-    const int ey = min((int)floor(ty), g.Ny - 1);
-    const int ez = min((int)floor(tz), g.Nz - 1);
-    xi[3 * b + 0] = (S)(2.0 * (tx - (double)ex) - 1.0);
-    xi[3 * b + 1] = (S)(2.0 * (ty - (double)ey) - 1.0);
-    xi[3 * b + 2] = (S)(2.0 * (tz - (double)ez) - 1.0);
+    xi[3 * b + 0] = (S)qx;
+    xi[3 * b + 1] = (S)qy;
+    xi[3 * b + 2] = (S)qz;
     const int e = ex + g.Nx * (ey + g.Ny * ez);
     elem[b] = e;
     return e;
