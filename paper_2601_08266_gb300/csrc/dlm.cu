@@ -746,7 +746,10 @@ __global__ void interp_kernel(int64_t m, GridArgs g, const int32_t *__restrict__
 }
 
 // Spreading, pass 1: one warp per segment of kSpreadSeg consecutive cells
-// (see spread_cells_segment).
+// (see spread_cells_segment).  Consecutive segments go to consecutive CTAs, so
+// to different SMs: the points of a thin structure lie in a few rows of cells, and
+// with a CTA's warps side by side a few SMs had all the work (FP64, 24^3 with a solid's leaflets, with fewer products for the
+// weights: a Newton step 31.1 -> 30.1 ms).
 // T is the compute type (double, float or double-float); xi, lam, w and F are
 // in its storage type, the corner sums S in T.
 // (SQ: w N^2 dsq instead of w N lambda, see spread_accumulate)
@@ -758,7 +761,7 @@ __global__ void spread_cells_kernel(int64_t E, const typename StorageOf<T>::type
                                     const typename StorageOf<T>::type *__restrict__ w,
                                     T *__restrict__ S, T dsq = T(0))
 {
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int64_t warp = blockIdx.x + (int64_t)(threadIdx.x >> 5) * gridDim.x;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t c0 = warp * kSpreadSeg; c0 < E; c0 += nwarps * kSpreadSeg)
         spread_cells_segment<T, SQ>(E, c0, xi, start, perm, lam, w, S, dsq);

@@ -440,10 +440,13 @@ __device__ __forceinline__ void interp_point(
         const T x0 = to_c<T>(xi[3 * b]), x1 = to_c<T>(xi[3 * b + 1]),
                 x2 = to_c<T>(xi[3 * b + 2]);
         const int n0 = ex + NX1 * ey + NXY1 * ez;
+        T sxy[4];  // tensor product, with the 1/8 in the x factors
+#pragma unroll
+        for (int a = 0; a < 4; ++a) sxy[a] = shape_1d(x0, a & 1) * T(0.125f) * shape_1d(x1, a >> 1);
 #pragma unroll
         for (int a = 0; a < 8; ++a) {
             const int ax = a & 1, ay = (a >> 1) & 1, az = (a >> 2) & 1;
-            const T Na = shape_1d(x0, ax) * shape_1d(x1, ay) * shape_1d(x2, az) * T(0.125f);
+            const T Na = sxy[a & 3] * shape_1d(x2, az);
             const auto v = ld4(U + n0 + ax + NX1 * ay + NXY1 * az);
             ux = madd(Na, to_c<T>(v.x), ux);
             uy = madd(Na, to_c<T>(v.y), uy);
@@ -520,11 +523,20 @@ __device__ __forceinline__ void spread_accumulate(
         l1 = to_c<T>(lam[3 * b + 1]);
         l2 = to_c<T>(lam[3 * b + 2]);
     }
+    // tensor product, with w / 8 in the x factors: 14 products instead of 20
+    T sx[2] = {shape_1d(x0, 0), shape_1d(x0, 1)};
+    if constexpr (!SQ) {
+        sx[0] = sx[0] * s;
+        sx[1] = sx[1] * s;
+    }
+    T sxy[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) sxy[a] = sx[a & 1] * shape_1d(x1, a >> 1);
 #pragma unroll
     for (int a = 0; a < 8; ++a) {
-        const T sh = shape_1d(x0, a & 1) * shape_1d(x1, (a >> 1) & 1) * shape_1d(x2, (a >> 2) & 1);
+        const T sh = sxy[a & 3] * shape_1d(x2, a >> 2);
         // N_a = sh / 8: w N_a = sh s, w N_a^2 = sh s (sh / 8)
-        const T Na = SQ ? sh * s * (sh * T(0.125f)) : sh * s;
+        const T Na = SQ ? sh * s * (sh * T(0.125f)) : sh;
         acc[3 * a] = madd(Na, l0, acc[3 * a]);
         acc[3 * a + 1] = madd(Na, l1, acc[3 * a + 1]);
         acc[3 * a + 2] = madd(Na, l2, acc[3 * a + 2]);
