@@ -54,6 +54,19 @@ __device__ __forceinline__ df64 df_split(double d)
     return df64(hi, (float)(d - (double)hi));
 }
 
+// (float)d by integer operations (round to nearest, ties to even): the FP64 unit
+// converts two values per SM and clock
+__device__ __forceinline__ float round_to_float(double d)
+{
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    const unsigned e = (hi >> 20) & 0x7ffu;
+    if (e - 897u < 254u) {  // a normal float before rounding (a carry may reach infinity, rightly)
+        const unsigned b = (hi & 0x80000000u) | ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+        return __uint_as_float(b + ((lo & 0x1fffffffu) + (b & 1u) > 0x10000000u ? 1u : 0u));
+    }
+    if (((hi << 1) | lo) == 0u) return __uint_as_float(hi);
+    return (float)d;
+}
 // s + e = a + b exactly (Knuth)
 __device__ __forceinline__ df64 df_two_sum(float a, float b)
 {

@@ -3,6 +3,7 @@
 // kernels (batch.cu).  See dlm.cu for the design.
 #pragma once
 
+#include <climits>
 #include <cmath>
 #include <cstring>
 
@@ -94,7 +95,7 @@ inline void set_reciprocals(GridArgs &g)
 // numerators divide.  (A zero comes out as +0.)
 __device__ __forceinline__ double grid_coord(double X, double x0, double h, double r, double y)
 {
-    const double d = X - x0;
+    const double d = x0 == 0.0 ? X : X - x0;
     if (r != 0.0) return d * r;
     const unsigned hw = (unsigned)__double2hiint(d) & 0x7fffffffu;
     if (y == 0.0 || (hw < (123u << 20) && (hw | (unsigned)__double2loint(d)) != 0u)) return d / h;
@@ -103,15 +104,32 @@ __device__ __forceinline__ double grid_coord(double X, double x0, double h, doub
     return fma(fma(-h, q, d), y, q);
 }
 
-// min(floor(t), N - 1) and 2 (t - that) - 1 for 0 <= t <= N, else false; the
-// comparisons on the bit patterns (NaN and negative values are above N's as
-// unsigned numbers; -0 is inside)
+// min(floor(t), N - 1) and 2 (t - that) - 1 for 0 <= t <= N, else false.  FP64
+// operations only where a value is rounded (64 instances with 5 M points, 11 an axis:
+// 296 us; 8: 260 us): the comparisons are on the bit patterns (NaN and negative
+// values are above N's as unsigned numbers; -0 is inside), floor(t) and the
+// element come from t's significand
 __device__ __forceinline__ bool cell_of(double t, long long nmax_bits, int N, int &e, double &xi)
 {
-    const unsigned long long bits = (unsigned long long)__double_as_longlong(t);
-    e = min(__double2int_rd(t), N - 1);
-    xi = fma(2.0, t - (double)e, -1.0);  // 2 (t - e) is exact
-    return bits <= (unsigned long long)nmax_bits || bits == 0x8000000000000000ull;
+    const long long bits = __double_as_longlong(t);
+    const int u = (int)((bits >> 52) & 0x7ff) - 1023;  // t = 1.f 2^u
+    const bool in = (unsigned long long)bits <= (unsigned long long)nmax_bits || bits == LLONG_MIN;
+    const int sh = 52 - (u < 0 ? 0 : (u > 30 ? 30 : u));
+    const long long sig = (bits & 0xfffffffffffffLL) | 0x10000000000000LL;
+    e = u < 0 ? 0 : (int)(sig >> sh);
+    const double fl = u < 0 ? 0.0 : __longlong_as_double(bits & ~((1LL << sh) - 1));
+    xi = fma(2.0, t - fl, -1.0);  // 2 (t - floor) is exact
+    if (e == N) {                 // t = N, in the last cell
+        e = N - 1;
+        xi = 1.0;
+    }
+    return in;
+}
+
+template <typename S> __device__ __forceinline__ S round_to(double d)
+{
+    if constexpr (sizeof(S) == 4) return round_to_float(d);
+    else return d;
 }
 
 // ------------------------------------------------------------ location
@@ -235,9 +253,9 @@ __device__ __forceinline__ int locate_point(const GridArgs &g, int64_t b,
             xi[3 * b + 2] = S(0);
             return -1;
         }
-        xi[3 * b + 0] = (S)qx;
-        xi[3 * b + 1] = (S)qy;
-        xi[3 * b + 2] = (S)qz;
+        xi[3 * b + 0] = round_to<S>(qx);
+        xi[3 * b + 1] = round_to<S>(qy);
+        xi[3 * b + 2] = round_to<S>(qz);
         const int e = ex + g.Nx * (ey + g.Ny * ez);
         elem[b] = e;
         return e;
@@ -255,9 +273,9 @@ __device__ __forceinline__ int locate_point(const GridArgs &g, int64_t b,
         xi[3 * b + 2] = S(0);
         return -1;
     }
-    xi[3 * b + 0] = (S)qx;
-    xi[3 * b + 1] = (S)qy;
-    xi[3 * b + 2] = (S)qz;
+    xi[3 * b + 0] = round_to<S>(qx);
+    xi[3 * b + 1] = round_to<S>(qy);
+    xi[3 * b + 2] = round_to<S>(qz);
     const int e = ex + g.Nx * (ey + g.Ny * ez);
     elem[b] = e;
     return e;

@@ -44,6 +44,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include "df64.cuh"
 #include "fsi_internal.cuh"
 #include "tc_common.cuh"
 
@@ -103,20 +104,6 @@ __global__ void pack_weights_kernel(const float *P, uint8_t *packed)
         }
         *reinterpret_cast<__nv_bfloat16 *>(packed + off) = v;
     }
-}
-
-// (float)d by integer operations (round to nearest, ties to even): the FP64
-// unit converts two values per SM and clock, and a tile has 14,336
-__device__ __forceinline__ float to_float(double d)
-{
-    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
-    const unsigned e = (hi >> 20) & 0x7ffu;
-    if (e - 897u < 254u) {  // a normal float before rounding (a carry may reach infinity, rightly)
-        const unsigned b = (hi & 0x80000000u) | ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
-        return __uint_as_float(b + ((lo & 0x1fffffffu) + (b & 1u) > 0x10000000u ? 1u : 0u));
-    }
-    if (((hi << 1) | lo) == 0u) return __uint_as_float(hi);
-    return (float)d;
 }
 
 struct TcArgs {
@@ -252,10 +239,10 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_predict_tc_kernel(const TcArg
                 const int f = c < c1 ? 8 * c + 4 * h : 0;
                 const float4 mn = *reinterpret_cast<const float4 *>(smean + f);
                 const float4 is = *reinterpret_cast<const float4 *>(sistd + f);
-                f8[4 * h] = (to_float(raw[u][h][0]) - mn.x) * is.x;
-                f8[4 * h + 1] = (to_float(raw[u][h][1]) - mn.y) * is.y;
-                f8[4 * h + 2] = (to_float(raw[u][h][2]) - mn.z) * is.z;
-                f8[4 * h + 3] = (to_float(raw[u][h][3]) - mn.w) * is.w;
+                f8[4 * h] = (round_to_float(raw[u][h][0]) - mn.x) * is.x;
+                f8[4 * h + 1] = (round_to_float(raw[u][h][1]) - mn.y) * is.y;
+                f8[4 * h + 2] = (round_to_float(raw[u][h][2]) - mn.z) * is.z;
+                f8[4 * h + 3] = (round_to_float(raw[u][h][3]) - mn.w) * is.w;
             }
             if (!live)
 #pragma unroll
