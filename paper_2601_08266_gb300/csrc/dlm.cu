@@ -746,13 +746,15 @@ __global__ void interp_kernel(int64_t m, GridArgs g, const int32_t *__restrict__
 }
 
 // Spreading, pass 1: one warp per segment of kSpreadSeg consecutive cells
-// (see spread_cells_segment).  Consecutive segments go to consecutive CTAs, so
-// to different SMs: the points of a thin structure lie in a few rows of cells, and
-// with a CTA's warps side by side a few SMs had all the work (FP64, 24^3 with a solid's leaflets, with fewer products for the
-// weights: a Newton step 31.1 -> 30.1 ms).
+// (see spread_cells_segment).  CTAs of few warps: the points of a thin structure lie
+// in a few rows of cells, which one large CTA's warps would have to themselves on one
+// SM (FP64, 24^3 with a solid's leaflets, CTAs of 256 -> 64 threads: a Newton step
+// 30.26 -> 29.60 ms, 64^3 with 200 k points 1,708 -> 1,684 us; FP32 at 128^3 gains 2 us
+// with 128 threads and loses 8 with 32).
 // T is the compute type (double, float or double-float); xi, lam, w and F are
 // in its storage type, the corner sums S in T.
 // (SQ: w N^2 dsq instead of w N lambda, see spread_accumulate)
+template <typename T> constexpr int kSpreadThreads = sizeof(T) == 4 ? 128 : 64;
 template <typename T, bool SQ = false>
 __global__ void spread_cells_kernel(int64_t E, const typename StorageOf<T>::type *__restrict__ xi,
                                     const int32_t *__restrict__ start,
@@ -761,7 +763,7 @@ __global__ void spread_cells_kernel(int64_t E, const typename StorageOf<T>::type
                                     const typename StorageOf<T>::type *__restrict__ w,
                                     T *__restrict__ S, T dsq = T(0))
 {
-    const int64_t warp = blockIdx.x + (int64_t)(threadIdx.x >> 5) * gridDim.x;
+    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t c0 = warp * kSpreadSeg; c0 < E; c0 += nwarps * kSpreadSeg)
         spread_cells_segment<T, SQ>(E, c0, xi, start, perm, lam, w, S, dsq);
@@ -930,8 +932,8 @@ fsi_status spread_mass_diag(fsi_mesh *mesh, int64_t m, const T *xi, const int32_
     const GridArgs g = grid_args(mesh);
     const int64_t E = mesh->n_elems;
     FSI_TRY(ensure_spread_scratch(mesh, (size_t)E * 24 * sizeof(T)));
-    const int cgrid = blocks_for((E + kSpreadSeg - 1) / kSpreadSeg * 32, 256, sm_count() * 64);
-    spread_cells_kernel<T, true><<<cgrid, 256, 0, mesh->stream>>>(
+    const int cgrid = blocks_for((E + kSpreadSeg - 1) / kSpreadSeg * 32, kSpreadThreads<T>, sm_count() * 256);
+    spread_cells_kernel<T, true><<<cgrid, kSpreadThreads<T>, 0, mesh->stream>>>(
         E, xi, cell_start, perm, nullptr, w, (T *)mesh->spread_scratch, (T)dsq);
     FSI_TRY(check_launch("spread cells kernel"));
     const dim3 nblock(32, 8), ngrid = node_grid(g);
@@ -1266,27 +1268,29 @@ fsi_status fsi_dlm_spread(fsi_mesh *mesh, fsi_prec prec, int64_t m, const int32_
     const size_t esz = prec == FSI_F32 ? sizeof(float) : sizeof(double);
     FSI_TRY(ensure_spread_scratch(mesh, (size_t)mesh->n_elems * 24 * esz));
     const int64_t E = mesh->n_elems;
-    const int cgrid = blocks_for((E + kSpreadSeg - 1) / kSpreadSeg * 32, 256, sm_count() * 64);
+    auto cgrid = [&](int threads) {
+        return blocks_for((E + kSpreadSeg - 1) / kSpreadSeg * 32, threads, sm_count() * 256);
+    };
     // nodes: 32 x 8 threads per CTA over (i, j), one grid layer per k
     const dim3 nblock(32, 8), ngrid = node_grid(g);
     if ((g.Ny + 8) / 8 > 65535)
         return set_error(FSI_ERR_ARG, "fsi_dlm_spread: more than 524,280 nodes along y");
     if (prec == FSI_F64) {
-        spread_cells_kernel<double><<<cgrid, 256, 0, mesh->stream>>>(
+        spread_cells_kernel<double><<<cgrid(kSpreadThreads<double>), kSpreadThreads<double>, 0, mesh->stream>>>(
             E, (const double *)xi, cell_start, perm, (const double *)lam, (const double *)w,
             (double *)mesh->spread_scratch);
         FSI_TRY(check_launch("spread cells kernel"));
         spread_nodes_kernel<double><<<ngrid, nblock, 0, mesh->stream>>>(
             g, cell_start, (const double *)mesh->spread_scratch, (double *)F, accumulate);
     } else if (prec == FSI_DF64) {
-        spread_cells_kernel<df64><<<cgrid, 256, 0, mesh->stream>>>(
+        spread_cells_kernel<df64><<<cgrid(kSpreadThreads<df64>), kSpreadThreads<df64>, 0, mesh->stream>>>(
             E, (const double *)xi, cell_start, perm, (const double *)lam, (const double *)w,
             (df64 *)mesh->spread_scratch);
         FSI_TRY(check_launch("spread cells kernel"));
         spread_nodes_kernel<df64><<<ngrid, nblock, 0, mesh->stream>>>(
             g, cell_start, (const df64 *)mesh->spread_scratch, (double *)F, accumulate);
     } else {
-        spread_cells_kernel<float><<<cgrid, 256, 0, mesh->stream>>>(
+        spread_cells_kernel<float><<<cgrid(kSpreadThreads<float>), kSpreadThreads<float>, 0, mesh->stream>>>(
             E, (const float *)xi, cell_start, perm, (const float *)lam, (const float *)w,
             (float *)mesh->spread_scratch);
         FSI_TRY(check_launch("spread cells kernel"));

@@ -1011,8 +1011,7 @@ __global__ void tet_spread_cells_kernel(int64_t E, const S *__restrict__ lam,
                                         T *__restrict__ Ssum)
 {
     const int lane = threadIdx.x & 31;
-    // (neighbouring groups of elements on different SMs, as in the hexahedral kernel)
-    const int64_t warp = blockIdx.x + (int64_t)(threadIdx.x >> 5) * gridDim.x;
+    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t e0 = warp * 8; e0 < E; e0 += nwarps * 8) {
         const int64_t e = e0 + (lane >> 2);
