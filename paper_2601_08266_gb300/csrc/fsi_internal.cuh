@@ -227,7 +227,7 @@ fsi_status mlp_predict_tc(cudaStream_t s, int device, const fsi_grid &g, int64_t
                           const float *params, const float *in_mean, const float *in_std,
                           const float *out_mean, const float *out_std, const double *Vn,
                           const double *y, const double *d1, const double *d2, double *y0,
-                          void *packed, int *dev_err);
+                          void *packed, void *feat, int *dev_err);
 
 // the coupled Jacobian (newton.cu) at st->y applied to k FP32 vectors after
 // one linearisation; used by the learned guess's fitted predictor

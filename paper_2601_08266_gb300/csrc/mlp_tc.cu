@@ -9,8 +9,8 @@
 // between.  Per tile:
 //
 //   features   the 112 features of each node (27-node stencil of V_n
-//              velocity and y_n pressure, the extrapolant 2 d1 - d2),
-//              normalised and rounded to BF16, into the A tile X [128 x 112].
+//              velocity and y_n pressure, in FP32 from
+//              node_features_kernel; the extrapolant 2 d1 - d2), normalised and rounded to BF16, into the A tile X [128 x 112].
 //              They are gathered one tile ahead, during the previous tile's
 //              MMAs and epilogues, and wait packed in 16 registers per thread
 //              (shared memory has no room for a second A tile);
@@ -27,10 +27,13 @@
 //              fixed order; the predictor y0 = y + e + (out_mean + out_std *
 //              out) is written in FP64, one component per thread.
 //
-// Bound: the phases of a tile follow one another, so their latencies add up.  The
-// gather with its FP64 -> FP32 conversions (two per SM and clock on GB300's FP64
-// unit, so they are done on the integer pipe) was the longest: gathered a tile
-// ahead, 2,146,689 nodes (129^3) take 1.12 ms instead of 1.29 ms.
+// Bound: the phases of a tile follow one another, so their latencies and instructions
+// add up.  2,146,689 nodes (129^3): 1.29 ms with every row converting its 27 nodes on
+// the FP64 unit when it needs them; 1.12 ms gathered a tile ahead and converted on the
+// integer pipe; 0.75 ms with each node converted once (node_features_kernel, 25 us
+// of that) and no FP64 operation left in a tile but the four of the result (the unit
+// does two per SM and clock: 25 a thread took 3 of a tile's 9 us), layer 3 on
+// paired FMAs with its biases read four at a time.
 //
 // The BF16 rounding points are those of the training kernels (inputs and
 // weights of every layer).  Weights are packed once per call into the
@@ -40,6 +43,7 @@
 // asynchronous copies.  Every wait is bounded: a wait that runs out sets an
 // error flag that the host reads, the CTA stops issuing work, waits (bounded)
 // for what it issued, frees its TMEM and returns.
+#include <algorithm>
 #include <atomic>
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -112,10 +116,45 @@ struct TcArgs {
     const float *P;  // FP32 parameters (biases, W3)
     const uint8_t *packed;
     const float *in_mean, *in_std, *out_mean, *out_std;
-    const double *Vn, *y, *d1, *d2;
+    const float4 *feat;  // (V_n, p_n) of every node in FP32
+    const double *y, *d1, *d2;
     double *y0;
     int *err;
 };
+
+// The stencil's inputs in FP32, each node converted once instead of by each of the
+// 27 rows that use it
+__global__ void __launch_bounds__(256) node_features_kernel(int64_t n, const double *__restrict__ Vn,
+                                                            const double *__restrict__ y,
+                                                            float4 *__restrict__ feat)
+{
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n;
+         q += (int64_t)gridDim.x * blockDim.x) {
+        const double2 v01 = __ldg(reinterpret_cast<const double2 *>(Vn + 4 * q));
+        feat[q] = make_float4(round_to_float(v01.x), round_to_float(v01.y),
+                              round_to_float(__ldg(Vn + 4 * q + 2)), round_to_float(__ldg(y + 4 * q + 3)));
+    }
+}
+
+// 2 d1 - d2 in FP32 (volatile: one warp in four wants it, and the FP64 unit would do it
+// for all)
+__device__ __forceinline__ float extrapolant(double d1, double d2)
+{
+    double d;
+    asm volatile("fma.rn.f64 %0, %1, %2, %3;" : "=d"(d) : "d"(d1), "d"(2.0), "d"(-d2));
+    return round_to_float(d);
+}
+
+// (double)f by integer operations
+__device__ __forceinline__ double widen(float f)
+{
+    const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+    double d;
+    asm volatile("cvt.f64.f32 %0, %1;" : "=d"(d) : "f"(f));
+    return d;
+}
 
 __global__ void __launch_bounds__(kThreads, 1) mlp_predict_tc_kernel(const TcArgs a)
 {
@@ -192,7 +231,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_predict_tc_kernel(const TcArg
     // issues a half's loads, convert() normalises them in FP32 ((value - mean) *
     // (1 / std): the result is rounded to BF16 right away) and packs them.
     const int c0 = kChunk[grp], c1 = kChunk[grp + 1];
-    double raw[2][2][4];
+    float4 raw[2][2];
+    double ex1[4], ex2[4];  // d1 and d2 of the extrapolant (the last stencil place, group 3)
     uint4 xf[4];
     auto gather = [&](int64_t tile, int half) {
         const int64_t node = tile * TM + row;
@@ -206,24 +246,19 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_predict_tc_kernel(const TcArg
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int s = 2 * c + h;
-#pragma unroll
-                for (int t = 0; t < 4; ++t) raw[u][h][t] = 0.0;
+                raw[u][h] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (c >= c1 || !live) continue;
                 if (s < 27) {
                     const int dz = s / 9, dy = (s - 9 * dz) / 3, dx = s - 9 * dz - 3 * dy;
                     const int ii = i + dx - 1, jj = j + dy - 1, kk = k + dz - 1;
-                    if (ii >= 0 && ii < nx && jj >= 0 && jj < ny && kk >= 0 && kk < nz) {
-                        const int64_t nb = ii + (int64_t)nx * (jj + (int64_t)ny * kk);
-                        const double2 v01 = __ldg(reinterpret_cast<const double2 *>(a.Vn + 4 * nb));
-                        raw[u][h][0] = v01.x;
-                        raw[u][h][1] = v01.y;
-                        raw[u][h][2] = __ldg(a.Vn + 4 * nb + 2);
-                        raw[u][h][3] = __ldg(a.y + 4 * nb + 3);
-                    }
-                } else {  // features 108..111: the extrapolant 2 d1 - d2
+                    if ((unsigned)ii < (unsigned)nx && (unsigned)jj < (unsigned)ny && (unsigned)kk < (unsigned)nz)
+                        raw[u][h] = __ldg(a.feat + ((int64_t)(kk * ny + jj) * nx + ii));
+                } else {
 #pragma unroll
-                    for (int t = 0; t < 4; ++t)
-                        raw[u][h][t] = 2.0 * __ldg(a.d1 + 4 * node + t) - __ldg(a.d2 + 4 * node + t);
+                    for (int t = 0; t < 4; ++t) {
+                        ex1[t] = __ldg(a.d1 + 4 * node + t);
+                        ex2[t] = __ldg(a.d2 + 4 * node + t);
+                    }
                 }
             }
         }
@@ -239,10 +274,15 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_predict_tc_kernel(const TcArg
                 const int f = c < c1 ? 8 * c + 4 * h : 0;
                 const float4 mn = *reinterpret_cast<const float4 *>(smean + f);
                 const float4 is = *reinterpret_cast<const float4 *>(sistd + f);
-                f8[4 * h] = (round_to_float(raw[u][h][0]) - mn.x) * is.x;
-                f8[4 * h + 1] = (round_to_float(raw[u][h][1]) - mn.y) * is.y;
-                f8[4 * h + 2] = (round_to_float(raw[u][h][2]) - mn.z) * is.z;
-                f8[4 * h + 3] = (round_to_float(raw[u][h][3]) - mn.w) * is.w;
+                float4 v = raw[u][h];
+                // features 108..111: the extrapolant 2 d1 - d2 (group 3's chunk 13)
+                if (half == 1 && u == 0 && h == 1 && c == 13 && live)
+                    v = make_float4(extrapolant(ex1[0], ex2[0]), extrapolant(ex1[1], ex2[1]),
+                                    extrapolant(ex1[2], ex2[2]), extrapolant(ex1[3], ex2[3]));
+                f8[4 * h] = (v.x - mn.x) * is.x;
+                f8[4 * h + 1] = (v.y - mn.y) * is.y;
+                f8[4 * h + 2] = (v.z - mn.z) * is.z;
+                f8[4 * h + 3] = (v.w - mn.w) * is.w;
             }
             if (!live)
 #pragma unroll
@@ -318,6 +358,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_predict_tc_kernel(const TcArg
                          sdesc(s0 + OFF_SW2A + ks * 256, 128, KC2 * 128), ks > 0);
             mma_commit(bar_m);
         }
+        const double p_base = p_y + (2.0 * p_d1 - p_d2);
         convert(next, 0);
         gather(next, 1);
         // second K-half of H1 (group g: columns 128 + 32 g ..) into registers
@@ -327,10 +368,10 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_predict_tc_kernel(const TcArg
             float v[32];
             tmem_ld32(tmem + lane_base + 128 + 32 * grp, v);
 #pragma unroll
-            for (int t = 0; t < 16; ++t) {
-                const int col = 128 + 32 * grp + 2 * t;
-                hp[t] = pack_bf16(fmaxf(v[2 * t] + sb1[col], 0.0f),
-                                  fmaxf(v[2 * t + 1] + sb1[col + 1], 0.0f));
+            for (int t = 0; t < 16; t += 2) {
+                const float4 b = *reinterpret_cast<const float4 *>(sb1 + 128 + 32 * grp + 2 * t);
+                hp[t] = pack_bf16(fmaxf(v[2 * t] + b.x, 0.0f), fmaxf(v[2 * t + 1] + b.y, 0.0f));
+                hp[t + 1] = pack_bf16(fmaxf(v[2 * t + 2] + b.z, 0.0f), fmaxf(v[2 * t + 3] + b.w, 0.0f));
             }
         }
         mma_pending = true;
@@ -372,24 +413,28 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_predict_tc_kernel(const TcArg
         // ---- layer 3: group g sums D2 columns 64 g .. 64 g + 63; groups 1..3
         // leave their partial sums in the X buffer (free now), group 0 adds
         // them in group order and writes the predictor
-        float o[4] = {0.f, 0.f, 0.f, 0.f};
+        float2 o01 = make_float2(0.f, 0.f), o23 = o01;
 #pragma unroll 1
         for (int c = 0; c < 2; ++c) {
             float v[32];
-            tmem_ld32(tmem + lane_base + NH + 64 * grp + 32 * c, v);
+            const int col = 64 * grp + 32 * c;
+            tmem_ld32(tmem + lane_base + NH + col, v);
 #pragma unroll
-            for (int t = 0; t < 32; ++t) {
-                const int col = 64 * grp + 32 * c + t;
-                const float h = bf16r(fmaxf(v[t] + sb2[col], 0.0f));
-                const float4 w = sW3[col];
-                o[0] = fmaf(h, w.x, o[0]);
-                o[1] = fmaf(h, w.y, o[1]);
-                o[2] = fmaf(h, w.z, o[2]);
-                o[3] = fmaf(h, w.w, o[3]);
+            for (int t = 0; t < 32; t += 4) {
+                const float4 b = *reinterpret_cast<const float4 *>(sb2 + col + t);
+                const uint32_t p[2] = {pack_bf16(fmaxf(v[t] + b.x, 0.0f), fmaxf(v[t + 1] + b.y, 0.0f)),
+                                       pack_bf16(fmaxf(v[t + 2] + b.z, 0.0f), fmaxf(v[t + 3] + b.w, 0.0f))};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float h = __uint_as_float(q & 1 ? p[q >> 1] & 0xffff0000u : p[q >> 1] << 16);
+                    const float4 w = sW3[col + t + q];
+                    o01 = __ffma2_rn(make_float2(h, h), make_float2(w.x, w.y), o01);
+                    o23 = __ffma2_rn(make_float2(h, h), make_float2(w.z, w.w), o23);
+                }
             }
         }
         float4 *part = reinterpret_cast<float4 *>(xh);
-        part[grp * TM + row] = make_float4(o[0], o[1], o[2], o[3]);
+        part[grp * TM + row] = make_float4(o01.x, o01.y, o23.x, o23.y);
         __syncthreads();
         {
             // component tid % 4 of row tid / 4: the groups' sums in group order
@@ -398,7 +443,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_predict_tc_kernel(const TcArg
 #pragma unroll
             for (int g = 1; g < kGroups; ++g) out += pp[4 * g * TM];
             out += b3;
-            if (plive) a.y0[pq] = p_y + (2.0 * p_d1 - p_d2) + (om + os * (double)out);
+            if (plive) a.y0[pq] = p_base + (om + os * widen(out));
         }
         // the next tile overwrites X (read by the finished MMAs and above) and D1
         fence_before();
@@ -443,7 +488,7 @@ fsi_status mlp_predict_tc(cudaStream_t s, int device, const fsi_grid &g, int64_t
                           const float *params, const float *in_mean, const float *in_std,
                           const float *out_mean, const float *out_std, const double *Vn,
                           const double *y, const double *d1, const double *d2, double *y0,
-                          void *packed, int *dev_err)
+                          void *packed, void *feat, int *dev_err)
 {
     if (n <= 0) return FSI_OK;
     // the attribute is per device; setting it twice (two threads racing on
@@ -458,8 +503,10 @@ fsi_status mlp_predict_tc(cudaStream_t s, int device, const fsi_grid &g, int64_t
     const int sms = sm_count();
     pack_weights_kernel<<<sm_count() * 4, 256, 0, s>>>(params, (uint8_t *)packed);
     FSI_TRY(check_launch("pack weights"));
+    node_features_kernel<<<(int)std::min<int64_t>((n + 255) / 256, 16 * sms), 256, 0, s>>>(n, Vn, y, (float4 *)feat);
+    FSI_TRY(check_launch("node features"));
     TcArgs a{g.N[0], g.N[1], g.N[2], n, params, (const uint8_t *)packed, in_mean, in_std,
-             out_mean, out_std, Vn, y, d1, d2, y0, dev_err};
+             out_mean, out_std, (const float4 *)feat, y, d1, d2, y0, dev_err};
     const int64_t tiles = (n + TM - 1) / TM;
     const int grid = (int)(tiles < sms ? tiles : sms);
     mlp_predict_tc_kernel<<<grid, kThreads, SMEM_BYTES, s>>>(a);
