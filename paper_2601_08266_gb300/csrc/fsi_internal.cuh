@@ -55,6 +55,40 @@ int sm_count();
 // device (once per kernel and device; thread-safe).
 fsi_status set_smem_limit(const void *kernel, int bytes);
 
+// ---------------------------------------------------------------- chained launches
+// A chain of short kernels spends much of its time between them.  A kernel launched by
+// launch_chain may start while the one before it in the stream runs out: its CTAs
+// take their places and do what needs no memory, and chain_wait() holds them until
+// the earlier kernels have finished and their results are visible.  Such a kernel calls
+// chain_wait() before its first access to global memory and passes it the pointers
+// that it reads and writes through, so that no access can be moved before it (loads
+// through read-only pointers otherwise might), and it reads what a kernel of the
+// chain may have written with __ldcg: two kernels back may still fill this SM's L1 with
+// lines from before that write.  Launched without the attribute, or
+// behind a kernel that does not chain, it waits for all of that kernel.
+template <typename P> __device__ __forceinline__ void chain_pin(P &p) { asm volatile("" : "+l"(p)); }
+template <typename... P> __device__ __forceinline__ void chain_wait(P &...p)
+{
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    (chain_pin(p), ...);
+}
+template <typename... P, typename... A>
+inline void launch_chain(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...a)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(a)...);
+}
+
 // ---------------------------------------------------------------- 4-vectors
 // 16/32-byte aligned node records so that one node is one vector load.
 template <typename T> struct alignas(4 * sizeof(T)) vec4 {

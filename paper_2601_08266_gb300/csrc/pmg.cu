@@ -274,8 +274,8 @@ __global__ void __launch_bounds__(32 * kMarchWarps) march_kernel(LevelArgs<T> L,
 #pragma unroll
         for (int r = 0; r < R + 2; ++r) {
             const bool g = inz && in[r];
-            if constexpr (VX != kVd) w.x[r] = g ? __ldg((VX == kVb ? M.b : M.x) + q + (int64_t)L.NX1 * r) : T(0);
-            if constexpr (VX == kVd || VX == kVxd) w.d[r] = g ? __ldg(M.d + q + (int64_t)L.NX1 * r) : T(0);
+            if constexpr (VX != kVd) w.x[r] = g ? __ldcg((VX == kVb ? M.b : M.x) + q + (int64_t)L.NX1 * r) : T(0);
+            if constexpr (VX == kVd || VX == kVxd) w.d[r] = g ? __ldcg(M.d + q + (int64_t)L.NX1 * r) : T(0);
         }
     };
     // v from a loaded plane's row
@@ -292,6 +292,7 @@ __global__ void __launch_bounds__(32 * kMarchWarps) march_kernel(LevelArgs<T> L,
 #pragma unroll
     for (int r = 0; r < R; ++r) acc[r] = PBk[r] = vk[r] = dk[r] = bk[r] = T(0);
     Raw nx;
+    chain_wait(M.x, M.d, M.b, M.y, M.x_next, M.d_next, M.x_final, M.z4, M.v4, M.m4);
     load(k0 - 1, nx);
     for (int kk = k0 - 1; kk <= k1; ++kk) {
         const Raw w = nx;
@@ -306,7 +307,7 @@ __global__ void __launch_bounds__(32 * kMarchWarps) march_kernel(LevelArgs<T> L,
             bn[r] = T(0);
             if constexpr (VX == kVb) bn[r] = w.x[r + 1];
             else if (M.b && mine && in[r + 1])
-                bn[r] = __ldg(M.b + off + plane_n * kk + (int64_t)L.NX1 * (r + 1));
+                bn[r] = __ldcg(M.b + off + plane_n * kk + (int64_t)L.NX1 * (r + 1));
         }
         T v[R + 2], X[R + 2];
 #pragma unroll
@@ -339,7 +340,7 @@ __global__ void __launch_bounds__(32 * kMarchWarps) march_kernel(LevelArgs<T> L,
                 } else {
                     const T dn = M.c1 * dk[r] + M.c2 * ((bk[r] - Av) * inv_D);
                     if (M.z4) {
-                        M.z4[4 * node + 3] = (M.m4 && M.m4[4 * node + 3]) ? M.v4[4 * node + 3]
+                        M.z4[4 * node + 3] = (M.m4 && M.m4[4 * node + 3]) ? __ldcg(M.v4 + 4 * node + 3)
                                                                          : (vk[r] + dn) * M.inv_sigma;
                     } else if (M.x_final) {
                         M.x_final[node] = vk[r] + dn;
@@ -369,7 +370,7 @@ fsi_status march_rows(const PressureMG &P, int l, cudaStream_t s, March<T> M)
     M.kz = (int)std::max<int64_t>(1, std::min<int64_t>(16, (int64_t)nz1 * gx * gy / (12 * sm_count())));
     const dim3 grid((unsigned)gx, (unsigned)((gy + kMarchWarps - 1) / kMarchWarps),
                     (unsigned)((nz1 + M.kz - 1) / M.kz));
-    march_kernel<T, MODE, VX, R><<<grid, dim3(32, kMarchWarps), 0, s>>>(level_args<T>(P, l), M);
+    launch_chain(march_kernel<T, MODE, VX, R>, grid, dim3(32, kMarchWarps), 0, s, level_args<T>(P, l), M);
     return check_launch("pressure stencil");
 }
 // Rows per warp: more rows share their neighbours' loads, fewer give short vectors
@@ -430,11 +431,13 @@ __global__ void restrict_kernel(LevelArgs<T> F, LevelArgs<T> C, int kz, const T 
     auto plane = [&](int k) {
         if (k < 0 || k >= F.NZ1) return T(0);
         const T *q = r + off + plane_n * k;
-        const T a = q[0] + wl * q[-xl] + wr * q[xr];
-        const T b = q[-yl] + wl * q[-yl - xl] + wr * q[xr - yl];
-        const T c = q[yr] + wl * q[yr - xl] + wr * q[yr + xr];
+        auto at = [&](int o) { return __ldcg(q + o); };
+        const T a = at(0) + wl * at(-xl) + wr * at(xr);
+        const T b = at(-yl) + wl * at(-yl - xl) + wr * at(xr - yl);
+        const T c = at(yr) + wl * at(yr - xl) + wr * at(yr + xr);
         return a + vl * b + vr * c;
     };
+    chain_wait(r, bc);
     T below = plane(2 * K0 - 1);
 #pragma unroll 2
     for (int K = K0; K < K1; ++K) {
@@ -463,15 +466,16 @@ __global__ void prolong_kernel(LevelArgs<T> F, LevelArgs<T> C, int kz, const T *
     T *f = x + i + (int64_t)F.NX1 * j;
     auto plane = [&](int K) {
         const T *q = c + plane_c * K;
-        return T(0.25) * ((q[0] + q[dx]) + (q[dy] + q[dy + dx]));
+        return T(0.25) * ((__ldcg(q) + __ldcg(q + dx)) + (__ldcg(q + dy) + __ldcg(q + dy + dx)));
     };
+    chain_wait(c, f);
     T at = plane(K0);
 #pragma unroll 2
     for (int K = K0; K < K1; ++K) {
-        f[plane_n * (2 * K)] += at;
+        f[plane_n * (2 * K)] = __ldcg(f + plane_n * (2 * K)) + at;
         if (2 * K + 1 < F.NZ1) {
             const T above = plane(K + 1);
-            f[plane_n * (2 * K + 1)] += T(0.5) * (at + above);
+            f[plane_n * (2 * K + 1)] = __ldcg(f + plane_n * (2 * K + 1)) + T(0.5) * (at + above);
             at = above;
         }
     }
@@ -817,15 +821,19 @@ __global__ void __launch_bounds__(kCoarseThreads, 1) coarse_cycle_kernel(const _
             if (k == s1 - 1 && s1 < NZ) *cl.map_shared_rank(at, rank + 1) = val;
         }
     };
-    // the dense inverse on its way (see off_inv)
-    if (rank == 0 && C.off_inv)
-        for (int q = tid; q < C.nd * C.nd; q += kCoarseThreads)
-            __pipeline_memcpy_async(cs + C.off_inv + q, C.inv + q, 4);
-    __pipeline_commit();
     for (int q = C.pads0 + tid; q < C.pads1; q += kCoarseThreads) cs[q] = 0.f;
     CoarseNode N;
     N.q = -1;
-    coarse_nodes(C.lev[0], s0, s1, N, [&](const CoarseNode &N) { cs[C.lev[0].b + N.q] = __ldg(C.b + N.q); });
+    coarse_nodes(C.lev[0], s0, s1, N, [&](const CoarseNode &) {});  // the weights
+    const float *gb = C.b, *ginv = C.inv;
+    float *gx = C.x;
+    chain_wait(gb, ginv, gx);
+    // the dense inverse on its way (see off_inv)
+    if (rank == 0 && C.off_inv)
+        for (int q = tid; q < C.nd * C.nd; q += kCoarseThreads)
+            __pipeline_memcpy_async(cs + C.off_inv + q, ginv + q, 4);
+    __pipeline_commit();
+    coarse_nodes(C.lev[0], s0, s1, N, [&](const CoarseNode &N) { cs[C.lev[0].b + N.q] = __ldcg(gb + N.q); });
     sync(true);
     // down: pre-smoothing from zero into t, residual into v, its restriction
     for (int l = 0; l < C.nlev; ++l) {
@@ -877,7 +885,7 @@ __global__ void __launch_bounds__(kCoarseThreads, 1) coarse_cycle_kernel(const _
     if (rank == 0) {
         const float *b = cs + C.off_d;
         float *x = cs + C.off_d + C.nd;
-        const float *inv = C.off_inv ? cs + C.off_inv : C.inv;
+        const float *inv = C.off_inv ? cs + C.off_inv : ginv;
         __pipeline_wait_prior(0);
         __syncthreads();
         for (int r0 = 0; r0 < C.nd; r0 += kCoarseThreads / 8) {
@@ -936,7 +944,7 @@ __global__ void __launch_bounds__(kCoarseThreads, 1) coarse_cycle_kernel(const _
         sync(split);
         coarse_nodes(L, z0, z1, N, [&](const CoarseNode &N) {
             const float y = v[N.p] + (L.c1 * e[N.q] + L.c2 * ((b[N.q] - coarse_row(L, N, v)) * N.iD));
-            if (l == 0) C.x[N.q] = y;
+            if (l == 0) gx[N.q] = y;
             else t[N.p] = y;
         });
         __syncthreads();
@@ -1012,12 +1020,14 @@ fsi_status coarse_cycle(fsi_mesh *m, int l0, const float *b, float *x)
     cfg.blockDim.x = kCoarseThreads;
     cfg.dynamicSmemBytes = bytes;
     cfg.stream = m->stream;
-    cudaLaunchAttribute at = {};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = cfg.gridDim.x;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cfg.gridDim.x;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_chain
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
     FSI_CUDA(cudaLaunchKernelEx(&cfg, coarse_cycle_kernel, C), "pressure coarse levels");
     return check_launch("pressure coarse levels");
 }
@@ -1055,11 +1065,11 @@ fsi_status vcycle_level(fsi_mesh *m, int l, const T *b, T *x, const SchurOut<T> 
     int kz = 1;
     FSI_TRY(level_apply<T>(P, l, m->stream, t, b, vec<T>(L.r)));
     const dim3 gr = transfer_grid(Lc, Lc, kz);
-    restrict_kernel<T><<<gr, kRowBlock, 0, m->stream>>>(A, Ac, kz, vec<T>(L.r), vec<T>(Lc.b));
+    launch_chain(restrict_kernel<T>, gr, kRowBlock, 0, m->stream, A, Ac, kz, vec<T>(L.r), vec<T>(Lc.b));
     FSI_TRY(check_launch("pressure restrict"));
     FSI_TRY(vcycle_level<T>(m, l + 1, vec<T>(Lc.b), vec<T>(Lc.x)));
     const dim3 gp = transfer_grid(L, Lc, kz);
-    prolong_kernel<T><<<gp, kRowBlock, 0, m->stream>>>(A, Ac, kz, vec<T>(Lc.x), t);
+    launch_chain(prolong_kernel<T>, gp, kRowBlock, 0, m->stream, A, Ac, kz, vec<T>(Lc.x), t);
     FSI_TRY(check_launch("pressure prolong"));
     return chebyshev<T>(m, l, kPmgNu, hi / 4.0, hi, b, t, x, so);
 }

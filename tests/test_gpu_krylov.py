@@ -56,3 +56,46 @@ def test_f32_vcycle_coarse_level_shapes(fsi, N, faces):
     torch.cuda.synchronize()
     assert torch.equal(x, x2)
     assert precond_case.rel(precond_case.H(x), mg.vcycle(b)) < 2e-5, N
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("N", [(8, 8, 8), (33, 20, 12), (48, 40, 24)])
+def test_vcycle_repeats_and_under_capture(fsi, prec, N):
+    """The V-cycle's launches overlap: back-to-back cycles on changing inputs,
+    eager and replayed from a CUDA graph, give the bits of a cycle by itself."""
+    import torch
+    mesh, mg = precond_case.setup(fsi, N, None)
+    n = mg.levels[0].n
+    dt = precond_case.dtype_of(prec)
+    rng = np.random.default_rng(5)
+    bs = [precond_case.T(rng.normal(size=n), dt) for _ in range(3)]
+    alone = []
+    for b in bs:
+        x = torch.empty(n, dtype=dt, device="cuda")
+        torch.cuda.synchronize()
+        fsi.fsi_pressure_vcycle(mesh, b, x)
+        torch.cuda.synchronize()
+        alone.append(x.clone())
+    xs = [torch.empty(n, dtype=dt, device="cuda") for _ in range(30)]
+    for q, x in enumerate(xs):
+        fsi.fsi_pressure_vcycle(mesh, bs[q % 3], x)
+    torch.cuda.synchronize()
+    assert all(torch.equal(x, alone[q % 3]) for q, x in enumerate(xs))
+    side = torch.cuda.Stream()
+    mesh2 = fsi.Mesh(N, device=0, stream=side.cuda_stream)
+    x = torch.empty(n, dtype=dt, device="cuda")
+    y = torch.empty(n, dtype=dt, device="cuda")
+    with torch.cuda.stream(side):
+        fsi.fsi_pressure_vcycle(mesh2, bs[0], x)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=side):
+        fsi.fsi_pressure_vcycle(mesh2, bs[0], x)
+        fsi.fsi_pressure_vcycle(mesh2, bs[1], y)
+    for _ in range(3):
+        x.zero_()
+        y.zero_()
+        torch.cuda.synchronize()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(x, alone[0]) and torch.equal(y, alone[1])
