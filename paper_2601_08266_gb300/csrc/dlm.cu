@@ -93,6 +93,7 @@ __global__ void locate_kernel(int64_t m, GridArgs g, const double *__restrict__ 
                               int32_t *__restrict__ count, unsigned long long *n_out,
                               int32_t *__restrict__ arrival)
 {
+    chain_trigger();
     const int64_t E = (int64_t)g.Nx * g.Ny * g.Nz;
     for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < m;
          b += (int64_t)gridDim.x * blockDim.x) {
@@ -421,6 +422,7 @@ __global__ void __launch_bounds__(kLbThreads) tile_sums_kernel(int64_t E,
 {
     __shared__ int warp_sums[kLbThreads / 32];
     int v[kLbPer];
+    chain_wait(count, tile_sum);
     tile_counts(E, count, blockIdx.x, v);
     int own = 0;
 #pragma unroll
@@ -444,6 +446,7 @@ __global__ void __launch_bounds__(kLbThreads) tile_scan_kernel(int64_t E,
                                                                const int32_t *__restrict__ tile_sum,
                                                                int32_t *__restrict__ start)
 {
+    chain_trigger();
     __shared__ int warp_sums[kLbThreads / 32];
     const int t = blockIdx.x;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -663,6 +666,7 @@ __global__ void scatter_arrival_kernel(int64_t m, int64_t E, const int32_t *__re
                                        const int32_t *__restrict__ start, int32_t *fill,
                                        int32_t *scr, int2 *__restrict__ tmp)
 {
+    chain_wait(elem, arrival, start, fill, scr, tmp);
     if (blockIdx.x == 0 && threadIdx.x == 0) scr[0] = 0;  // the dense list starts empty
     for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < m;
          b += (int64_t)gridDim.x * blockDim.x) {
@@ -679,6 +683,7 @@ __global__ void rank_place_kernel(int64_t m, int64_t E, const int32_t *__restric
                                   const int2 *__restrict__ tmp, int32_t *__restrict__ perm,
                                   int32_t *dense, int32_t *scr)
 {
+    chain_trigger();
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < m;
          k += (int64_t)gridDim.x * blockDim.x) {
         const int2 p = tmp[k];
@@ -712,6 +717,7 @@ __global__ void __launch_bounds__(1024) dense_pairs_kernel(int64_t E, int64_t m,
                                                            const int32_t *dense_count)
 {
     extern __shared__ int32_t sort_sh[];
+    chain_wait(start, tmp, perm, dense, dense_count);
     const int n = *dense_count;
     for (int k = blockIdx.x; k < n; k += gridDim.x) {
         const int c = dense[k];
@@ -763,6 +769,7 @@ __global__ void spread_cells_kernel(int64_t E, const typename StorageOf<T>::type
                                     const typename StorageOf<T>::type *__restrict__ w,
                                     T *__restrict__ S, T dsq = T(0))
 {
+    chain_trigger();
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t c0 = warp * kSpreadSeg; c0 < E; c0 += nwarps * kSpreadSeg)
@@ -780,6 +787,7 @@ __global__ void spread_nodes_kernel(GridArgs g, const int32_t *__restrict__ star
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     if (i > g.Nx || j > g.Ny) return;
+    chain_wait(start, S, F);
     for (int k = blockIdx.z; k <= g.Nz; k += gridDim.z)
         spread_node<T>(g, i, j, k, start, S, F, accumulate);
 }
@@ -879,7 +887,7 @@ fsi_status build_cell_table(cudaStream_t s, int64_t E, int64_t m, const int32_t 
     const int64_t ntiles = cell_tiles(E);
     if (ntiles > INT32_MAX) return set_error(FSI_ERR_ARG, "cell table: too many cells");
     int32_t *tile_sum = scan_tmp + kScanHdr;
-    tile_sums_kernel<<<(int)ntiles, kLbThreads, 0, s>>>(E, fill, tile_sum);
+    launch_chain(tile_sums_kernel, (int)ntiles, kLbThreads, 0, s, E, fill, tile_sum);
     FSI_TRY(check_launch("cell tile sums kernel"));
     if (ntiles <= kDirectTiles) {
         tile_scan_kernel<true><<<(int)ntiles, kLbThreads, 0, s>>>(E, fill, tile_sum, cell_start);
@@ -890,7 +898,7 @@ fsi_status build_cell_table(cudaStream_t s, int64_t E, int64_t m, const int32_t 
     }
     FSI_TRY(check_launch("cell scan kernel"));
     if (m > 0 && tmp) {
-        scatter_arrival_kernel<<<blocks_for(m, 256), 256, 0, s>>>(m, E, elem, perm, cell_start,
+        launch_chain(scatter_arrival_kernel, blocks_for(m, 256), 256, 0, s, m, E, elem, perm, cell_start,
                                                                   fill, scan_tmp, tmp);
         FSI_TRY(check_launch("scatter kernel"));
         rank_place_kernel<<<blocks_for(m, 256, sm_count() * 32), 256, 0, s>>>(
@@ -899,7 +907,7 @@ fsi_status build_cell_table(cudaStream_t s, int64_t E, int64_t m, const int32_t 
         if (m > kWarpSortMax) {
             const int smem = kBlockSortMax * (int)sizeof(int32_t);
             FSI_TRY(set_smem_limit((const void *)dense_pairs_kernel, smem));
-            dense_pairs_kernel<<<sm_count(), 1024, smem, s>>>(E, m, cell_start, tmp, perm, fill,
+            launch_chain(dense_pairs_kernel, sm_count(), 1024, smem, s, E, m, cell_start, tmp, perm, fill,
                                                              scan_tmp);
             FSI_TRY(check_launch("dense cell sort kernel"));
         }
@@ -939,7 +947,7 @@ fsi_status spread_mass_diag(fsi_mesh *mesh, int64_t m, const T *xi, const int32_
     const dim3 nblock(32, 8), ngrid = node_grid(g);
     if ((g.Ny + 8) / 8 > 65535)
         return set_error(FSI_ERR_ARG, "spreading: more than 524,280 nodes along y");
-    spread_nodes_kernel<T><<<ngrid, nblock, 0, mesh->stream>>>(g, cell_start,
+    launch_chain(spread_nodes_kernel<T>, ngrid, nblock, 0, mesh->stream, g, cell_start,
                                                               (const T *)mesh->spread_scratch, F, 0);
     return check_launch("spread nodes kernel");
 }
@@ -1280,21 +1288,21 @@ fsi_status fsi_dlm_spread(fsi_mesh *mesh, fsi_prec prec, int64_t m, const int32_
             E, (const double *)xi, cell_start, perm, (const double *)lam, (const double *)w,
             (double *)mesh->spread_scratch);
         FSI_TRY(check_launch("spread cells kernel"));
-        spread_nodes_kernel<double><<<ngrid, nblock, 0, mesh->stream>>>(
+        launch_chain(spread_nodes_kernel<double>, ngrid, nblock, 0, mesh->stream, 
             g, cell_start, (const double *)mesh->spread_scratch, (double *)F, accumulate);
     } else if (prec == FSI_DF64) {
         spread_cells_kernel<df64><<<cgrid(kSpreadThreads<df64>), kSpreadThreads<df64>, 0, mesh->stream>>>(
             E, (const double *)xi, cell_start, perm, (const double *)lam, (const double *)w,
             (df64 *)mesh->spread_scratch);
         FSI_TRY(check_launch("spread cells kernel"));
-        spread_nodes_kernel<df64><<<ngrid, nblock, 0, mesh->stream>>>(
+        launch_chain(spread_nodes_kernel<df64>, ngrid, nblock, 0, mesh->stream, 
             g, cell_start, (const df64 *)mesh->spread_scratch, (double *)F, accumulate);
     } else {
         spread_cells_kernel<float><<<cgrid(kSpreadThreads<float>), kSpreadThreads<float>, 0, mesh->stream>>>(
             E, (const float *)xi, cell_start, perm, (const float *)lam, (const float *)w,
             (float *)mesh->spread_scratch);
         FSI_TRY(check_launch("spread cells kernel"));
-        spread_nodes_kernel<float><<<ngrid, nblock, 0, mesh->stream>>>(
+        launch_chain(spread_nodes_kernel<float>, ngrid, nblock, 0, mesh->stream, 
             g, cell_start, (const float *)mesh->spread_scratch, (float *)F, accumulate);
     }
     return check_launch("spread nodes kernel");

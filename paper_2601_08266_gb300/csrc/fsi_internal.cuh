@@ -66,10 +66,13 @@ fsi_status set_smem_limit(const void *kernel, int bytes);
 // chain may have written with __ldcg: two kernels back may still fill this SM's L1 with
 // lines from before that write.  Launched without the attribute, or
 // behind a kernel that does not chain, it waits for all of that kernel.
+// chain_trigger() lets the next kernel start; a kernel that triggers and was itself
+// launched the ordinary way needs no wait, and the L1 rule does not concern the one
+// behind it unless it reads what it writes.
 template <typename P> __device__ __forceinline__ void chain_pin(P &p) { asm volatile("" : "+l"(p)); }
+__device__ __forceinline__ void chain_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
 template <typename... P> __device__ __forceinline__ void chain_wait(P &...p)
 {
-    asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     (chain_pin(p), ...);
 }

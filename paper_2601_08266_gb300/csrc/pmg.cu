@@ -292,6 +292,7 @@ __global__ void __launch_bounds__(32 * kMarchWarps) march_kernel(LevelArgs<T> L,
 #pragma unroll
     for (int r = 0; r < R; ++r) acc[r] = PBk[r] = vk[r] = dk[r] = bk[r] = T(0);
     Raw nx;
+    chain_trigger();
     chain_wait(M.x, M.d, M.b, M.y, M.x_next, M.d_next, M.x_final, M.z4, M.v4, M.m4);
     load(k0 - 1, nx);
     for (int kk = k0 - 1; kk <= k1; ++kk) {
@@ -437,6 +438,7 @@ __global__ void restrict_kernel(LevelArgs<T> F, LevelArgs<T> C, int kz, const T 
         const T c = at(yr) + wl * at(yr - xl) + wr * at(yr + xr);
         return a + vl * b + vr * c;
     };
+    chain_trigger();
     chain_wait(r, bc);
     T below = plane(2 * K0 - 1);
 #pragma unroll 2
@@ -468,6 +470,7 @@ __global__ void prolong_kernel(LevelArgs<T> F, LevelArgs<T> C, int kz, const T *
         const T *q = c + plane_c * K;
         return T(0.25) * ((__ldcg(q) + __ldcg(q + dx)) + (__ldcg(q + dy) + __ldcg(q + dy + dx)));
     };
+    chain_trigger();
     chain_wait(c, f);
     T at = plane(K0);
 #pragma unroll 2
@@ -827,6 +830,7 @@ __global__ void __launch_bounds__(kCoarseThreads, 1) coarse_cycle_kernel(const _
     coarse_nodes(C.lev[0], s0, s1, N, [&](const CoarseNode &) {});  // the weights
     const float *gb = C.b, *ginv = C.inv;
     float *gx = C.x;
+    chain_trigger();
     chain_wait(gb, ginv, gx);
     // the dense inverse on its way (see off_inv)
     if (rank == 0 && C.off_inv)

@@ -42,6 +42,7 @@ constexpr int kBrickCtas = sizeof(T) == 4 ? 4 : (std::is_same<T, double>::value 
 template <typename T, bool JAC, bool MAPPED, bool FUSED = false>
 __global__ void __launch_bounds__(kBrickThreads, (kBrickCtas<T, FUSED>)) vms_brick_kernel(const VmsArgs<T> P)
 {
+    chain_trigger();
     extern __shared__ __align__(32) unsigned char smem_raw[];
     brick_body<T, JAC, MAPPED, FUSED>(P, blockIdx.x, smem_raw);
 }
@@ -116,7 +117,9 @@ template <typename T, bool FUSED = false>
 __global__ void __launch_bounds__(256) vms_gather_kernel(const VmsArgs<T> P, int n)
 {
     const int q = blockIdx.x * 256 + threadIdx.x;
-    if (q < n) gather_shared<T, FUSED>(P, q);
+    VmsArgs<T> Q = P;
+    chain_wait(Q.blocks, Q.blocks2, Q.out, Q.out2);
+    if (q < n) gather_shared<T, FUSED>(Q, q);
 }
 
 // FUSED: the residual (R) and the Jacobian apply (out) at the same state in
@@ -147,8 +150,7 @@ fsi_status launch_geo(fsi_mesh *m, const void *U, const void *A, const void *f, 
     FSI_TRY(check_launch("vms brick kernel"));
     const int64_t shared = shared_nodes(P);
     if (shared == 0) return FSI_OK;
-    vms_gather_kernel<T, FUSED>
-        <<<(int)((shared + 255) / 256), 256, 0, m->stream>>>(P, (int)shared);
+    launch_chain(vms_gather_kernel<T, FUSED>, (int)((shared + 255) / 256), 256, 0, m->stream, P, (int)shared);
     return check_launch("vms gather kernel");
 }
 
