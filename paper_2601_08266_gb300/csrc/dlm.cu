@@ -73,10 +73,10 @@ fsi_status launch_locate(cudaStream_t s, int64_t m, const GridArgs &g, const dou
                          int32_t *arrival = nullptr)
 {
     if (g.shifted && g.zero_origin)
-        locate_kernel<true><<<blocks_for(m, 256), 256, 0, s>>>(m, g, X, elem, xi, count, n_out,
+        launch_chain(locate_kernel<true>, blocks_for(m, 256), 256, 0, s, m, g, X, elem, xi, count, n_out,
                                                                arrival);
     else
-        locate_kernel<false><<<blocks_for(m, 256), 256, 0, s>>>(m, g, X, elem, xi, count, n_out,
+        launch_chain(locate_kernel<false>, blocks_for(m, 256), 256, 0, s, m, g, X, elem, xi, count, n_out,
                                                                 arrival);
     return check_launch("locate kernel");
 }
@@ -93,6 +93,7 @@ __global__ void locate_kernel(int64_t m, GridArgs g, const double *__restrict__ 
                               int32_t *__restrict__ count, unsigned long long *n_out,
                               int32_t *__restrict__ arrival)
 {
+    chain_wait(X, elem, xi, count, n_out, arrival);
     chain_trigger();
     const int64_t E = (int64_t)g.Nx * g.Ny * g.Nz;
     for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < m;
@@ -423,6 +424,7 @@ __global__ void __launch_bounds__(kLbThreads) tile_sums_kernel(int64_t E,
     __shared__ int warp_sums[kLbThreads / 32];
     int v[kLbPer];
     chain_wait(count, tile_sum);
+    chain_trigger();
     tile_counts(E, count, blockIdx.x, v);
     int own = 0;
 #pragma unroll
@@ -446,6 +448,7 @@ __global__ void __launch_bounds__(kLbThreads) tile_scan_kernel(int64_t E,
                                                                const int32_t *__restrict__ tile_sum,
                                                                int32_t *__restrict__ start)
 {
+    chain_wait(count, tile_sum, start);
     chain_trigger();
     __shared__ int warp_sums[kLbThreads / 32];
     const int t = blockIdx.x;
@@ -667,6 +670,7 @@ __global__ void scatter_arrival_kernel(int64_t m, int64_t E, const int32_t *__re
                                        int32_t *scr, int2 *__restrict__ tmp)
 {
     chain_wait(elem, arrival, start, fill, scr, tmp);
+    chain_trigger();
     if (blockIdx.x == 0 && threadIdx.x == 0) scr[0] = 0;  // the dense list starts empty
     for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < m;
          b += (int64_t)gridDim.x * blockDim.x) {
@@ -683,6 +687,7 @@ __global__ void rank_place_kernel(int64_t m, int64_t E, const int32_t *__restric
                                   const int2 *__restrict__ tmp, int32_t *__restrict__ perm,
                                   int32_t *dense, int32_t *scr)
 {
+    chain_wait(start, tmp, perm, dense, scr);
     chain_trigger();
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < m;
          k += (int64_t)gridDim.x * blockDim.x) {
@@ -717,6 +722,7 @@ __global__ void __launch_bounds__(1024) dense_pairs_kernel(int64_t E, int64_t m,
                                                            const int32_t *dense_count)
 {
     extern __shared__ int32_t sort_sh[];
+    // (no trigger: it reads perm where it writes it)
     chain_wait(start, tmp, perm, dense, dense_count);
     const int n = *dense_count;
     for (int k = blockIdx.x; k < n; k += gridDim.x) {
@@ -738,6 +744,8 @@ __global__ void interp_kernel(int64_t m, GridArgs g, const int32_t *__restrict__
                               const S *__restrict__ xi, const vec4<S> *__restrict__ U,
                               S *__restrict__ u)
 {
+    chain_wait(elem, xi, U, u);
+    chain_trigger();
     if constexpr (std::is_same<T, float>::value) {
         const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
         const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -769,6 +777,7 @@ __global__ void spread_cells_kernel(int64_t E, const typename StorageOf<T>::type
                                     const typename StorageOf<T>::type *__restrict__ w,
                                     T *__restrict__ S, T dsq = T(0))
 {
+    chain_wait(xi, start, perm, lam, w, S);
     chain_trigger();
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -890,18 +899,18 @@ fsi_status build_cell_table(cudaStream_t s, int64_t E, int64_t m, const int32_t 
     launch_chain(tile_sums_kernel, (int)ntiles, kLbThreads, 0, s, E, fill, tile_sum);
     FSI_TRY(check_launch("cell tile sums kernel"));
     if (ntiles <= kDirectTiles) {
-        tile_scan_kernel<true><<<(int)ntiles, kLbThreads, 0, s>>>(E, fill, tile_sum, cell_start);
+        launch_chain(tile_scan_kernel<true>, (int)ntiles, kLbThreads, 0, s, E, fill, tile_sum, cell_start);
     } else {
         tile_prefix_kernel<<<1, 1024, 0, s>>>(ntiles, tile_sum);
         FSI_TRY(check_launch("cell tile prefix kernel"));
-        tile_scan_kernel<false><<<(int)ntiles, kLbThreads, 0, s>>>(E, fill, tile_sum, cell_start);
+        launch_chain(tile_scan_kernel<false>, (int)ntiles, kLbThreads, 0, s, E, fill, tile_sum, cell_start);
     }
     FSI_TRY(check_launch("cell scan kernel"));
     if (m > 0 && tmp) {
         launch_chain(scatter_arrival_kernel, blocks_for(m, 256), 256, 0, s, m, E, elem, perm, cell_start,
                                                                   fill, scan_tmp, tmp);
         FSI_TRY(check_launch("scatter kernel"));
-        rank_place_kernel<<<blocks_for(m, 256, sm_count() * 32), 256, 0, s>>>(
+        launch_chain(rank_place_kernel, blocks_for(m, 256, sm_count() * 32), 256, 0, s, 
             m, E, cell_start, tmp, perm, fill, scan_tmp);
         FSI_TRY(check_launch("rank place kernel"));
         if (m > kWarpSortMax) {
@@ -941,7 +950,7 @@ fsi_status spread_mass_diag(fsi_mesh *mesh, int64_t m, const T *xi, const int32_
     const int64_t E = mesh->n_elems;
     FSI_TRY(ensure_spread_scratch(mesh, (size_t)E * 24 * sizeof(T)));
     const int cgrid = blocks_for((E + kSpreadSeg - 1) / kSpreadSeg * 32, kSpreadThreads<T>, sm_count() * 256);
-    spread_cells_kernel<T, true><<<cgrid, kSpreadThreads<T>, 0, mesh->stream>>>(
+    launch_chain(spread_cells_kernel<T, true>, cgrid, kSpreadThreads<T>, 0, mesh->stream, 
         E, xi, cell_start, perm, nullptr, w, (T *)mesh->spread_scratch, (T)dsq);
     FSI_TRY(check_launch("spread cells kernel"));
     const dim3 nblock(32, 8), ngrid = node_grid(g);
@@ -1244,13 +1253,13 @@ fsi_status fsi_dlm_interp(fsi_mesh *mesh, fsi_prec prec, int64_t m, const int32_
     if (mesh->tet) return fsi_tet_interp(mesh->tet, prec, m, elem, xi, U, u);
     GridArgs g = grid_args(mesh);
     if (prec == FSI_F64)
-        interp_kernel<double><<<blocks_for(m, 256), 256, 0, mesh->stream>>>(
+        launch_chain(interp_kernel<double>, blocks_for(m, 256), 256, 0, mesh->stream, 
             m, g, elem, (const double *)xi, (const vec4<double> *)U, (double *)u);
     else if (prec == FSI_DF64)
-        interp_kernel<df64><<<blocks_for(m, 256), 256, 0, mesh->stream>>>(
+        launch_chain(interp_kernel<df64>, blocks_for(m, 256), 256, 0, mesh->stream, 
             m, g, elem, (const double *)xi, (const vec4<double> *)U, (double *)u);
     else
-        interp_kernel<float><<<blocks_for(2 * m, 256), 256, 0, mesh->stream>>>(
+        launch_chain(interp_kernel<float>, blocks_for(2 * m, 256), 256, 0, mesh->stream, 
             m, g, elem, (const float *)xi, (const vec4<float> *)U, (float *)u);
     return check_launch("interp kernel");
 }
@@ -1284,23 +1293,23 @@ fsi_status fsi_dlm_spread(fsi_mesh *mesh, fsi_prec prec, int64_t m, const int32_
     if ((g.Ny + 8) / 8 > 65535)
         return set_error(FSI_ERR_ARG, "fsi_dlm_spread: more than 524,280 nodes along y");
     if (prec == FSI_F64) {
-        spread_cells_kernel<double><<<cgrid(kSpreadThreads<double>), kSpreadThreads<double>, 0, mesh->stream>>>(
+        launch_chain(spread_cells_kernel<double>, cgrid(kSpreadThreads<double>), kSpreadThreads<double>, 0, mesh->stream, 
             E, (const double *)xi, cell_start, perm, (const double *)lam, (const double *)w,
-            (double *)mesh->spread_scratch);
+            (double *)mesh->spread_scratch, 0.0);
         FSI_TRY(check_launch("spread cells kernel"));
         launch_chain(spread_nodes_kernel<double>, ngrid, nblock, 0, mesh->stream, 
             g, cell_start, (const double *)mesh->spread_scratch, (double *)F, accumulate);
     } else if (prec == FSI_DF64) {
-        spread_cells_kernel<df64><<<cgrid(kSpreadThreads<df64>), kSpreadThreads<df64>, 0, mesh->stream>>>(
+        launch_chain(spread_cells_kernel<df64>, cgrid(kSpreadThreads<df64>), kSpreadThreads<df64>, 0, mesh->stream, 
             E, (const double *)xi, cell_start, perm, (const double *)lam, (const double *)w,
-            (df64 *)mesh->spread_scratch);
+            (df64 *)mesh->spread_scratch, df64(0));
         FSI_TRY(check_launch("spread cells kernel"));
         launch_chain(spread_nodes_kernel<df64>, ngrid, nblock, 0, mesh->stream, 
             g, cell_start, (const df64 *)mesh->spread_scratch, (double *)F, accumulate);
     } else {
-        spread_cells_kernel<float><<<cgrid(kSpreadThreads<float>), kSpreadThreads<float>, 0, mesh->stream>>>(
+        launch_chain(spread_cells_kernel<float>, cgrid(kSpreadThreads<float>), kSpreadThreads<float>, 0, mesh->stream, 
             E, (const float *)xi, cell_start, perm, (const float *)lam, (const float *)w,
-            (float *)mesh->spread_scratch);
+            (float *)mesh->spread_scratch, 0.0f);
         FSI_TRY(check_launch("spread cells kernel"));
         launch_chain(spread_nodes_kernel<float>, ngrid, nblock, 0, mesh->stream, 
             g, cell_start, (const float *)mesh->spread_scratch, (float *)F, accumulate);

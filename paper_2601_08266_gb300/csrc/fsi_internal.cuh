@@ -62,13 +62,13 @@ fsi_status set_smem_limit(const void *kernel, int bytes);
 // the earlier kernels have finished and their results are visible.  Such a kernel calls
 // chain_wait() before its first access to global memory and passes it the pointers
 // that it reads and writes through, so that no access can be moved before it (loads
-// through read-only pointers otherwise might), and it reads what a kernel of the
-// chain may have written with __ldcg: two kernels back may still fill this SM's L1 with
-// lines from before that write.  Launched without the attribute, or
-// behind a kernel that does not chain, it waits for all of that kernel.
-// chain_trigger() lets the next kernel start; a kernel that triggers and was itself
-// launched the ordinary way needs no wait, and the L1 rule does not concern the one
-// behind it unless it reads what it writes.
+// through read-only pointers otherwise might).
+//
+// chain_trigger() lets the next kernel start.  After chain_wait() only these two can
+// be running then, and the next one's reads are safe if this one does not read
+// what it writes: its CTAs start with an empty L1.  Before chain_wait() (the V-cycle) two
+// kernels back may still be running and fill this SM's L1 with lines that the one
+// between them then writes, so what the chain writes is read with __ldcg.
 template <typename P> __device__ __forceinline__ void chain_pin(P &p) { asm volatile("" : "+l"(p)); }
 __device__ __forceinline__ void chain_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
 template <typename... P> __device__ __forceinline__ void chain_wait(P &...p)

@@ -292,8 +292,11 @@ __global__ void __launch_bounds__(32 * kMarchWarps) march_kernel(LevelArgs<T> L,
 #pragma unroll
     for (int r = 0; r < R; ++r) acc[r] = PBk[r] = vk[r] = dk[r] = bk[r] = T(0);
     Raw nx;
-    chain_trigger();
+    // (a cycle's last kernel lets the next start only when those before it are done)
+    const bool last = M.x_final || M.z4;
+    if (!last) chain_trigger();
     chain_wait(M.x, M.d, M.b, M.y, M.x_next, M.d_next, M.x_final, M.z4, M.v4, M.m4);
+    if (last) chain_trigger();
     load(k0 - 1, nx);
     for (int kk = k0 - 1; kk <= k1; ++kk) {
         const Raw w = nx;

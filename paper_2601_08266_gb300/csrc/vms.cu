@@ -119,6 +119,7 @@ __global__ void __launch_bounds__(256) vms_gather_kernel(const VmsArgs<T> P, int
     const int q = blockIdx.x * 256 + threadIdx.x;
     VmsArgs<T> Q = P;
     chain_wait(Q.blocks, Q.blocks2, Q.out, Q.out2);
+    chain_trigger();
     if (q < n) gather_shared<T, FUSED>(Q, q);
 }
 
