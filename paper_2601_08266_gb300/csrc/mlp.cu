@@ -549,11 +549,11 @@ fsi_status fsi_mlp_predict(fsi_mlp *h, fsi_mesh *mesh, const float *params, cons
     if (h->device != mesh->device) return set_error(FSI_ERR_ARG, "mlp and mesh on other devices");
     FSI_DEVICE(mesh->device);
     // fused features -> network -> predictor on the tcgen05 tensor cores
-    // (the FP32 nodes go into the mesh's spreading scratch, on the mesh's stream: 16 B a
-    // node, and it has 192 B an element from the start)
+    // the FP32 nodes go behind the corner sums in the mesh's spreading scratch
+    void *feat = (char *)mesh->spread_scratch + (size_t)mesh->n_elems * 24 * sizeof(double);
     return mlp_predict_tc(mesh->stream, mesh->device, mesh->grid, mesh->n_nodes, params, in_mean,
                           in_std, out_mean, out_std, Vn, y, d1, d2, y0, h->packed,
-                          mesh->spread_scratch, h->tc_err);
+                          feat, h->tc_err);
 }
 
 fsi_status fsi_mlp_guess(fsi_mlp *h, fsi_mesh *mesh, const float *params, const float *in_mean,

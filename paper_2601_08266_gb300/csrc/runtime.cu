@@ -276,7 +276,10 @@ fsi_status fsi_mesh_create(const fsi_grid *grid, const fsi_physics *phys, int de
         st = check_cuda(cudaMalloc(&m->vms_scratch, need), "VMS scratch allocation");
         if (st == FSI_OK) m->vms_scratch_bytes = need;
     }
-    if (st == FSI_OK) st = ensure_spread_scratch(m, (size_t)E * 24 * sizeof(double));
+    // the spreading's corner sums, and behind them the predictor's FP32 nodes (both may
+    // be in use at once, on different streams)
+    if (st == FSI_OK)
+        st = ensure_spread_scratch(m, (size_t)E * 24 * sizeof(double) + (size_t)m->n_nodes * sizeof(float4));
     if (st != FSI_OK) {
         fsi_mesh_destroy(m);
         return st;

@@ -99,3 +99,47 @@ def test_vcycle_repeats_and_under_capture(fsi, prec, N):
         g.replay()
         torch.cuda.synchronize()
         assert torch.equal(x, alone[0]) and torch.equal(y, alone[1])
+
+
+# 45^3 and 35^3 nodes: more records than the one-launch orthogonalisation holds, so the
+# passes of long vectors run (8 vectors and fewer, then up to 16)
+@pytest.mark.parametrize("mixed,N", [(True, 44), (False, 34)])
+def test_newton_step_on_long_vectors(fsi, mixed, N):
+    import torch
+    from paper_2601_08266_gb300 import inputs
+    n, m = (N + 1) ** 3, 20000
+    rng = np.random.default_rng(2)
+    ax = np.arange(N + 1) / N
+    Z, Y, X = np.meshgrid(ax, ax, ax, indexing="ij")
+    X, Y, Z = X.ravel(), Y.ravel(), Z.ravel()
+    wall = (Y < 1e-12) | (Y > 1 - 1e-12) | (Z < 1e-12) | (Z > 1 - 1e-12)
+    inflow = (X < 1e-12) & ~wall
+    mask = np.zeros((n, 4), dtype=np.uint8)
+    mask[wall | inflow, :3] = 1
+    prof = 16 * Y * (1 - Y) * Z * (1 - Z)
+    Vn = np.zeros((n, 4))
+    Vn[:, 0] = prof
+    Vn[:, :3] += 0.05 * rng.normal(size=(n, 3))
+    Vn[mask[:, 0].astype(bool), :3] = 0
+    Vn[inflow, 0] = prof[inflow]
+    f64 = lambda a: precond_case.T(a, torch.float64)
+    mesh = fsi.Mesh(N, rho=1.0, mu=1e-3, dt=1e-3, rho_inf=0.5, device=0)
+    e = torch.empty(m, dtype=torch.int32, device="cuda")
+    xi = torch.empty((m, 3), dtype=torch.float64, device="cuda")
+    cs = torch.empty(N ** 3 + 1, dtype=torch.int32, device="cuda")
+    pm = torch.empty(m, dtype=torch.int32, device="cuda")
+    fsi.fsi_locate(mesh, f64(inputs.leaflet_points(m, seed=5)), e, xi, cs, pm)
+    y = torch.zeros((n, 4), dtype=torch.float64, device="cuda")
+    keep = [f64(Vn), f64(np.zeros((n, 4))), precond_case.T(mask, torch.uint8),
+            f64(np.zeros((n, 4))), torch.full((m,), 0.024 / m, dtype=torch.float64, device="cuda")]
+    st = fsi.StepState(y, keep[0], keep[1], mask=keep[2], yD=keep[3], elem=e, xi=xi, cell_start=cs,
+                       perm=pm, w=keep[4], drho_s=0.5)
+    code, rep = fsi.fsi_newton_step(mesh, st, mixed=mixed, restart=50, max_newton=10, max_krylov=400,
+                                    newton_rtol=1e-8, krylov_rtol=1e-3, precond=fsi.PRECOND_SCHUR)
+    assert code == 0 and rep["converged"] == 1
+    assert rep["krylov_iters"] <= 20 * rep["newton_iters"], rep  # ~10 a solve; no stagnation
+    R = torch.empty_like(y)
+    fsi.fsi_coupled_residual(mesh, st, R)
+    torch.cuda.synchronize()
+    assert R.norm().item() <= 1.01e-8 * rep["r_ref"]
+    mesh.close()
