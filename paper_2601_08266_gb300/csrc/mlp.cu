@@ -65,6 +65,8 @@ __global__ void loss_kernel(int64_t B, const float *O, const float *T, float *dO
                             double *partial)
 {
     __shared__ double red[256];
+    chain_wait(O, T, dO, partial);
+    chain_trigger();
     double acc = 0.0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < B * NO;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -102,6 +104,8 @@ __global__ void colsum_partial_kernel(int64_t M, ColSums c, float *part)
     while (q < 2 && (int)blockIdx.x >= c.cta0[q + 1]) ++q;
     const int N = c.N[q];
     const float *dZ = c.dZ[q];
+    chain_wait(dZ, part);
+    chain_trigger();
     const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
     const int j = (blockIdx.x - c.cta0[q]) * 32 + x;
     const int64_t per = (M + gridDim.y - 1) / gridDim.y;
@@ -124,6 +128,8 @@ __global__ void colsum_partial_kernel(int64_t M, ColSums c, float *part)
 __global__ void grad_final_kernel(ColSums c, int slices, const float *part, int nb,
                                   const double *partial, float *loss)
 {
+    chain_wait(part, partial, loss);
+    chain_trigger();
     if (blockIdx.x == 0) {
         __shared__ double red[256];
         double v = 0.0;
@@ -151,6 +157,7 @@ __global__ void grad_final_kernel(ColSums c, int slices, const float *part, int 
 __global__ void adam_kernel(int64_t n, float *p, const float *g, float *m, float *v, float lr,
                             float b1, float b2, float eps, float c1, float c2)
 {
+    chain_wait(p, g, m, v);  // (no trigger: it reads what it writes)
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const float gi = g[i];
@@ -479,7 +486,7 @@ fsi_status fsi_mlp_loss_grad(fsi_mlp *h, const float *params, const float *X, co
     const float *P = params;
     FSI_TRY(forward_impl(h, P, X, B, true));
     const int nb = 256;
-    loss_kernel<<<nb, 256, 0, s>>>(B, h->O, T, h->dO, h->loss_partial);
+    launch_chain(loss_kernel, nb, 256, 0, s, B, h->O, T, h->dO, h->loss_partial);
     FSI_TRY(check_launch("loss kernel"));
     const int M = (int)B;
     // dZ2 = (dO W3^T) * (Z2 > 0), dZ1 = (dZ2 W2^T) * (Z1 > 0)
@@ -500,8 +507,8 @@ fsi_status fsi_mlp_loss_grad(fsi_mlp *h, const float *params, const float *X, co
                        {0, NH / 32, 2 * (NH / 32), 2 * (NH / 32) + 1},
                        2 * NH + NO};
     float *part = h->gemm_work;  // the split-K workspace, free again in stream order
-    colsum_partial_kernel<<<dim3(c.cta0[3], kColSlices), 256, 0, s>>>(B, c, part);
-    grad_final_kernel<<<1 + (c.cols + 255) / 256, 256, 0, s>>>(c, kColSlices, part, nb,
+    launch_chain(colsum_partial_kernel, dim3(c.cta0[3], kColSlices), 256, 0, s, B, c, part);
+    launch_chain(grad_final_kernel, 1 + (c.cols + 255) / 256, 256, 0, s, c, kColSlices, part, nb,
                                                               h->loss_partial, loss);
     return check_launch("bias gradients");
 }
@@ -513,7 +520,7 @@ fsi_status fsi_mlp_adam(fsi_mlp *h, float *params, const float *grad, float *m, 
     if (!params || !grad || !m || !v || step < 1) return set_error(FSI_ERR_ARG, "bad argument");
     FSI_DEVICE(h->device);
     const float c1 = 1.f - powf(beta1, (float)step), c2 = 1.f - powf(beta2, (float)step);
-    adam_kernel<<<blocks(N_PARAMS), 256, 0, h->stream>>>(N_PARAMS, params, grad, m, v, lr, beta1,
+    launch_chain(adam_kernel, blocks(N_PARAMS), 256, 0, h->stream, N_PARAMS, params, grad, m, v, lr, beta1,
                                                         beta2, eps, c1, c2);
     return check_launch("adam kernel");
 }

@@ -285,7 +285,9 @@ __global__ void __launch_bounds__(kThreads) tc_gemm_kernel(const Group G, int *e
     __shared__ int abort_flag;
     int q = 0;
     while (q + 1 < G.n && (int)blockIdx.x >= G.start[q + 1]) ++q;
-    const TcGemm &g = G.g[q];
+    TcGemm g = G.g[q];
+    chain_wait(g.A, g.B, g.bias, g.mask, g.work, g.C, g.Cpre);
+    chain_trigger();
     const int cta = blockIdx.x - G.start[q];
     if (g.transA) {
         if (g.transB) gemm_body<false, true>(g, cta, err, sm, bars, &tmem_holder, &abort_flag);
@@ -300,8 +302,11 @@ __global__ void __launch_bounds__(kThreads) tc_gemm_kernel(const Group G, int *e
 // of the group that was split
 __global__ void tc_gemm_reduce_kernel(const Group G)
 {
+    chain_wait();
+    chain_trigger();
     for (int q = 0; q < G.n; ++q) {
-        const TcGemm &g = G.g[q];
+        TcGemm g = G.g[q];
+        chain_pin(g.work);
         if (g.splits < 2) continue;
         const int64_t total = (int64_t)g.M * g.N;
         for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
@@ -358,11 +363,11 @@ fsi_status tc_gemm_group(cudaStream_t s, const TcGemm *gs, int n, float *work, i
         G.start[q + 1] = G.start[q] + mt * nt * splits;
     }
     FSI_TRY(set_smem_limit((const void *)tc_gemm_kernel, SMEM_BYTES));
-    tc_gemm_kernel<<<G.start[n], kThreads, SMEM_BYTES, s>>>(G, err);
+    launch_chain(tc_gemm_kernel, G.start[n], kThreads, SMEM_BYTES, s, G, err);
     FSI_TRY(check_launch("tensor-core gemm"));
     if (reduce > 0) {
         const int blocks = (int)std::min<int64_t>((reduce + 255) / 256, sm_count() * 8);
-        tc_gemm_reduce_kernel<<<blocks, 256, 0, s>>>(G);
+        launch_chain(tc_gemm_reduce_kernel, blocks, 256, 0, s, G);
         FSI_TRY(check_launch("tensor-core gemm reduce"));
     }
     return FSI_OK;
