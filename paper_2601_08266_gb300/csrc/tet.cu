@@ -196,6 +196,7 @@ template <typename T> struct TetArgs {
 // element's gradients (the rule: tet_by_element).
 template <typename T, bool JAC> __global__ void __launch_bounds__(256) tet_vms_kernel(TetArgs<T> P)
 {
+    chain_trigger();
     using S = typename StorageOf<T>::type;
     const VmsArgs<T> &V = P.V;
     const int a = threadIdx.x & 3;
@@ -375,6 +376,7 @@ template <typename T, bool JAC>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 || (!JAC && std::is_same<T, df64>::value) ? 4 : 3)
     tet_vms_elem_kernel(TetArgs<T> P)
 {
+    chain_trigger();
     using S = typename StorageOf<T>::type;
     using PT = Points<T>;
     using C = typename PT::C;
@@ -728,6 +730,7 @@ __global__ void __launch_bounds__(256)
     tet_gather_kernel(int64_t n, const int32_t *__restrict__ start, const int32_t *__restrict__ slot,
                       const vec4<T> *__restrict__ in, typename StorageOf<T>::type *__restrict__ out)
 {
+    chain_wait(start, slot, in, out);
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, i = t >> 2;
     const int q = (int)(t & 3);
     int k = 0, k1 = 0;
@@ -842,6 +845,7 @@ __global__ void __launch_bounds__(kLocThreads)
                       double *__restrict__ lam_out, int32_t *__restrict__ count,
                       unsigned long long *n_out)
 {
+    chain_trigger();
     constexpr unsigned kAll = 0xffffffffu;
     __shared__ int cand_s[kLocThreads / 32][32 * kLocCand], pair_s[kLocThreads / 32][32 * kLocCand];
     __shared__ uint8_t owner_s[kLocThreads / 32][32 * kLocCand];
@@ -1010,6 +1014,7 @@ __global__ void tet_spread_cells_kernel(int64_t E, const S *__restrict__ lam,
                                         const S *__restrict__ lamv, const S *__restrict__ w,
                                         T *__restrict__ Ssum)
 {
+    chain_trigger();
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1067,6 +1072,7 @@ __global__ void __launch_bounds__(256)
                             const int32_t *__restrict__ nslot, const int32_t *__restrict__ start,
                             const T *__restrict__ Ssum, S *__restrict__ F, int accumulate)
 {
+    chain_wait(nstart, nslot, start, Ssum, F);
     // four lanes per node, four slots a lane in flight, as in tet_gather_kernel
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, i = t >> 2;
     const int q = (int)(t & 3);
@@ -1192,7 +1198,7 @@ fsi_status tet_vms(fsi_tetmesh *m, const void *U, const void *A, const void *f, 
         tet_vms_kernel<T, JAC><<<grid_for(threads, 256, sm_count() * 64), 256, 0, m->stream>>>(P);
     }
     FSI_TRY(check_launch("tet vms kernel"));
-    tet_gather_kernel<T><<<(int)((4 * m->n_nodes + 255) / 256), 256, 0, m->stream>>>(
+    launch_chain(tet_gather_kernel<T>, (int)((4 * m->n_nodes + 255) / 256), 256, 0, m->stream,
         m->n_nodes, m->node_start, m->node_slot, P.slots, (S *)out);
     return check_launch("tet gather kernel");
 }
@@ -1595,7 +1601,7 @@ fsi_status fsi_tet_spread(fsi_tetmesh *m, fsi_prec prec, int64_t np, const int32
                                                            (const double *)w,
                                                            (double *)m->corner_scratch);
         FSI_TRY(check_launch("tet spread cells kernel"));
-        tet_spread_nodes_kernel<double><<<ng, 256, 0, s>>>(m->n_nodes, m->node_start, m->node_slot,
+        launch_chain(tet_spread_nodes_kernel<double>, ng, 256, 0, s, m->n_nodes, m->node_start, m->node_slot,
                                                            cell_start,
                                                            (const double *)m->corner_scratch,
                                                            (double *)F, accumulate);
@@ -1604,7 +1610,7 @@ fsi_status fsi_tet_spread(fsi_tetmesh *m, fsi_prec prec, int64_t np, const int32
                                                          (const double *)lamv, (const double *)w,
                                                          (df64 *)m->corner_scratch);
         FSI_TRY(check_launch("tet spread cells kernel"));
-        tet_spread_nodes_kernel<df64><<<ng, 256, 0, s>>>(m->n_nodes, m->node_start, m->node_slot,
+        launch_chain(tet_spread_nodes_kernel<df64>, ng, 256, 0, s, m->n_nodes, m->node_start, m->node_slot,
                                                          cell_start,
                                                          (const df64 *)m->corner_scratch,
                                                          (double *)F, accumulate);
@@ -1613,7 +1619,7 @@ fsi_status fsi_tet_spread(fsi_tetmesh *m, fsi_prec prec, int64_t np, const int32
                                                           (const float *)lamv, (const float *)w,
                                                           (float *)m->corner_scratch);
         FSI_TRY(check_launch("tet spread cells kernel"));
-        tet_spread_nodes_kernel<float><<<ng, 256, 0, s>>>(m->n_nodes, m->node_start, m->node_slot,
+        launch_chain(tet_spread_nodes_kernel<float>, ng, 256, 0, s, m->n_nodes, m->node_start, m->node_slot,
                                                           cell_start,
                                                           (const float *)m->corner_scratch,
                                                           (float *)F, accumulate);
