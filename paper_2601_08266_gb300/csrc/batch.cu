@@ -254,7 +254,7 @@ __global__ void batch_interp_kernel(const DlmDesc<T> *desc, const int64_t *prefi
 }
 
 template <typename T>
-__global__ void batch_spread_cells_kernel(const DlmDesc<T> *desc, const int64_t *prefix,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) batch_spread_cells_kernel(const DlmDesc<T> *desc, const int64_t *prefix,
                                           int count)
 {
     const int64_t total = prefix[count];

@@ -522,24 +522,41 @@ __device__ __forceinline__ void interp_point_pair(
     }
 }
 
+// One point's inputs as stored
+template <typename S> struct SpreadPoint {
+    S x[3], l[3], w;
+};
+template <typename S, bool SQ>
+__device__ __forceinline__ SpreadPoint<S> spread_load(int b, const S *__restrict__ xi,
+                                                      const S *__restrict__ lam,
+                                                      const S *__restrict__ w)
+{
+    SpreadPoint<S> q;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        q.x[k] = xi[3 * b + k];
+        q.l[k] = SQ ? S(0) : lam[3 * b + k];
+    }
+    q.w = w ? w[b] : S(1);
+    return q;
+}
+
 // Corner contributions w_B N_a(xi_B) lambda_B of one point B added to acc
 // (T the compute type; inputs in StorageOf<T>).  SQ: w_B N_a(xi_B)^2 dsq
 // instead (lam unused): the diagonal of C W C^T scaled by dsq.
 template <typename T, bool SQ = false>
 __device__ __forceinline__ void spread_accumulate(
-    int b, const typename StorageOf<T>::type *__restrict__ xi,
-    const typename StorageOf<T>::type *__restrict__ lam,
-    const typename StorageOf<T>::type *__restrict__ w, T (&acc)[24], T dsq = T(0))
+    const SpreadPoint<typename StorageOf<T>::type> &q, bool weighted, T (&acc)[24], T dsq = T(0))
 {
-    const T x0 = to_c<T>(xi[3 * b]), x1 = to_c<T>(xi[3 * b + 1]), x2 = to_c<T>(xi[3 * b + 2]);
-    const T s = w ? to_c<T>(w[b]) * T(0.125f) : T(0.125f);
+    const T x0 = to_c<T>(q.x[0]), x1 = to_c<T>(q.x[1]), x2 = to_c<T>(q.x[2]);
+    const T s = weighted ? to_c<T>(q.w) * T(0.125f) : T(0.125f);
     T l0, l1, l2;
     if constexpr (SQ) {
         l0 = l1 = l2 = dsq;
     } else {
-        l0 = to_c<T>(lam[3 * b]);
-        l1 = to_c<T>(lam[3 * b + 1]);
-        l2 = to_c<T>(lam[3 * b + 2]);
+        l0 = to_c<T>(q.l[0]);
+        l1 = to_c<T>(q.l[1]);
+        l2 = to_c<T>(q.l[2]);
     }
     // tensor product, with w / 8 in the x factors: 14 products instead of 20
     T sx[2] = {shape_1d(x0, 0), shape_1d(x0, 1)};
@@ -558,6 +575,29 @@ __device__ __forceinline__ void spread_accumulate(
         acc[3 * a] = madd(Na, l0, acc[3 * a]);
         acc[3 * a + 1] = madd(Na, l1, acc[3 * a + 1]);
         acc[3 * a + 2] = madd(Na, l2, acc[3 * a + 2]);
+    }
+}
+
+// The points perm[p], perm[p + step], ... < hi, each one's inputs loaded while the one
+// before it is summed and its index one earlier still (two dependent reads in random
+// order took longer than a point's sums)
+template <typename T, bool SQ>
+__device__ __forceinline__ void spread_run(int p, int hi, int step,
+                                           const typename StorageOf<T>::type *__restrict__ xi,
+                                           const int32_t *__restrict__ perm,
+                                           const typename StorageOf<T>::type *__restrict__ lam,
+                                           const typename StorageOf<T>::type *__restrict__ w,
+                                           T (&acc)[24], T dsq)
+{
+    using St = typename StorageOf<T>::type;
+    if (p >= hi) return;
+    SpreadPoint<St> next = spread_load<St, SQ>(perm[p], xi, lam, w);
+    int b = hi - p > step ? perm[p + step] : 0;
+    for (; p < hi; p += step) {
+        const SpreadPoint<St> q = next;
+        if (hi - p > step) next = spread_load<St, SQ>(b, xi, lam, w);
+        if (hi - p > 2 * step) b = perm[p + 2 * step];
+        spread_accumulate<T, SQ>(q, w != nullptr, acc, dsq);
     }
 }
 
@@ -596,7 +636,7 @@ __device__ __forceinline__ void spread_cells_segment(
 #pragma unroll
         for (int k = 0; k < 24; ++k) acc[k] = T(0);
         if (group)
-            for (int p = lo + (lane & 3); p < hi; p += 4) spread_accumulate<T, SQ>(perm[p], xi, lam, w, acc, dsq);
+            spread_run<T, SQ>(lo + (lane & 3), hi, 4, xi, perm, lam, w, acc, dsq);
         const bool b1 = lane & 2, b0 = lane & 1;
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
@@ -626,7 +666,7 @@ __device__ __forceinline__ void spread_cells_segment(
         T acc[24];
 #pragma unroll
         for (int k = 0; k < 24; ++k) acc[k] = T(0);
-        for (int p = plo + lane; p < phi; p += 32) spread_accumulate<T, SQ>(perm[p], xi, lam, w, acc, dsq);
+        spread_run<T, SQ>(plo + lane, phi, 32, xi, perm, lam, w, acc, dsq);
         // each level halves the values a lane carries (12, 6, 3), then a
         // butterfly over the last two bits
         const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
