@@ -204,22 +204,33 @@ template <typename T>
 __global__ void __launch_bounds__(1024) batch_dense_sort_kernel(const DlmDesc<T> *desc, int count)
 {
     extern __shared__ int32_t sort_sh[];
-    // the instances' lists read as one: CTA b takes entries b, b + grid, ...
+    __shared__ int listed[1024];
+    // the instances' lists read as one: CTA b takes entries b, b + grid, ...; their
+    // lengths together (one dependent read after the other, 64 instances took most of
+    // the kernel's 61 us)
     int64_t g = blockIdx.x, base = 0;
-    for (int inst = 0; inst < count; ++inst) {
-        const DlmDesc<T> &D = desc[inst];
-        if (!D.X) continue;
-        const int n = D.tiles[D.ntiles];
-        for (; g < base + n; g += gridDim.x) {
-            const int c = D.fill[g - base];
-            const int lo = D.start[c];
-            const int len = (c < D.E ? D.start[c + 1] : (int)D.m) - lo;
-            int32_t *perm = const_cast<int32_t *>(D.perm);
-            for (int i = threadIdx.x; i < len; i += blockDim.x) perm[lo + i] = D.pairs[lo + i].x;
-            __syncthreads();
-            dlmd::block_sort_cell(D.E, D.m, D.start, perm, c, sort_sh);
+    for (int i0 = 0; i0 < count; i0 += 1024) {
+        const int ni = min(1024, count - i0);
+        if ((int)threadIdx.x < ni) {
+            const DlmDesc<T> &D = desc[i0 + threadIdx.x];
+            listed[threadIdx.x] = D.X ? D.tiles[D.ntiles] : 0;
         }
-        base += n;
+        __syncthreads();
+        for (int i = 0; i < ni; ++i) {
+            const int n = listed[i];
+            for (; g < base + n; g += gridDim.x) {
+                const DlmDesc<T> &D = desc[i0 + i];
+                const int c = D.fill[g - base];
+                const int lo = D.start[c];
+                const int len = (c < D.E ? D.start[c + 1] : (int)D.m) - lo;
+                int32_t *perm = const_cast<int32_t *>(D.perm);
+                for (int k = threadIdx.x; k < len; k += blockDim.x) perm[lo + k] = D.pairs[lo + k].x;
+                __syncthreads();
+                dlmd::block_sort_cell(D.E, D.m, D.start, perm, c, sort_sh);
+            }
+            base += n;
+        }
+        __syncthreads();  // `listed` is written again
     }
 }
 
