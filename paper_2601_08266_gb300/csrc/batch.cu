@@ -680,7 +680,9 @@ fsi_status fsi_batch_create(fsi_mesh *const *meshes, const fsi_batch_item *items
     {
         std::vector<int32_t> N(3 * (size_t)count);
         for (int i = 0; i < count; ++i) std::copy_n(meshes[i]->grid.N, 3, &N[3 * (size_t)i]);
-        b->brick = default_brick((const int32_t (*)[3])N.data(), count, prec, 2, b->sms);
+        Brick best[3][3];
+        default_bricks((const int32_t (*)[3])N.data(), count, b->sms, best);
+        b->brick = best[2][prec];
     }
     const size_t vsz = prec == FSI_F64 ? sizeof(vmsd::VmsArgs<double>) : sizeof(vmsd::VmsArgs<float>);
     const size_t dsz = prec == FSI_F64 ? sizeof(DlmDesc<double>) : sizeof(DlmDesc<float>);

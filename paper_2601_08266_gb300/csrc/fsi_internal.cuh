@@ -119,10 +119,10 @@ struct Brick {
     int threads;     // CTA size (multiple of 32; 4 lanes per bx x by column)
 };
 
-// Default brick schedule of one VMS operator (op 0 residual, 1 Jacobian apply, 2
-// both) in compute type prec for `count` grids run together (one mesh, or a
-// batch's instances), on sms SMs (vms.cu)
-Brick default_brick(const int32_t (*N)[3], int count, int prec, int op, int sms);
+// Default brick schedules of the VMS operators (best[op][prec], op 0 residual, 1
+// Jacobian apply, 2 both) for `count` grids run together (one mesh, or a batch's
+// instances), on sms SMs (vms.cu)
+void default_bricks(const int32_t (*N)[3], int count, int sms, Brick (&best)[3][3]);
 
 struct NewtonWorkspace;
 struct PressureMG;

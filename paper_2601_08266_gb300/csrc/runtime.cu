@@ -244,10 +244,7 @@ fsi_status fsi_mesh_create(const fsi_grid *grid, const fsi_physics *phys, int de
     m->n_nodes = n;
     m->n_elems = E;
     derive(m);
-    for (int op = 0; op < 3; ++op)
-        for (int p = 0; p < 3; ++p)
-            m->brick[op][p] = op == 1 ? m->brick[0][p]  // the residual's rule too
-                                      : default_brick(&m->grid.N, 1, p, op, sm_count());
+    default_bricks(&m->grid.N, 1, sm_count(), m->brick);
     fsi_status st = FSI_OK;
     // cell-hash scratch: fill counters [E+1], scan scratch, counters; both
     // start at zero and every cell-table build leaves them so

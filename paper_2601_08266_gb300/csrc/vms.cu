@@ -18,6 +18,7 @@
 //     that contain it in a fixed brick order.  The result is deterministic
 //     (bitwise reproducible) and atomic-free.
 #include <algorithm>
+#include <vector>
 #include <cmath>
 #include <cstring>
 #include <type_traits>
@@ -173,6 +174,8 @@ fsi_status launch_fused(fsi_mesh *m, const void *U, const void *A, const void *f
     return launch_geo<T, true, false, true>(m, U, A, f, x, Jx, R);
 }
 
+}  // namespace
+
 // Cost of a schedule in units of one warp's share of an element layer (8
 // columns): the warps' work over the SMs plus a quarter of one CTA's own
 // duration as the tail, but no less than one CTA alone takes.  `alone` is how much
@@ -181,38 +184,57 @@ fsi_status launch_fused(fsi_mesh *m, const void *U, const void *A, const void *f
 // 10 : 1 in double-float and 16 : 1 in FP32.  A brick of bz layers spends 0.3 of a
 // layer more (its lowest plane, the carried parts), and its rim nodes go through
 // the node blocks.
-double brick_cost(const int32_t (*N)[3], int count, const Brick &b, double alone, int sms)
+// One sweep over the schedules for every type and operator (they share all but
+// `alone` and the height): each mesh created runs it.
+void default_bricks(const int32_t (*N)[3], int count, int sms, Brick (&best)[3][3])
 {
-    const double layer = b.bz + 0.3;
-    const double rim = 1.0 + 0.06 * ((b.bx + 1.0) * (b.by + 1.0) / (b.bx * b.by) - 1.0);
-    double ctas = 0.0;
-    for (int i = 0; i < count; ++i)
-        ctas += (double)((N[i][0] + b.bx - 1) / b.bx) * ((N[i][1] + b.by - 1) / b.by) *
-                ((N[i][2] + b.bz - 1) / b.bz);
-    const double work = ctas / sms * (b.threads / 32) * layer * rim;
-    return std::max(work + 0.25 * alone * layer, alone * layer) + 0.01 * work;
-}
-
-}  // namespace
-
-Brick default_brick(const int32_t (*N)[3], int count, int prec, int op, int sms)
-{
-    const double alone = prec == FSI_F64 ? 4.0 : (prec == FSI_DF64 ? 10.0 : 16.0);
-    // both operators in an 8-byte type: taller bricks leave one CTA per SM
-    const int max_bz = op == 2 && prec != FSI_F32 ? 4 : 8;
-    Brick best{8, 4, max_bz, 128};
-    double cost = 1e300;
-    for (int bz = max_bz; bz >= 1; --bz)
-        for (int by = 1; by <= 16; ++by)
+    // of an 8-byte type both operators at once take lower bricks
+    // (taller ones leave one CTA per SM); the Jacobian goes by the residual's rule
+    constexpr int kRules = 5;
+    const struct {
+        double alone;
+        int max_bz;
+    } rule[kRules] = {{4.0, 8}, {16.0, 8}, {10.0, 8}, {4.0, 4}, {10.0, 4}};
+    Brick pick[kRules];
+    double cost[kRules];
+    for (int q = 0; q < kRules; ++q) {
+        pick[q] = {8, 4, rule[q].max_bz, 128};
+        cost[q] = 1e300;
+    }
+    // bricks along each axis by brick size
+    std::vector<double> along[3], yz(count);
+    for (int d = 0; d < 3; ++d) {
+        along[d].resize((size_t)16 * count);
+        for (int v = 1; v <= 16; ++v)
+            for (int i = 0; i < count; ++i) along[d][(size_t)(v - 1) * count + i] = (N[i][d] + v - 1) / v;
+    }
+    for (int bz = 8; bz >= 1; --bz)
+        for (int by = 1; by <= 16; ++by) {
+            for (int i = 0; i < count; ++i)
+                yz[i] = along[1][(size_t)(by - 1) * count + i] * along[2][(size_t)(bz - 1) * count + i];
             for (int bx = 1; bx * by <= 32 && bx <= 16; ++bx) {
                 const Brick b{bx, by, bz, (4 * bx * by + 31) / 32 * 32};
-                const double c = brick_cost(N, count, b, alone, sms);
-                if (c < cost * (1.0 - 1e-9)) {
-                    cost = c;
-                    best = b;
+                double ctas = 0.0;
+                for (int i = 0; i < count; ++i) ctas += along[0][(size_t)(bx - 1) * count + i] * yz[i];
+                const double layer = bz + 0.3;
+                const double rim = 1.0 + 0.06 * ((bx + 1.0) * (by + 1.0) / (bx * by) - 1.0);
+                const double work = ctas / sms * (b.threads / 32) * layer * rim;
+                for (int q = 0; q < kRules; ++q) {
+                    if (bz > rule[q].max_bz) continue;
+                    const double alone = rule[q].alone * layer,
+                                 c = std::max(work + 0.25 * rule[q].alone * layer, alone) + 0.01 * work;
+                    if (c < cost[q] * (1.0 - 1e-9)) {
+                        cost[q] = c;
+                        pick[q] = b;
+                    }
                 }
             }
-    return best;
+        }
+    for (int op = 0; op < 3; ++op) {
+        best[op][FSI_F64] = pick[op == 2 ? 3 : 0];
+        best[op][FSI_F32] = pick[1];
+        best[op][FSI_DF64] = pick[op == 2 ? 4 : 2];
+    }
 }
 
 namespace {
