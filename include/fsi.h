@@ -812,11 +812,12 @@ fsi_status fsi_mesh_set_brick(fsi_mesh *mesh, int op, fsi_prec prec, int bx, int
 
 /* Autotuner of a single structured mesh: times the VMS residual (op 0),
  * Jacobian apply (op 1) or both fused (op 2, fsi_residual_jacobian_apply) in
- * compute type `prec` on scratch inputs for a fixed
- * set of brick shapes (8x8x4, 8x4x4, 8x8x2, 4x4x4, 4x4x8, 16x4x4 at 256
- * threads; 8x4x4, 4x4x4, 8x4x2, 4x4x2 at 128) and keeps the fastest, as
- * fsi_mesh_set_brick would.  Each compute type (FSI_F64, FSI_F32,
- * FSI_DF64) has its own schedule per operator.  The report's cand_ctas holds each
+ * compute type `prec` on scratch inputs for the mesh's present schedule, which
+ * is the first candidate, and nine of a fixed set (8x8x4, 8x4x4, 8x8x2, 16x4x4,
+ * 8x4x2 at 128 threads, 4x4x4, 4x4x8, 4x4x2, 8x2x4 at 64, 4x2x4 at 32), and
+ * keeps the fastest, as fsi_mesh_set_brick would.  Each compute type (FSI_F64,
+ * FSI_F32, FSI_DF64) has its own schedule per operator.  The report names the
+ * schedules as they run (threads included); its cand_ctas holds each
  * candidate's CTA size, ctas_per_sm is 0; seconds is per launch (brick and
  * gather kernels, mean of reps after one warm-up).  Synchronises; results
  * of later calls do not depend on the schedule's choice beyond rounding

@@ -239,11 +239,13 @@ void default_bricks(const int32_t (*N)[3], int count, int sms, Brick (&best)[3][
 
 namespace {
 
-// candidate brick shapes of the single-mesh autotuner (fit_brick halves the ones
-// wider than a CTA has lanes for)
+// Candidate schedules of the single-mesh autotuner beside the one the mesh has: the
+// first of these, as fit_brick makes them, that differ from it and from each other, up
+// to kMeshCandidates in all
+constexpr int kMeshCandidates = 10;
 const Brick kMeshBricks[] = {
-    {8, 8, 4, 256}, {8, 4, 4, 256}, {8, 8, 2, 256}, {4, 4, 4, 256}, {4, 4, 8, 256},
-    {16, 4, 4, 256}, {8, 4, 4, 128}, {4, 4, 4, 128}, {8, 4, 2, 128}, {4, 4, 2, 128},
+    {8, 8, 4, 128}, {8, 4, 4, 128}, {8, 8, 2, 128}, {4, 4, 4, 64}, {4, 4, 8, 64},
+    {16, 4, 4, 128}, {8, 4, 2, 128}, {4, 4, 2, 64}, {8, 2, 4, 64}, {4, 2, 4, 32},
 };
 
 template <typename S> __global__ void fill_state_kernel(int64_t n, vec4<S> *U, vec4<S> *A, vec4<S> *x)
@@ -278,6 +280,7 @@ fsi_status time_op(fsi_mesh *m, int op, int reps, const void *U, const void *A, 
     return FSI_OK;
 }
 
+static_assert(kMeshCandidates <= FSI_TUNE_MAX_CANDIDATES, "the report holds every candidate");
 template <typename T> fsi_status autotune(fsi_mesh *m, int op, int reps, fsi_tune_report *rep)
 {
     using S = typename StorageOf<T>::type;
@@ -295,27 +298,39 @@ template <typename T> fsi_status autotune(fsi_mesh *m, int op, int reps, fsi_tun
     if (st == FSI_OK &&
         (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess))
         st = set_error(FSI_ERR_CUDA, "fsi_mesh_autotune: cudaEventCreate failed");
+    // the present schedule is the first candidate and the one to beat
+    const bool jac = op > 0, fused = op == 2;
+    std::vector<Brick> cands(1, fit_brick(start, (int)sizeof(T), jac, fused));
+    for (const Brick &b : kMeshBricks) {
+        const Brick c = fit_brick(b, (int)sizeof(T), jac, fused);
+        bool seen = false;
+        for (const Brick &o : cands)
+            seen = seen || (o.bx == c.bx && o.by == c.by && o.bz == c.bz && o.threads == c.threads);
+        if (!seen && (int)cands.size() < kMeshCandidates) cands.push_back(c);
+    }
     double best = 1e30;
     Brick best_brick = start;
     int tried = 0;
+    auto time_brick = [&](const Brick &b, double *t) {
+        m->brick[op][slot] = b;
+        return time_op<T>(m, op, reps, buf[0], buf[1], buf[2], buf[3], buf[4], e0, e1, t);
+    };
     if (st == FSI_OK) {
         fill_state_kernel<S><<<sm_count() * 4, 256, 0, m->stream>>>(m->n_nodes, (vec4<S> *)buf[0],
                                                              (vec4<S> *)buf[1], (vec4<S> *)buf[2]);
         st = check_launch("autotune fill");
     }
-    for (const Brick &cand : kMeshBricks) {
+    double t = 0.0;
+    if (st == FSI_OK) st = time_brick(start, &t);  // not counted: the clocks come up
+    for (const Brick &cand : cands) {
         if (st != FSI_OK) break;
-        m->brick[op][slot] = cand;
-        double t = 0.0;
-        st = time_op<T>(m, op, reps, buf[0], buf[1], buf[2], buf[3], buf[4], e0, e1, &t);
+        st = time_brick(cand, &t);
         if (st != FSI_OK) break;
-        if (tried < FSI_TUNE_MAX_CANDIDATES) {
-            rep->cand_bx[tried] = cand.bx;
-            rep->cand_by[tried] = cand.by;
-            rep->cand_bz[tried] = cand.bz;
-            rep->cand_ctas[tried] = cand.threads;
-            rep->cand_seconds[tried] = t;
-        }
+        rep->cand_bx[tried] = cand.bx;
+        rep->cand_by[tried] = cand.by;
+        rep->cand_bz[tried] = cand.bz;
+        rep->cand_ctas[tried] = cand.threads;
+        rep->cand_seconds[tried] = t;
         ++tried;
         if (t < best) {
             best = t;
@@ -328,7 +343,7 @@ template <typename T> fsi_status autotune(fsi_mesh *m, int op, int reps, fsi_tun
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     if (st != FSI_OK) return st;
-    rep->n_candidates = tried < FSI_TUNE_MAX_CANDIDATES ? tried : FSI_TUNE_MAX_CANDIDATES;
+    rep->n_candidates = tried;
     rep->bx = best_brick.bx;
     rep->by = best_brick.by;
     rep->bz = best_brick.bz;
