@@ -793,9 +793,11 @@ typedef struct {
     double cand_seconds[FSI_TUNE_MAX_CANDIDATES];
 } fsi_tune_report;
 
-/* Autotuner: times every candidate brick shape (elements per CTA along each
- * axis, CTA size) and persistent grid size (CTAs per SM) on this batch's
- * residual + Jacobian phases and keeps the fastest.  When the environment
+/* Autotuner: times the batch's present schedule, which is the first candidate,
+ * then its brick and a fixed set of brick shapes (elements per CTA along each
+ * axis) with every persistent grid size (CTAs of 128 threads per SM: 1, 2, 4, 8) on
+ * this batch's residual + Jacobian phases and keeps the fastest.  The report names
+ * the schedules as they run.  When the environment
  * variable FSI_TUNE_CACHE names a file, the choice is appended to it as one
  * JSON object per line.  Synchronises.                                     */
 fsi_status fsi_batch_autotune(fsi_batch *batch, int reps, fsi_tune_report *report);

@@ -632,10 +632,14 @@ fsi_status time_mode(fsi_batch *b, int mode, int phases, int reps, double *out)
     return st;
 }
 
+// candidate bricks of the batch autotuner beside the batch's own
 const fsi::Brick kBrickCandidates[] = {
-    {8, 8, 4, 256}, {8, 4, 4, 128}, {4, 4, 4, 64}, {16, 4, 4, 256}, {8, 8, 2, 128},
-    {16, 8, 2, 256}, {4, 4, 8, 128}, {8, 4, 8, 256},
+    {8, 8, 4, 128}, {8, 4, 4, 128}, {4, 4, 4, 64}, {16, 4, 4, 128}, {8, 8, 2, 128},
+    {16, 8, 2, 128}, {4, 4, 8, 64}, {8, 4, 8, 128},
 };
+constexpr int kCtasPerSm[] = {1, 2, 4, 8};
+static_assert((std::size(kBrickCandidates) + 1) * std::size(kCtasPerSm) + 1 <= FSI_TUNE_MAX_CANDIDATES,
+              "the report holds every candidate");
 
 }  // namespace
 }  // namespace fsi
@@ -732,36 +736,56 @@ fsi_status fsi_batch_autotune(fsi_batch *b, int reps, fsi_tune_report *rep)
     std::memset(rep, 0, sizeof *rep);
     const Brick start = b->brick;
     const int start_ctas = b->ctas_per_sm;
+    // the present schedule is the first candidate and the one to beat; then its brick
+    // and the listed ones with every grid size, each launch once
+    struct Cand {
+        Brick b;
+        int ctas;
+    };
+    auto as_run = [&](const Brick &c) {
+        return vmsd::fit_brick(c, b->prec == FSI_F64 ? 8 : 4, true, true);
+    };
+    std::vector<Cand> cands(1, Cand{as_run(start), start_ctas});
+    auto add = [&](const Brick &c, int ctas) {
+        for (const Cand &o : cands)
+            if (o.b.bx == c.bx && o.b.by == c.by && o.b.bz == c.bz && o.b.threads == c.threads &&
+                o.ctas == ctas)
+                return;
+        cands.push_back(Cand{c, ctas});
+    };
+    for (int ctas : kCtasPerSm) add(as_run(start), ctas);
+    for (const Brick &c : kBrickCandidates)
+        for (int ctas : kCtasPerSm) add(as_run(c), ctas);
     double best = 1e30;
     Brick best_brick = start;
     int best_ctas = start_ctas;
     int tried = 0;
-    for (const Brick &cand : kBrickCandidates) {
-        for (int ctas : {1, 2, 4, 8}) {
-            b->brick = cand;
-            b->ctas_per_sm = ctas;
-            FSI_TRY(b->prec == FSI_F64 ? build_batch<double>(b) : build_batch<float>(b));
-            double t = 0.0;
-            FSI_TRY(time_mode(b, FSI_BATCH_PERSISTENT, 1, reps, &t));
-            if (tried < FSI_TUNE_MAX_CANDIDATES) {
-                rep->cand_bx[tried] = cand.bx;
-                rep->cand_by[tried] = cand.by;
-                rep->cand_bz[tried] = cand.bz;
-                rep->cand_ctas[tried] = ctas;
-                rep->cand_seconds[tried] = t;
-            }
-            ++tried;
-            if (t < best) {
-                best = t;
-                best_brick = cand;
-                best_ctas = ctas;
-            }
+    auto time_cand = [&](const Cand &c, double *t) -> fsi_status {
+        b->brick = c.b;
+        b->ctas_per_sm = c.ctas;
+        FSI_TRY(b->prec == FSI_F64 ? build_batch<double>(b) : build_batch<float>(b));
+        return time_mode(b, FSI_BATCH_PERSISTENT, 1, reps, t);
+    };
+    double t = 0.0;
+    FSI_TRY(time_cand(cands[0], &t));  // not counted: the clocks come up
+    for (const Cand &c : cands) {
+        FSI_TRY(time_cand(c, &t));
+        rep->cand_bx[tried] = c.b.bx;
+        rep->cand_by[tried] = c.b.by;
+        rep->cand_bz[tried] = c.b.bz;
+        rep->cand_ctas[tried] = c.ctas;
+        rep->cand_seconds[tried] = t;
+        ++tried;
+        if (t < best) {
+            best = t;
+            best_brick = c.b;
+            best_ctas = c.ctas;
         }
     }
     b->brick = best_brick;
     b->ctas_per_sm = best_ctas;
     FSI_TRY(b->prec == FSI_F64 ? build_batch<double>(b) : build_batch<float>(b));
-    rep->n_candidates = tried < FSI_TUNE_MAX_CANDIDATES ? tried : FSI_TUNE_MAX_CANDIDATES;
+    rep->n_candidates = tried;
     rep->bx = best_brick.bx;
     rep->by = best_brick.by;
     rep->bz = best_brick.bz;

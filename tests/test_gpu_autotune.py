@@ -38,3 +38,32 @@ def test_mesh_autotune_starts_from_the_present_brick(fsi, op, prec, brick, runs)
     again = fsi.fsi_mesh_autotune(mesh, op, P, reps=2)["candidates"][0]
     assert (again[0], again[1]) == (t["brick"], t["threads"])
     mesh.close()
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+def test_batch_autotune_starts_from_the_present_schedule(fsi, prec):
+    import torch
+    P, dt = (fsi.FSI_F64, torch.float64) if prec == "f64" else (fsi.FSI_F32, torch.float32)
+    s = torch.cuda.Stream()
+    meshes, items = [], []
+    for N in [(3, 5, 2), (6, 2, 7), (5, 5, 5)]:
+        mesh = fsi.Mesh(N, device=0, stream=s.cuda_stream)
+        nodal = lambda: torch.rand((mesh.n_nodes, 4), dtype=dt, device="cuda")
+        it = {k: nodal() for k in ("U", "A", "x", "R", "Jx", "F")}
+        it["cell_start"] = torch.zeros(mesh.n_elems + 1, dtype=torch.int32, device="cuda")
+        meshes.append(mesh)
+        items.append(it)
+    torch.cuda.synchronize()
+    b = fsi.Batch(meshes, items, P, s.cuda_stream)
+    t = b.autotune(reps=2)
+    c = t["candidates"]
+    # grids this small start with bricks of their own size, which the fixed list
+    # (at least 4 x 4 x 4) does not hold
+    assert c[0][0] * c[0][1] * c[0][2] < 64 and c[0][3] == 4
+    assert len({k[:4] for k in c}) == len(c)
+    assert t["seconds"] <= c[0][4]
+    again = b.autotune(reps=2)["candidates"][0]
+    assert (again[:3], again[3]) == (t["brick"], t["ctas_per_sm"])
+    b.close()
+    for m in meshes:
+        m.close()
