@@ -94,7 +94,7 @@ __global__ void locate_kernel(int64_t m, GridArgs g, const double *__restrict__ 
                               int32_t *__restrict__ arrival)
 {
     chain_wait(X, elem, xi, count, n_out, arrival);
-    chain_trigger();
+    if (count) chain_trigger();  // the cell table follows; else it may be any kernel
     const int64_t E = (int64_t)g.Nx * g.Ny * g.Nz;
     for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < m;
          b += (int64_t)gridDim.x * blockDim.x) {
@@ -688,7 +688,7 @@ __global__ void rank_place_kernel(int64_t m, int64_t E, const int32_t *__restric
                                   int32_t *dense, int32_t *scr)
 {
     chain_wait(start, tmp, perm, dense, scr);
-    chain_trigger();
+    if (m > kWarpSortMax) chain_trigger();  // dense_pairs_kernel follows; else any kernel
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < m;
          k += (int64_t)gridDim.x * blockDim.x) {
         const int2 p = tmp[k];
@@ -745,7 +745,6 @@ __global__ void interp_kernel(int64_t m, GridArgs g, const int32_t *__restrict__
                               S *__restrict__ u)
 {
     chain_wait(elem, xi, U, u);
-    chain_trigger();
     if constexpr (std::is_same<T, float>::value) {
         const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
         const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -757,6 +756,8 @@ __global__ void interp_kernel(int64_t m, GridArgs g, const int32_t *__restrict__
              b += (int64_t)gridDim.x * blockDim.x)
             interp_point<T>(g, b, elem, xi, U, u);
     }
+    __syncthreads();  // the CTA has read everything (see chain_trigger)
+    chain_trigger();
 }
 
 // Spreading, pass 1: one warp per segment of kSpreadSeg consecutive cells

@@ -64,11 +64,22 @@ fsi_status set_smem_limit(const void *kernel, int bytes);
 // that it reads and writes through, so that no access can be moved before it (loads
 // through read-only pointers otherwise might).
 //
-// chain_trigger() lets the next kernel start.  After chain_wait() only these two can
-// be running then, and the next one's reads are safe if this one does not read
-// what it writes: its CTAs start with an empty L1.  Before chain_wait() (the V-cycle) two
-// kernels back may still be running and fill this SM's L1 with lines that the one
-// between them then writes, so what the chain writes is read with __ldcg.
+// chain_trigger() lets the next kernel start, and with it the time in which this
+// kernel's reads fill the L1 that the next one will read through.  Where it stands:
+//   - After chain_wait(), at once, in a kernel that reads no 32-byte sector which the
+//     next kernel reads and this one writes: the next kernel is known and reads
+//     scratch of the library's own, or this one reads nothing else.  (Only these
+//     two can be running then.)
+//   - After the last read of the CTA (__syncthreads() before it) or not at all in
+//     a kernel that reads a caller's arrays and writes a caller's arrays while the
+//     next kernel is the caller's choice: two of the arrays may share a sector (packed
+//     into one allocation), and the next kernel may read the one just written.
+//   - Not at all in a kernel that reads what it writes.
+//   - Before chain_wait() in the V-cycle, whose kernels read what the chain writes
+//     with __ldcg (past the L1): two kernels back may still be running then.
+// A kernel that starts to read what it writes, or gets another successor, needs its
+// trigger looked at again; test_gpu_overlap.py runs the chains back to back, on
+// packed arrays and under capture.
 template <typename P> __device__ __forceinline__ void chain_pin(P &p) { asm volatile("" : "+l"(p)); }
 __device__ __forceinline__ void chain_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
 template <typename... P> __device__ __forceinline__ void chain_wait(P &...p)

@@ -43,7 +43,7 @@ constexpr int kBrickCtas = sizeof(T) == 4 ? 4 : (std::is_same<T, double>::value 
 template <typename T, bool JAC, bool MAPPED, bool FUSED = false>
 __global__ void __launch_bounds__(kBrickThreads, (kBrickCtas<T, FUSED>)) vms_brick_kernel(const VmsArgs<T> P)
 {
-    chain_trigger();
+    if (P.nbx * P.nby * P.nbz > 1) chain_trigger();  // the gather follows; else any kernel
     extern __shared__ __align__(32) unsigned char smem_raw[];
     brick_body<T, JAC, MAPPED, FUSED>(P, blockIdx.x, smem_raw);
 }
