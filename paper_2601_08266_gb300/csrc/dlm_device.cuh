@@ -465,7 +465,7 @@ __device__ __forceinline__ void interp_point(
         for (int a = 0; a < 8; ++a) {
             const int ax = a & 1, ay = (a >> 1) & 1, az = (a >> 2) & 1;
             const T Na = sxy[a & 3] * shape_1d(x2, az);
-            const auto v = ld4(U + n0 + ax + NX1 * ay + NXY1 * az);
+            const auto v = ld4_chain(U + n0 + ax + NX1 * ay + NXY1 * az);
             ux = madd(Na, to_c<T>(v.x), ux);
             uy = madd(Na, to_c<T>(v.y), uy);
             uz = madd(Na, to_c<T>(v.z), uz);
@@ -506,7 +506,7 @@ __device__ __forceinline__ void interp_point_pair(
         for (int q = 0; q < 4; ++q) {
             const int ay = q & 1, az = q >> 1;
             const T Na = sx * shape_1d(x1, ay) * shape_1d(x2, az) * T(0.125f);
-            const auto v = ld4(U + n0 + NX1 * ay + NXY1 * az);
+            const auto v = ld4_chain(U + n0 + NX1 * ay + NXY1 * az);
             ux = madd(Na, to_c<T>(v.x), ux);
             uy = madd(Na, to_c<T>(v.y), uy);
             uz = madd(Na, to_c<T>(v.z), uz);

@@ -100,7 +100,7 @@ __device__ __forceinline__ void load_tasks(const float *__restrict__ p, int64_t 
             for (int h = 0; h < 2; ++h) {
                 float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (in && gk + 4 * h < K)
-                    f = __ldg(reinterpret_cast<const float4 *>(p + (int64_t)gr * ld + gk + 4 * h));
+                    f = *reinterpret_cast<const float4 *>(p + (int64_t)gr * ld + gk + 4 * h);
                 v[t][4 * h] = f.x;
                 v[t][4 * h + 1] = f.y;
                 v[t][4 * h + 2] = f.z;
@@ -111,7 +111,7 @@ __device__ __forceinline__ void load_tasks(const float *__restrict__ p, int64_t 
             for (int j = 0; j < 8; ++j) {
                 v[t][j] = 0.f;
                 if (in && gk + j < K)
-                    v[t][j] = __ldg(KC ? p + (int64_t)gr * ld + gk + j : p + (int64_t)(gk + j) * ld + gr);
+                    v[t][j] = KC ? p[(int64_t)gr * ld + gk + j] : p[(int64_t)(gk + j) * ld + gr];
             }
         }
     }
@@ -236,8 +236,8 @@ __device__ __forceinline__ void gemm_body(const TcGemm &g, int cta, int *err, ui
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 if (gj0 + j >= g.N) break;
-                if (g.epi == TC_EPI_BIAS || g.epi == TC_EPI_BIAS_RELU) v[j] += __ldg(g.bias + gj0 + j);
-                if (g.epi == TC_EPI_MASK) v[j] = __ldg(g.mask + o + j) > 0.f ? v[j] : 0.f;
+                if (g.epi == TC_EPI_BIAS || g.epi == TC_EPI_BIAS_RELU) v[j] += g.bias[gj0 + j];
+                if (g.epi == TC_EPI_MASK) v[j] = g.mask[o + j] > 0.f ? v[j] : 0.f;
             }
             if (g.vec & 4) {  // whole 16-byte pieces: N and ldc multiples of 8
                 if (g.epi == TC_EPI_BIAS_RELU) {

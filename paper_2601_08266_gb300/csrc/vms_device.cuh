@@ -26,17 +26,17 @@ template <typename T> __device__ __forceinline__ T cB2() { return T(kB2); }
 template <> __device__ __forceinline__ df64 cB1<df64>() { return df64(kB1h, kB1l); }
 template <> __device__ __forceinline__ df64 cB2<df64>() { return df64(kB2h, kB2l); }
 
-// node record of double-float values (two float4 loads)
-__device__ __forceinline__ vec4<df64> ld4_df(const vec4<df64> *p)
+// record that the kernel before in the chain wrote, in compute type (double-float:
+// two float4 loads)
+template <typename T> __device__ __forceinline__ vec4<T> ld4_blk(const vec4<T> *p)
 {
-    const float4 *q = reinterpret_cast<const float4 *>(p);
-    const float4 a = __ldg(q), b = __ldg(q + 1);
-    return {df64(a.x, a.y), df64(a.z, a.w), df64(b.x, b.y), df64(b.z, b.w)};
+    return ld4_chain(p);
 }
-template <typename T> __device__ __forceinline__ vec4<T> ld4_blk(const vec4<T> *p) { return ld4(p); }
 template <> __device__ __forceinline__ vec4<df64> ld4_blk<df64>(const vec4<df64> *p)
 {
-    return ld4_df(p);
+    const float4 *q = reinterpret_cast<const float4 *>(p);
+    const float4 a = ldg_chain(q), b = ldg_chain(q + 1);
+    return {df64(a.x, a.y), df64(a.z, a.w), df64(b.x, b.y), df64(b.z, b.w)};
 }
 
 // Per-Gauss-point geometry of a mapped grid, built once per coordinate set and
