@@ -52,7 +52,7 @@ constexpr int BK = 64;        // K per stage (4 MMAs of K = 16)
 constexpr int KCH = BK / 8;   // 16-byte chunks along K in a stage
 constexpr int kThreads = 256;
 constexpr uint32_t SZ_A = TM * BK * 2;      // 16 KB
-constexpr int kMaxBN = 64;
+constexpr int kMaxBN = kGemmMaxBN;
 constexpr uint32_t SZ_B = kMaxBN * BK * 2;  // 8 KB
 constexpr uint32_t SZ_STAGE = SZ_A + SZ_B;
 constexpr uint32_t SMEM_BYTES = 2 * SZ_STAGE;  // 48 KB
@@ -224,22 +224,23 @@ __device__ __forceinline__ void gemm_body(const TcGemm &g, int cta, int *err, ui
 #pragma unroll
                 for (int j = 0; j < 8; ++j) v[j] = 0.f;
             if (gi >= g.M) continue;
-            const int gj0 = n0 + 8 * c8;
+            const int gj0 = n0 + 8 * c8, nc = gemm_piece_columns(gj0, g.N);
+            if (nc == 0) continue;
             if (g.splits > 1) {  // partial sum of a K slice
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
-                    if (gj0 + j < g.N) g.work[((int64_t)z * g.M + gi) * g.N + gj0 + j] = v[j];
+                    if (j < nc) g.work[((int64_t)z * g.M + gi) * g.N + gj0 + j] = v[j];
                 continue;
             }
             const int64_t o = (int64_t)gi * g.ldc + gj0;
             // bias, pre-activation, ReLU or mask
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                if (gj0 + j >= g.N) break;
+                if (j >= nc) break;
                 if (g.epi == TC_EPI_BIAS || g.epi == TC_EPI_BIAS_RELU) v[j] += g.bias[gj0 + j];
                 if (g.epi == TC_EPI_MASK) v[j] = g.mask[o + j] > 0.f ? v[j] : 0.f;
             }
-            if (g.vec & 4) {  // whole 16-byte pieces: N and ldc multiples of 8
+            if ((g.vec & 4) && nc == 8) {  // whole 16-byte pieces, see tc_gemm_group
                 if (g.epi == TC_EPI_BIAS_RELU) {
                     if (g.Cpre) {
                         *reinterpret_cast<float4 *>(g.Cpre + o) = make_float4(v[0], v[1], v[2], v[3]);
@@ -254,7 +255,7 @@ __device__ __forceinline__ void gemm_body(const TcGemm &g, int cta, int *err, ui
             }
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                if (gj0 + j >= g.N) break;
+                if (j >= nc) break;
                 if (g.epi == TC_EPI_BIAS_RELU) {
                     if (g.Cpre) g.Cpre[o + j] = v[j];
                     v[j] = v[j] > 0.f ? v[j] : 0.f;
@@ -336,7 +337,7 @@ fsi_status tc_gemm_group(cudaStream_t s, const TcGemm *gs, int n, float *work, i
         g = gs[q];
         if (g.M <= 0 || g.N <= 0 || g.K <= 0 || g.N > 256)
             return set_error(FSI_ERR_ARG, "tensor-core GEMM: bad shape %d x %d x %d", g.M, g.N, g.K);
-        g.BN = g.N >= kMaxBN ? kMaxBN : (g.N + 15) / 16 * 16;
+        g.BN = gemm_tile_columns(g.N);
         const int mt = (g.M + TM - 1) / TM, nt = (g.N + g.BN - 1) / g.BN;
         const int nchunks = (g.K + BK - 1) / BK;
         // split K when 256-column tiles alone would leave most SMs idle and K is

@@ -27,6 +27,19 @@ __host__ __device__ __forceinline__ uint32_t kmaj(uint32_t row, uint32_t k, uint
     return (row >> 3) * (kc * 128u) + (k >> 3) * 128u + (row & 7u) * 16u + (k & 7u) * 2u;
 }
 
+// GEMM output tiles: the columns of a tile of an N-column output (N <= 256), and how
+// many of the 8 columns from j on the output has (a tile is a multiple of 16
+// wide, so its last pieces of 8 may lie beyond the output)
+constexpr int kGemmMaxBN = 64;
+__host__ __device__ __forceinline__ int gemm_tile_columns(int N)
+{
+    return N >= kGemmMaxBN ? kGemmMaxBN : (N + 15) / 16 * 16;
+}
+__host__ __device__ __forceinline__ int gemm_piece_columns(int j, int N)
+{
+    return j >= N ? 0 : (N - j < 8 ? N - j : 8);
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
 {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
