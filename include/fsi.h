@@ -805,10 +805,13 @@ fsi_status fsi_batch_autotune(fsi_batch *batch, int reps, fsi_tune_report *repor
 /* Brick schedule of a single mesh for op 0 (residual), 1 (Jacobian) or 2
  * (both fused; twice the shared memory) in compute type
  * `prec` (FSI_F64, FSI_F32 or FSI_DF64, each its own): bx*by columns of bz elements per CTA of `threads` threads (4 lanes
- * per column; threads a multiple of 32 and at most 256).  A brick wider than the
- * CTA has lanes for, or than its shared memory holds, is halved along its longest
- * side until it fits; CTAs larger than 128 threads are not used.  Scratch grows
- * as needed.  Without this call the library picks a schedule from the grid's size. */
+ * per column; threads a multiple of 32 and at most 256).  FSI_ERR_ARG for a brick
+ * of more than 800 elements (FSI_F32: 1,600; op 2: half of either).  A CTA runs
+ * with at most 128 threads and no more than the brick's columns have lanes for; a
+ * wider brick takes several passes over its columns.  A brick whose sums do
+ * not fit the shared memory (200 KB) is halved along its longest side until they
+ * do.  Scratch grows as needed.  Without this call the library picks a schedule
+ * from the grid's size.                                                    */
 fsi_status fsi_mesh_set_brick(fsi_mesh *mesh, int op, fsi_prec prec, int bx, int by, int bz,
                               int threads);
 

@@ -378,10 +378,10 @@ fsi_status fsi_mesh_set_brick(fsi_mesh *m, int op, fsi_prec prec, int bx, int by
         return set_error(FSI_ERR_ARG, "bad op or precision");
     if (bx < 1 || by < 1 || bz < 1 || threads < 32 || threads > 256 || threads % 32 != 0)
         return set_error(FSI_ERR_ARG, "bad brick %dx%dx%d / %d threads", bx, by, bz, threads);
-    const size_t smem = (op == 2 ? 2 : 1) * (size_t)bx * by * bz * 8 * 4 * (prec == FSI_F32 ? 4 : 8);
-    if (smem > 200 * 1024)
-        return set_error(FSI_ERR_ARG, "brick %dx%dx%d needs %zu bytes of shared memory", bx, by,
-                         bz, smem);
+    const int most = (prec == FSI_F32 ? 1600 : 800) / (op == 2 ? 2 : 1);
+    if (bx > most || by > most || bz > most || (int64_t)bx * by * bz > most)
+        return set_error(FSI_ERR_ARG, "brick %dx%dx%d: more than %d elements (operator %d in this type)",
+                         bx, by, bz, most, op);
     m->brick[op][prec] = Brick{bx, by, bz, threads};
     return FSI_OK;
 }

@@ -49,3 +49,21 @@ def test_brick_schedules(oracle, prec, N):
             e = parity.rel_local(got.double().cpu().numpy(), ref, N)
             assert e < TOL[prec], (b, e)
     mesh.close()
+
+
+# as include/fsi.h states them
+@pytest.mark.parametrize("prec,op,most", [("f64", 0, 800), ("f64", 2, 400), ("df64", 1, 800),
+                                          ("df64", 2, 400), ("f32", 1, 1600), ("f32", 2, 800)])
+def test_brick_size_limit(prec, op, most):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2601_08266_gb300 as fsi
+    P = {"f64": fsi.FSI_F64, "f32": fsi.FSI_F32, "df64": fsi.FSI_DF64}[prec]
+    mesh = fsi.Mesh((3, 2, 2), device=0)
+    for b in [(most // 8, 4, 2), (1, 1, most), (20, most // 20, 1)]:
+        fsi.fsi_mesh_set_brick(mesh, op, P, *b, 128)
+    for b in [(most // 8, 4, 3), (1, 1, most + 1), (2 ** 20, 2 ** 20, 2 ** 20), (2 ** 30, 4, 1)]:
+        with pytest.raises(fsi.FsiError, match=f"more than {most} elements"):
+            fsi.fsi_mesh_set_brick(mesh, op, P, *b, 128)
+    mesh.close()
