@@ -365,6 +365,13 @@ fsi_status fsi_tet_spread(fsi_tetmesh *mesh, fsi_prec prec, int64_t m, const int
  * returns, and the context stays usable.  *timed_out = 1 when that happened,
  * *seconds = the kernel's time.  Synchronises the device.                   */
 fsi_status fsi_wait_selftest(int device, int *timed_out, double *seconds);
+/* The same for the bounded wait between the CTAs of the Krylov solver's
+ * orthogonalisation, on the mesh's own solver workspace: of eight CTAs one leaves before
+ * it arrives, the others' waits give up after a short poll limit, the kernel
+ * returns, and the status that a step takes from it is FSI_ERR_TIMEOUT
+ * (*timed_out = 1).  Then all eight meet three times on the workspace as that
+ * status left it (*recovered = 1).  Synchronises the mesh's stream.          */
+fsi_status fsi_grid_wait_selftest(fsi_mesh *mesh, int *timed_out, int *recovered);
 
 /* ----------------------------------------------------------------------- */
 /* One implicit step: the reduced FSI system of Sec. 2.4.                    */

@@ -139,6 +139,7 @@ _SIGS = {
     "fsi_solid_positions": ([_VP, _VP, _VP], _INT),
     "fsi_mesh_set_coordinates": ([_VP, _VP], _INT),
     "fsi_wait_selftest": ([_INT, ctypes.POINTER(_INT), ctypes.POINTER(ctypes.c_double)], _INT),
+    "fsi_grid_wait_selftest": ([_VP, ctypes.POINTER(_INT), ctypes.POINTER(_INT)], _INT),
     "fsi_mesh_create_tet": ([_I64, _VP, _I64, _VP, ctypes.POINTER(fsi_physics), _INT, _VP,
                              ctypes.POINTER(_VP)], _INT),
     "fsi_tetmesh_create": ([_I64, _VP, _I64, _VP, ctypes.POINTER(fsi_physics), _INT, _VP,
@@ -457,6 +458,13 @@ def fsi_wait_selftest(device=0):
     sec = ctypes.c_double(0.0)
     _check(lib().fsi_wait_selftest(device, ctypes.byref(t), ctypes.byref(sec)))
     return bool(t.value), sec.value
+
+
+def fsi_grid_wait_selftest(mesh: Mesh):
+    """(timed_out, recovered) of the wait between CTAs (see fsi.h)."""
+    t, r = _INT(0), _INT(0)
+    _check(lib().fsi_grid_wait_selftest(mesh.handle, ctypes.byref(t), ctypes.byref(r)))
+    return bool(t.value), bool(r.value)
 
 
 def fsi_measure_fma_peak(device, prec):

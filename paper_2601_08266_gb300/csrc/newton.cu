@@ -838,7 +838,8 @@ template <typename T> struct OrthoArgs {
 // The wait is bounded: when it runs out *err is set, later waits are skipped and the
 // kernel ends with meaningless results.
 template <typename F>
-__device__ __forceinline__ void grid_step(unsigned *bar, double *err, int &last_or_bad, F fin)
+__device__ __forceinline__ void grid_step(unsigned *bar, double *err, int &last_or_bad, F fin,
+                                          unsigned limit = kOrthoPolls)
 {
     __syncthreads();
     unsigned gen = 0;
@@ -863,7 +864,7 @@ __device__ __forceinline__ void grid_step(unsigned *bar, double *err, int &last_
     } else if (threadIdx.x == 0 && !bad) {
         unsigned polls = 0;
         while (*(volatile unsigned *)(bar + 1) == gen)
-            if (++polls == kOrthoPolls) {
+            if (++polls == limit) {
                 *err = 1.0;
                 last_or_bad = 2;
                 break;
@@ -1006,6 +1007,18 @@ __global__ void __launch_bounds__(kOrthoThreads, 2) ortho_kernel(const OrthoArgs
 #pragma unroll
     for (int q = 0; q < R; ++q)
         if (i + q * NT < P.n) scale_split_node<T>(i + q * NT, w[q], den, P.Vnew, P.inv, P.z, P.bp);
+}
+
+// grid_step by itself: `steps` meetings, each counted by the last CTA; the CTA
+// `absent` (if any) leaves before the first one, and the others' waits run out
+__global__ void grid_wait_kernel(unsigned *bar, double *err, int steps, int absent, unsigned limit,
+                                 double *count)
+{
+    __shared__ int state;
+    if ((int)blockIdx.x == absent) return;
+    if (threadIdx.x == 0) state = 0;
+    for (int k = 0; k < steps; ++k)
+        grid_step(bar, err, state, [&]() { if (threadIdx.x == 0) *count += 1.0; }, limit);
 }
 
 // z_p = V-cycle result / sigma, or z_p = v_p on Dirichlet pressure rows
@@ -1487,6 +1500,16 @@ bool ortho_launch(fsi_mesh *mesh, int cnt, const T *V, int64_t ld, double *flag,
     return true;
 }
 
+// After the column (W.hcol) is in W.hhost: did a wait between CTAs run out?  The
+// arrivals and the tickets are then cleared for the next call.
+fsi_status wait_status(fsi_mesh *mesh, int restart)
+{
+    Work &W = mesh->newton->w;
+    if (W.hhost[restart + 3] == 0.0) return FSI_OK;
+    FSI_CUDA(cudaMemsetAsync(W.ticket, 0, 4 * sizeof(unsigned), mesh->stream), "memset");
+    return set_error(FSI_ERR_TIMEOUT, "GMRES: a wait between CTAs ran out");
+}
+
 template <typename T> fsi_status norm2(fsi_mesh *mesh, const T *x, double *dev_out)
 {
     return multi_dot<T>(mesh, 1, x, 0, x, dev_out, 1);
@@ -1610,10 +1633,7 @@ fsi_status gmres(fsi_mesh *mesh, const fsi_step_state *st, int restart, int max_
                                      cudaMemcpyDeviceToHost, s),
                      "memcpy");
             FSI_CUDA(cudaStreamSynchronize(s), "GMRES sync");
-            if (W.hhost[restart + 3] != 0.0) {
-                cudaMemsetAsync(W.ticket, 0, 4 * sizeof(unsigned), s);
-                return set_error(FSI_ERR_TIMEOUT, "GMRES: a wait between CTAs ran out");
-            }
+            FSI_TRY(wait_status(mesh, restart));
             if (W.hhost[restart + 2] != 0.0) ++W.reorth;
             ++its;
             double *h = &H[(size_t)j * (restart + 1)];
@@ -1825,6 +1845,42 @@ fsi_status fsi_coupled_jacobian_apply(fsi_mesh *mesh, fsi_prec prec, const fsi_s
     }
     FSI_TRY(prepare_linearisation<float>(mesh, st));
     return coupled_jacobian_impl<float>(mesh, st, (const float *)x, (float *)Jx);
+}
+
+fsi_status fsi_grid_wait_selftest(fsi_mesh *mesh, int *timed_out, int *recovered)
+{
+    FSI_TRY(validate_mesh(mesh));
+    if (!timed_out || !recovered)
+        return set_error(FSI_ERR_ARG, "fsi_grid_wait_selftest: NULL output");
+    FSI_DEVICE(mesh->device);
+    FSI_TRY(ensure_work(mesh, 0, 1));
+    Work &W = mesh->newton->w;
+    cudaStream_t s = mesh->stream;
+    const int restart = W.restart, ctas = 8;
+    int steps = 3;
+    unsigned *bar = W.ticket + 2, limit = 1u << 16;  // some tens of milliseconds
+    double *count = W.hcol, *err = W.hcol + restart + 3;
+    auto run = [&](int absent, double *meetings) -> fsi_status {
+        FSI_CUDA(cudaMemsetAsync(W.hcol, 0, (restart + 4) * sizeof(double), s), "memset");
+        void *args[] = {&bar, &err, &steps, &absent, &limit, &count};
+        FSI_CUDA(cudaLaunchCooperativeKernel((const void *)grid_wait_kernel, dim3(ctas),
+                                             dim3(kOrthoThreads), args, 0, s),
+                 "grid wait self-test");
+        FSI_CUDA(cudaMemcpyAsync(W.hhost, W.hcol, (restart + 4) * sizeof(double),
+                                 cudaMemcpyDeviceToHost, s),
+                 "memcpy");
+        FSI_CUDA(cudaStreamSynchronize(s), "sync");
+        *meetings = W.hhost[0];
+        return wait_status(mesh, restart);
+    };
+    double meetings = 0.0;
+    fsi_status st = run(3, &meetings);
+    if (st != FSI_OK && st != FSI_ERR_TIMEOUT) return st;
+    *timed_out = st == FSI_ERR_TIMEOUT && meetings == 0.0;
+    st = run(-1, &meetings);
+    if (st != FSI_OK && st != FSI_ERR_TIMEOUT) return st;
+    *recovered = st == FSI_OK && meetings == steps;
+    return FSI_OK;
 }
 
 fsi_status fsi_block_diagonal(fsi_mesh *mesh, fsi_prec prec, const fsi_step_state *st,
