@@ -877,7 +877,8 @@ __device__ __forceinline__ void grid_step(unsigned *bar, double *err, int &last_
 template <typename T>
 __global__ void __launch_bounds__(kOrthoThreads, 2) ortho_kernel(const OrthoArgs<T> P)
 {
-    chain_trigger();
+    // (no chain_trigger: a copy to the host follows, and a chained kernel's CTAs would
+    // only take places from the ones that meet here)
     constexpr int G = kOrthoMax, R = kOrthoRec<T>, NT = kOrthoThreads, NW = NT / 32, Q = (G + NW) / NW;
     using Acc = typename DotAcc<T>::type;
     __shared__ double red[G + 1][NW];
