@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(1024) batch_dense_sort_kernel(const DlmDesc<T>
     extern __shared__ int32_t sort_sh[];
     __shared__ int listed[1024];
     // the instances' lists read as one: CTA b takes entries b, b + grid, ...; their
-    // lengths together (one dependent read after the other, 64 instances took most of
+    // lengths together (one dependent read after the other, 64 instances took 21 of
     // the kernel's 61 us)
     int64_t g = blockIdx.x, base = 0;
     for (int i0 = 0; i0 < count; i0 += 1024) {

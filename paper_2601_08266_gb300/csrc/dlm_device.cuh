@@ -105,8 +105,8 @@ __device__ __forceinline__ double grid_coord(double X, double x0, double h, doub
 }
 
 // min(floor(t), N - 1) and 2 (t - that) - 1 for 0 <= t <= N, else false.  FP64
-// operations only where a value is rounded (64 instances with 5 M points, 11 an axis:
-// 296 us; 8: 260 us): the comparisons are on the bit patterns (NaN and negative
+// operations only where a value is rounded (64 instances with 3.9 M points, 11 an
+// axis: 296 us; 8: 260 us): the comparisons are on the bit patterns (NaN and negative
 // values are above N's as unsigned numbers; -0 is inside), floor(t) and the
 // element come from t's significand
 __device__ __forceinline__ bool cell_of(double t, long long nmax_bits, int N, int &e, double &xi)

@@ -125,7 +125,7 @@ __global__ void colsum_partial_kernel(int64_t M, ColSums c, float *part)
 
 // bias gradients from the slices (CTAs 1 ..), loss from its nb partial sums
 // (CTA 0: 256 threads, a fixed tree)
-__global__ void grad_final_kernel(ColSums c, int slices, const float *part, int nb,
+__global__ void grad_final_kernel(ColSums c, const float *part, int nb,
                                   const double *partial, float *loss)
 {
     chain_wait(part, partial, loss);
@@ -150,7 +150,6 @@ __global__ void grad_final_kernel(ColSums c, int slices, const float *part, int 
     float s = 0.f;
 #pragma unroll
     for (int r = 0; r < kColSlices; ++r) s += part[(int64_t)r * c.cols + k];
-    (void)slices;
     c.db[q][k - c.col0[q]] = s;
 }
 
@@ -508,8 +507,8 @@ fsi_status fsi_mlp_loss_grad(fsi_mlp *h, const float *params, const float *X, co
                        2 * NH + NO};
     float *part = h->gemm_work;  // the split-K workspace, free again in stream order
     launch_chain(colsum_partial_kernel, dim3(c.cta0[3], kColSlices), 256, 0, s, B, c, part);
-    launch_chain(grad_final_kernel, 1 + (c.cols + 255) / 256, 256, 0, s, c, kColSlices, part, nb,
-                                                              h->loss_partial, loss);
+    launch_chain(grad_final_kernel, 1 + (c.cols + 255) / 256, 256, 0, s, c, part, nb,
+                 h->loss_partial, loss);
     return check_launch("bias gradients");
 }
 

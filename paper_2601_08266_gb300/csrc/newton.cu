@@ -1056,10 +1056,10 @@ struct Work {
                                             // then arrivals and generation of ortho_kernel
     double *hhost = nullptr;                // pinned
     int precond = 0;                        // 0 block-Jacobi, 1 Schur (pmg.cu)
+    void *ftmp = nullptr;                   // [n][4]: the point masses' part of the diagonal blocks
     // the point-mass coupling of the Jacobian apply runs on a side stream
-    // while the VMS Jacobian runs on the mesh's stream; its spread goes to
-    // ftmp [n][4] (components 0..2), added to Jx after the join
-    void *ftmp = nullptr;
+    // while the VMS Jacobian runs on the mesh's stream; its corner forces (in the mesh's
+    // spreading scratch) are added to Jx after the join
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     int64_t reorth = 0;                     // second Gram-Schmidt passes taken

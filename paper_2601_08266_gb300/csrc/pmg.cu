@@ -31,8 +31,10 @@
 //              [hi/30, hi].
 //
 // The V-cycle is a fixed linear operator (symmetric), so it can precondition
-// plain GMRES.  Every kernel is one thread per node, deterministic; FP64 or
-// FP32 arithmetic follows the caller's precision.
+// plain GMRES.  The stencil and transfer kernels march up columns of nodes, a thread
+// or lane each; the FP32 levels of at most 17^3 nodes run as one cluster of CTAs
+// (coarse_cycle_kernel); the rest is a thread per node.  Deterministic; FP64 or FP32
+// arithmetic follows the caller's precision.
 #include <algorithm>
 #include <cmath>
 #include <cooperative_groups.h>
