@@ -49,20 +49,30 @@ N_GRID = 64
 M_POINTS = 200_000
 SEED = 2026
 # Kernel launches per step issued by the library (stage 1, residual + Jacobian
-# fused 2, locate 1 + scan 3 + scatter 1 + sort 1, interp 1, spread 2).
+# fused 2, locate 1 + scan 2 + scatter 1 + rank 1 + dense cells 1, interp 1, spread 2).
 LAUNCHES_PER_STEP = 12
 # dram__bytes_read.sum + dram__bytes_write.sum of one fused native FP64
-# residual + Jacobian launch on the 64^3 workload, per brick schedule the
-# autotuner picks (4x4x4 bricks, 128 threads: brick 26.43 + 0.23 MB, gather
-# 32.79 + 0 MB; 8x4x2, 128 threads: brick 26.43 + 0.40 MB, gather 35.41 +
-# 0.004 MB), from ncu captures of the current kernels with a cache flush
-# between the two (profiles/vms_fused_f64_64cubed_ncu.md)
-TRAFFIC_FUSED_F64_64 = {(4, 4, 4, 128): 26_429_696 + 226_304 + 32_786_432 + 0,
-                        (8, 4, 2, 128): 26_429_952 + 403_712 + 35_407_616 + 4_096}
-# FP64 operations the fused FP64 brick kernel executes per element (ncu,
-# same capture: DFMA 1,808 (x2), DMUL 1,232, DADD 950): context for the
-# roofline, whose achieved rate counts the oracle's operations
-KERNEL_FP64_FLOPS_PER_ELEM = 2 * 1808 + 1232 + 950
+# residual + Jacobian launch on the 64^3 workload, per brick schedule (the first is
+# the library's default there): brick kernel, then gather, from ncu captures with
+# cold caches (profiles/vms_operators_marching_ncu.md)
+TRAFFIC_FUSED_F64_64 = {
+    (8, 4, 4, 128): 26_458_880 + 479_232 + 23_997_952 + 8_704,
+    (4, 4, 8, 64): 26_456_064 + 1_173_504 + 29_122_048 + 6_144,
+    (4, 4, 4, 64): 26_477_568 + 1_577_216 + 32_397_312 + 36_352,
+    (8, 4, 2, 128): 26_456_576 + 989_952 + 31_662_080 + 41_472,
+    (8, 2, 4, 64): 26_456_576 + 887_040 + 31_663_872 + 14_080,
+    (4, 2, 4, 32): 26_473_216 + 2_480_640 + 39_081_472 + 110_848,
+    (8, 8, 4, 128): 26_456_320 + 313_088 + 20_226_816 + 768,
+}
+
+
+def kernel_fp64_flops_per_elem(layers):
+    """FP64 operations the fused FP64 brick kernel executes per element in bricks of
+    `layers` element layers (ncu, 64^3: DFMA x 2 + DMUL + DADD are 1,590, 603, 790 with 4
+    layers and 1,660, 662, 840 with 2, so 1,520, 544, 740 a layer and 280, 236, 200 a
+    brick column): context for the roofline, whose achieved rate counts the oracle's
+    operations."""
+    return (2 * 1520 + 544 + 740) + (2 * 280 + 236 + 200) / layers
 
 
 def dist_env():
@@ -274,7 +284,7 @@ def run_ours(args):
         for op, name in ((0, "residual"), (1, "jacobian"), (2, "vms")):
             key = f"{name}_{tag}"
             if args.no_autotune:
-                schedule[key] = {"brick": [8, 4, 4] if op == 2 else [8, 8, 4], "threads": 256}
+                schedule[key] = {"brick": None}  # the library's rule on the grid's size
             else:
                 t = fsi.fsi_mesh_autotune(mesh, op, prec, reps=3 if tag == "f64" else 5)
                 schedule[key] = {"brick": list(t["brick"]), "threads": t["threads"],
@@ -565,8 +575,12 @@ def finish(args, W, ws, rank, local, mesh, ms64, per64, ms32, per32, ops, ops32,
     achieved = flops_elem["fused"] * E / (vms_ms * 1e-3)
     # DRAM bytes of one fused FP64 launch (brick + gather kernels), from an
     # ncu capture of this workload; only meaningful for the 64^3 grid
-    vms_sched = tuple(schedule["vms_f64"]["brick"]) + (schedule["vms_f64"]["threads"],)
+    vms_sched = schedule["vms_f64"]
+    vms_sched = tuple(vms_sched["brick"]) + (vms_sched["threads"],) if vms_sched["brick"] else None
+    if N == N_GRID and vms_sched is None:
+        vms_sched = next(iter(TRAFFIC_FUSED_F64_64))
     traffic = TRAFFIC_FUSED_F64_64.get(vms_sched) if N == N_GRID else None
+    kernel_flops = kernel_fp64_flops_per_elem(vms_sched[2]) if vms_sched else None
     peaks = measured_peaks()
     hbm = peaks.get("hbm_gbs", 6800.0)
 
@@ -668,11 +682,12 @@ def finish(args, W, ws, rank, local, mesh, ms64, per64, ms32, per32, ops, ops32,
                                      "kernel executes fewer operations than this count",
                      "peak_source": "FP64 FMA rate probed in this run (fsi_measure_fma_peak; "
                                     "MEASURED_PEAKS.json has no FP64 figure)",
-                     "kernel_flops_per_element": KERNEL_FP64_FLOPS_PER_ELEM,
-                     "kernel_flop_frac": KERNEL_FP64_FLOPS_PER_ELEM * E / (vms_ms * 1e-3) / fma64,
+                     "kernel_flops_per_element": kernel_flops,
+                     "kernel_flop_frac": (kernel_flops * E / (vms_ms * 1e-3) / fma64
+                                          if kernel_flops else None),
                      "kernel_flops_source": "ncu FP64 instruction counts of the fused brick kernel "
-                                            "at 64^3 (DFMA x 2 + DMUL + DADD); its FP64 pipe is "
-                                            "85 % active"},
+                                            "at 64^3 (DFMA x 2 + DMUL + DADD, by the bricks' "
+                                            "layers); its FP64 pipe is 86 % active"},
         "schedule": schedule,
         "step_df64": {
             "ms": native[0], "gdof_s": gdofs(native[0]),
@@ -1587,7 +1602,7 @@ def mlp_section(args, dev, stream, W):
 def profile_case(args):
     """Small fixed cases for ncu captures (nothing is timed): 'vms_f64' runs the
     fused FP64 residual + Jacobian pass twice on the --grid grid with the
-    --profile-brick schedule (default 4x4x4 bricks of 128 threads); 'vms_f32' runs the FP32 Jacobian apply twice on
+    --profile-brick schedule (default: the library's at 64^3); 'vms_f32' runs the FP32 Jacobian apply twice on
     the --grid grid with the default schedule; 'dlm' runs location with the cell table, and FP32
     and double-float interpolation and spreading, twice, on the --grid grid
     with --points leaflet points; 'blas1' runs the Krylov multi-dot and
@@ -1700,7 +1715,7 @@ def main():
     ap.add_argument("--batch-count", type=int, default=64)
     ap.add_argument("--batch-reps", type=int, default=3)
     ap.add_argument("--batch-tune-f64", action="store_true")
-    ap.add_argument("--profile-brick", default="4,4,4,128",
+    ap.add_argument("--profile-brick", default="8,4,4,128",
                     help="brick schedule bx,by,bz,threads of the vms_f64 profile case")
     ap.add_argument("--profile-case", choices=["vms_f64", "vms_f32", "dlm", "blas1", "pmg"],
                     default=None,
