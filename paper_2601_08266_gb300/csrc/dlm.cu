@@ -786,6 +786,19 @@ __global__ void spread_cells_kernel(int64_t E, const typename StorageOf<T>::type
         spread_cells_segment<T, SQ>(E, c0, xi, start, perm, lam, w, S, dsq);
 }
 
+// CTAs of the cell pass: up to 64 per SM, each striding over segments.  A grid of many
+// more, one CTA per few segments, is only CTAs that find nothing where few cells hold
+// points (128^3, FP32, 100 points: 256 CTAs an SM 55 us, 64 31 us; 1 M points 62 and
+// 51 us).  In FP64, whose occupied segments are long work, it evens out that work once
+// the points fill them: from a point per segment on (128^3, 1 M points: 64 225 us, 256
+// 208 us; 300,000: 123 and 119 us; 60,000: 80 us either way; 5,000: 60 and 66 us).
+template <typename T> int spread_cells_grid(int64_t E, int64_t m)
+{
+    const bool many = std::is_same<T, double>::value && m >= E / kSpreadSeg;
+    return blocks_for((E + kSpreadSeg - 1) / kSpreadSeg * 32, kSpreadThreads<T>,
+                      sm_count() * (many ? 256 : 64));
+}
+
 // Spreading, pass 2: every node sums the corner sums of its occupied cells.
 // 3D launch: x over the row's nodes, y over j, z (strided) over k: no index
 // division.
@@ -945,13 +958,11 @@ template <typename T>
 fsi_status spread_mass_diag(fsi_mesh *mesh, int64_t m, const T *xi, const int32_t *cell_start,
                             const int32_t *perm, const T *w, double dsq, T *F)
 {
-    (void)m;  // the cell table lists the points
     FSI_DEVICE(mesh->device);
     const GridArgs g = grid_args(mesh);
     const int64_t E = mesh->n_elems;
     FSI_TRY(ensure_spread_scratch(mesh, (size_t)E * 24 * sizeof(T)));
-    const int cgrid = blocks_for((E + kSpreadSeg - 1) / kSpreadSeg * 32, kSpreadThreads<T>, sm_count() * 256);
-    launch_chain(spread_cells_kernel<T, true>, cgrid, kSpreadThreads<T>, 0, mesh->stream, 
+    launch_chain(spread_cells_kernel<T, true>, spread_cells_grid<T>(E, m), kSpreadThreads<T>, 0, mesh->stream, 
         E, xi, cell_start, perm, nullptr, w, (T *)mesh->spread_scratch, (T)dsq);
     FSI_TRY(check_launch("spread cells kernel"));
     const dim3 nblock(32, 8), ngrid = node_grid(g);
@@ -1286,29 +1297,26 @@ fsi_status fsi_dlm_spread(fsi_mesh *mesh, fsi_prec prec, int64_t m, const int32_
     const size_t esz = prec == FSI_F32 ? sizeof(float) : sizeof(double);
     FSI_TRY(ensure_spread_scratch(mesh, (size_t)mesh->n_elems * 24 * esz));
     const int64_t E = mesh->n_elems;
-    auto cgrid = [&](int threads) {
-        return blocks_for((E + kSpreadSeg - 1) / kSpreadSeg * 32, threads, sm_count() * 256);
-    };
     // nodes: 32 x 8 threads per CTA over (i, j), one grid layer per k
     const dim3 nblock(32, 8), ngrid = node_grid(g);
     if ((g.Ny + 8) / 8 > 65535)
         return set_error(FSI_ERR_ARG, "fsi_dlm_spread: more than 524,280 nodes along y");
     if (prec == FSI_F64) {
-        launch_chain(spread_cells_kernel<double>, cgrid(kSpreadThreads<double>), kSpreadThreads<double>, 0, mesh->stream, 
+        launch_chain(spread_cells_kernel<double>, spread_cells_grid<double>(E, m), kSpreadThreads<double>, 0, mesh->stream, 
             E, (const double *)xi, cell_start, perm, (const double *)lam, (const double *)w,
             (double *)mesh->spread_scratch, 0.0);
         FSI_TRY(check_launch("spread cells kernel"));
         launch_chain(spread_nodes_kernel<double>, ngrid, nblock, 0, mesh->stream, 
             g, cell_start, (const double *)mesh->spread_scratch, (double *)F, accumulate);
     } else if (prec == FSI_DF64) {
-        launch_chain(spread_cells_kernel<df64>, cgrid(kSpreadThreads<df64>), kSpreadThreads<df64>, 0, mesh->stream, 
+        launch_chain(spread_cells_kernel<df64>, spread_cells_grid<df64>(E, m), kSpreadThreads<df64>, 0, mesh->stream, 
             E, (const double *)xi, cell_start, perm, (const double *)lam, (const double *)w,
             (df64 *)mesh->spread_scratch, df64(0));
         FSI_TRY(check_launch("spread cells kernel"));
         launch_chain(spread_nodes_kernel<df64>, ngrid, nblock, 0, mesh->stream, 
             g, cell_start, (const df64 *)mesh->spread_scratch, (double *)F, accumulate);
     } else {
-        launch_chain(spread_cells_kernel<float>, cgrid(kSpreadThreads<float>), kSpreadThreads<float>, 0, mesh->stream, 
+        launch_chain(spread_cells_kernel<float>, spread_cells_grid<float>(E, m), kSpreadThreads<float>, 0, mesh->stream, 
             E, (const float *)xi, cell_start, perm, (const float *)lam, (const float *)w,
             (float *)mesh->spread_scratch, 0.0f);
         FSI_TRY(check_launch("spread cells kernel"));
