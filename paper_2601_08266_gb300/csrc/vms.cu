@@ -36,12 +36,14 @@ using namespace vmsd;
 // registers; 3 or 5 were within 1 %).  FP64: 2, since 8 warps keep its pipe busy
 // (85 % active) and no value has to be spilled.  Double-float: 3 (168 registers),
 // both operators at once 2 (254; at 3 it spills and takes 420 instead of 406 us at
-// 64^3).  On mapped grids FP32 spills a little at 4 and is still faster than at 3.
-template <typename T, bool FUSED>
-constexpr int kBrickCtas = sizeof(T) == 4 ? 4 : (std::is_same<T, double>::value || FUSED ? 2 : 3);
+// 64^3).  On mapped grids FP32 spills a little at 4 and is still faster than at 3, but
+// for both operators at once: 3 (at 4 it spills 628 bytes; 128^3 812 -> 555 us).
+template <typename T, bool FUSED, bool MAPPED>
+constexpr int kBrickCtas = sizeof(T) == 4 ? (FUSED && MAPPED ? 3 : 4)
+                                          : (std::is_same<T, double>::value || FUSED ? 2 : 3);
 
 template <typename T, bool JAC, bool MAPPED, bool FUSED = false>
-__global__ void __launch_bounds__(kBrickThreads, (kBrickCtas<T, FUSED>)) vms_brick_kernel(const VmsArgs<T> P)
+__global__ void __launch_bounds__(kBrickThreads, (kBrickCtas<T, FUSED, MAPPED>)) vms_brick_kernel(const VmsArgs<T> P)
 {
     if (P.nbx * P.nby * P.nbz > 1) chain_trigger();  // the gather follows; else any kernel
     extern __shared__ __align__(32) unsigned char smem_raw[];
