@@ -294,8 +294,11 @@ __global__ void __launch_bounds__(32 * kMarchWarps) march_kernel(LevelArgs<T> L,
 #pragma unroll
     for (int r = 0; r < R; ++r) acc[r] = PBk[r] = vk[r] = dk[r] = bk[r] = T(0);
     Raw nx;
-    // (a cycle's last kernel lets the next start only when those before it are done)
-    const bool last = M.x_final || M.z4;
+    // A call's last kernel (a smoothing's, or y = A x for a caller) lets the next start
+    // only when those before it are done: that one is the caller's choice, and
+    // applications in a row that were all let in at once shared the SMs unevenly (FP64,
+    // 25^3 nodes 12.8 -> 8.4 us, 65^3 44.9 -> 38.3 us).
+    const bool last = M.x_final || M.z4 || (MODE == kMarchApply && !M.b);
     if (!last) chain_trigger();
     chain_wait(M.x, M.d, M.b, M.y, M.x_next, M.d_next, M.x_final, M.z4, M.v4, M.m4);
     if (last) chain_trigger();
