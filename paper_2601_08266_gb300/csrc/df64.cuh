@@ -41,6 +41,18 @@ __device__ __forceinline__ float float_of(double d)
     return r;
 }
 
+// df_split where a conversion is needed (zero, the ends of the float range)
+__device__ __forceinline__ df64 df_split_rare(double d)
+{
+    const unsigned hw = (unsigned)__double2hiint(d), lw = (unsigned)__double2loint(d);
+    const unsigned e = (hw >> 20) & 0x7FFu;
+    if (((hw << 1) | lw) == 0u) return df64(__uint_as_float(hw), 0.0f);
+    const float hi = float_of(d);
+    if (e < 897u || e > 1150u) return df64(hi, 0.0f);
+    return df64(hi, float_of(d - (double)hi));
+}
+static __device__ __noinline__ df64 df_split_rare_ool(double d) { return df_split_rare(d); }
+
 // Split of a double into hi + lo without an FP64 instruction: hi keeps the sign,
 // the exponent and the leading 24 significant bits (truncated), lo is the
 // remaining 29 bits rounded to a float (an integer, converted and scaled by a
@@ -48,8 +60,12 @@ __device__ __forceinline__ float float_of(double d)
 // takes the place of finding and shifting the leading bit, half of the split's
 // instructions: four-lane tetrahedral operators at 279,936 elements 136/193 ->
 // 126/181 us, a step on a ragged 47 x 61 x 38 grid 307 -> 300 us.  Zero and
-// magnitudes at the ends of the float range take the float conversion path.
-__device__ __forceinline__ df64 df_split(double d)
+// magnitudes at the ends of the float range take the float conversion path, with
+// RARE_CALL out of line: where a kernel splits some thirty values in a row (node
+// records) the inlined rare branches cost registers and instruction cache (location on
+// a mapped grid, 300,000 points: 331 -> 324 us; double-float operators 1 to 4 %); the
+// coupling's few values lose 2 % by it.
+template <bool RARE_CALL = false> __device__ __forceinline__ df64 df_split(double d)
 {
     const unsigned hw = (unsigned)__double2hiint(d), lw = (unsigned)__double2loint(d);
     const unsigned e = (hw >> 20) & 0x7FFu;
@@ -59,10 +75,8 @@ __device__ __forceinline__ df64 df_split(double d)
         // d - hi = (low 29 bits) * 2^(e - 1075)
         return df64(hi, __int2float_rn((int)(lw & 0x1FFFFFFFu)) * __uint_as_float(sign | ((e - 948u) << 23)));
     }
-    if (((hw << 1) | lw) == 0u) return df64(__uint_as_float(hw), 0.0f);
-    const float hi = float_of(d);
-    if (e < 897u || e > 1150u) return df64(hi, 0.0f);
-    return df64(hi, float_of(d - (double)hi));
+    if constexpr (RARE_CALL) return df_split_rare_ool(d);
+    else return df_split_rare(d);
 }
 
 // (float)d by integer operations (round to nearest, ties to even): the FP64 unit

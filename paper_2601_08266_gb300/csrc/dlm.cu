@@ -220,11 +220,11 @@ __device__ bool newton_df(const HexNodes &H, const double X[3], double (&xi)[3])
 #pragma unroll
     for (int a = 0; a < 8; ++a)
 #pragma unroll
-        for (int i = 0; i < 3; ++i) xa[a][i] = df_split(H.d[a][i]);
+        for (int i = 0; i < 3; ++i) xa[a][i] = df_split<true>(H.d[a][i]);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        Y[i] = df_split(X[i] - H.o[i]);
-        q[i] = df_split(xi[i]);
+        Y[i] = df_split<true>(X[i] - H.o[i]);
+        q[i] = df_split<true>(xi[i]);
     }
     const df64 one(1), eighth(0.125f);
     float last = 1.0f;

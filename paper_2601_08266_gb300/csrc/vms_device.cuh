@@ -165,7 +165,9 @@ template <typename T>
 __device__ __forceinline__ vec4<T> load_c(const vec4<typename StorageOf<T>::type> *p)
 {
     const auto v = ld4(p);
-    return {to_c<T>(v.x), to_c<T>(v.y), to_c<T>(v.z), to_c<T>(v.w)};
+    if constexpr (std::is_same<T, df64>::value)
+        return {df_split<true>(v.x), df_split<true>(v.y), df_split<true>(v.z), df_split<true>(v.w)};
+    else return {to_c<T>(v.x), to_c<T>(v.y), to_c<T>(v.z), to_c<T>(v.w)};
 }
 
 template <typename T> struct VG {
