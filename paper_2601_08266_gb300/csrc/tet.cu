@@ -1562,7 +1562,9 @@ fsi_status fsi_tet_locate(fsi_tetmesh *m, int64_t np, const double *P, int32_t *
         }
         int npw = 4;
         while (npw < 16 && np > (int64_t)npw * 16 * sm_count()) npw *= 2;
-        tet_locate_kernel<<<grid_for((np + npw - 1) / npw * 32, kLocThreads), kLocThreads, 0, s>>>(
+        // (16 CTAs an SM, warps striding: 300,000 points in 24,576 elements 201 us with 32, 188)
+        tet_locate_kernel<<<grid_for((np + npw - 1) / npw * 32, kLocThreads, sm_count() * 16),
+                            kLocThreads, 0, s>>>(
             np, B, m->X64, m->X32, m->tets, m->bucket_start, m->bucket_tets, P, npw, elem, lam,
             table ? m->fill : nullptr, m->nout);
         FSI_TRY(check_launch("tet locate kernel"));
