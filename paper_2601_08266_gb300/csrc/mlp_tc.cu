@@ -10,7 +10,7 @@
 //
 //   features   the 112 features of each node (27-node stencil of V_n
 //              velocity and y_n pressure, in FP32 from
-//              node_features_kernel; the extrapolant 2 d1 - d2), normalised and rounded to BF16, into the A tile X [128 x 112].
+//              prepare_kernel; the extrapolant 2 d1 - d2), normalised and rounded to BF16, into the A tile X [128 x 112].
 //              They are gathered one tile ahead, during the previous tile's
 //              MMAs and epilogues, and wait packed in 16 registers per thread
 //              (shared memory has no room for a second A tile);
@@ -30,7 +30,7 @@
 // Bound: the phases of a tile follow one another, so their latencies and instructions
 // add up.  2,146,689 nodes (129^3): 1.29 ms with every row converting its 27 nodes on
 // the FP64 unit when it needs them; 1.12 ms gathered a tile ahead and converted on the
-// integer pipe; 0.75 ms with each node converted once (node_features_kernel, 25 us
+// integer pipe; 0.75 ms with each node converted once (prepare_kernel, 25 us
 // of that) and no FP64 operation left in a tile but the four of the result (the unit
 // does two per SM and clock: 25 a thread took 3 of a tile's 9 us), layer 3 on
 // paired FMAs with its biases read four at a time.
@@ -90,24 +90,24 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b
 // W1 [NI][NH] and W2 [NH][NH] (input-major, as trained) -> B operands
 // [N = out][K = in] BF16 in the canonical layout: W1 (K = 112), then the two
 // K-halves of W2 (K = 0..127, 128..255)
-__global__ void pack_weights_kernel(const float *P, uint8_t *packed)
+constexpr int kPrepThreads = 256;
+constexpr int kPackCtas = NH * (NI + NH) / kPrepThreads;  // an entry per thread
+static_assert(kPackCtas * kPrepThreads == NH * (NI + NH), "every entry");
+__device__ __forceinline__ void pack_weight(int e, const float *P, uint8_t *packed)
 {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)NH * (NI + NH);
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int n = (int)(e % NH);
-        const int k = (int)(e / NH);
-        __nv_bfloat16 v;
-        uint32_t off;
-        if (k < NI) {
-            v = __float2bfloat16_rn(P[OFF_W1 + (int64_t)k * NH + n]);
-            off = OFF_SW1 + kmaj(n, k, KC1);
-        } else {
-            const int k2 = k - NI;
-            v = __float2bfloat16_rn(P[OFF_W2 + (int64_t)k2 * NH + n]);
-            off = (k2 < 128 ? OFF_SW2A : OFF_SW2B) + kmaj(n, k2 & 127, KC2);
-        }
-        *reinterpret_cast<__nv_bfloat16 *>(packed + off) = v;
+    const int n = e % NH;
+    const int k = e / NH;
+    __nv_bfloat16 v;
+    uint32_t off;
+    if (k < NI) {
+        v = __float2bfloat16_rn(P[OFF_W1 + (int64_t)k * NH + n]);
+        off = OFF_SW1 + kmaj(n, k, KC1);
+    } else {
+        const int k2 = k - NI;
+        v = __float2bfloat16_rn(P[OFF_W2 + (int64_t)k2 * NH + n]);
+        off = (k2 < 128 ? OFF_SW2A : OFF_SW2B) + kmaj(n, k2 & 127, KC2);
     }
+    *reinterpret_cast<__nv_bfloat16 *>(packed + off) = v;
 }
 
 struct TcArgs {
@@ -122,14 +122,19 @@ struct TcArgs {
     int *err;
 };
 
-// The stencil's inputs in FP32, each node converted once instead of by each of the
-// 27 rows that use it
-__global__ void __launch_bounds__(256) node_features_kernel(int64_t n, const double *__restrict__ Vn,
-                                                            const double *__restrict__ y,
-                                                            float4 *__restrict__ feat)
+// One launch before the network: the weights (the first kPackCtas CTAs), and the
+// stencil's inputs in FP32, each node converted once instead of by each of the 27
+// rows that use it.  (On a grid of 5^3 nodes a launch each made a prediction 22.6 us.)
+__global__ void __launch_bounds__(kPrepThreads)
+    prepare_kernel(const float *P, uint8_t *packed, int64_t n, const double *__restrict__ Vn,
+                   const double *__restrict__ y, float4 *__restrict__ feat)
 {
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n;
-         q += (int64_t)gridDim.x * blockDim.x) {
+    if (blockIdx.x < kPackCtas) {
+        pack_weight(blockIdx.x * kPrepThreads + threadIdx.x, P, packed);
+        return;
+    }
+    for (int64_t q = (blockIdx.x - kPackCtas) * (int64_t)kPrepThreads + threadIdx.x; q < n;
+         q += (int64_t)(gridDim.x - kPackCtas) * kPrepThreads) {
         const double2 v01 = __ldg(reinterpret_cast<const double2 *>(Vn + 4 * q));
         feat[q] = make_float4(round_to_float(v01.x), round_to_float(v01.y),
                               round_to_float(__ldg(Vn + 4 * q + 2)), round_to_float(__ldg(y + 4 * q + 3)));
@@ -501,10 +506,10 @@ fsi_status mlp_predict_tc(cudaStream_t s, int device, const fsi_grid &g, int64_t
         if (device >= 0 && device < 64) attr_set[device].store(true, std::memory_order_release);
     }
     const int sms = sm_count();
-    pack_weights_kernel<<<sm_count() * 4, 256, 0, s>>>(params, (uint8_t *)packed);
-    FSI_TRY(check_launch("pack weights"));
-    node_features_kernel<<<(int)std::min<int64_t>((n + 255) / 256, 16 * sms), 256, 0, s>>>(n, Vn, y, (float4 *)feat);
-    FSI_TRY(check_launch("node features"));
+    const int nodes = (int)std::min<int64_t>((n + kPrepThreads - 1) / kPrepThreads, 16 * sms);
+    prepare_kernel<<<kPackCtas + nodes, kPrepThreads, 0, s>>>(params, (uint8_t *)packed, n, Vn, y,
+                                                             (float4 *)feat);
+    FSI_TRY(check_launch("predictor inputs"));
     TcArgs a{g.N[0], g.N[1], g.N[2], n, params, (const uint8_t *)packed, in_mean, in_std,
              out_mean, out_std, (const float4 *)feat, y, d1, d2, y0, dev_err};
     const int64_t tiles = (n + TM - 1) / TM;
