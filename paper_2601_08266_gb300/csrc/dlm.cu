@@ -738,11 +738,15 @@ __global__ void __launch_bounds__(1024) dense_pairs_kernel(int64_t E, int64_t m,
 
 // --------------------------------------------------------------- interp / spread
 // FP32: two lanes per point (interp_point_pair; the loop bound is
-// warp-uniform); double-float and FP64: one lane per point
+// warp-uniform); double-float and FP64: one lane per point.  CTAs per SM: as the
+// registers fall, but five in double-float (its ordinary loads took 56 registers and a CTA
+// less: 128^3, 1 M random points 57.8 -> 53.7 us)
+template <typename T>
+constexpr int kInterpCtas = std::is_same<T, float>::value ? 6 : (std::is_same<T, double>::value ? 4 : 5);
 template <typename T, typename S = typename StorageOf<T>::type>
-__global__ void interp_kernel(int64_t m, GridArgs g, const int32_t *__restrict__ elem,
-                              const S *__restrict__ xi, const vec4<S> *__restrict__ U,
-                              S *__restrict__ u)
+__global__ void __launch_bounds__(256, kInterpCtas<T>)
+    interp_kernel(int64_t m, GridArgs g, const int32_t *__restrict__ elem, const S *__restrict__ xi,
+                  const vec4<S> *__restrict__ U, S *__restrict__ u)
 {
     chain_wait(elem, xi, U, u);
     if constexpr (std::is_same<T, float>::value) {
@@ -786,17 +790,17 @@ __global__ void spread_cells_kernel(int64_t E, const typename StorageOf<T>::type
         spread_cells_segment<T, SQ>(E, c0, xi, start, perm, lam, w, S, dsq);
 }
 
-// CTAs of the cell pass: up to 64 per SM, each striding over segments.  A grid of many
-// more, one CTA per few segments, is only CTAs that find nothing where few cells hold
-// points (128^3, FP32, 100 points: 256 CTAs an SM 55 us, 64 31 us; 1 M points 62 and
-// 51 us).  In FP64, whose occupied segments are long work, it evens out that work once
+// CTAs of the cell pass: up to 64 per SM (FP32, of twice the threads, 32), each striding
+// over segments.  A grid of many more, one CTA per few segments, is only CTAs that find
+// nothing where few cells hold points (128^3, FP32, 100 points: 256 CTAs an SM 55 us,
+// 32 31 us; 1 M points 62 and 51 us; 64^3, 5,000 points: 13.8 and 10 us).  In FP64, whose occupied segments are long work, it evens out that work once
 // the points fill them: from a point per segment on (128^3, 1 M points: 64 225 us, 256
 // 208 us; 300,000: 123 and 119 us; 60,000: 80 us either way; 5,000: 60 and 66 us).
 template <typename T> int spread_cells_grid(int64_t E, int64_t m)
 {
     const bool many = std::is_same<T, double>::value && m >= E / kSpreadSeg;
     return blocks_for((E + kSpreadSeg - 1) / kSpreadSeg * 32, kSpreadThreads<T>,
-                      sm_count() * (many ? 256 : 64));
+                      sm_count() * (many ? 256 : (sizeof(T) == 4 ? 32 : 64)));
 }
 
 // Spreading, pass 2: every node sums the corner sums of its occupied cells.

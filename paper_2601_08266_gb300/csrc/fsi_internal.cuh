@@ -126,10 +126,11 @@ template <> __device__ __forceinline__ vec4<double> ld4(const vec4<double> *p)
     return {a.x, a.y, b.x, b.y};
 }
 
-// The same by ordinary loads, for what an earlier kernel of a chain wrote.  As
+// The same by ordinary loads, for what an earlier kernel of a chain wrote.  In FP32 as
 // instructions of their own, which may be moved among the kernel's stores (in C++ they
-// stay in order with them: 128^3 step with 1 M points 400.5 -> 405.1 us), but not before
-// the chain_wait() that the pointer went through.
+// stay in order with them: 128^3 step with 1 M points 405.1 -> 400.5 us), but not before
+// the chain_wait() that the pointer went through.  (In FP64 moving them costs registers
+// and gains nothing.)
 __device__ __forceinline__ float4 ldg_chain(const float4 *p)
 {
     float4 v;
@@ -143,11 +144,9 @@ __device__ __forceinline__ vec4<float> ld4_chain(const vec4<float> *p)
 }
 __device__ __forceinline__ vec4<double> ld4_chain(const vec4<double> *p)
 {
-    vec4<double> v;
     const double2 *q = reinterpret_cast<const double2 *>(p);
-    asm("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(q));
-    asm("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.z), "=d"(v.w) : "l"(q + 1));
-    return v;
+    const double2 a = q[0], b = q[1];
+    return {a.x, a.y, b.x, b.y};
 }
 
 template <typename T> __device__ __forceinline__ void st4(vec4<T> *p, vec4<T> v) { *p = v; }
