@@ -649,8 +649,6 @@ __device__ __forceinline__ F face_project(F P1, F P2, F P3, F sx, F sy)
         return face_project_body(P1, P2, P3, sx, sy);
 }
 
-// z stage: the two Gauss points between the plane values lo and hi
-template <typename T> __device__ __forceinline__ typename PairOf<T>::type z_val(T lo, T hi)
 // (a, b, c) times a 3 x 3 matrix m (row-major), or m times it (RIGHT), in the physical
 // gradients and the projections of mapped grids: out of line for double-float pairs, as
 // face_ool (128^3, both operators at once 5,835 -> 4,745 us; inline the eight uses
@@ -684,6 +682,8 @@ __device__ __forceinline__ Row3<F> times3(F a, F b, F c, const F (&m)[9])
         return times3_body<RIGHT>(a, b, c, m);
 }
 
+// z stage: the two Gauss points between the plane values lo and hi
+template <typename T> __device__ __forceinline__ typename PairOf<T>::type z_val(T lo, T hi)
 {
     const T d = hi - lo;
     return PairOf<T>::pack(fma_t(cB2<T>(), d, lo), fma_t(cB1<T>(), d, lo));
