@@ -5,11 +5,11 @@
 // Location is closed-form on the uniform grid (integer work on the bits of
 // the coordinates when the spacings are powers of two; a bounded element
 // walk with Newton inversion on a mapped grid).  The cell table is a stable
-// counting sort: histogram (integer atomics, order-free), a single-pass
-// exclusive scan with decoupled look-back, a scatter that counts the
-// per-cell counters back down, and a per-cell sort of each cell's slice by
-// point index, which restores the stable order exactly (a warp rank sort up
-// to 128 points, a CTA bitonic network or a shell sort beyond).  Spreading
+// counting sort: histogram with arrival slots (one returning integer atomic a point), a
+// two-kernel exclusive scan, a scatter to the slots, and a rank pass that restores
+// the stable order by point index (a CTA bitonic network or a shell sort for cells of
+// more than 128 points); without point scratch the scatter counts the counters back down
+// and a warp sorts each segment's slices in place.  Spreading
 // is atomic-free in two passes:
 // per-cell corner sums (four lanes per cell of up to 128 points, the warp for
 // fuller cells, fixed transpose-reduce trees), then a node gather over the
